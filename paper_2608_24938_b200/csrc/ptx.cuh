@@ -282,4 +282,31 @@ __device__ __host__ constexpr uint32_t make_idesc_bf16(int M, int N) {
 
 }  // namespace ptx
 
+// ------------------------------------------------------------------ epilogue staging
+// An epilogue warp owns 32 accumulator rows, one per lane. Stored straight from registers, a 16-byte store instruction
+// touches 32 different rows: 32 cache lines in the SM's store path and 32 half-filled sectors on the way to L2. The warp
+// therefore passes 128 bytes of each row (64 bf16 or 32 fp32 columns) through 4 KB of shared memory, 16-byte chunks
+// XOR-swizzled by the row so that both directions are free of bank conflicts, and stores whole 128-byte lines, four rows
+// per instruction.
+constexpr int kStageOutBytes = 4096;  // per epilogue warp
+__device__ __forceinline__ void stage_put(unsigned char* buf, int lane, int chunk, const uint4& v) {
+    *reinterpret_cast<uint4*>(buf + lane * 128 + ((chunk ^ (lane & 7)) << 4)) = v;
+}
+// Rows with their bit in `valid` go to dst + row * row_bytes (row: this lane's target row); the lanes have written all
+// eight chunks. Warp-uniform call.
+__device__ __forceinline__ void stage_flush(const unsigned char* buf, int lane, unsigned valid, int row, char* dst,
+                                            size_t row_bytes) {
+    __syncwarp();
+    const int c = lane & 7;
+#pragma unroll
+    for (int it = 0; it < 8; ++it) {
+        const int r = it * 4 + (lane >> 3);
+        const int target = __shfl_sync(0xffffffffu, row, r);
+        if ((valid >> r) & 1u)
+            *reinterpret_cast<uint4*>(dst + (size_t)target * row_bytes + c * 16) =
+                *reinterpret_cast<const uint4*>(buf + r * 128 + ((c ^ (r & 7)) << 4));
+    }
+    __syncwarp();
+}
+
 }  // namespace exfold
