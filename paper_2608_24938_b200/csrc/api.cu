@@ -259,6 +259,80 @@ bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 
         if (e__ != cudaSuccess) return EXFOLD_ERR_CUDA;   \
     } while (0)
 
+// Row tiles of a grouped GEMM over `rows` sorted rows of G groups: on average half a tile per group is a ragged last one
+int64_t expected_tiles(int64_t rows, int G) { return rows / kTileM + G / 2; }
+
+// Whether the two GEMMs run their whole pairs of row tiles on CTA pairs (gemm_pair.cu: a third less operand traffic per
+// SM, a deeper ring) with the groups' odd last tiles beside them, or every tile on the one-CTA kernel. The pairs pay once
+// a group owns a tile or more on average (before, most tiles are odd ones, and the weights of a group with three tiles
+// are read by both passes) and the GEMMs are long enough for the second stream's fork and join: from ~400 k-blocks per
+// SM. Measured, pair / one-CTA time of the call: Qwen3 shape (K' = 4) 1024 tokens 206 / 168 us, 4096 328 / 300, 6144
+// 408 / 409, 8192 467 / 502; GLM shape 2048 tokens 1025 / 899 us, 4096 1229 / 1289; Mixtral shape (K' = 1) 512 tokens
+// 511 / 496 us, 1024 630 / 695, 4096 1277 / 1852; 64 experts of 1024 x 512, 8192 tokens 160 / 157 us. With few tiles in
+// all, the sizes of the last tiles decide (Mixtral shape, 17 tiles: 1179 / 1078 us): one-CTA below 24.
+bool use_pairs(int64_t rows, int G, int d, int I) {
+    const int64_t tiles = rows / kTileM;
+    const int64_t kblocks = (int64_t)((I + 127) / 128) * (d / kGemmBK) + (int64_t)((d + 255) / 256) * (I / kGemmBK);
+    return kGemmBK == 64 && tiles >= G && expected_tiles(rows, G) >= 24 && tiles * kblocks >= (int64_t)400 * sm_count();
+}
+
+// The two grouped GEMMs of bf16 expert rows (prefill, calibration): g = GEMM-1, g2 = GEMM-2 on `rows` sorted rows.
+// Without `pairs` every row tile runs on the one-CTA kernel. With it, whole pairs of row tiles run on CTA pairs on the
+// caller's stream and the groups' odd last tiles beside them on a second stream.
+int enqueue_expert_gemms(GroupedGemmParams& g, GroupedGemmParams& g2, int64_t rows, bool pairs, int shared_pairs,
+                         cudaStream_t s) {
+    const int G = g.G, nt1 = g.n_ntiles, nt2 = g2.n_ntiles, d = g.d, I = g.I;
+    if (!pairs) {
+        const int64_t max_tiles = rows / kTileM + G;
+        { ProfScope ps(3, s); EXFOLD_CUDA(launch_grouped_gemm1(g, (int)std::min<int64_t>(sm_count(), max_tiles * nt1), s)); }
+        { ProfScope ps(4, s); EXFOLD_CUDA(launch_grouped_gemm2(g2, (int)std::min<int64_t>(sm_count(), max_tiles * nt2), s)); }
+        return EXFOLD_OK;
+    }
+    // Both passes are launched over all SMs, the pair pass on the caller's stream and the odd-tile pass on a
+    // second one; on the device each keeps its share of the SM pairs (pair_pass_clusters of the actual tile
+    // counts) and its other CTAs leave at once, so the two grids settle side by side whatever the routing.
+    // Rows of whole tile pairs and rows of odd last tiles never meet before the combine step, so each pass
+    // of GEMM-2 follows the same pass of GEMM-1 on its own stream: caller's stream: GEMM-1 pairs -> GEMM-2
+    // pairs; side stream: GEMM-1 odd tiles -> GEMM-2 odd tiles; joined before the combine kernel (or the
+    // end of the call). With per-kernel timing on, and in calibration, whose fp32 outputs overwrite the rows that
+    // GEMM-1 reads, the streams also join between the two GEMMs.
+    const bool join_mid = g_prof.on || g2.o32 != nullptr;
+    const int sms = sm_count() & ~1;
+    ThreadDeviceState* sidep = side_stream();
+    if (!sidep) return EXFOLD_ERR_CUDA;
+    ThreadDeviceState& side = *sidep;
+    GroupedGemmParams go1 = g, go2 = g2;
+    go1.odd_only = go2.odd_only = 1;
+    // The odd-tile pass is launched with about twice the CTAs its expected share of the work needs (its share
+    // is decided on the device, where the tile counts are known): CTAs without work leave at once, but every
+    // one of them has to pass through one of the pass's few SMs first.
+    const double odd_est = std::max<double>(1.0, G / 2.0),
+                 pair_est = std::max<double>(1.0, (expected_tiles(rows, G) - G / 2.0) / 2.0);
+    const double q_est = sms * odd_est / (odd_est + 2 * 0.73 * pair_est);
+    const int odd_grid = std::min(sms, 2 * (int)std::ceil(q_est) + 8) & ~1;
+    const SideBySide sbs{nt1, d / kGemmBK, nt2, I / kGemmBK, sms / 2, odd_grid, shared_pairs};
+    g.sbs = g2.sbs = go1.sbs = go2.sbs = sbs;
+    SideJoin joiner{sidep, s};
+    EXFOLD_CUDA(cudaEventRecord(side.fork, s));
+    EXFOLD_CUDA(cudaStreamWaitEvent(side.side, side.fork, 0));
+    {
+        ProfScope ps(3, s);
+        { ProfScope pp(12, s); EXFOLD_CUDA(launch_grouped_gemm1_pair(g, sms, s)); }
+        EXFOLD_CUDA(launch_grouped_gemm1_odd(go1, odd_grid, side.side));
+        if (join_mid) {
+            EXFOLD_CUDA(cudaEventRecord(side.mid, side.side));
+            EXFOLD_CUDA(cudaEventRecord(side.fork, s));
+            EXFOLD_CUDA(cudaStreamWaitEvent(s, side.mid, 0));
+            EXFOLD_CUDA(cudaStreamWaitEvent(side.side, side.fork, 0));
+        }
+    }
+    ProfScope ps(4, s);
+    { ProfScope pp(13, s); EXFOLD_CUDA(launch_grouped_gemm2_pair(g2, sms, s)); }
+    EXFOLD_CUDA(launch_grouped_gemm2_odd(go2, odd_grid, side.side));
+    EXFOLD_CUDA(joiner.join());
+    return EXFOLD_OK;
+}
+
 int copy_meta(void* dst, const void* src, size_t bytes, cudaStream_t s) {
     if (dst == nullptr || bytes == 0) return EXFOLD_OK;
     EXFOLD_CUDA(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToDevice, s));
@@ -389,14 +463,8 @@ int exfold_moe_prefill_ex(const exfold_layer* layer, const void* x, const float*
     const bool direct = bf16 && Kp == 1 && l.n_shared == 0;  // every token is written exactly once
 
     CUtensorMap tm_xs, tm_x, tm_wg, tm_wu, tm_h, tm_wd, tm_wd_half;
-    // A call with enough work (>= 24 row tiles of 128 sorted rows) runs every group's row tiles two at a time on CTA
-    // pairs (gemm_pair.cu: a third less operand traffic per SM, a deeper ring, the tensor pipe busy > 95 % of the
-    // main loop) and only a group's odd last tile on the one-CTA kernel, the two passes side by side (below).
-    // Measured against the one-CTA kernel alone: Mixtral shape 4096 / 8192 / 16384 / 32768 tokens -3 / -9 / -14 /
-    // -16 %, GLM shape -8 %, Qwen3 shape (half of the experts own a single tile) -1 %.
-    const int64_t tiles_est = Rtot / kTileM + G / 2;
     const int mode = opts == nullptr || opts->gemm_path < 0 || opts->gemm_path > 2 ? 0 : opts->gemm_path;
-    const bool pairs = bf16 && kGemmBK == 64 && (mode == 2 ? Rtot >= 2 * kTileM : mode == 0 && tiles_est >= 24);
+    const bool pairs = bf16 && (mode == 2 ? kGemmBK == 64 && Rtot >= 2 * kTileM : mode == 0 && use_pairs(Rtot, G, d, I));
     const int sms = sm_count() & ~1;
     if (bf16) {
         const uint64_t E = (uint64_t)G;
@@ -466,62 +534,18 @@ int exfold_moe_prefill_ex(const exfold_layer* layer, const void* x, const float*
         g.grp_expert = nullptr; g.n_groups_dev = nullptr;
         g.H = at<__nv_bfloat16>(ws, pl.H); g.row_tok = cp.row_tok; g.row_w = cp.row_w;
         g.y = nullptr; g.status = at<DeviceStatus>(ws, pl.status);
-        const int64_t max_tiles = Rtot / kTileM + G;
-        const int nt1 = (I + 127) / 128, nt2 = (d + 255) / 256;
         GroupedGemmParams g2 = g;  // GEMM-2: H x W_down -> y (or the per-route buffer O)
-        g2.tm_a = tm_h; g2.tm_b0 = tm_wd; g2.tm_b1 = tm_wd_half; g2.n_ntiles = nt2;
+        g2.tm_a = tm_h; g2.tm_b0 = tm_wd; g2.tm_b1 = tm_wd_half; g2.n_ntiles = (d + 255) / 256;
         // K' = 1 without a shared expert: every token is written once, straight into y. Otherwise each
         // route's weighted output goes to O (bf16, sorted rows) and the combine kernel sums per token.
         g2.y = direct ? reinterpret_cast<__nv_bfloat16*>(y) : at<__nv_bfloat16>(ws, pl.obuf);
         g2.store_rows = direct ? 0 : 1;
-        if (!pairs) {
-            { ProfScope ps(3, s); EXFOLD_CUDA(launch_grouped_gemm1(g, (int)std::min<int64_t>(sm_count(), max_tiles * nt1), s)); }
-            { ProfScope ps(4, s); EXFOLD_CUDA(launch_grouped_gemm2(g2, (int)std::min<int64_t>(sm_count(), max_tiles * nt2), s)); }
-        } else {
-            // Both passes are launched over all SMs, the pair pass on the caller's stream and the odd-tile pass on a
-            // second one; on the device each keeps its share of the SM pairs (pair_pass_clusters of the actual tile
-            // counts) and its other CTAs leave at once, so the two grids settle side by side whatever the routing.
-            // Rows of whole tile pairs and rows of odd last tiles never meet before the combine step, so each pass
-            // of GEMM-2 follows the same pass of GEMM-1 on its own stream: caller's stream: GEMM-1 pairs -> GEMM-2
-            // pairs; side stream: GEMM-1 odd tiles -> GEMM-2 odd tiles; joined before the combine kernel (or the
-            // end of the call). With per-kernel timing on, the streams also join between the two GEMMs.
-            ThreadDeviceState* sidep = side_stream();
-            if (!sidep) return EXFOLD_ERR_CUDA;
-            ThreadDeviceState& side = *sidep;
-            GroupedGemmParams go1 = g, go2 = g2;
-            go1.odd_only = go2.odd_only = 1;
-            // The odd-tile pass is launched with about twice the CTAs its expected share of the work needs (its share
-            // is decided on the device, where the tile counts are known): CTAs without work leave at once, but every
-            // one of them has to pass through one of the pass's few SMs first.
-            const double odd_est = std::max<double>(1.0, G / 2.0), pair_est = std::max<double>(1.0, (tiles_est - G / 2.0) / 2.0);
-            const double q_est = sms * odd_est / (odd_est + 2 * 0.73 * pair_est);
-            const int odd_grid = std::min(sms, 2 * (int)std::ceil(q_est) + 8) & ~1;
-            const SideBySide sbs{nt1, d / kGemmBK, nt2, I / kGemmBK, sms / 2, odd_grid, shared_pairs};
-            g.sbs = g2.sbs = go1.sbs = go2.sbs = sbs;
-            if (shared_pairs > 0) {  // the shared expert's pairs of GEMM-1 are done (or running) on the second stream
-                g.shared_split = 2;
-                EXFOLD_CUDA(cudaStreamWaitEvent(s, side.mid, 0));
-            }
-            EXFOLD_CUDA(cudaEventRecord(side.fork, s));
-            EXFOLD_CUDA(cudaStreamWaitEvent(side.side, side.fork, 0));
-            SideJoin joiner{sidep, s};
-            early_join.armed = false;
-            {
-                ProfScope ps(3, s);
-                { ProfScope pp(12, s); EXFOLD_CUDA(launch_grouped_gemm1_pair(g, sms, s)); }
-                EXFOLD_CUDA(launch_grouped_gemm1_odd(go1, odd_grid, side.side));
-                if (g_prof.on) {
-                    EXFOLD_CUDA(cudaEventRecord(side.mid, side.side));
-                    EXFOLD_CUDA(cudaStreamWaitEvent(s, side.mid, 0));
-                }
-            }
-            {
-                ProfScope ps(4, s);
-                { ProfScope pp(13, s); EXFOLD_CUDA(launch_grouped_gemm2_pair(g2, sms, s)); }
-                EXFOLD_CUDA(launch_grouped_gemm2_odd(go2, odd_grid, side.side));
-                EXFOLD_CUDA(joiner.join());
-            }
+        if (shared_pairs > 0) {  // the shared expert's pairs of GEMM-1 are done (or running) on the second stream
+            g.shared_split = 2;
+            EXFOLD_CUDA(cudaStreamWaitEvent(s, early_side->mid, 0));
         }
+        if ((rc = enqueue_expert_gemms(g, g2, Rtot, pairs, shared_pairs, s)) != EXFOLD_OK) return rc;
+        early_join.armed = false;  // the passes above have joined the second stream
         if (!direct) {
             ProfScope ps(5, s);
             EXFOLD_CUDA(launch_combine_rows(at<__nv_bfloat16>(ws, pl.obuf), cp.inv_pos, T, Kp, d, l.n_shared, nullptr, 1, 0,
@@ -759,12 +783,12 @@ static int calibrate_enqueue(const exfold_layer* layer, const void* x_cal, const
         // Expert outputs on the tensor cores: rows sorted by expert -> GEMM-1 (SwiGLU, H in bf16) -> GEMM-2
         // with the raw fp32 accumulators stored per sorted row. Mode 0 sorts the routed rows like prefill;
         // in mode 1 every expert's rows are the tokens themselves, read from x_cal without a copy.
-        CUtensorMap tm_xs, tm_x, tm_wg, tm_wu, tm_h, tm_wd;
+        CUtensorMap tm_xs, tm_x, tm_wg, tm_wu, tm_h, tm_wd, tm_wd_half;
         const uint64_t E = (uint64_t)N;
         bool ok = make_tmap(&tm_xs, at<char>(ws, pl.xs), (uint64_t)Rc, d, 128) &&
                   make_tmap(&tm_x, x_cal, (uint64_t)m, d, 128) && make_tmap(&tm_wg, w_gate, E * I, d, 128) &&
                   make_tmap(&tm_wu, w_up, E * I, d, 128) && make_tmap(&tm_h, at<char>(ws, pl.H), (uint64_t)Rc, I, 128) &&
-                  make_tmap(&tm_wd, w_down, E * d, I, 256);
+                  make_tmap(&tm_wd, w_down, E * d, I, 256) && make_tmap(&tm_wd_half, w_down, E * d, I, 128);
         if (!ok) return EXFOLD_ERR_CUDA;
         int32_t* offsets = at<int32_t>(ws, pl.offsets);
         int32_t* work_start = at<int32_t>(ws, pl.work_start);
@@ -793,12 +817,12 @@ static int calibrate_enqueue(const exfold_layer* layer, const void* x_cal, const
         g.d = d; g.I = I; g.n_ntiles = (I + 127) / 128; g.ksplit = 1; g.a_rows = kTileM;
         g.H = at<__nv_bfloat16>(ws, pl.H); g.row_tok = at<int32_t>(ws, pl.row_tok); g.row_w = at<float>(ws, pl.row_w);
         g.status = at<DeviceStatus>(ws, pl.status);
-        const int64_t max_tiles = Rc / kTileM + N;
-        EXFOLD_CUDA(launch_grouped_gemm1(g, (int)std::min<int64_t>(sm_count(), max_tiles * g.n_ntiles), s));
-        g.tm_a = tm_h; g.tm_b0 = tm_wd; g.n_ntiles = (d + 255) / 256;
-        g.o32 = at<float>(ws, pl.xs);  // spans the xs and obuf regions (GEMM-1 is done with xs)
-        EXFOLD_CUDA(launch_grouped_gemm2(g, (int)std::min<int64_t>(sm_count(), max_tiles * g.n_ntiles), s));
-        cs.out = g.o32;
+        GroupedGemmParams g2 = g;
+        g2.tm_a = tm_h; g2.tm_b0 = tm_wd; g2.tm_b1 = tm_wd_half; g2.n_ntiles = (d + 255) / 256;
+        g2.o32 = at<float>(ws, pl.xs);  // spans the xs and obuf regions (GEMM-1 is done with xs)
+        const int rc = enqueue_expert_gemms(g, g2, Rc, use_pairs(Rc, N, d, I), 0, s);
+        if (rc != EXFOLD_OK) return rc;
+        cs.out = g2.o32;
     } else {
         SimtFfnParams fp{};
         fp.x = x_cal; fp.wg = w_gate; fp.wu = w_up; fp.wd = w_down; fp.dtype = l.dtype; fp.d = d; fp.I = I;
@@ -968,9 +992,6 @@ int exfold_moe_prefill_host(const exfold_layer* layer, const void* x_host, const
     // metadata describes the whole call (one permutation over all routes), so a call that asks for it is not split.
     const int64_t chunk_tokens = 2048;
     int chunks = meta != nullptr ? 1 : (int)std::min<int64_t>(kMaxHostChunks, T / chunk_tokens);
-    // a chunk of at least 12 row tiles still runs its whole tile pairs on the CTA-pair kernel
-    const int64_t chunk_rows = chunks > 1 ? (T / chunks) * (k_pre + layer->n_shared) : 0;
-    exfold_fold_opts chunk_opts{INFINITY, 0, 0, chunk_rows >= 12 * kTileM ? 2 : 0};
     if (chunks <= 1) {
         EXFOLD_CUDA(cudaMemcpyAsync(xd, x_host, xb, cudaMemcpyHostToDevice, s));
         EXFOLD_CUDA(cudaMemcpyAsync(ld, logits_host, lb, cudaMemcpyHostToDevice, s));
@@ -1003,9 +1024,8 @@ int exfold_moe_prefill_host(const exfold_layer* layer, const void* x_host, const
         if (n <= 0) break;
         EXFOLD_CUDA(cudaStreamWaitEvent(s, h.copied[c], 0));
         t_keep_status = c > 0;  // an error recorded by an earlier chunk stays visible
-        int rc = exfold_moe_prefill_ex(layer, xd + t0 * row_x, reinterpret_cast<const float*>(ld + t0 * row_l), n, w_gate,
-                                       w_up, w_down, tables, k_pre, &chunk_opts, yd + t0 * row_x, nullptr, ws, main_bytes,
-                                       cuda_stream);
+        int rc = exfold_moe_prefill(layer, xd + t0 * row_x, reinterpret_cast<const float*>(ld + t0 * row_l), n, w_gate,
+                                    w_up, w_down, tables, k_pre, yd + t0 * row_x, nullptr, ws, main_bytes, cuda_stream);
         t_keep_status = false;
         if (rc != EXFOLD_OK) return rc;
         EXFOLD_CUDA(cudaEventRecord(h.computed[c], s));
