@@ -333,6 +333,19 @@ int enqueue_expert_gemms(GroupedGemmParams& g, GroupedGemmParams& g2, int64_t ro
     return EXFOLD_OK;
 }
 
+struct PdlScope {  // programmatic dependent launch for the launches of this scope
+    explicit PdlScope(bool on) { set_pdl(on); }
+    ~PdlScope() { set_pdl(false); }
+};
+
+FfnF32Params f32_params(const void* x, const void* wg, const void* wu, const void* wd, int d, int I, int G, int tile_rows) {
+    FfnF32Params p{};
+    p.x = reinterpret_cast<const float*>(x); p.wg = reinterpret_cast<const float*>(wg);
+    p.wu = reinterpret_cast<const float*>(wu); p.wd = reinterpret_cast<const float*>(wd);
+    p.d = d; p.I = I; p.G = G; p.tile_rows = tile_rows; p.x_rows = 1;
+    return p;
+}
+
 int copy_meta(void* dst, const void* src, size_t bytes, cudaStream_t s) {
     if (dst == nullptr || bytes == 0) return EXFOLD_OK;
     EXFOLD_CUDA(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToDevice, s));
@@ -460,7 +473,7 @@ int exfold_moe_prefill_ex(const exfold_layer* layer, const void* x, const float*
     if (ws_bytes < pl.total) return EXFOLD_ERR_WORKSPACE_TOO_SMALL;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(cuda_stream);
     const bool bf16 = l.dtype == EXFOLD_BF16;
-    const bool direct = bf16 && Kp == 1 && l.n_shared == 0;  // every token is written exactly once
+    const bool direct = Kp == 1 && l.n_shared == 0;  // every token is written exactly once
 
     CUtensorMap tm_xs, tm_x, tm_wg, tm_wu, tm_h, tm_wd, tm_wd_half;
     const int mode = opts == nullptr || opts->gemm_path < 0 || opts->gemm_path > 2 ? 0 : opts->gemm_path;
@@ -476,6 +489,9 @@ int exfold_moe_prefill_ex(const exfold_layer* layer, const void* x, const float*
     }
 
     prof_reset();
+    // The kernels of an fp32 layer are short: chained by programmatic dependent launch. The bf16 path launches plainly
+    // (early-resident successors compete with the running kernels: 19-32 us slower).
+    PdlScope pdl_scope(!bf16);
 
     PrefillRouteParams rp{};
     rp.logits = logits; rp.S = tables->S; rp.L = tables->L; rp.lnh = tables->lnh;
@@ -517,6 +533,7 @@ int exfold_moe_prefill_ex(const exfold_layer* layer, const void* x, const float*
 
     PrefillScatterParams cp{};
     cp.T = T; cp.N = N; cp.n_shared = l.n_shared; cp.Kp = Kp; cp.d_bytes = bf16 ? d * 2 : 0;
+    cp.tile_rows = bf16 ? kTileM : ffn_f32_tile_rows(Rtot, G, I);
     cp.nblk = (int)((T + kRouteTokensPerBlock - 1) / kRouteTokensPerBlock);
     cp.ids = rp.ids; cp.w = rp.w; cp.block_hist = rp.block_hist; cp.sb_hist = rp.sb_hist;
     cp.offsets = at<int32_t>(ws, pl.offsets); cp.work_start = at<int32_t>(ws, pl.work_start);
@@ -552,11 +569,16 @@ int exfold_moe_prefill_ex(const exfold_layer* layer, const void* x, const float*
                                             reinterpret_cast<__nv_bfloat16*>(y), s));
         }
     } else {
-        SimtFfnParams fp{};
-        fp.x = x; fp.wg = w_gate; fp.wu = w_up; fp.wd = w_down; fp.dtype = l.dtype; fp.d = d; fp.I = I;
-        fp.T = T; fp.Kr = Kp; fp.n_shared = l.n_shared; fp.N = N; fp.ids = rp.ids; fp.out = at<float>(ws, pl.out);
-        { ProfScope ps(10, s); EXFOLD_CUDA(launch_simt_ffn(fp, s)); }
-        { ProfScope ps(11, s); EXFOLD_CUDA(launch_combine_routes(fp.out, rp.w, T, Kp, d, l.n_shared, y, l.dtype, s)); }
+        FfnF32Params fp = f32_params(x, w_gate, w_up, w_down, d, I, G, cp.tile_rows);
+        fp.offsets = cp.offsets; fp.tile_start = cp.work_start; fp.row_tok = cp.row_tok; fp.row_w = cp.row_w;
+        if (direct) fp.y = reinterpret_cast<float*>(y);
+        else fp.out = at<float>(ws, pl.out);
+        { ProfScope ps(10, s); EXFOLD_CUDA(launch_ffn_f32(fp, Rtot, s)); }
+        if (!direct) {
+            ProfScope ps(11, s);
+            EXFOLD_CUDA(launch_combine_f32(fp.out, cp.inv_pos, cp.row_w, T, Kp, d, l.n_shared, nullptr,
+                                           reinterpret_cast<float*>(y), s));
+        }
     }
     if (meta) {
         if ((rc = copy_meta(meta->ids, rp.ids, (size_t)R * 4, s))) return rc;
@@ -608,10 +630,7 @@ static int decode_impl(const exfold_layer* layer, const void* x, const float* lo
         if (!ok) return EXFOLD_ERR_CUDA;
     }
     prof_reset();
-    struct PdlScope {
-        PdlScope() { set_pdl(true); }
-        ~PdlScope() { set_pdl(false); }
-    } pdl_scope;
+    PdlScope pdl_scope(true);
 
     DecodeRouteParams rp{};
     rp.logits = logits; rp.S = tables->S; rp.L = tables->L; rp.h = tables->h;
@@ -625,6 +644,7 @@ static int decode_impl(const exfold_layer* layer, const void* x, const float* lo
     rp.row_tok = at<int32_t>(ws, pl.row_tok); rp.row_w = at<float>(ws, pl.row_w);
     rp.grp_expert = at<int32_t>(ws, pl.grp_expert); rp.grp_off = at<int32_t>(ws, pl.grp_off);
     rp.grp_tiles = at<int32_t>(ws, pl.grp_tiles); rp.n_groups = at<int32_t>(ws, pl.n_groups);
+    rp.slot_row = at<int32_t>(ws, pl.inv_pos);
     rp.status = at<DeviceStatus>(ws, pl.status);
     if (bf16) {
         // Token-parallel Top-K (with the router scores when w_router is given) -> gate/up kernel that finishes the
@@ -655,7 +675,7 @@ static int decode_impl(const exfold_layer* layer, const void* x, const float* lo
         // the remapped slots go to a second array: the Top-K ids are read by every CTA while CTA 0 writes
         fp.out_ids = at<int32_t>(ws, pl.perm); fp.out_w = rp.w; fp.target = rp.target; fp.scale = rp.scale;
         fp.H = at<__nv_bfloat16>(ws, pl.H); fp.row_tok = rp.row_tok; fp.row_w = rp.row_w;
-        fp.slot_row = at<int32_t>(ws, pl.inv_pos);
+        fp.slot_row = rp.slot_row;
         fp.grp_expert = rp.grp_expert; fp.grp_off = rp.grp_off; fp.grp_tiles = rp.grp_tiles; fp.n_groups = rp.n_groups;
         fp.status = rp.status;
         { ProfScope ps(14, s); EXFOLD_CUDA(launch_decode_ffn(fp, sm_count(), s)); }
@@ -684,19 +704,19 @@ static int decode_impl(const exfold_layer* layer, const void* x, const float* lo
                                                        max_rows, reinterpret_cast<__nv_bfloat16*>(y), s)); }
         rp.ids = fp.out_ids;  // for the metadata copies below
     } else {
-    if (w_router != nullptr) {
-        rc = router_enqueue(layer, x, w_router, B, const_cast<float*>(logits), ws, ws_bytes, s, false);
-        if (rc != EXFOLD_OK) return rc;
-    }
-    { ProfScope ps(6, s); EXFOLD_CUDA(launch_decode_route(rp, s)); }
-
-    {
-        SimtFfnParams fp{};
-        fp.x = x; fp.wg = w_gate; fp.wu = w_up; fp.wd = w_down; fp.dtype = l.dtype; fp.d = d; fp.I = I;
-        fp.T = B; fp.Kr = K; fp.n_shared = l.n_shared; fp.N = N; fp.ids = rp.ids; fp.out = at<float>(ws, pl.out);
-        { ProfScope ps(10, s); EXFOLD_CUDA(launch_simt_ffn(fp, s)); }
-        { ProfScope ps(11, s); EXFOLD_CUDA(launch_combine_routes(fp.out, rp.w, B, K, d, l.n_shared, y, l.dtype, s)); }
-    }
+        if (w_router != nullptr) {
+            rc = router_enqueue(layer, x, w_router, B, const_cast<float*>(logits), ws, ws_bytes, s, false);
+            if (rc != EXFOLD_OK) return rc;
+        }
+        const int max_groups = std::min(pool_m, N) + l.n_shared;
+        rp.tile_rows = ffn_f32_tile_rows(max_rows, max_groups, I);
+        { ProfScope ps(6, s); EXFOLD_CUDA(launch_decode_route(rp, s)); }
+        FfnF32Params fp = f32_params(x, w_gate, w_up, w_down, d, I, max_groups, rp.tile_rows);
+        fp.offsets = rp.grp_off; fp.tile_start = rp.grp_tiles; fp.grp_expert = rp.grp_expert; fp.n_groups_dev = rp.n_groups;
+        fp.row_tok = rp.row_tok; fp.row_w = rp.row_w; fp.out = at<float>(ws, pl.out);
+        { ProfScope ps(10, s); EXFOLD_CUDA(launch_ffn_f32(fp, max_rows, s)); }
+        { ProfScope ps(11, s); EXFOLD_CUDA(launch_combine_f32(fp.out, rp.slot_row, rp.row_w, B, K, d, l.n_shared, rp.n_groups + 2,
+                                                              reinterpret_cast<float*>(y), s)); }
     }
     if (meta) {
         if ((rc = copy_meta(meta->pool_ids, rp.pool_ids, (size_t)pool_m * 4, s))) return rc;
@@ -779,10 +799,31 @@ static int calibrate_enqueue(const exfold_layer* layer, const void* x_cal, const
     const int64_t Rc = m * Ke;
     if (tensor_path && Rc > (int64_t)1 << 30) return EXFOLD_ERR_UNSUPPORTED;
     CalibStatsParams cs{};
+    // Expert outputs, one fp32 row per (token, expert), sorted by expert. Mode 0 sorts the routed rows like prefill; in
+    // mode 1 every expert's rows are the tokens themselves, read from x_cal without a copy.
+    int32_t* offsets = at<int32_t>(ws, pl.offsets);
+    int32_t* work_start = at<int32_t>(ws, pl.work_start);
+    int32_t* row_tok = at<int32_t>(ws, pl.row_tok);
+    const int tile_rows = tensor_path ? kTileM : ffn_f32_tile_rows(Rc, N, I);
+    if (opts->mode == 0) {
+        PrefillScatterParams cp{};
+        cp.T = m; cp.N = N; cp.n_shared = 0; cp.Kp = K; cp.d_bytes = tensor_path ? d * 2 : 0; cp.tile_rows = tile_rows;
+        cp.nblk = (int)((m + kRouteTokensPerBlock - 1) / kRouteTokensPerBlock);
+        cp.ids = ids; cp.w = at<float>(ws, pl.w); cp.block_hist = at<int32_t>(ws, pl.block_hist);
+        cp.sb_hist = at<int32_t>(ws, pl.sb_hist);
+        cp.offsets = offsets; cp.work_start = work_start;
+        cp.x = x_cal; cp.xs = tensor_path ? at<char>(ws, pl.xs) : nullptr;
+        cp.perm = at<int32_t>(ws, pl.perm); cp.row_tok = row_tok;
+        cp.row_w = at<float>(ws, pl.row_w); cp.row_exp = at<int32_t>(ws, pl.row_exp);
+        cp.inv_pos = at<int32_t>(ws, pl.inv_pos);
+        EXFOLD_CUDA(launch_prefill_scatter(cp, s));
+        cs.inv_pos = cp.inv_pos;
+    } else {
+        EXFOLD_CUDA(launch_calib_common_rows(offsets, work_start, m, N, tile_rows, s));
+        cs.inv_pos = nullptr; cs.tok_stride = 1; cs.slot_stride = m;
+    }
     if (tensor_path) {
-        // Expert outputs on the tensor cores: rows sorted by expert -> GEMM-1 (SwiGLU, H in bf16) -> GEMM-2
-        // with the raw fp32 accumulators stored per sorted row. Mode 0 sorts the routed rows like prefill;
-        // in mode 1 every expert's rows are the tokens themselves, read from x_cal without a copy.
+        // GEMM-1 (SwiGLU, H in bf16) -> GEMM-2 with the raw fp32 accumulators stored per sorted row
         CUtensorMap tm_xs, tm_x, tm_wg, tm_wu, tm_h, tm_wd, tm_wd_half;
         const uint64_t E = (uint64_t)N;
         bool ok = make_tmap(&tm_xs, at<char>(ws, pl.xs), (uint64_t)Rc, d, 128) &&
@@ -790,32 +831,13 @@ static int calibrate_enqueue(const exfold_layer* layer, const void* x_cal, const
                   make_tmap(&tm_wu, w_up, E * I, d, 128) && make_tmap(&tm_h, at<char>(ws, pl.H), (uint64_t)Rc, I, 128) &&
                   make_tmap(&tm_wd, w_down, E * d, I, 256) && make_tmap(&tm_wd_half, w_down, E * d, I, 128);
         if (!ok) return EXFOLD_ERR_CUDA;
-        int32_t* offsets = at<int32_t>(ws, pl.offsets);
-        int32_t* work_start = at<int32_t>(ws, pl.work_start);
-        if (opts->mode == 0) {
-            PrefillScatterParams cp{};
-            cp.T = m; cp.N = N; cp.n_shared = 0; cp.Kp = K; cp.d_bytes = d * 2;
-            cp.nblk = (int)((m + kRouteTokensPerBlock - 1) / kRouteTokensPerBlock);
-            cp.ids = ids; cp.w = at<float>(ws, pl.w); cp.block_hist = at<int32_t>(ws, pl.block_hist);
-            cp.sb_hist = at<int32_t>(ws, pl.sb_hist);
-            cp.offsets = offsets; cp.work_start = work_start;
-            cp.x = x_cal; cp.xs = at<char>(ws, pl.xs);
-            cp.perm = at<int32_t>(ws, pl.perm); cp.row_tok = at<int32_t>(ws, pl.row_tok);
-            cp.row_w = at<float>(ws, pl.row_w); cp.row_exp = at<int32_t>(ws, pl.row_exp);
-            cp.inv_pos = at<int32_t>(ws, pl.inv_pos);
-            EXFOLD_CUDA(launch_prefill_scatter(cp, s));
-            cs.inv_pos = cp.inv_pos;
-        } else {
-            EXFOLD_CUDA(launch_calib_common_rows(offsets, work_start, m, N, s));
-            cs.inv_pos = nullptr; cs.tok_stride = 1; cs.slot_stride = m;
-        }
         GroupedGemmParams g{};
         g.tm_a = tm_xs; g.tm_a2 = tm_x; g.tm_b0 = tm_wg; g.tm_b1 = tm_wu;
         g.offsets = offsets; g.work_start = work_start; g.G = N;
         g.n_routed = opts->mode == 0 ? N : 0;  // mode 1: every group reads x_cal directly
         g.R = 0; g.x_rows = (int)m;
         g.d = d; g.I = I; g.n_ntiles = (I + 127) / 128; g.ksplit = 1; g.a_rows = kTileM;
-        g.H = at<__nv_bfloat16>(ws, pl.H); g.row_tok = at<int32_t>(ws, pl.row_tok); g.row_w = at<float>(ws, pl.row_w);
+        g.H = at<__nv_bfloat16>(ws, pl.H); g.row_tok = row_tok; g.row_w = at<float>(ws, pl.row_w);
         g.status = at<DeviceStatus>(ws, pl.status);
         GroupedGemmParams g2 = g;
         g2.tm_a = tm_h; g2.tm_b0 = tm_wd; g2.tm_b1 = tm_wd_half; g2.n_ntiles = (d + 255) / 256;
@@ -824,11 +846,12 @@ static int calibrate_enqueue(const exfold_layer* layer, const void* x_cal, const
         if (rc != EXFOLD_OK) return rc;
         cs.out = g2.o32;
     } else {
-        SimtFfnParams fp{};
-        fp.x = x_cal; fp.wg = w_gate; fp.wu = w_up; fp.wd = w_down; fp.dtype = l.dtype; fp.d = d; fp.I = I;
-        fp.T = m; fp.Kr = Ke; fp.n_shared = 0; fp.N = N; fp.ids = ids; fp.out = at<float>(ws, pl.out);
-        EXFOLD_CUDA(launch_simt_ffn(fp, s));
-        cs.out = fp.out; cs.inv_pos = nullptr; cs.tok_stride = Ke; cs.slot_stride = 1;
+        FfnF32Params fp = f32_params(x_cal, w_gate, w_up, w_down, d, I, N, tile_rows);
+        fp.offsets = offsets; fp.tile_start = work_start; fp.x_rows = m;
+        fp.row_tok = opts->mode == 0 ? row_tok : nullptr;
+        fp.out = at<float>(ws, pl.out);
+        EXFOLD_CUDA(launch_ffn_f32(fp, Rc, s));
+        cs.out = fp.out;
     }
 
     char* cb = at<char>(ws, pl.calib);

@@ -365,19 +365,19 @@ __global__ void __launch_bounds__(256) calib_common_finish_kernel(CalibStatsPara
     }
 }
 
-// common-input mode on the grouped GEMMs: group e = all m tokens in order
-__global__ void calib_common_rows_kernel(int32_t* offsets, int32_t* work_start, int64_t m, int N) {
+// common-input mode: group e = all m tokens in order
+__global__ void calib_common_rows_kernel(int32_t* offsets, int32_t* work_start, int64_t m, int N, int tile_rows) {
     const int g = blockIdx.x * blockDim.x + threadIdx.x;
     if (g <= N) {
         offsets[g] = (int32_t)(g * m);
-        work_start[g] = (int32_t)(g * ((m + kTileM - 1) / kTileM));
+        work_start[g] = (int32_t)(g * ((m + tile_rows - 1) / tile_rows));
     }
 }
 
 }  // namespace
 
-cudaError_t launch_calib_common_rows(int32_t* offsets, int32_t* work_start, int64_t m, int N, cudaStream_t s) {
-    calib_common_rows_kernel<<<(N + 1 + 255) / 256, 256, 0, s>>>(offsets, work_start, m, N);
+cudaError_t launch_calib_common_rows(int32_t* offsets, int32_t* work_start, int64_t m, int N, int tile_rows, cudaStream_t s) {
+    calib_common_rows_kernel<<<(N + 1 + 255) / 256, 256, 0, s>>>(offsets, work_start, m, N, tile_rows);
     count_launch();
     return cudaGetLastError();
 }

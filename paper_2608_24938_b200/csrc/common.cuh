@@ -151,12 +151,13 @@ struct PrefillScatterParams {
     int64_t T;
     int N, n_shared, Kp, d_bytes;  // d_bytes: bytes of one x row (0: no gather)
     int nblk;                   // blocks of the route kernel (= blocks of this kernel)
+    int tile_rows;              // rows per tile of the work list (kTileM, or the fp32 FFN's)
     const int32_t* ids;         // [T][Kp]
     const float* w;             // [T][Kp]
     const int32_t* block_hist;  // [nblk][N] retained routes per (block, expert)
     const int32_t* sb_hist;     // [ceil(nblk / kRouteSuperBlock)][N] the same per super-block
     int32_t* offsets;           // [G+1] out: first sorted row of each group
-    int32_t* work_start;        // [G+1] out: prefix of 128-row tiles per group
+    int32_t* work_start;        // [G+1] out: prefix of row tiles per group
     const void* x;      // [T][d]
     void* xs;           // [R][d] gathered rows (may be null)
     int32_t* perm;      // [R]
@@ -176,6 +177,7 @@ struct DecodeRouteParams {
     const float* L;
     const float* h;
     int B, N, K, M, n_shared;
+    int tile_rows;              // rows per tile of grp_tiles
     // static pool (all null for the dynamic pool of Eq. 11): precomputed pool, targets and scalars
     const int32_t* st_pool;    // [M]
     const int32_t* st_target;  // [N]
@@ -193,8 +195,9 @@ struct DecodeRouteParams {
     float* row_w;         // [B*K + B]
     int32_t* grp_expert;  // [N+1] expert id of each group (pool order; shared last)
     int32_t* grp_off;     // [N+2] first row of each group
-    int32_t* grp_tiles;   // [N+2] prefix of 128-row tiles per group (work list of the grouped GEMMs)
-    int32_t* n_groups;    // [2]: number of groups, total rows
+    int32_t* grp_tiles;   // [N+2] prefix of row tiles per group (work list of the expert FFN)
+    int32_t* slot_row;    // [B][K] row of each routed slot, -1 for a slot merged into an earlier one
+    int32_t* n_groups;    // [3]: number of groups, total rows, first row of the shared expert's group
     DeviceStatus* status; // cleared here (first kernel of a decode call)
 };
 cudaError_t launch_decode_route(const DecodeRouteParams& p, cudaStream_t s);
@@ -259,23 +262,31 @@ size_t decode_ffn_smem_plan(int B, int K, int N, int* stages, int* scratch_off, 
 cudaError_t launch_static_pool(int N, int M, const float* S, const float* L, const float* h, int32_t* pool_ids,
                                int32_t* target, float* scale, cudaStream_t s);
 
-// ---------------------------------------------------------------- SIMT expert FFN (fp32 accumulate)
-struct SimtFfnParams {
-    const void* x;  // [T][d]
-    const void* wg;
-    const void* wu;
-    const void* wd;
-    int dtype, d, I;
-    int64_t T;           // tokens
-    int Kr;              // routes per token; row r < T*Kr is route (r / Kr, r % Kr)
-    int n_shared, N;     // rows T*Kr + i run the shared expert (index N) on token i
-    const int32_t* ids;  // [T][Kr] expert of each route
-    float* out;          // [T*Kr + T*n_shared][d] unweighted expert outputs
+// ---------------------------------------------------------------- fp32 expert FFN (CUDA cores)
+struct FfnF32Params {
+    const float* x;  // [x_rows][d]
+    const float* wg;
+    const float* wu;
+    const float* wd;
+    int d, I, G;                  // G: groups (upper bound when n_groups_dev is given)
+    int tile_rows;                // rows per tile
+    int fpc, push, hld;           // set by the launcher: features per CTA, where H lies and its row pitch
+    int64_t x_rows;               // without row_tok: row r reads token r % x_rows
+    const int32_t* offsets;       // [G+1] first sorted row of each group
+    const int32_t* tile_start;    // [G+1] prefix of row tiles (tile_rows each)
+    const int32_t* grp_expert;    // [G] expert of each group (null: the group itself)
+    const int32_t* n_groups_dev;  // groups known only on the device (decode)
+    const int32_t* row_tok;       // [rows] token of each sorted row, or null
+    const float* row_w;           // [rows]; read when y is set
+    float* out;                   // [rows][d] unweighted expert outputs, or
+    float* y;                     // [tokens][d]: every token has one row, stored weighted (out unused)
 };
-cudaError_t launch_simt_ffn(const SimtFfnParams& p, cudaStream_t s);
-// y[i] = sum_j w[i][j] out[i*Kr+j] (+ out[T*Kr+i] for the shared expert); y in the layer dtype
-cudaError_t launch_combine_routes(const float* out, const float* w, int64_t T, int Kr, int d, int n_shared,
-                                  void* y, int dtype, cudaStream_t s);
+int ffn_f32_tile_rows(int64_t rows, int G, int I);
+cudaError_t launch_ffn_f32(FfnF32Params p, int64_t rows, cudaStream_t s);
+cudaError_t launch_combine_f32(const float* out, const int32_t* inv_pos, const float* row_w, int64_t T, int Kr, int d,
+                               int n_shared, const int32_t* shared0_dev, float* y, cudaStream_t s);
+
+// ---------------------------------------------------------------- router scores, final sums of the bf16 path
 cudaError_t launch_router_simt(const void* x, const void* wr, int dtype, int64_t T, int N, int d, float* out,
                                cudaStream_t s);
 // y[i] = sum_j O[inv_pos[i*Kr+j]] (entries < 0 skipped) (+ O[shared0 + i] for the shared expert), fp32 sum in slot
@@ -309,8 +320,8 @@ cudaError_t launch_calib_stats_common(const CalibStatsParams& p, double* nrm, in
 cudaError_t launch_calib_finalize(const CalibStatsParams& p, const exfold_calib_opts& o, float* S, float* L,
                                   float* h, float* lnh, int32_t* n_obs, int32_t* unobserved, cudaStream_t s);
 cudaError_t launch_iota_ids(int32_t* ids, int64_t m, int N, cudaStream_t s);
-// Common-input calibration on the grouped GEMMs: every expert e owns rows [e*m, (e+1)*m) = all tokens in order
-cudaError_t launch_calib_common_rows(int32_t* offsets, int32_t* work_start, int64_t m, int N, cudaStream_t s);
+// Common-input calibration: every expert e owns rows [e*m, (e+1)*m) = all tokens in order
+cudaError_t launch_calib_common_rows(int32_t* offsets, int32_t* work_start, int64_t m, int N, int tile_rows, cudaStream_t s);
 
 // ---------------------------------------------------------------- tcgen05 grouped GEMMs (bf16)
 // SM pairs, of n_clusters, that the CTA-pair passes keep when the odd-tile passes run beside them on the other

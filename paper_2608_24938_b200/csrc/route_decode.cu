@@ -272,17 +272,24 @@ __global__ void __launch_bounds__(kDecThreads) decode_route_kernel(DecodeRoutePa
                 int i = i0 + lane;
                 bool has = false;
                 float ws = 0.f;
+                unsigned slots = 0;  // the token's slots with this target
                 if (i < B)
                     for (int k = 0; k < K; ++k)
                         if (sm.ids[i * K + k] == t) {
                             ws = has ? __fadd_rn(ws, sm.wrm[i * K + k]) : sm.wrm[i * K + k];
                             has = true;
+                            slots |= 1u << k;
                         }
                 unsigned m = __ballot_sync(0xffffffffu, has);
                 if (pass && has) {
                     int q = run + __popc(m & ((1u << lane) - 1u));
                     p.row_tok[q] = i;
                     p.row_w[q] = ws;
+                    const int first = __ffs(slots) - 1;
+                    for (unsigned rest = slots; rest != 0; rest &= rest - 1) {
+                        const int k = __ffs(rest) - 1;
+                        p.slot_row[i * K + k] = k == first ? q : -1;
+                    }
                 }
                 run += __popc(m);
             }
@@ -318,11 +325,11 @@ __global__ void __launch_bounds__(kDecThreads) decode_route_kernel(DecodeRoutePa
         p.grp_off[g] = sm.goff[g];
         if (g < G) p.grp_expert[g] = g < P ? sm.pool[g] : N;
     }
-    if (threadIdx.x == 0) {  // prefix of 128-row tiles per group
+    if (threadIdx.x == 0) {  // prefix of row tiles per group
         int tiles = 0;
         for (int g = 0; g < G; ++g) {
             p.grp_tiles[g] = tiles;
-            tiles += (sm.goff[g + 1] - sm.goff[g] + kTileM - 1) / kTileM;
+            tiles += (sm.goff[g + 1] - sm.goff[g] + p.tile_rows - 1) / p.tile_rows;
         }
         p.grp_tiles[G] = tiles;
     }
@@ -334,6 +341,7 @@ __global__ void __launch_bounds__(kDecThreads) decode_route_kernel(DecodeRoutePa
     if (threadIdx.x == 0) {
         p.n_groups[0] = G;
         p.n_groups[1] = sm.goff[G];  // total rows
+        p.n_groups[2] = sm.goff[P];  // first row of the shared expert's group
     }
 }
 

@@ -239,7 +239,7 @@ __global__ void __launch_bounds__(kRouteThreads) prefill_scatter_kernel(PrefillS
             p.offsets[g] = off;
             p.work_start[g] = tiles;
             off += rows;
-            tiles += (rows + kTileM - 1) / kTileM;
+            tiles += (rows + p.tile_rows - 1) / p.tile_rows;
         }
         p.offsets[G] = off;
         p.work_start[G] = tiles;

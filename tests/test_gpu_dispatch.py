@@ -5,7 +5,7 @@ import torch
 
 import oracle
 import synth_inputs as si
-from harness import A, Case
+from harness import A, Case, check_decode_meta, check_output, check_prefill_meta
 
 pytestmark = pytest.mark.gpu
 
@@ -34,3 +34,26 @@ def test_calibration_sums_by_top_k(K):
     np.testing.assert_allclose(L.cpu().numpy(), ref["L"], rtol=1e-4, atol=2e-5)
     np.testing.assert_allclose(h.cpu().numpy(), ref["h"], rtol=1e-5)
     np.testing.assert_allclose(lnh.cpu().numpy(), ref["lnh"], rtol=1e-5, atol=1e-6)
+
+
+@pytest.mark.parametrize("shape", [
+    # N, shared, d, I, K, T, K', B, M
+    (8, 0, 128, 256, 2, 64, 1, 16, 4),      # 8-row tiles, one row per token straight into y
+    (8, 1, 132, 100, 3, 37, 2, 7, 3),       # widths off every multiple: ragged K chunks, CTAs without columns
+    (4, 0, 64, 33, 2, 9, 2, 1, 4),          # I % 4 != 0: element-wise staging; slices of H past I
+    (6, 1, 100, 40, 2, 300, 2, 90, 6),      # 32-row tiles with ragged last tiles, fewer slices than CTAs
+    (5, 0, 256, 390, 3, 257, 3, 256, 2),    # 32-row tiles, element-wise staging, merged decode slots
+    (40, 0, 36, 1100, 5, 130, 4, 33, 17),   # 16-row tiles, several feature passes per CTA
+    (16, 0, 384, 640, 2, 50, 2, 40, 5),     # 8-row tiles, two feature passes
+])
+def test_f32_layer_shapes(shape):
+    """fp32 layers: row-tile sizes, vector and element-wise staging, ragged widths, shared expert; routing bit-exact,
+    outputs to fp32 rounding (two-level sums of at most ~1100 terms: 2e-6 of the norm; seen ~3e-7)."""
+    N, ns, d, I, K, T, Kp, B, M = shape
+    case = Case(si.LayerConfig("f32s", N, ns, d, I, K, "f32", T, (Kp,), B, (M,)))
+    got, ref = case.run_prefill(Kp), case.oracle_prefill(Kp)
+    check_prefill_meta(got, ref)
+    assert check_output(got["y"], ref["y"], "f32")[1] < 2e-6
+    got, ref = case.run_decode(M), case.oracle_decode(M)
+    check_decode_meta(got, ref, M)
+    assert check_output(got["y"], ref["y"], "f32")[1] < 2e-6
