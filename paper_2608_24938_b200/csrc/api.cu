@@ -533,7 +533,7 @@ int exfold_moe_prefill_ex(const exfold_layer* layer, const void* x, const float*
 
     PrefillScatterParams cp{};
     cp.T = T; cp.N = N; cp.n_shared = l.n_shared; cp.Kp = Kp; cp.d_bytes = bf16 ? d * 2 : 0;
-    cp.tile_rows = bf16 ? kTileM : ffn_f32_tile_rows(Rtot, G, I);
+    cp.tile_rows = bf16 ? kTileM : ffn_f32_tile_rows(Rtot, G, d, I);
     cp.nblk = (int)((T + kRouteTokensPerBlock - 1) / kRouteTokensPerBlock);
     cp.ids = rp.ids; cp.w = rp.w; cp.block_hist = rp.block_hist; cp.sb_hist = rp.sb_hist;
     cp.offsets = at<int32_t>(ws, pl.offsets); cp.work_start = at<int32_t>(ws, pl.work_start);
@@ -709,7 +709,7 @@ static int decode_impl(const exfold_layer* layer, const void* x, const float* lo
             if (rc != EXFOLD_OK) return rc;
         }
         const int max_groups = std::min(pool_m, N) + l.n_shared;
-        rp.tile_rows = ffn_f32_tile_rows(max_rows, max_groups, I);
+        rp.tile_rows = ffn_f32_tile_rows(max_rows, max_groups, d, I);
         { ProfScope ps(6, s); EXFOLD_CUDA(launch_decode_route(rp, s)); }
         FfnF32Params fp = f32_params(x, w_gate, w_up, w_down, d, I, max_groups, rp.tile_rows);
         fp.offsets = rp.grp_off; fp.tile_start = rp.grp_tiles; fp.grp_expert = rp.grp_expert; fp.n_groups_dev = rp.n_groups;
@@ -804,7 +804,7 @@ static int calibrate_enqueue(const exfold_layer* layer, const void* x_cal, const
     int32_t* offsets = at<int32_t>(ws, pl.offsets);
     int32_t* work_start = at<int32_t>(ws, pl.work_start);
     int32_t* row_tok = at<int32_t>(ws, pl.row_tok);
-    const int tile_rows = tensor_path ? kTileM : ffn_f32_tile_rows(Rc, N, I);
+    const int tile_rows = tensor_path ? kTileM : ffn_f32_tile_rows(Rc, N, d, I);
     if (opts->mode == 0) {
         PrefillScatterParams cp{};
         cp.T = m; cp.N = N; cp.n_shared = 0; cp.Kp = K; cp.d_bytes = tensor_path ? d * 2 : 0; cp.tile_rows = tile_rows;

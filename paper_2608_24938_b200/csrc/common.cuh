@@ -270,7 +270,7 @@ struct FfnF32Params {
     const float* wd;
     int d, I, G;                  // G: groups (upper bound when n_groups_dev is given)
     int tile_rows;                // rows per tile
-    int fpc, push, hld;           // set by the launcher: features per CTA, where H lies and its row pitch
+    int fpc, hld;                 // set by the launcher: features per CTA (tall tiles), row pitch of H in shared memory
     int64_t x_rows;               // without row_tok: row r reads token r % x_rows
     const int32_t* offsets;       // [G+1] first sorted row of each group
     const int32_t* tile_start;    // [G+1] prefix of row tiles (tile_rows each)
@@ -281,7 +281,7 @@ struct FfnF32Params {
     float* out;                   // [rows][d] unweighted expert outputs, or
     float* y;                     // [tokens][d]: every token has one row, stored weighted (out unused)
 };
-int ffn_f32_tile_rows(int64_t rows, int G, int I);
+int ffn_f32_tile_rows(int64_t rows, int G, int d, int I);
 cudaError_t launch_ffn_f32(FfnF32Params p, int64_t rows, cudaStream_t s);
 cudaError_t launch_combine_f32(const float* out, const int32_t* inv_pos, const float* row_w, int64_t T, int Kr, int d,
                                int n_shared, const int32_t* shared0_dev, float* y, cudaStream_t s);

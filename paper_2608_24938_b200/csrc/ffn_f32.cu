@@ -1,23 +1,29 @@
 // Expert FFN of fp32 layers (Eq. 1) on the CUDA cores: tensor cores would round fp32 inputs.
 //
 // A cluster of 8 CTAs per row tile (up to tile_rows sorted rows of one expert). Phase 0: CTA r computes its eighth of the
-// intermediate features, gate and up, for all rows of the tile, and keeps silu(gate) * up in shared memory. Phase 1,
+// intermediate features, gate and up, for all rows of the tile, and leaves silu(gate) * up in shared memory. Phase 1,
 // after a cluster barrier: CTA r computes its eighth of the output features with all of I as K. The activation crosses the
-// cluster through distributed shared memory: small tiles (up to kPushBytes) are written to every CTA's copy as they are
-// computed, so that phase 1 waits for nothing but weights; of larger ones a CTA keeps its slice and the others read it
-// chunk by chunk. The activation never goes to memory, one launch does the whole FFN, and a tile's weights are read once
-// per tile instead of once per row.
+// cluster through distributed shared memory and never goes to memory; one launch does the whole FFN, and a tile's weights
+// are read once per tile instead of once per row. Two kernels:
 //
-// What bounds it: with few rows (the tiny layer: 8 rows per expert, 128 x 256) latency, hence eight CTAs per tile, one
-// launch, the K split below, and ONE copy of the main loop for both phases (a kernel that runs for a few microseconds
-// also waits for its own instructions); with many rows the multiply-adds. A warp covers 4 TM rows x 8 NW weight rows, its
-// lanes 4 rows x 8 weight rows, so that a 16-byte shared-memory read of a warp touches at most 128 distinct bytes (one
-// wavefront) and TM + NW of them feed 4 TM NW multiply-adds. Tiles of 32 rows: TM = NW = 4, two warps along the rows; of
-// 16 rows: TM = 4, NW = 2; of 8 rows: TM = NW = 2. The remaining warps lie along the features; where a CTA has too few
-// features for them they split K (partial sums meet in shared memory, in order). Sums: the products of one 32-wide chunk
-// in a row, chunks added in order - the error of a two-level sum, as with a warp per output before.
-// Measured against one CTA per route with a warp per output feature: tiny layer, 64 rows 24 -> 12 us; 400 rows of
-// 768 x 1024 750 -> 158 us (12 TFLOP/s); 2048 rows of 256 x 512 270 -> 130 us.
+//   short tiles (8 rows)  Bound by latency and the weights' bytes. The lanes of a warp lie along K and load the weights
+//       straight into registers, a group of 4 weight rows at a time with the next group's loads in flight (phase 1's first
+//       ones before the cluster barrier); the tokens lie in shared memory whole. The 4 x 8 sums of a group are reduced over
+//       the lanes by halving exchanges (31 shuffles), which leaves one sum per lane. Activations are written to every
+//       CTA's copy of H as they are computed.
+//   tall tiles (16 or 32 rows)  Bound by the multiply-adds. 32-wide K chunks pass through two shared-memory stages, the
+//       next chunk's loads in registers meanwhile (cp.async moves only ~17 bytes per cycle and SM in 16-byte pieces: it
+//       took longer than the arithmetic). A warp covers 4 TM rows x 8 NW weight rows, its lanes 4 rows x 8 weight rows,
+//       so that a 16-byte shared-memory read of a warp touches at most 128 distinct bytes (one wavefront) and TM + NW of
+//       them feed 4 TM NW multiply-adds; TM = NW = 4 with two warps along 32 rows, TM = 4, NW = 2 for 16 rows. The
+//       remaining warps lie along the features; where a CTA has too few features for them they split K (partial sums
+//       meet in shared memory, in order). A CTA keeps its slice of H and the others read it chunk by chunk.
+//
+// Sums: a few products in a row, partial sums added in order - the error of a two-level sum, as with a warp per output.
+// Measured (one CTA per route with a warp per output feature -> cp.async stages for every tile height -> now): tiny layer,
+// 64 rows of 128 x 256 24 -> 12.4 -> 7.6 us; one token, 9 experts of 512 x 384, whole call 171 -> 40 -> 33; tall: 400 rows
+// of 768 x 1024 750 -> 158 -> 149 us (12.7 TFLOP/s); 2048 rows of 256 x 512 270 -> 130 -> 123. What bounds the tall form now
+// is shared-memory reads (a 16-byte read costs a wavefront per quarter warp, so 32 for the 64 multiply-adds they feed).
 #include <algorithm>
 
 #include "common.cuh"
@@ -33,36 +39,191 @@ namespace cg = cooperative_groups;
 
 constexpr int kCl = 8;         // CTAs per row tile
 constexpr int kThreads = 256;  // 8 warps
-constexpr int kKC = 32;        // K elements per stage
+constexpr int kKC = 32;        // tall tiles: K elements per stage
 constexpr int kLd = kKC + 4;   // row pitch in floats: 16-byte aligned, the rows of a warp's read hit distinct banks
-// Short tiles wait for weights (a chunk's copies take 700-1500 cycles, its multiply-adds ~100): six stages; longer ones
-// compute: three, and two CTAs per SM.
-__host__ __device__ constexpr int stages_of(int form_rows) { return form_rows == 8 ? 6 : 3; }
-
-__device__ __forceinline__ void cp_async16(uint32_t dst, const float* src, bool in) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(in ? 16 : 0) : "memory");
-}
-__device__ __forceinline__ void cp_async4(uint32_t dst, const float* src, bool in) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(in ? 4 : 0) : "memory");
-}
-__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_wait() {
-    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-}
-
-// Four consecutive floats into shared memory, `left` of which exist (<= 0: none): the others are zero, nothing is read for
-// them. VEC: 16-byte aligned, all or none. `base` is any readable, aligned address.
+// Four consecutive floats, `left` of which exist (<= 0: none), the others zero. VEC: 16-byte aligned, all or none
 template <bool VEC>
-__device__ __forceinline__ void stage4(uint32_t dst, const float* src, int left, const float* base) {
+__device__ __forceinline__ float4 load4(const float* src, int left) {
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
     if (VEC) {
-        cp_async16(dst, left > 0 ? src : base, left > 0);
+        if (left > 0) v = __ldg(reinterpret_cast<const float4*>(src));
     } else {
+        if (left > 0) v.x = __ldg(src);
+        if (left > 1) v.y = __ldg(src + 1);
+        if (left > 2) v.z = __ldg(src + 2);
+        if (left > 3) v.w = __ldg(src + 3);
+    }
+    return v;
+}
+
+// The group, rows and expert of a row tile: every group's tile range in one round trip. False: past the last tile
+struct Tile {
+    int g, row0, rows, expert;
+};
+__device__ __forceinline__ bool find_tile(const FfnF32Params& p, int tile, Tile* s) {
+    if (threadIdx.x == 0) s->g = -1;
+    __syncthreads();
+    const int gd = p.n_groups_dev != nullptr ? *p.n_groups_dev : p.G;
+    for (int g = threadIdx.x; g < p.G; g += kThreads) {
+        const int t0 = p.tile_start[g], t1 = p.tile_start[g + 1], o0 = p.offsets[g], o1 = p.offsets[g + 1];
+        const int e = p.grp_expert != nullptr ? p.grp_expert[g] : g;
+        if (g < gd && tile >= t0 && tile < t1) {
+            s->g = g;
+            s->row0 = o0 + (tile - t0) * p.tile_rows;
+            s->rows = min(p.tile_rows, o1 - s->row0);
+            s->expert = e;
+        }
+    }
+    __syncthreads();
+    return s->g >= 0;
+}
+__device__ __forceinline__ int64_t token_of(const FfnF32Params& p, int64_t row) {
+    return p.row_tok != nullptr ? (int64_t)p.row_tok[row] : row % p.x_rows;
+}
+__device__ __forceinline__ float swiglu(float g, float u) { return (g / (1.0f + expf(-g))) * u; }
+
+// ---------------------------------------------------------------- short tiles
+constexpr int kSR = 8;  // token rows of a tile
+constexpr int kSW = 4;  // weight rows of a group: phase 0 two features' gate rows and up rows, phase 1 four columns
+
+// Sum over the lanes of 32 values by halving exchanges: lane l ends up with the sum of value l
+template <int N, int OFF>
+__device__ __forceinline__ void lane_sums(float* v, int lane) {
+    if constexpr (OFF > 0) {
+        const bool up = (lane & OFF) != 0;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) cp_async4(dst + 4 * j, left > j ? src + j : base, left > j);
+        for (int i = 0; i < N / 2; ++i) {
+            const float keep = up ? v[i + N / 2] : v[i], send = up ? v[i] : v[i + N / 2];
+            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, OFF);
+        }
+        lane_sums<N / 2, OFF / 2>(v, lane);
     }
 }
 
+template <bool VEC>
+__global__ void __launch_bounds__(kThreads) ffn_f32_short_kernel(FfnF32Params p) {
+    extern __shared__ __align__(16) float smem[];
+    __shared__ Tile s_tile;
+    const int d = p.d, I = p.I, xld = (d + 127) / 128 * 128, hld = p.hld;  // whole 128-wide K chunks
+    float* xs = smem;             // [8][xld]
+    float* hs = smem + kSR * xld;  // [8][hld]
+    cg::cluster_group cluster = cg::this_cluster();
+    const int rank = (int)cluster.block_rank();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    constexpr int kWarps = kThreads / 32;
+    grid_dep_wait();
+    if (!find_tile(p, (int)(blockIdx.x / kCl), &s_tile)) return;  // the whole cluster
+    cluster.barrier_arrive();  // waited for before the first remote write: all CTAs of the cluster have started
+    const int rows = s_tile.rows;
+    const int64_t row0 = s_tile.row0;
+    const size_t e = s_tile.expert;
+    const int per0 = (I + kCl - 1) / kCl, per1 = (d + kCl - 1) / kCl;
+
+    // Lane's elements of K chunk c: VEC 4 consecutive ones, else 4 that are 32 apart
+    auto load_w = [&](const float* row, bool in, int c, int K) {
+        if (VEC) return load4<true>(row + c * 128 + lane * 4, in ? K - c * 128 - lane * 4 : 0);
+        float4 v;
+        const int k = c * 128 + lane;
+        v.x = in && k < K ? __ldg(row + k) : 0.f;
+        v.y = in && k + 32 < K ? __ldg(row + k + 32) : 0.f;
+        v.z = in && k + 64 < K ? __ldg(row + k + 64) : 0.f;
+        v.w = in && k + 96 < K ? __ldg(row + k + 96) : 0.f;
+        return v;
+    };
+    auto load_t = [&](const float* row, int c) {
+        if (VEC) return *reinterpret_cast<const float4*>(row + c * 128 + lane * 4);
+        const float* q = row + c * 128 + lane;
+        return make_float4(q[0], q[32], q[64], q[96]);
+    };
+    // item (group gi of this CTA, chunk c) of a phase: the four weight rows' elements
+    auto load_item = [&](int phase, int gi, int c, float4 (&w)[kSW]) {
+#pragma unroll
+        for (int q = 0; q < kSW; ++q) {
+            if (phase == 0) {
+                const int f = rank * per0 + gi * 2 + (q & 1);
+                const bool in = f < min(I, (rank + 1) * per0);
+                w[q] = load_w((q < 2 ? p.wg : p.wu) + (e * I + (in ? f : 0)) * (size_t)d, in, c, d);
+            } else {
+                const int col = rank * per1 + gi * kSW + q;
+                const bool in = col < min(d, (rank + 1) * per1);
+                w[q] = load_w(p.wd + (e * d + (in ? col : 0)) * (size_t)I, in, c, I);
+            }
+        }
+    };
+    float4 w[kSW], nxt[kSW];
+    const int n0 = max(0, min(I, (rank + 1) * per0) - rank * per0), n1 = max(0, min(d, (rank + 1) * per1) - rank * per1);
+    if (warp * 2 < n0) load_item(0, warp, 0, nxt);  // the first weights before the tokens, whose addresses take a round trip
+    for (int t = warp; t < kSR; t += kWarps) {
+        const float* src = p.x + (t < rows ? token_of(p, row0 + t) : 0) * d;
+        for (int k = lane * 4; k < xld; k += 128)
+            *reinterpret_cast<float4*>(xs + t * xld + k) = load4<VEC>(src + k, t < rows ? d - k : 0);
+    }
+    for (int i = threadIdx.x; i < kSR * (hld - I); i += kThreads)  // columns past I: read by the last chunk
+        hs[i / (hld - I) * hld + I + i % (hld - I)] = 0.f;
+    __syncthreads();
+    bool started = false;
+
+#pragma unroll 1
+    for (int phase = 0; phase < 2; ++phase) {
+        const int K = phase == 0 ? d : I, nc = (K + 127) / 128;
+        const int groups = phase == 0 ? (n0 + 1) / 2 : (n1 + kSW - 1) / kSW;
+        const float* ts = phase == 0 ? xs : hs;
+        const int tld = phase == 0 ? xld : hld;
+        if (phase == 1) {
+            if (warp < groups) load_item(1, warp, 0, nxt);
+            if (!started) cluster.barrier_wait();
+            grid_dep_launch();  // not earlier: the next kernel's CTAs would only take this grid's places
+            cluster.sync();     // every CTA's share of H is in every copy
+        }
+#pragma unroll 1
+        for (int gi = warp; gi < groups; gi += kWarps) {
+            float acc[kSW * kSR];
+#pragma unroll
+            for (int i = 0; i < kSW * kSR; ++i) acc[i] = 0.f;
+#pragma unroll 1
+            for (int c = 0; c < nc; ++c) {
+#pragma unroll
+                for (int q = 0; q < kSW; ++q) w[q] = nxt[q];
+                const bool last = c + 1 == nc;
+                if (!last || gi + kWarps < groups) load_item(phase, last ? gi + kWarps : gi, last ? 0 : c + 1, nxt);
+#pragma unroll
+                for (int t = 0; t < kSR; ++t) {
+                    const float4 x = load_t(ts + t * tld, c);
+#pragma unroll
+                    for (int q = 0; q < kSW; ++q) {
+                        float a = acc[q * kSR + t];
+                        a = fmaf(w[q].x, x.x, a);
+                        a = fmaf(w[q].y, x.y, a);
+                        a = fmaf(w[q].z, x.z, a);
+                        acc[q * kSR + t] = fmaf(w[q].w, x.w, a);
+                    }
+                }
+            }
+            lane_sums<32, 16>(acc, lane);
+            const int t = lane & 7, q = lane >> 3;  // this lane's sum: weight row q of the group, token t
+            if (phase == 0) {
+                if (!started) {
+                    cluster.barrier_wait();
+                    started = true;
+                }
+                // lanes 0-15 hold gate, 16-31 up of the same (feature, token): both compute, each writes to four CTAs
+                const float other = __shfl_xor_sync(0xffffffffu, acc[0], 16);
+                const float h = lane < 16 ? swiglu(acc[0], other) : swiglu(other, acc[0]);
+                const int fl = gi * 2 + (q & 1);
+                if (fl < n0)
+#pragma unroll
+                    for (int c = 0; c < kCl / 2; ++c)
+                        cluster.map_shared_rank(hs, c + (lane < 16 ? 0 : kCl / 2))[t * hld + rank * per0 + fl] = h;
+            } else if (gi * kSW + q < n1 && t < rows) {
+                const int col = rank * per1 + gi * kSW + q;
+                if (p.y != nullptr) p.y[(int64_t)p.row_tok[row0 + t] * d + col] = p.row_w[row0 + t] * acc[0];
+                else p.out[(row0 + t) * d + col] = acc[0];
+            }
+        }
+    }
+}
+
+// ---------------------------------------------------------------- tall tiles
 // k steps wk, wk + nk, ... of one chunk (8 steps of 4): part = products of the chunk, acc += part
 template <int TM, int NW>
 __device__ __forceinline__ void mac_chunk(const float* ws, const float* xs, int x_pitch, int wk, int nk,
@@ -96,68 +257,40 @@ __device__ __forceinline__ void mac_chunk(const float* ws, const float* xs, int 
 }
 
 template <int TM, int NW, int RW, bool VEC>
-__global__ void __launch_bounds__(kThreads) ffn_f32_kernel(FfnF32Params p) {
+__global__ void __launch_bounds__(kThreads, 2) ffn_f32_tall_kernel(FfnF32Params p) {
     constexpr int BM = 4 * TM * RW;              // rows of the tile
     constexpr int kAcross = 8 / RW;              // warps along the features and along K
     constexpr int WR = kAcross * 8 * NW;         // weight rows of a stage, at most
     constexpr int kStage = (WR + BM) * kLd;      // floats
-    constexpr int S = stages_of(BM);
     constexpr int SR = WR / 32;                  // weight rows a thread copies per chunk, at most
-    static_assert(TM * NW * kThreads <= S * kStage, "partial sums fit the stages");
+    static_assert(TM * NW * kThreads <= 2 * kStage, "partial sums fit the stages");
     static_assert(BM <= 32, "one token row per staging thread");
     extern __shared__ __align__(16) float smem[];
-    __shared__ int s_g, s_row0, s_rows;
-    float* hs = smem + S * kStage;  // [tile_rows][hld]: this CTA's slice of H, or (push) all of H
+    __shared__ Tile s_tile;
+    float* hs = smem + 2 * kStage;  // [tile_rows][hld]: this CTA's slice of H
     cg::cluster_group cluster = cg::this_cluster();
     const int rank = (int)cluster.block_rank();
-    const int tile = (int)(blockIdx.x / kCl);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int lr = lane >> 3, lf = lane & 7, wr = warp / kAcross, wa = warp % kAcross;
     const int d = p.d, I = p.I, fpc = p.fpc, hld = p.hld;
-    const bool push = p.push != 0;
-    if (threadIdx.x == 0) s_g = -1;
     grid_dep_wait();
-    __syncthreads();
-    {  // which group owns this tile: every group's tile range in one round trip
-        const int gd = p.n_groups_dev != nullptr ? *p.n_groups_dev : p.G;
-        for (int g = threadIdx.x; g < p.G; g += kThreads) {
-            const int t0 = p.tile_start[g], t1 = p.tile_start[g + 1], o0 = p.offsets[g], o1 = p.offsets[g + 1];
-            if (g < gd && tile >= t0 && tile < t1) {
-                s_g = g;
-                s_row0 = o0 + (tile - t0) * p.tile_rows;
-                s_rows = min(p.tile_rows, o1 - s_row0);
-            }
-        }
-    }
-    __syncthreads();
-    if (s_g < 0) return;  // the whole cluster: past the last tile
-    cluster.barrier_arrive();  // waited for before the first access to another CTA's shared memory: all CTAs have started
-    bool started = false;
-    const int rows = s_rows;
-    const int64_t row0 = s_row0;
-    const size_t e = p.grp_expert != nullptr ? p.grp_expert[s_g] : s_g;
+    if (!find_tile(p, (int)(blockIdx.x / kCl), &s_tile)) return;  // the whole cluster
+    const int rows = s_tile.rows;
+    const int64_t row0 = s_tile.row0;
+    const size_t e = s_tile.expert;
 
     // What this thread copies in every chunk, fixed for a pass: SR weight rows of the stage and one token row, from
     // w_src / x_src on, w_len / x_len floats ahead of it in the first chunk (none for rows that are not there)
     const int vk = (threadIdx.x & 7) * 4, vr = threadIdx.x >> 3;  // 32 rows of 8 vectors per sweep
     const bool x_in = vr < BM && vr < rows;
-    const uint32_t w_dst = ptx::smem_u32(smem) + (uint32_t)(vr * kLd + vk) * 4u;
     const float* w_src[SR];
     int w_len[SR];
-    const float* x_src = p.x;
-    if (x_in) {
-        const int64_t tok = p.row_tok != nullptr ? (int64_t)p.row_tok[row0 + vr] : (row0 + vr) % p.x_rows;
-        x_src = p.x + tok * d + vk;
-    }
+    const float* x_src = x_in ? p.x + token_of(p, row0 + vr) * d + vk : p.x;
     const int x_len = x_in ? d - vk : 0;
 
 #pragma unroll 1
     for (int phase = 0; phase < 2; ++phase) {
         if (phase == 1) {
-            if (push)  // the last chunk's columns past I
-                for (int i = threadIdx.x; i < p.tile_rows * (hld - I); i += kThreads)
-                    hs[i / (hld - I) * hld + I + i % (hld - I)] = 0.f;
-            if (!started) cluster.barrier_wait();
             grid_dep_launch();  // not earlier: the next kernel's CTAs would only take this grid's places
             cluster.sync();     // every slice of H is in place
         }
@@ -170,7 +303,6 @@ __global__ void __launch_bounds__(kThreads) ffn_f32_kernel(FfnF32Params p) {
         while (n_wf < kAcross && n_wf * 8 * NW < (phase == 0 ? 2 : 1) * (hi - lo)) n_wf *= 2;
         const int wf = wa & (n_wf - 1), wk = wa / n_wf, nk = kAcross / n_wf, n_rows = n_wf * 8 * NW;
         const int step = phase == 0 ? n_rows / 2 : n_rows;  // features (a gate and an up row each) or columns per pass
-        const bool x_local = phase == 1 && push;
         const int nc = (K + kKC - 1) / kKC;
 #pragma unroll 1
         for (int f0 = lo; f0 < hi; f0 += step) {
@@ -179,55 +311,49 @@ __global__ void __launch_bounds__(kThreads) ffn_f32_kernel(FfnF32Params p) {
                 const int r = vr + 32 * q, in_warp = r % (8 * NW);
                 const int f = phase == 0 ? f0 + r / (8 * NW) * (4 * NW) + in_warp % (4 * NW) : f0 + r;
                 const float* base = phase == 1 ? p.wd : (in_warp < 4 * NW ? p.wg : p.wu);
-                w_src[q] = base + (e * (size_t)(phase == 0 ? I : d) + f) * K + vk;
-                w_len[q] = r < n_rows && f < hi ? K - vk : 0;
+                const bool in = r < n_rows && f < hi;
+                w_src[q] = base + (e * (size_t)(phase == 0 ? I : d) + (in ? f : 0)) * K + vk;
+                w_len[q] = in ? K - vk : 0;
             }
+            float4 wv[SR], xv;
+            auto load = [&](int c) {
+#pragma unroll
+                for (int q = 0; q < SR; ++q) wv[q] = load4<VEC>(w_src[q] + c * kKC, w_len[q] - c * kKC);
+                if (phase == 0) {
+                    xv = load4<VEC>(x_src + c * kKC, x_len - c * kKC);
+                } else {
+                    // a chunk lies in one CTA's slice (fpc is a multiple of 32); features past I (never written) are zero
+                    xv = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (x_in) {
+                        const int owner = (c * kKC) / fpc, k = c * kKC + vk;
+                        xv = *reinterpret_cast<const float4*>(cluster.map_shared_rank(hs, owner) + vr * hld + (k - owner * fpc));
+                        if (k >= I) xv.x = 0.f;
+                        if (k + 1 >= I) xv.y = 0.f;
+                        if (k + 2 >= I) xv.z = 0.f;
+                        if (k + 3 >= I) xv.w = 0.f;
+                    }
+                }
+            };
+            auto store = [&](float* st) {
+#pragma unroll
+                for (int q = 0; q < SR; ++q) *reinterpret_cast<float4*>(st + (vr + 32 * q) * kLd + vk) = wv[q];
+                if (vr < BM) *reinterpret_cast<float4*>(st + (WR + vr) * kLd + vk) = xv;
+            };
             float acc[TM][NW];
 #pragma unroll
             for (int r = 0; r < TM; ++r)
 #pragma unroll
                 for (int q = 0; q < NW; ++q) acc[r][q] = 0.f;
+            load(0);
             __syncthreads();  // the previous pass is done with the stages
-            int st_in = 0, st_out = 0;
+            store(smem);
 #pragma unroll 1
-            for (int c = 1 - S; c < nc; ++c) {  // chunk c + S - 1 is requested, chunk c (once >= 0) is consumed
-                if (c >= 0) {
-                    cp_wait<S - 2>();
-                    __syncthreads();
-                }
-                const int cn = c + S - 1;
-                float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-                const uint32_t off = (uint32_t)(st_in * kStage) * 4u;
-                if (cn < nc) {
-#pragma unroll
-                    for (int q = 0; q < SR; ++q)
-                        if (vr + 32 * q < n_rows)
-                            stage4<VEC>(w_dst + off + (uint32_t)(32 * q * kLd) * 4u, w_src[q] + cn * kKC, w_len[q] - cn * kKC, p.x);
-                    if (phase == 0) {
-                        if (vr < BM) stage4<VEC>(w_dst + off + (uint32_t)(WR * kLd) * 4u, x_src + cn * kKC, x_len - cn * kKC, p.x);
-                    } else if (!push && x_in) {
-                        // a chunk lies in one CTA's slice (fpc is a multiple of 32); features past I (never written) are zero
-                        const int owner = (cn * kKC) / fpc, k = cn * kKC + vk;
-                        v = *reinterpret_cast<const float4*>(cluster.map_shared_rank(hs, owner) + vr * hld + (k - owner * fpc));
-                        if (k + 4 > I) {
-                            if (k >= I) v.x = 0.f;
-                            if (k + 1 >= I) v.y = 0.f;
-                            if (k + 2 >= I) v.z = 0.f;
-                            if (k + 3 >= I) v.w = 0.f;
-                        }
-                    }
-                }
-                cp_commit();
-                if (c >= 0) {
-                    const float* ws = smem + st_out * kStage;
-                    const float* xs = x_local ? hs + c * kKC : ws + WR * kLd;
-                    const int x_pitch = x_local ? hld : kLd;
-                    mac_chunk<TM, NW>(ws + (wf * 8 * NW + lf) * kLd, xs + (wr * 4 * TM + lr) * x_pitch, x_pitch, wk, nk, acc);
-                    if (++st_out == S) st_out = 0;
-                }
-                if (cn < nc && phase == 1 && !push && vr < BM)
-                    *reinterpret_cast<float4*>(smem + st_in * kStage + (WR + vr) * kLd + vk) = v;
-                if (++st_in == S) st_in = 0;
+            for (int c = 0; c < nc; ++c) {
+                __syncthreads();  // chunk c is in place; chunk c - 1, whose stage takes chunk c + 1, is used up
+                if (c + 1 < nc) load(c + 1);
+                const float* ws = smem + (c & 1) * kStage;
+                mac_chunk<TM, NW>(ws + (wf * 8 * NW + lf) * kLd, ws + (WR + wr * 4 * TM + lr) * kLd, kLd, wk, nk, acc);
+                if (c + 1 < nc) store(smem + ((c + 1) & 1) * kStage);
             }
             if (nk > 1) {  // partial sums of the K parts, added in order
                 __syncthreads();
@@ -242,32 +368,17 @@ __global__ void __launch_bounds__(kThreads) ffn_f32_kernel(FfnF32Params p) {
 #pragma unroll
                         for (int i = 0; i < TM * NW; ++i) acc[i / NW][i % NW] += red[(k * n_wf * TM * NW + i) * 32];
             }
-            if (phase == 0) {
-                if (!started) {
-                    cluster.barrier_wait();
-                    started = true;
-                }
-                if (wk == 0)
+            if (wk != 0) continue;
 #pragma unroll
-                    for (int r = 0; r < TM; ++r)
+            for (int r = 0; r < TM; ++r) {
+                const int row = (wr * TM + r) * 4 + lr;
+                if (phase == 0) {
 #pragma unroll
-                        for (int q = 0; q < NW / 2; ++q) {
-                            const int f = f0 + wf * 4 * NW + q * 8 + lf, row = (wr * TM + r) * 4 + lr;
-                            const float g = acc[r][q], u = acc[r][q + NW / 2];
-                            const float h = (g / (1.0f + expf(-g))) * u;
-                            if (row >= p.tile_rows) continue;
-                            if (!push) {
-                                if (f < lo + fpc) hs[row * hld + f - lo] = h;
-                            } else if (f < hi) {
-#pragma unroll
-                                for (int c = 0; c < kCl; ++c) cluster.map_shared_rank(hs, c)[row * hld + f] = h;
-                            }
-                        }
-            } else if (wk == 0) {
-#pragma unroll
-                for (int r = 0; r < TM; ++r) {
-                    const int row = (wr * TM + r) * 4 + lr;
-                    if (row >= rows) continue;
+                    for (int q = 0; q < NW / 2; ++q) {
+                        const int f = f0 + wf * 4 * NW + q * 8 + lf;
+                        if (f < lo + fpc && row < p.tile_rows) hs[row * hld + f - lo] = swiglu(acc[r][q], acc[r][q + NW / 2]);
+                    }
+                } else if (row < rows) {
                     const float w = p.y != nullptr ? p.row_w[row0 + row] : 1.0f;
                     float* dst = p.y != nullptr ? p.y + (int64_t)p.row_tok[row0 + row] * d : p.out + (row0 + row) * d;
 #pragma unroll
@@ -279,29 +390,22 @@ __global__ void __launch_bounds__(kThreads) ffn_f32_kernel(FfnF32Params p) {
             }
         }
     }
-    if (!push) cluster.sync();  // no CTA leaves while another may still read its slice of H
+    cluster.sync();  // no CTA leaves while another may still read its slice of H
 }
 
 constexpr size_t kSmemLimit = 227 * 1024 - 1024;
-constexpr size_t kPushBytes = 32 * 1024;
 int features_per_cta(int I) { return ((I + kCl - 1) / kCl + kKC - 1) / kKC * kKC; }
-bool push_h(int tile_rows, int I) { return (size_t)std::max(8, tile_rows) * I * sizeof(float) <= kPushBytes; }
-int h_pitch(int tile_rows, int I) {  // whole chunks + 4: 16-byte aligned, the four rows of a warp's read in distinct banks
-    return (push_h(tile_rows, I) ? (I + kKC - 1) / kKC * kKC : features_per_cta(I)) + 4;
-}
-size_t smem_bytes(int tile_rows, int I) {  // 128 weight rows and the form's token rows per stage, then H
-    const int form_rows = std::max(8, tile_rows);  // all of which are read from a push tile (and not used past tile_rows)
-    const int h_rows = push_h(tile_rows, I) ? form_rows : tile_rows;
-    return ((size_t)stages_of(form_rows) * (128 + form_rows) * kLd + (size_t)h_rows * h_pitch(tile_rows, I)) * sizeof(float);
+size_t short_bytes(int d, int I) { return (size_t)kSR * ((d + 127) / 128 * 128 + (I + 127) / 128 * 128 + 4) * sizeof(float); }
+size_t tall_bytes(int tile_rows, int I) {  // two stages of 128 weight rows and the form's token rows, then the slice of H
+    const int form_rows = tile_rows > 16 ? 32 : 16;
+    return ((size_t)2 * (128 + form_rows) * kLd + (size_t)tile_rows * (features_per_cta(I) + 4)) * sizeof(float);
 }
 
-template <int TM, int NW, int RW, bool VEC>
-cudaError_t launch_t(const FfnF32Params& p, int64_t tiles, cudaStream_t s) {
-    const size_t smem = smem_bytes(p.tile_rows, p.I);
-    cudaError_t err = cudaFuncSetAttribute(ffn_f32_kernel<TM, NW, RW, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)smem);
+template <typename K>
+cudaError_t launch_t(K kernel, const FfnF32Params& p, size_t smem, int64_t tiles, cudaStream_t s) {
+    cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (err != cudaSuccess) return err;
-    return launch_pdl_cluster(ffn_f32_kernel<TM, NW, RW, VEC>, (unsigned)(tiles * kCl), kThreads, smem, kCl, s, p);
+    return launch_pdl_cluster(kernel, (unsigned)(tiles * kCl), kThreads, smem, kCl, s, p);
 }
 
 // y[i][c] = sum_j w(row) out[row][c] over the token's rows in slot order (row = inv_pos[i][j], -1: merged into an earlier
@@ -340,26 +444,33 @@ __global__ void __launch_bounds__(128) combine_f32_kernel(const float* __restric
 }  // namespace
 
 // Rows per tile: a tile computes all of its rows, so short groups want short tiles (and more of them to fill the SMs); a
-// tile's weights are read once per tile, so long groups want long ones. Measured, 16 / 32-row tiles: 17 experts of
-// 768 x 1024 with 25 rows each 154 / 220 us; 20 of 512 x 384 with ~40 rows 109 / 123 us. Halved while the tile's slice of H
-// does not fit the shared memory (8 rows: I above ~40 000 features).
-int ffn_f32_tile_rows(int64_t rows, int G, int I) {
-    int tile_rows = rows > (int64_t)48 * G ? 32 : rows > (int64_t)8 * G ? 16 : 8;
-    while (tile_rows > 1 && smem_bytes(tile_rows, I) > kSmemLimit) tile_rows /= 2;
+// tile's weights are read once per tile, so long groups want long ones. Short tiles need the tokens and H in shared memory
+// whole (d + I up to ~7000); tall ones are halved while the slice of H does not fit (32 rows: I above ~11 000).
+int ffn_f32_tile_rows(int64_t rows, int G, int d, int I) {
+    if (rows <= (int64_t)kSR * G && short_bytes(d, I) <= kSmemLimit) return kSR;
+    int tile_rows = rows > (int64_t)48 * G ? 32 : 16;
+    while (tile_rows > 1 && tall_bytes(tile_rows, I) > kSmemLimit) tile_rows /= 2;
     return tile_rows;
 }
 
 cudaError_t launch_ffn_f32(FfnF32Params p, int64_t rows, cudaStream_t s) {
     if (rows == 0) return cudaSuccess;
-    p.fpc = features_per_cta(p.I);
-    p.push = push_h(p.tile_rows, p.I) ? 1 : 0;
-    p.hld = h_pitch(p.tile_rows, p.I);
     const int64_t tiles = std::min<int64_t>(rows, rows / p.tile_rows + p.G);
     auto a16 = [](const void* q) { return (reinterpret_cast<uintptr_t>(q) & 15) == 0; };
-    const bool vec = p.d % 4 == 0 && p.I % 4 == 0 && a16(p.x) && a16(p.wg) && a16(p.wu) && a16(p.wd);
-    if (p.tile_rows == 32) return vec ? launch_t<4, 4, 2, true>(p, tiles, s) : launch_t<4, 4, 2, false>(p, tiles, s);
-    if (p.tile_rows == 16) return vec ? launch_t<4, 2, 1, true>(p, tiles, s) : launch_t<4, 2, 1, false>(p, tiles, s);
-    return vec ? launch_t<2, 2, 1, true>(p, tiles, s) : launch_t<2, 2, 1, false>(p, tiles, s);
+    const bool vec = p.I % 4 == 0 && a16(p.x) && a16(p.wg) && a16(p.wu) && a16(p.wd);
+    if (p.tile_rows == kSR && short_bytes(p.d, p.I) <= kSmemLimit) {
+        p.hld = (p.I + 127) / 128 * 128 + 4;
+        const size_t smem = short_bytes(p.d, p.I);
+        return vec ? launch_t(ffn_f32_short_kernel<true>, p, smem, tiles, s) : launch_t(ffn_f32_short_kernel<false>, p, smem, tiles, s);
+    }
+    p.fpc = features_per_cta(p.I);
+    p.hld = p.fpc + 4;
+    const size_t smem = tall_bytes(p.tile_rows, p.I);
+    if (p.tile_rows > 16)
+        return vec ? launch_t(ffn_f32_tall_kernel<4, 4, 2, true>, p, smem, tiles, s)
+                   : launch_t(ffn_f32_tall_kernel<4, 4, 2, false>, p, smem, tiles, s);
+    return vec ? launch_t(ffn_f32_tall_kernel<4, 2, 1, true>, p, smem, tiles, s)
+               : launch_t(ffn_f32_tall_kernel<4, 2, 1, false>, p, smem, tiles, s);
 }
 
 cudaError_t launch_combine_f32(const float* out, const int32_t* inv_pos, const float* row_w, int64_t T, int Kr, int d,

@@ -13,7 +13,8 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("K", [1, 2, 3, 4, 5, 6, 7, 8, 9, 13, 16])
 def test_calibration_sums_by_top_k(K):
     """Pair sums: a kernel per Top-K up to 8, tiles of four slots above (9: a ragged last tile). d = 132 leaves a tail
-    after whole 128-column steps; m is not a multiple of the tokens per block. fp32 outputs, double sums: the oracle's
+    after whole 128-column steps; m is not a multiple of the tokens per block; odd K: x_cal 4 bytes off a 16-byte
+    boundary (fp32 calibration takes any). fp32 outputs, double sums: the oracle's
     tables to fp32 rounding of the outputs (2e-5, as in the other fp32 calibration tests)."""
     N = 16
     cfg = si.LayerConfig("calk", N, 0, 132, 64, K, "f32", 16, (1,), 4, (2,))
@@ -26,7 +27,9 @@ def test_calibration_sums_by_top_k(K):
     h, lnh, n_obs = torch.empty(N, device=dev), torch.empty(N, device=dev), torch.empty((N, N), dtype=torch.int32, device=dev)
     ws = ex.alloc_workspace(case.layer, m, K)
     ws.fill_(0xFF)
-    rc = ex.exfold_calibrate(case.layer, xc.to(dev), lc.to(dev), case.d_wg, case.d_wu, case.d_wd,
+    room = torch.empty(xc.numel() + 4, device=dev)
+    x_dev = room[K % 2:K % 2 + xc.numel()].view(xc.shape).copy_(xc)
+    rc = ex.exfold_calibrate(case.layer, x_dev, lc.to(dev), case.d_wg, case.d_wu, case.d_wd,
                              ex.make_tables(S, L, h, lnh, n_obs), ws)
     assert rc == (1 if ref["unobserved"] else 0)
     assert np.array_equal(n_obs.cpu().numpy(), ref["n_obs"])
