@@ -140,11 +140,13 @@ struct PrefillRouteParams {
     int32_t* omit_tgt;  // [T][K-Kp] or null
     int32_t* block_hist;  // [nblk][N]
     int32_t* sb_hist;     // [ceil(nblk / kRouteSuperBlock)][N] retained routes per (super-block, expert); the
-                          //   launcher clears it, the blocks add to it
+                          //   launcher clears it, the blocks add to it (not with a single super-block)
     DeviceStatus* status; // cleared by block 0 (first kernel of a call); may be null
 };
 constexpr int kRouteTokensPerBlock = 32;
 constexpr int kRouteThreads = 512;
+constexpr int kRouteMaxThreads = 1024;  // a warp per token of the block
+constexpr int kRouteFewBlocks = 148;    // up to this many blocks the kernels spread them over more threads or blocks
 constexpr int kRouteSuperBlock = 64;  // blocks per super-block of the two-level histogram
 
 struct PrefillScatterParams {
@@ -152,6 +154,7 @@ struct PrefillScatterParams {
     int N, n_shared, Kp, d_bytes;  // d_bytes: bytes of one x row (0: no gather)
     int nblk;                   // blocks of the route kernel (= blocks of this kernel)
     int tile_rows;              // rows per tile of the work list (kTileM, or the fp32 FFN's)
+    int split;                  // blocks per token block (set by the launcher)
     const int32_t* ids;         // [T][Kp]
     const float* w;             // [T][Kp]
     const int32_t* block_hist;  // [nblk][N] retained routes per (block, expert)
@@ -167,8 +170,8 @@ struct PrefillScatterParams {
     int32_t* inv_pos;   // [R] sorted row of each route (inverse of perm); may be null
 };
 
-cudaError_t launch_prefill_route(const PrefillRouteParams& p, cudaStream_t s);
-cudaError_t launch_prefill_scatter(const PrefillScatterParams& p, cudaStream_t s);
+cudaError_t launch_prefill_route(PrefillRouteParams p, cudaStream_t s);
+cudaError_t launch_prefill_scatter(PrefillScatterParams p, cudaStream_t s);
 
 // ---------------------------------------------------------------- routing (decode)
 struct DecodeRouteParams {

@@ -494,14 +494,18 @@ __global__ void __launch_bounds__(256) static_pool_kernel(int N, int M, const fl
 
 cudaError_t launch_decode_route(const DecodeRouteParams& p, cudaStream_t s) {
     const int npl = (p.N + 31) / 32;
+    // A small batch on a small layer is one CTA's work: the cluster barriers cost more than the other seven CTAs bring
+    // (whole decode call, 8 / 1 CTAs: 8 experts, Top-2, 64 tokens 42.4 / 35.9 us, 16 tokens 17.4 / 17.1; 30 experts, Top-6,
+    // 60 tokens 34.2 / 36.3)
+    const int ncl = p.N <= 32 && p.B * p.K <= 128 ? 1 : kDecCluster;
     // state + this CTA's rows of the two tables
-    const size_t smem = kDecSmemBytes + 2 * (size_t)((p.N + kDecCluster - 1) / kDecCluster) * p.N * sizeof(float);
+    const size_t smem = kDecSmemBytes + 2 * (size_t)((p.N + ncl - 1) / ncl) * p.N * sizeof(float);
     cudaError_t err = cudaSuccess;
 #define EXFOLD_DEC_LAUNCH(NPL)                                                                              \
     err = cudaFuncSetAttribute(decode_route_kernel<NPL>, cudaFuncAttributeMaxDynamicSharedMemorySize,       \
                                (int)smem);                                                                  \
     if (err != cudaSuccess) return err;                                                                     \
-    err = launch_pdl_cluster(decode_route_kernel<NPL>, kDecCluster, kDecThreads, smem, kDecCluster, s, p);
+    err = launch_pdl_cluster(decode_route_kernel<NPL>, ncl, kDecThreads, smem, ncl, s, p);
     switch (npl) {
         case 1: EXFOLD_DEC_LAUNCH(1) break;
         case 2: EXFOLD_DEC_LAUNCH(2) break;

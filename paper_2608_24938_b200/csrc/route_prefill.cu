@@ -13,6 +13,8 @@
 //                  row-tile prefix for the GEMM work list). It then ranks its routes in (token,
 //                  slot) order, so the permutation is the stable sort by expert and is
 //                  bit-reproducible; it also gathers the token rows into sorted order.
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace exfold {
@@ -20,11 +22,11 @@ namespace exfold {
 namespace {
 
 template <int NPL>  // logits per lane = ceil(N / 32)
-__global__ void __launch_bounds__(kRouteThreads) prefill_route_kernel(PrefillRouteParams p) {
+__global__ void __launch_bounds__(kRouteMaxThreads) prefill_route_kernel(PrefillRouteParams p) {
     __shared__ int hist[kMaxExperts];
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
-    constexpr int kWarps = kRouteThreads / 32;
+    const int kWarps = blockDim.x >> 5;
     grid_dep_launch();
     for (int e = threadIdx.x; e < p.N; e += blockDim.x) hist[e] = 0;
     __syncthreads();
@@ -174,6 +176,33 @@ __global__ void __launch_bounds__(kRouteThreads) prefill_route_kernel(PrefillRou
     }
 }
 
+// Exclusive prefix over N <= 256 counters held one per thread (threads e < N), all threads of the block call it;
+// *total receives the sum. `warp_tot` is shared scratch of kMaxExperts / 32 words.
+__device__ __forceinline__ int block_prefix(int v, int N, int* warp_tot, int* total) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int incl = 0;
+    if (warp * 32 < N) {
+        incl = v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int u = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += u;
+        }
+        if (lane == 31) warp_tot[warp] = incl;
+    }
+    __syncthreads();
+    int before = 0, all = 0;
+    for (int w = 0; w * 32 < N; ++w) {
+        if (w < warp) before += warp_tot[w];
+        all += warp_tot[w];
+    }
+    __syncthreads();
+    *total = all;
+    return before + incl - v;
+}
+
+// `split` blocks share a block of tokens: each derives the same bases and positions, the first writes the metadata, and the
+// rows to gather are dealt over them (few tokens would otherwise leave most SMs without rows to copy).
 __global__ void __launch_bounds__(kRouteThreads) prefill_scatter_kernel(PrefillScatterParams p) {
     __shared__ int cnt[kMaxExperts];
     __shared__ int pos[kRouteTokensPerBlock * kMaxTopK];
@@ -182,7 +211,8 @@ __global__ void __launch_bounds__(kRouteThreads) prefill_scatter_kernel(PrefillS
     __shared__ int warp_tot[kMaxExperts / 32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int N = p.N, Kp = p.Kp;
-    const int64_t tok0 = (int64_t)blockIdx.x * kRouteTokensPerBlock;
+    const int blk = (int)blockIdx.x / p.split, part = (int)blockIdx.x - blk * p.split;
+    const int64_t tok0 = (int64_t)blk * kRouteTokensPerBlock;
     const int ntok = (int)min((int64_t)kRouteTokensPerBlock, p.T - tok0);
     const int n = ntok * Kp;
     const int64_t r0 = tok0 * Kp;
@@ -192,14 +222,22 @@ __global__ void __launch_bounds__(kRouteThreads) prefill_scatter_kernel(PrefillS
     grid_dep_wait();
     // Bases of this block: first sorted position of expert e = (rows of experts < e) + (rows of e in
     // earlier blocks). Super-block rows first (nsb of them), then the block rows before this one inside
-    // its super-block: nsb + 63 rows of N counters at most, whatever the token count.
+    // its super-block: nsb + 63 rows of N counters at most, whatever the token count. With a single
+    // super-block the block rows serve both sums.
     {
-        const int sb = (int)blockIdx.x / kRouteSuperBlock, nsb = (p.nblk + kRouteSuperBlock - 1) / kRouteSuperBlock;
-        const int b0 = sb * kRouteSuperBlock, n_inner = (int)blockIdx.x - b0;
-        const int n_rows = nsb + n_inner;
+        const int sb = blk / kRouteSuperBlock, nsb = (p.nblk + kRouteSuperBlock - 1) / kRouteSuperBlock;
+        const bool one = nsb == 1;
+        const int b0 = sb * kRouteSuperBlock;
+        const int n_rows = one ? p.nblk : nsb + blk - b0;
         for (int idx = threadIdx.x; idx < n_rows * N; idx += blockDim.x) {
             const int row = idx / N, e = idx - row * N;
-            if (row < nsb) {
+            if (one) {
+                const int v = p.block_hist[idx];
+                if (v != 0) {
+                    atomicAdd(&tot[e], v);
+                    if (row < blk) atomicAdd(&pre[e], v);
+                }
+            } else if (row < nsb) {
                 const int v = p.sb_hist[(size_t)row * N + e];
                 if (v != 0) {
                     atomicAdd(&tot[e], v);
@@ -212,37 +250,28 @@ __global__ void __launch_bounds__(kRouteThreads) prefill_scatter_kernel(PrefillS
         }
     }
     __syncthreads();
-    // exclusive prefix of tot over the experts: warp w scans experts [32w, 32w + 32)
-    if (warp * 32 < N) {
-        const int e = warp * 32 + lane;
-        const int v = e < N ? tot[e] : 0;
-        int incl = v;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int u = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += u;
+    {
+        const int e = threadIdx.x;  // N <= 256 <= the block
+        const int rows = e < N ? tot[e] : 0;
+        int all_rows, all_tiles;
+        const int off = block_prefix(rows, N, warp_tot, &all_rows);
+        if (e < N) cnt[e] = off + pre[e];
+        if (blockIdx.x == 0) {  // group offsets and the row-tile prefix for the GEMM work list
+            const int tiles = (rows + p.tile_rows - 1) / p.tile_rows;
+            const int tile0 = block_prefix(tiles, N, warp_tot, &all_tiles);
+            if (e < N) {
+                p.offsets[e] = off;
+                p.work_start[e] = tile0;
+            }
+            if (e == 0) {
+                p.offsets[N] = all_rows;
+                p.work_start[N] = all_tiles;
+                if (p.n_shared) {
+                    p.offsets[N + 1] = all_rows + (int)p.T;
+                    p.work_start[N + 1] = all_tiles + (int)((p.T + p.tile_rows - 1) / p.tile_rows);
+                }
+            }
         }
-        if (e < N) cnt[e] = incl - v;
-        if (lane == 31) warp_tot[warp] = incl;
-    }
-    __syncthreads();
-    for (int e = threadIdx.x; e < N; e += blockDim.x) {
-        int off = 0;
-        for (int w = 0; w < (e >> 5); ++w) off += warp_tot[w];
-        cnt[e] += off + pre[e];
-    }
-    if (blockIdx.x == 0 && threadIdx.x == 0) {  // group offsets and the row-tile prefix for the GEMM work list
-        const int G = N + p.n_shared;
-        int off = 0, tiles = 0;
-        for (int g = 0; g < G; ++g) {
-            const int rows = g < N ? tot[g] : (int)p.T;
-            p.offsets[g] = off;
-            p.work_start[g] = tiles;
-            off += rows;
-            tiles += (rows + p.tile_rows - 1) / p.tile_rows;
-        }
-        p.offsets[G] = off;
-        p.work_start[G] = tiles;
     }
     __syncthreads();
     if (warp == 0) {
@@ -262,7 +291,7 @@ __global__ void __launch_bounds__(kRouteThreads) prefill_scatter_kernel(PrefillS
         }
     }
     __syncthreads();
-    for (int r = threadIdx.x; r < n; r += blockDim.x) {
+    for (int r = threadIdx.x; part == 0 && r < n; r += blockDim.x) {
         int q = pos[r];
         int64_t route = r0 + r;
         p.perm[q] = (int32_t)route;
@@ -271,7 +300,7 @@ __global__ void __launch_bounds__(kRouteThreads) prefill_scatter_kernel(PrefillS
         p.row_w[q] = p.w[route];
         p.row_exp[q] = p.ids[route];
     }
-    if (p.n_shared) {  // shared-expert rows follow the routed rows, identity order, weight 1
+    if (p.n_shared && part == 0) {  // shared-expert rows follow the routed rows, identity order, weight 1
         const int64_t R = p.T * Kp;
         for (int t = threadIdx.x; t < ntok; t += blockDim.x) {
             p.row_tok[R + tok0 + t] = (int32_t)(tok0 + t);
@@ -283,7 +312,7 @@ __global__ void __launch_bounds__(kRouteThreads) prefill_scatter_kernel(PrefillS
         // gather: sorted row pos[r] <- token row; one warp per route, 16-byte chunks
         const int chunks = p.d_bytes >> 4;
         const int nwarps = blockDim.x >> 5;
-        for (int r = warp; r < n; r += nwarps) {
+        for (int r = part * nwarps + warp; r < n; r += p.split * nwarps) {
             const uint4* src = reinterpret_cast<const uint4*>(
                 reinterpret_cast<const char*>(p.x) + (size_t)((r0 + r) / Kp) * p.d_bytes);
             uint4* dst = reinterpret_cast<uint4*>(reinterpret_cast<char*>(p.xs) + (size_t)pos[r] * p.d_bytes);
@@ -294,25 +323,36 @@ __global__ void __launch_bounds__(kRouteThreads) prefill_scatter_kernel(PrefillS
 
 }  // namespace
 
-cudaError_t launch_prefill_route(const PrefillRouteParams& p, cudaStream_t s) {
+cudaError_t launch_prefill_route(PrefillRouteParams p, cudaStream_t s) {
     const int nblk = (int)((p.T + kRouteTokensPerBlock - 1) / kRouteTokensPerBlock);
     const int npl = (p.N + 31) / 32;
-    if (p.sb_hist != nullptr) {  // the super-block histograms are added up with atomics: they start at zero
+    // No more blocks than SMs: a warp per token, the time is one token's chain of loads and reductions (777 tokens of 128
+    // experts 9.6 -> 7.9 us). More blocks fill the SMs either way (8192 tokens 17.2 us, with a warp per token 17.7).
+    const int threads = nblk <= kRouteFewBlocks ? kRouteMaxThreads : kRouteThreads;
+    if (nblk <= kRouteSuperBlock) {
+        p.sb_hist = nullptr;  // one super-block: the scatter kernel adds up the block rows itself
+    } else {  // the super-block histograms are added up with atomics: they start at zero
         const size_t nsb = (size_t)(nblk + kRouteSuperBlock - 1) / kRouteSuperBlock;
         cudaError_t e = cudaMemsetAsync(p.sb_hist, 0, nsb * p.N * sizeof(int32_t), s);
         if (e != cudaSuccess) return e;
     }
     switch (npl) {
-        case 1: return launch_pdl(prefill_route_kernel<1>, nblk, kRouteThreads, 0, s, p);
-        case 2: return launch_pdl(prefill_route_kernel<2>, nblk, kRouteThreads, 0, s, p);
-        case 3: case 4: return launch_pdl(prefill_route_kernel<4>, nblk, kRouteThreads, 0, s, p);
-        default: return launch_pdl(prefill_route_kernel<8>, nblk, kRouteThreads, 0, s, p);
+        case 1: return launch_pdl(prefill_route_kernel<1>, nblk, threads, 0, s, p);
+        case 2: return launch_pdl(prefill_route_kernel<2>, nblk, threads, 0, s, p);
+        case 3: case 4: return launch_pdl(prefill_route_kernel<4>, nblk, threads, 0, s, p);
+        default: return launch_pdl(prefill_route_kernel<8>, nblk, threads, 0, s, p);
     }
 }
 
-cudaError_t launch_prefill_scatter(const PrefillScatterParams& p, cudaStream_t s) {
+cudaError_t launch_prefill_scatter(PrefillScatterParams p, cudaStream_t s) {
     const int nblk = (int)((p.T + kRouteTokensPerBlock - 1) / kRouteTokensPerBlock);
-    return launch_pdl(prefill_scatter_kernel, nblk, kRouteThreads, 0, s, p);
+    // a warp copies a row at a time: as many blocks per token block as leave every warp a row or two, on ~2 blocks per SM
+    // (777 tokens x 6 rows of 4 KB: 25 blocks 22.2 us, 275 blocks 12.1)
+    const int64_t rows_per_block = (int64_t)kRouteTokensPerBlock * p.Kp;
+    p.split = 1;
+    if (p.xs != nullptr && p.d_bytes > 0)
+        p.split = (int)std::max<int64_t>(1, std::min<int64_t>(2 * kRouteFewBlocks / nblk, rows_per_block / (kRouteThreads / 32)));
+    return launch_pdl(prefill_scatter_kernel, nblk * p.split, kRouteThreads, 0, s, p);
 }
 
 }  // namespace exfold

@@ -60,3 +60,15 @@ def test_f32_layer_shapes(shape):
     got, ref = case.run_decode(M), case.oracle_decode(M)
     check_decode_meta(got, ref, M)
     assert check_output(got["y"], ref["y"], "f32")[1] < 2e-6
+
+
+@pytest.mark.parametrize("T", [1, 31, 33, 777, 2048, 2049, 4800])
+def test_routing_block_forms(T):
+    """Route / scatter kernels around their block rules: one token, part blocks, token blocks shared by several blocks,
+    the last call with a single super-block (2048 tokens) and the first ones with two, more blocks than SMs. Bit-exact
+    permutation and offsets; every row gathered (outputs to the bf16 bound)."""
+    cfg = si.LayerConfig("blocks", 40, 1, 128, 64, 5, "bf16", T, (3,), 4, (2,), logits="zipf")
+    case = Case(cfg)
+    got, ref = case.run_prefill(3), case.oracle_prefill(3)
+    check_prefill_meta(got, ref)
+    check_output(got["y"], ref["y"], "bf16")
