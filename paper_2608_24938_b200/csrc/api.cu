@@ -489,9 +489,11 @@ int exfold_moe_prefill_ex(const exfold_layer* layer, const void* x, const float*
     }
 
     prof_reset();
-    // The kernels of an fp32 layer are short: chained by programmatic dependent launch. The bf16 path launches plainly
-    // (early-resident successors compete with the running kernels: 19-32 us slower).
-    PdlScope pdl_scope(!bf16);
+    // Calls without the CTA-pair passes (fp32 layers, shorter bf16 prompts) are a chain of short kernels on one stream:
+    // programmatic dependent launch hides their launches and set-up (Qwen3 shape 20 tokens 66.8 -> 56.5 us, 777 tokens 279
+    // -> 270; Mixtral shape 200 tokens 532 -> 514). The large calls launch plainly: early-resident successors compete with
+    // the running kernels (19-32 us slower).
+    PdlScope pdl_scope(!pairs);
 
     PrefillRouteParams rp{};
     rp.logits = logits; rp.S = tables->S; rp.L = tables->L; rp.lnh = tables->lnh;
