@@ -218,7 +218,8 @@ int exfold_moe_prefill_ex(const exfold_layer *layer, const void *x, const float 
  * read, each byte once. bf16 layers: four kernels chained by programmatic dependent launch
  * (per-token Top-K; gate/up projection with the batch-level routing in its prologue, x read in
  * place; grouped down projection over one row per distinct (token, pool expert); per-token sum
- * of those rows in slot order). No atomics are used: the same inputs give the same bits.
+ * of those rows in slot order); batches of at most 8 tokens (weights 32-byte aligned): two (routing
+ * with the gate/up projection; down projection with the sum over a token's experts). No atomics are used: the same inputs give the same bits.
  */
 int exfold_moe_decode(const exfold_layer *layer, const void *x, const float *logits, int64_t B,
                       const void *w_gate, const void *w_up, const void *w_down,
@@ -374,8 +375,8 @@ int64_t exfold_launch_count(void);
  * 6 decode pool/remap, 7 decode row gather, 8 decode GEMM-1 (gate/up stream), 9 decode GEMM-2 (down stream),
  * 10 SIMT expert FFN, 11 SIMT combine, 12 / 13 the CTA-pair pass of GEMM-1 / GEMM-2 alone (slots 3 and 4 cover a
  * whole GEMM: the pair pass, when it runs, and the one-CTA pass), 14 decode expert FFN of bf16 layers (one kernel:
- * pool / remap prologue + gate, up and down weight stream; slot 6 is then the per-token Top-K kernel and slots
- * 7-9 stay empty). Returns EXFOLD_OK or EXFOLD_ERR_CUDA.
+ * pool / remap prologue + gate and up weight stream, slot 6 is then the per-token Top-K kernel; batches of at most 8
+ * tokens: both kernels). Returns EXFOLD_OK or EXFOLD_ERR_CUDA.
  */
 #define EXFOLD_PROFILE_SLOTS 15
 int exfold_profile_enable(int enable);

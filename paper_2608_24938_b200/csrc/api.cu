@@ -649,62 +649,83 @@ static int decode_impl(const exfold_layer* layer, const void* x, const float* lo
     rp.slot_row = at<int32_t>(ws, pl.inv_pos);
     rp.status = at<DeviceStatus>(ws, pl.status);
     if (bf16) {
-        // Token-parallel Top-K (with the router scores when w_router is given) -> gate/up kernel that finishes the
-        // routing in its prologue and streams the pool's gate and up weights against x in place -> grouped down
-        // projection over the compact rows -> per-token sum of the rows.
-        int stages = 0, scratch_off = 0, ar = 0;
-        decode_ffn_smem_plan((int)B, K, N, &stages, &scratch_off, &ar);
-        if (stages < 2) return EXFOLD_ERR_UNSUPPORTED;
-        CUtensorMap tm_x, tm_wg64, tm_wu64, tm_wg96, tm_wu96;
-        const uint64_t E = (uint64_t)G;
-        if (!make_tmap(&tm_x, x, (uint64_t)B, d, ar) || !make_tmap(&tm_wg64, w_gate, E * I, d, 64) ||
-            !make_tmap(&tm_wu64, w_up, E * I, d, 64) || !make_tmap(&tm_wg96, w_gate, E * I, d, 96) ||
-            !make_tmap(&tm_wu96, w_up, E * I, d, 96))
-            return EXFOLD_ERR_CUDA;
         DecodeTopkParams tp{};
         tp.logits = logits; tp.x = reinterpret_cast<const __nv_bfloat16*>(x);
         tp.w_router = reinterpret_cast<const __nv_bfloat16*>(w_router); tp.logits_out = const_cast<float*>(logits);
         tp.B = (int)B; tp.N = N; tp.K = K; tp.d = d;
         tp.ids = rp.ids; tp.w64 = at<double>(ws, pl.w64); tp.status = rp.status;
-        { ProfScope ps(6, s); EXFOLD_CUDA(launch_decode_topk(tp, s)); }
-        DecodeFfnParams fp{};
-        fp.tm_x = tm_x; fp.tm_wg = tm_wg; fp.tm_wu = tm_wu; fp.tm_wg64 = tm_wg64; fp.tm_wu64 = tm_wu64; fp.tm_wg96 = tm_wg96; fp.tm_wu96 = tm_wu96;
-        fp.ids = rp.ids; fp.w64 = tp.w64; fp.S = tables->S; fp.L = tables->L; fp.h = tables->h;
-        fp.st_pool = rp.st_pool; fp.st_target = rp.st_target; fp.st_scale = rp.st_scale;
-        fp.B = (int)B; fp.N = N; fp.K = K; fp.M = pool_m; fp.n_shared = l.n_shared; fp.d = d; fp.I = I; fp.a_rows = ar;
-        fp.stages = stages; fp.scratch_off = scratch_off;
-        fp.pool_ids = rp.pool_ids; fp.pool_size = rp.pool_size; fp.pool_mask = rp.pool_mask;
-        // the remapped slots go to a second array: the Top-K ids are read by every CTA while CTA 0 writes
-        fp.out_ids = at<int32_t>(ws, pl.perm); fp.out_w = rp.w; fp.target = rp.target; fp.scale = rp.scale;
-        fp.H = at<__nv_bfloat16>(ws, pl.H); fp.row_tok = rp.row_tok; fp.row_w = rp.row_w;
-        fp.slot_row = rp.slot_row;
-        fp.grp_expert = rp.grp_expert; fp.grp_off = rp.grp_off; fp.grp_tiles = rp.grp_tiles; fp.n_groups = rp.n_groups;
-        fp.status = rp.status;
-        { ProfScope ps(14, s); EXFOLD_CUDA(launch_decode_ffn(fp, sm_count(), s)); }
-        // Down projection on the grouped GEMM-2 kernel over the compact rows (the whole intermediate dimension is
-        // its K, so no partial outputs meet in memory); each row's weighted output is stored once, in bf16, and a
-        // token's rows are then summed in slot order: no atomics, so a decode step is reproducible bit for bit.
-        const int max_groups = std::min(pool_m, N) + l.n_shared;
-        const int tiles_per_group = (int)((B + kTileM - 1) / kTileM);
-        const int sms = std::min(sm_count(), kMaxCtas);
-        GroupedGemmParams g{};
-        g.tm_a = tm_h; g.tm_a2 = tm_h; g.tm_b0 = tm_wd; g.tm_b1 = tm_wd; g.x_rows = 1; g.o32 = nullptr;
-        g.offsets = rp.grp_off; g.work_start = rp.grp_tiles; g.G = max_groups; g.n_routed = 0x7fffffff;
-        g.R = max_rows; g.d = d; g.I = I; g.n_ntiles = (d + 255) / 256; g.ksplit = 1; g.a_rows = a_rows;
-        g.grp_expert = rp.grp_expert; g.n_groups_dev = rp.n_groups;
-        g.H = fp.H; g.row_tok = rp.row_tok; g.row_w = rp.row_w;
-        g.y = at<__nv_bfloat16>(ws, pl.obuf); g.store_rows = 1; g.status = rp.status;
-        // Fewer (expert, column tile) items than half the SMs (few experts, large I): K is split in two so that
-        // enough SMs stream W_down; each part's rows go to a plane of their own (the two planes are the row buffer
-        // and the unused gathered-rows region before it) and are summed, in order, by the kernel after.
-        const int nkb2 = I / 64;
-        const int64_t base_items = (int64_t)max_groups * tiles_per_group * g.n_ntiles;
-        g.ksplit = (2 * base_items < sms && nkb2 >= 8) ? kMaxDecodeKsplit : 1;
-        g.y = g.ksplit > 1 ? at<__nv_bfloat16>(ws, pl.obuf) - (size_t)max_rows * d : at<__nv_bfloat16>(ws, pl.obuf);
-        { ProfScope ps(9, s); EXFOLD_CUDA(launch_grouped_gemm2(g, (int)std::min<int64_t>(sms, base_items * g.ksplit), s)); }
-        { ProfScope ps(5, s); EXFOLD_CUDA(launch_combine_rows(g.y, fp.slot_row, B, K, d, l.n_shared, rp.n_groups + 2, g.ksplit,
-                                                       max_rows, reinterpret_cast<__nv_bfloat16*>(y), s)); }
-        rp.ids = fp.out_ids;  // for the metadata copies below
+        // the remapped slots go to a second array: the Top-K ids are read by every CTA while one of them writes
+        int32_t* const out_ids = at<int32_t>(ws, pl.perm);
+        if (decode_small_fits((int)B, K, d, w_gate, w_up, w_down)) {
+            if (w_router != nullptr) { ProfScope ps(6, s); EXFOLD_CUDA(launch_decode_topk(tp, s)); }
+            DecodeSmallParams sp{};
+            sp.x = tp.x; sp.wg = reinterpret_cast<const __nv_bfloat16*>(w_gate); sp.wu = reinterpret_cast<const __nv_bfloat16*>(w_up);
+            sp.wd = reinterpret_cast<const __nv_bfloat16*>(w_down); sp.y = reinterpret_cast<__nv_bfloat16*>(y);
+            sp.logits = w_router == nullptr ? logits : nullptr; sp.ids = tp.ids; sp.w64 = tp.w64;
+            sp.S = tables->S; sp.L = tables->L; sp.h = tables->h;
+            sp.st_pool = rp.st_pool; sp.st_target = rp.st_target; sp.st_scale = rp.st_scale;
+            sp.B = (int)B; sp.N = N; sp.K = K; sp.M = pool_m; sp.n_shared = l.n_shared; sp.d = d; sp.I = I;
+            sp.max_groups = (int)std::min<int64_t>(std::min(pool_m, N), B * K) + l.n_shared; sp.max_rows = max_rows;
+            if (meta) {
+                sp.pool_ids = rp.pool_ids; sp.pool_size = rp.pool_size; sp.pool_mask = rp.pool_mask;
+                sp.out_ids = out_ids; sp.out_w = rp.w; sp.target = rp.target; sp.scale = rp.scale;
+            }
+            sp.H = at<__nv_bfloat16>(ws, pl.H); sp.row_tok = rp.row_tok; sp.row_w = rp.row_w;
+            sp.row_grp = at<int32_t>(ws, pl.row_exp); sp.grp_expert = rp.grp_expert; sp.n_groups = rp.n_groups;
+            sp.status = w_router == nullptr ? rp.status : nullptr;
+            { ProfScope ps(14, s); EXFOLD_CUDA(launch_decode_small(sp, sm_count(), s)); }
+        } else {
+            // Token-parallel Top-K (with the router scores when w_router is given) -> gate/up kernel that finishes the
+            // routing in its prologue and streams the pool's gate and up weights against x in place -> grouped down
+            // projection over the compact rows -> per-token sum of the rows.
+            int stages = 0, scratch_off = 0, ar = 0;
+            decode_ffn_smem_plan((int)B, K, N, &stages, &scratch_off, &ar);
+            if (stages < 2) return EXFOLD_ERR_UNSUPPORTED;
+            CUtensorMap tm_x, tm_wg64, tm_wu64, tm_wg96, tm_wu96;
+            const uint64_t E = (uint64_t)G;
+            if (!make_tmap(&tm_x, x, (uint64_t)B, d, ar) || !make_tmap(&tm_wg64, w_gate, E * I, d, 64) ||
+                !make_tmap(&tm_wu64, w_up, E * I, d, 64) || !make_tmap(&tm_wg96, w_gate, E * I, d, 96) ||
+                !make_tmap(&tm_wu96, w_up, E * I, d, 96))
+                return EXFOLD_ERR_CUDA;
+            { ProfScope ps(6, s); EXFOLD_CUDA(launch_decode_topk(tp, s)); }
+            DecodeFfnParams fp{};
+            fp.tm_x = tm_x; fp.tm_wg = tm_wg; fp.tm_wu = tm_wu; fp.tm_wg64 = tm_wg64; fp.tm_wu64 = tm_wu64; fp.tm_wg96 = tm_wg96; fp.tm_wu96 = tm_wu96;
+            fp.ids = rp.ids; fp.w64 = tp.w64; fp.S = tables->S; fp.L = tables->L; fp.h = tables->h;
+            fp.st_pool = rp.st_pool; fp.st_target = rp.st_target; fp.st_scale = rp.st_scale;
+            fp.B = (int)B; fp.N = N; fp.K = K; fp.M = pool_m; fp.n_shared = l.n_shared; fp.d = d; fp.I = I; fp.a_rows = ar;
+            fp.stages = stages; fp.scratch_off = scratch_off;
+            fp.pool_ids = rp.pool_ids; fp.pool_size = rp.pool_size; fp.pool_mask = rp.pool_mask;
+            fp.out_ids = out_ids; fp.out_w = rp.w; fp.target = rp.target; fp.scale = rp.scale;
+            fp.H = at<__nv_bfloat16>(ws, pl.H); fp.row_tok = rp.row_tok; fp.row_w = rp.row_w;
+            fp.slot_row = rp.slot_row;
+            fp.grp_expert = rp.grp_expert; fp.grp_off = rp.grp_off; fp.grp_tiles = rp.grp_tiles; fp.n_groups = rp.n_groups;
+            fp.status = rp.status;
+            { ProfScope ps(14, s); EXFOLD_CUDA(launch_decode_ffn(fp, sm_count(), s)); }
+            // Down projection on the grouped GEMM-2 kernel over the compact rows (the whole intermediate dimension is
+            // its K, so no partial outputs meet in memory); each row's weighted output is stored once, in bf16, and a
+            // token's rows are then summed in slot order: no atomics, so a decode step is reproducible bit for bit.
+            const int max_groups = std::min(pool_m, N) + l.n_shared;
+            const int tiles_per_group = (int)((B + kTileM - 1) / kTileM);
+            const int sms = std::min(sm_count(), kMaxCtas);
+            GroupedGemmParams g{};
+            g.tm_a = tm_h; g.tm_a2 = tm_h; g.tm_b0 = tm_wd; g.tm_b1 = tm_wd; g.x_rows = 1; g.o32 = nullptr;
+            g.offsets = rp.grp_off; g.work_start = rp.grp_tiles; g.G = max_groups; g.n_routed = 0x7fffffff;
+            g.R = max_rows; g.d = d; g.I = I; g.n_ntiles = (d + 255) / 256; g.ksplit = 1; g.a_rows = a_rows;
+            g.grp_expert = rp.grp_expert; g.n_groups_dev = rp.n_groups;
+            g.H = fp.H; g.row_tok = rp.row_tok; g.row_w = rp.row_w;
+            g.y = at<__nv_bfloat16>(ws, pl.obuf); g.store_rows = 1; g.status = rp.status;
+            // Fewer (expert, column tile) items than half the SMs (few experts, large I): K is split in two so that
+            // enough SMs stream W_down; each part's rows go to a plane of their own (the two planes are the row buffer
+            // and the unused gathered-rows region before it) and are summed, in order, by the kernel after.
+            const int nkb2 = I / 64;
+            const int64_t base_items = (int64_t)max_groups * tiles_per_group * g.n_ntiles;
+            g.ksplit = (2 * base_items < sms && nkb2 >= 8) ? kMaxDecodeKsplit : 1;
+            g.y = g.ksplit > 1 ? at<__nv_bfloat16>(ws, pl.obuf) - (size_t)max_rows * d : at<__nv_bfloat16>(ws, pl.obuf);
+            { ProfScope ps(9, s); EXFOLD_CUDA(launch_grouped_gemm2(g, (int)std::min<int64_t>(sms, base_items * g.ksplit), s)); }
+            { ProfScope ps(5, s); EXFOLD_CUDA(launch_combine_rows(g.y, fp.slot_row, B, K, d, l.n_shared, rp.n_groups + 2, g.ksplit,
+                                                           max_rows, reinterpret_cast<__nv_bfloat16*>(y), s)); }
+        }
+        rp.ids = out_ids;  // for the metadata copies below
     } else {
         if (w_router != nullptr) {
             rc = router_enqueue(layer, x, w_router, B, const_cast<float*>(logits), ws, ws_bytes, s, false);

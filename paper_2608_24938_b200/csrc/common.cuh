@@ -81,6 +81,46 @@ __device__ __forceinline__ int warp_argmin(bool has, uint32_t key, int id) {
     return __reduce_min_sync(0xffffffffu, (has && key == m) ? id : 0x7fffffff);
 }
 
+// A token's Top-K and its softmax weights in double, by one warp: v[q] = score of expert lane + 32 q (NPL = ceil(N / 32) or
+// more). Lane k < K returns the weight of route k (router order, ties -> lower id) and its expert through *id.
+template <int NPL>
+__device__ __forceinline__ double warp_topk_softmax(const float (&v)[NPL], int N, int K, int lane, int* id) {
+    uint32_t key_q[NPL];
+    uint32_t used = 0;
+#pragma unroll
+    for (int q = 0; q < NPL; ++q) {
+        key_q[q] = float_order_key(v[q]);
+        if (lane + 32 * q >= N) used |= 1u << q;
+    }
+    int my_id = -1;
+    float my_r = 0.f;
+    for (int k = 0; k < K; ++k) {
+        uint32_t bk = 0;
+        int be = 0x7fffffff;
+#pragma unroll
+        for (int q = 0; q < NPL; ++q) {
+            const bool free_q = !((used >> q) & 1u);
+            if (free_q && (be == 0x7fffffff || key_q[q] > bk)) {
+                bk = key_q[q];
+                be = lane + 32 * q;
+            }
+        }
+        uint32_t mk;
+        be = warp_argmax(be != 0x7fffffff, bk, be, &mk);
+        if ((be & 31) == lane) used |= 1u << (be >> 5);
+        if (lane == k) {
+            my_id = be;
+            my_r = float_from_order_key(mk);
+        }
+    }
+    const float rmax = __shfl_sync(0xffffffffu, my_r, 0);
+    const double ex = lane < K ? exp((double)my_r - (double)rmax) : 0.0;
+    double sum = 0.0;
+    for (int k = 0; k < K; ++k) sum += __shfl_sync(0xffffffffu, ex, k);  // slot order, like the definition
+    *id = my_id;
+    return ex / sum;
+}
+
 template <typename... KArgs, typename... Args>
 cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Args... args) {
     cudaLaunchConfig_t cfg = {};
@@ -121,6 +161,7 @@ cudaError_t launch_pdl_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 block, 
     return e;
 }
 
+__host__ __device__ inline size_t align16(size_t v) { return (v + 15) / 16 * 16; }
 inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
 // ---------------------------------------------------------------- routing (prefill)
@@ -262,6 +303,45 @@ struct DecodeFfnParams {
 };
 cudaError_t launch_decode_ffn(const DecodeFfnParams& p, int sms, cudaStream_t s);
 size_t decode_ffn_smem_plan(int B, int K, int N, int* stages, int* scratch_off, int* a_rows);
+// Decode of at most kSmallDecodeBatch tokens, bf16 layers: two kernels (decode_small.cu)
+constexpr int kSmallDecodeBatch = 8;
+struct DecodeSmallParams {
+    const __nv_bfloat16* x;
+    const __nv_bfloat16* wg;
+    const __nv_bfloat16* wu;
+    const __nv_bfloat16* wd;
+    __nv_bfloat16* y;
+    const float* logits;  // [B][N], or null: ids and w64 come from the top-k kernel
+    const int32_t* ids;
+    const double* w64;
+    const float* S;
+    const float* L;
+    const float* h;
+    const int32_t* st_pool;    // static pool (all null for the dynamic pool)
+    const int32_t* st_target;
+    const float* st_scale;
+    int B, N, K, M, n_shared, d, I;
+    int max_groups, max_rows;  // bounds of the lists below
+    int split;                 // set by the launcher
+    // metadata (all null when the caller asks for none)
+    int32_t* pool_ids;
+    int32_t* pool_size;
+    uint32_t* pool_mask;
+    int32_t* out_ids;
+    float* out_w;
+    int32_t* target;
+    float* scale;
+    // one row per distinct (token, pool expert)
+    __nv_bfloat16* H;     // [rows][I]
+    int32_t* row_tok;
+    float* row_w;
+    int32_t* row_grp;
+    int32_t* grp_expert;
+    int32_t* n_groups;    // [2]: groups, rows
+    DeviceStatus* status; // cleared here when this is the call's first kernel (else null)
+};
+bool decode_small_fits(int B, int K, int d, const void* wg, const void* wu, const void* wd);
+cudaError_t launch_decode_small(DecodeSmallParams p, int sms, cudaStream_t s);
 cudaError_t launch_static_pool(int N, int M, const float* S, const float* L, const float* h, int32_t* pool_ids,
                                int32_t* target, float* scale, cudaStream_t s);
 

@@ -403,41 +403,11 @@ __global__ void __launch_bounds__(256) decode_topk_kernel(DecodeTopkParams p) {
         const int e = lane + 32 * q;
         v[q] = e < N ? (ROUTER ? s_lg[e] : p.logits[(size_t)i * N + e]) : -INFINITY;
     }
-    uint32_t key_q[NPL];
-    uint32_t used = 0;
-#pragma unroll
-    for (int q = 0; q < NPL; ++q) {
-        key_q[q] = float_order_key(v[q]);
-        if (lane + 32 * q >= N) used |= 1u << q;
-    }
-    int my_id = -1;
-    float my_r = 0.f;
-    for (int k = 0; k < K; ++k) {
-        uint32_t bk = 0;
-        int be = 0x7fffffff;
-#pragma unroll
-        for (int q = 0; q < NPL; ++q) {
-            const bool free_q = !((used >> q) & 1u);
-            if (free_q && (be == 0x7fffffff || key_q[q] > bk)) {
-                bk = key_q[q];
-                be = lane + 32 * q;
-            }
-        }
-        uint32_t mk;
-        be = warp_argmax(be != 0x7fffffff, bk, be, &mk);
-        if ((be & 31) == lane) used |= 1u << (be >> 5);
-        if (lane == k) {
-            my_id = be;
-            my_r = float_from_order_key(mk);
-        }
-    }
-    const float rmax = __shfl_sync(0xffffffffu, my_r, 0);
-    const double ex = lane < K ? exp((double)my_r - (double)rmax) : 0.0;
-    double sum = 0.0;
-    for (int k = 0; k < K; ++k) sum += __shfl_sync(0xffffffffu, ex, k);  // slot order, like the definition
+    int my_id;
+    const double w = warp_topk_softmax<NPL>(v, N, K, lane, &my_id);
     if (lane < K) {
         p.ids[(size_t)i * K + lane] = my_id;
-        p.w64[(size_t)i * K + lane] = ex / sum;
+        p.w64[(size_t)i * K + lane] = w;
     }
 }
 

@@ -72,3 +72,62 @@ def test_routing_block_forms(T):
     got, ref = case.run_prefill(3), case.oracle_prefill(3)
     check_prefill_meta(got, ref)
     check_output(got["y"], ref["y"], "bf16")
+
+
+@pytest.mark.parametrize("shape", [
+    # N, shared, d, I, K, B, M
+    (16, 0, 256, 384, 4, 1, 6),      # one token; a cluster of CTAs per down item
+    (16, 1, 64, 64, 4, 3, 2),        # a single K chunk, shared expert, merged slots
+    (40, 0, 1088, 192, 5, 8, 40),    # 17 chunks (ragged stages), full 8-column operand, pool = the batch's union
+    (40, 1, 192, 320, 6, 7, 7),
+    (256, 0, 128, 64, 32, 8, 200),   # largest N, K and batch
+    (256, 1, 128, 64, 32, 8, 3),
+    (16, 0, 2432, 128, 4, 5, 16),    # more down items than SMs: two CTAs of 8 warps
+    (16, 0, 256, 384, 4, 9, 6),      # first batch of the four-kernel chain
+    (16, 0, 8192, 64, 2, 8, 5),      # tokens too large for shared memory twice per SM: the chain
+])
+@pytest.mark.parametrize("mode", ["dynamic", "static", "router", "unaligned"])
+def test_small_decode_batches(shape, mode):
+    """Two-kernel decode of at most 8 tokens against the oracle: routing bit-exact, outputs to the bf16 bound. "router":
+    scores from the router matrix, outputs bit-identical to the call on those scores. "unaligned": weights 16 but not 32
+    bytes aligned take the chain."""
+    N, ns, d, I, K, B, M = shape
+    case = Case(si.LayerConfig("smalldec", N, ns, d, I, K, "bf16", 8, (1,), B, (M,)))
+    ex, dev, cfg = case.ex, case.dev, case.cfg
+    if mode == "unaligned":
+        room = torch.empty(case.d_wg.numel() + 16, dtype=torch.bfloat16, device=dev)
+        at = 8 if room.data_ptr() % 32 == 0 else 0
+        case.d_wg = room[at:at + case.d_wg.numel()].view(case.d_wg.shape).copy_(case.d_wg)
+        assert case.d_wg.data_ptr() % 32 == 16
+    if mode == "static":
+        pool = [torch.empty(M, dtype=torch.int32, device=dev), torch.empty(N, dtype=torch.int32, device=dev), torch.empty(N, device=dev)]
+        sp = ex.exfold_static_pool_build(case.layer, case.tables, M, *pool)
+        y = torch.full((B, d), float("nan"), dtype=torch.bfloat16, device=dev)
+        ids = torch.full((B, K), -7, dtype=torch.int32, device=dev)
+        w = torch.full((B, K), float("nan"), device=dev)
+        ws = case.workspace(B, K)
+        ex.exfold_moe_decode_static(case.layer, case.d_xd, case.d_lgd, case.d_wg, case.d_wu, case.d_wd, sp, y, ws, meta=dict(ids=ids, w=w))
+        assert ex.exfold_device_status(ws) == 0
+        top = oracle.decode_fold(case.lgd.numpy(), K, N, *[t.numpy() for t in case.tables_host[:3]])  # unfolded: the routes
+        tgt, scl = pool[1].cpu().numpy(), pool[2].cpu().numpy()
+        assert np.array_equal(ids.cpu().numpy(), tgt[top["ids"]])
+        np.testing.assert_allclose(w.cpu().numpy(), top["w"] * scl[top["ids"]], rtol=1e-6, atol=1e-7)
+        yr = oracle.moe_apply(A(case.xd), A(case.wg), A(case.wu), A(case.wd), tgt[top["ids"]], w.cpu().numpy(), N, ns)
+        check_output(y.float().cpu().numpy(), yr, "bf16")
+        return
+    if mode == "router":
+        wr = si.router_weights(cfg).to(dev)
+        lg = torch.full((B, N), float("nan"), device=dev)
+        y = torch.full((B, d), float("nan"), dtype=torch.bfloat16, device=dev)
+        ws = case.workspace(B, K)
+        ex.exfold_moe_decode_layer(case.layer, case.d_xd, wr, case.d_wg, case.d_wu, case.d_wd, case.tables, M, y, ws, lg)
+        assert ex.exfold_device_status(ws) == 0
+        case.d_lgd = lg
+        case.lgd = lg.cpu()
+    got, ref = case.run_decode(M), case.oracle_decode(M)
+    check_decode_meta(got, ref, M)
+    check_output(got["y"], ref["y"], "bf16")
+    if mode == "router":
+        assert np.array_equal(got["y"], y.float().cpu().numpy())
+    plain = case.run_decode(M, with_meta=False)  # without metadata only the batch's experts get targets
+    assert np.array_equal(got["y"], plain["y"])
