@@ -350,58 +350,91 @@ __global__ void __launch_bounds__(kDecThreads) decode_route_kernel(DecodeRoutePa
 // Per token: (optionally) the router scores of Eq. 2 as fixed-order dot products - the same lane partition, the
 // same fused multiply-adds and the same shuffle tree as router_simt_kernel, so the scores are those of
 // exfold_router_logits bit for bit -, then the token's Top-K and its softmax weights in double (slot order).
-// Without the router: one CTA per token. With it: a cluster of 8 CTAs per token, each taking an eighth of the
+// Without the router: one CTA per token. With it: a cluster of 8 CTAs per TT tokens, each taking an eighth of the
 // experts (one CTA alone would walk the whole router matrix with a handful of loads in flight); the scores meet
-// in the shared memory of the cluster's first CTA, which then ranks them. CTA 0 also clears the status record.
+// in the shared memory of the cluster's first CTA, which then ranks them. TT = 1 spreads a small batch over the most SMs: a
+// warp takes two experts at a time. TT = 8: a warp takes 4 experts x 4 tokens, so that a conversion serves four products
+// and the router matrix is read through L2 once per 8 tokens. CTA 0 also clears the status record.
 // The batch-level half (pool, targets, remap) runs in the prologue of the gate/up kernel (ffn_decode.cu).
 constexpr int kTopkCluster = 8;
 
-template <int NPL, bool ROUTER>
+template <int NPL, bool ROUTER, int TT>
 __global__ void __launch_bounds__(256) decode_topk_kernel(DecodeTopkParams p) {
-    __shared__ float s_lg[kMaxExperts];
+    __shared__ float s_lg[TT][kMaxExperts];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int N = p.N, K = p.K, d = p.d;
-    const int i = ROUTER ? (int)blockIdx.x / kTopkCluster : (int)blockIdx.x;
+    const int i0 = (ROUTER ? (int)blockIdx.x / kTopkCluster : (int)blockIdx.x) * TT;
     grid_dep_launch();
     grid_dep_wait();  // x may be the previous layer's output; the workspace may still be read by the previous call
     if (blockIdx.x == 0 && threadIdx.x < 4) reinterpret_cast<int*>(p.status)[threadIdx.x] = 0;
     if (ROUTER) {
+        constexpr int EW = TT == 1 ? 2 : 4, TW = TT == 1 ? 1 : 4;  // experts and tokens of a warp
+        constexpr int kTokGroups = TT / TW, kExpGroups = 8 / kTokGroups;
         cg::cluster_group cluster = cg::this_cluster();
         const int rank = (int)cluster.block_rank();
-        float* lead = cluster.map_shared_rank(s_lg, 0);
+        float* lead = cluster.map_shared_rank(&s_lg[0][0], 0);
         const int per = (N + kTopkCluster - 1) / kTopkCluster;
         const int e_lo = rank * per, e_hi = min(N, e_lo + per);
-        const __nv_bfloat16* xi = p.x + (size_t)i * d;
-        for (int e = e_lo + warp; e < e_hi; e += 8) {
-            const __nv_bfloat16* we = p.w_router + (size_t)e * d;
-            float acc = 0.f;
+        const int t0 = warp / kExpGroups * TW;
+        const __nv_bfloat16* xi[TW];
+#pragma unroll
+        for (int t = 0; t < TW; ++t) xi[t] = p.x + (size_t)min(i0 + t0 + t, p.B - 1) * d;
+        for (int e0 = e_lo + warp % kExpGroups * EW; e0 < e_hi; e0 += kExpGroups * EW) {
+            const __nv_bfloat16* we[EW];
+#pragma unroll
+            for (int u = 0; u < EW; ++u) we[u] = p.w_router + (size_t)min(e0 + u, e_hi - 1) * d;
+            float acc[EW][TW];
+#pragma unroll
+            for (int u = 0; u < EW; ++u)
+#pragma unroll
+                for (int t = 0; t < TW; ++t) acc[u][t] = 0.f;
+#pragma unroll 2
             for (int c = lane * 8; c < d; c += 256) {
-                const uint4 a = *reinterpret_cast<const uint4*>(we + c), b = *reinterpret_cast<const uint4*>(xi + c);
-                const __nv_bfloat162* pa = reinterpret_cast<const __nv_bfloat162*>(&a);
-                const __nv_bfloat162* pb = reinterpret_cast<const __nv_bfloat162*>(&b);
+                uint4 a[EW], b[TW];
+#pragma unroll
+                for (int u = 0; u < EW; ++u) a[u] = *reinterpret_cast<const uint4*>(we[u] + c);
+#pragma unroll
+                for (int t = 0; t < TW; ++t) b[t] = *reinterpret_cast<const uint4*>(xi[t] + c);
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
-                    const float2 fa = __bfloat1622float2(pa[j]), fb = __bfloat1622float2(pb[j]);
-                    acc = fmaf(fa.x, fb.x, acc);
-                    acc = fmaf(fa.y, fb.y, acc);
+                    float2 fa[EW];
+#pragma unroll
+                    for (int u = 0; u < EW; ++u) fa[u] = __bfloat1622float2(reinterpret_cast<const __nv_bfloat162*>(&a[u])[j]);
+#pragma unroll
+                    for (int t = 0; t < TW; ++t) {
+                        const float2 fb = __bfloat1622float2(reinterpret_cast<const __nv_bfloat162*>(&b[t])[j]);
+#pragma unroll
+                        for (int u = 0; u < EW; ++u) {
+                            acc[u][t] = fmaf(fa[u].x, fb.x, acc[u][t]);
+                            acc[u][t] = fmaf(fa[u].y, fb.y, acc[u][t]);
+                        }
+                    }
                 }
             }
 #pragma unroll
-            for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-            if (lane == 0) {
-                lead[e] = acc;
-                p.logits_out[(size_t)i * N + e] = acc;
-            }
+            for (int u = 0; u < EW; ++u)
+#pragma unroll
+                for (int t = 0; t < TW; ++t) {
+                    float v = acc[u][t];
+#pragma unroll
+                    for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+                    const int e = e0 + u, i = i0 + t0 + t;
+                    if (lane == 0 && e < e_hi && i < p.B) {
+                        lead[(t0 + t) * kMaxExperts + e] = v;
+                        p.logits_out[(size_t)i * N + e] = v;
+                    }
+                }
         }
-        cluster.sync();  // every score of the token is in the first CTA's shared memory
+        cluster.sync();  // every score of the tokens is in the first CTA's shared memory
         if (rank != 0) return;
     }
-    if (warp != 0) return;
+    const int i = i0 + warp;
+    if (warp >= TT || i >= p.B) return;
     float v[NPL];
 #pragma unroll
     for (int q = 0; q < NPL; ++q) {
         const int e = lane + 32 * q;
-        v[q] = e < N ? (ROUTER ? s_lg[e] : p.logits[(size_t)i * N + e]) : -INFINITY;
+        v[q] = e < N ? (ROUTER ? s_lg[warp][e] : p.logits[(size_t)i * N + e]) : -INFINITY;
     }
     int my_id;
     const double w = warp_topk_softmax<NPL>(v, N, K, lane, &my_id);
@@ -486,22 +519,24 @@ cudaError_t launch_decode_route(const DecodeRouteParams& p, cudaStream_t s) {
     return err;
 }
 
+// From this batch on (and with enough experts to fill the tiles) clusters take 8 tokens. Whole decode call with the router,
+// TT = 1 / 8: Qwen3 shape 40 tokens 50.5 / 51.8 us, 64 tokens 51.2 / 52.6, 120 tokens 58.3 / 54.2, 256 tokens 207 / 199; GLM
+// shape 40 tokens 139 / 141, 128 tokens 251 / 244.
+constexpr int kTopkTileBatch = 81;
+template <int NPL>
+static cudaError_t launch_topk_t(const DecodeTopkParams& p, cudaStream_t s) {
+    if (p.w_router == nullptr) return launch_pdl(decode_topk_kernel<NPL, false, 1>, p.B, 256, 0, s, p);
+    if (p.B < kTopkTileBatch || p.N < 32)
+        return launch_pdl_cluster(decode_topk_kernel<NPL, true, 1>, (unsigned)p.B * kTopkCluster, 256, 0, kTopkCluster, s, p);
+    return launch_pdl_cluster(decode_topk_kernel<NPL, true, 8>, (unsigned)(p.B + 7) / 8 * kTopkCluster, 256, 0, kTopkCluster, s, p);
+}
+
 cudaError_t launch_decode_topk(const DecodeTopkParams& p, cudaStream_t s) {
-    const int npl = (p.N + 31) / 32;
-    if (p.w_router != nullptr) {
-        const unsigned grid = (unsigned)p.B * kTopkCluster;
-        switch (npl) {
-            case 1: return launch_pdl_cluster(decode_topk_kernel<1, true>, grid, 256, 0, kTopkCluster, s, p);
-            case 2: return launch_pdl_cluster(decode_topk_kernel<2, true>, grid, 256, 0, kTopkCluster, s, p);
-            case 3: case 4: return launch_pdl_cluster(decode_topk_kernel<4, true>, grid, 256, 0, kTopkCluster, s, p);
-            default: return launch_pdl_cluster(decode_topk_kernel<8, true>, grid, 256, 0, kTopkCluster, s, p);
-        }
-    }
-    switch (npl) {
-        case 1: return launch_pdl(decode_topk_kernel<1, false>, p.B, 256, 0, s, p);
-        case 2: return launch_pdl(decode_topk_kernel<2, false>, p.B, 256, 0, s, p);
-        case 3: case 4: return launch_pdl(decode_topk_kernel<4, false>, p.B, 256, 0, s, p);
-        default: return launch_pdl(decode_topk_kernel<8, false>, p.B, 256, 0, s, p);
+    switch ((p.N + 31) / 32) {
+        case 1: return launch_topk_t<1>(p, s);
+        case 2: return launch_topk_t<2>(p, s);
+        case 3: case 4: return launch_topk_t<4>(p, s);
+        default: return launch_topk_t<8>(p, s);
     }
 }
 

@@ -131,3 +131,23 @@ def test_small_decode_batches(shape, mode):
         assert np.array_equal(got["y"], y.float().cpu().numpy())
     plain = case.run_decode(M, with_meta=False)  # without metadata only the batch's experts get targets
     assert np.array_equal(got["y"], plain["y"])
+
+
+@pytest.mark.parametrize("B", [80, 81, 87, 128])
+@pytest.mark.parametrize("N", [31, 32, 100, 256])
+def test_decode_router_scores_by_batch(B, N):
+    """Router scores inside the decode call, a token per cluster or eight (from 81 tokens and 32 experts on; ragged last
+    cluster, experts not a multiple of the tiles): the bits of exfold_router_logits."""
+    case = Case(si.LayerConfig("rt", N, 0, 320, 64, 4, "bf16", 8, (1,), B, (6,)))
+    ex, dev = case.ex, case.dev
+    wr = si.router_weights(case.cfg).to(dev)
+    lg, want = torch.full((B, N), float("nan"), device=dev), torch.full((B, N), float("nan"), device=dev)
+    y = torch.empty((B, 320), dtype=torch.bfloat16, device=dev)
+    ws = case.workspace(B, 4)
+    ex.exfold_moe_decode_layer(case.layer, case.d_xd, wr, case.d_wg, case.d_wu, case.d_wd, case.tables, 6, y, ws, lg)
+    assert ex.exfold_device_status(ws) == 0
+    ex.exfold_router_logits(case.layer, case.d_xd, wr, want, ws)
+    assert torch.equal(lg, want)
+    case.lgd, case.d_lgd = lg.cpu(), lg
+    ref = case.oracle_decode(6)
+    check_output(y.float().cpu().numpy(), ref["y"], "bf16")
