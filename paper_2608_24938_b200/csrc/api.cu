@@ -694,8 +694,10 @@ static int decode_impl(const exfold_layer* layer, const void* x, const float* lo
             fp.st_pool = rp.st_pool; fp.st_target = rp.st_target; fp.st_scale = rp.st_scale;
             fp.B = (int)B; fp.N = N; fp.K = K; fp.M = pool_m; fp.n_shared = l.n_shared; fp.d = d; fp.I = I; fp.a_rows = ar;
             fp.stages = stages; fp.scratch_off = scratch_off;
-            fp.pool_ids = rp.pool_ids; fp.pool_size = rp.pool_size; fp.pool_mask = rp.pool_mask;
-            fp.out_ids = out_ids; fp.out_w = rp.w; fp.target = rp.target; fp.scale = rp.scale;
+            if (meta) {
+                fp.pool_ids = rp.pool_ids; fp.pool_size = rp.pool_size; fp.pool_mask = rp.pool_mask;
+                fp.out_ids = out_ids; fp.out_w = rp.w; fp.target = rp.target; fp.scale = rp.scale;
+            }
             fp.H = at<__nv_bfloat16>(ws, pl.H); fp.row_tok = rp.row_tok; fp.row_w = rp.row_w;
             fp.slot_row = rp.slot_row;
             fp.grp_expert = rp.grp_expert; fp.grp_off = rp.grp_off; fp.grp_tiles = rp.grp_tiles; fp.n_groups = rp.n_groups;

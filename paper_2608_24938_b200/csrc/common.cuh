@@ -282,7 +282,7 @@ struct DecodeFfnParams {
     const float* st_scale;
     int B, N, K, M, n_shared, d, I, a_rows;
     int stages, scratch_off;  // shared-memory plan made by the launcher
-    // metadata written by CTA 0 (workspace copies)
+    // metadata written by CTA 0 (workspace copies; all null when the caller asks for none)
     int32_t* pool_ids;    // [N] (-1 padded)
     int32_t* pool_size;   // [1]
     uint32_t* pool_mask;  // [8]

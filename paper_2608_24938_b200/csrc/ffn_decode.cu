@@ -26,6 +26,11 @@
 // that own a group's first slice write its execution lists (row -> token, merged weight, slot -> row); CTA 0 writes
 // the routing metadata and the group table.
 //
+// Routing prologue, dependency wait -> pool known -> first weights multiplied -> row lists done: 64 tokens 3.2 -> 5.9 -> 12 us
+// before the members-only ranking, the eight-lane target search and the token masks; 256 tokens 4.5, 19 (nothing streams
+// before the lists there), 17 us. Whole call then -> now: Qwen3 shape 64 tokens, pool 16 43.4 -> 42.4 us; 256 tokens with the
+// router, pool 64 192 -> 180, pool 16 74 -> 66 (also a fourth ring stage, from the slot tables' bytes).
+//
 // Item sizes: full slices of 128 features; the last partial round of full items is cut into halves (s = 64) when
 // that lets more SMs share it, and a trailing 64-wide slice of I is a half by itself.
 #include <algorithm>
@@ -49,7 +54,7 @@ static_assert(kGemmBK == 64, "the decode FFN kernel stages 64 K elements per k-b
 static_assert(kMaxDecodeBatch <= 256, "two token tiles per group at most");
 
 struct Scratch {  // per-batch routing state, one copy per CTA
-    long long key[kMaxExperts];        // order-preserving integer image of score_e (LLONG_MIN: not in the union)
+    long long key[kMaxExperts];        // by union member: order-preserving integer image of score_e
     unsigned acc32[3 * kMaxExperts];   // sum_i w_{i,e} in 2^-53 units, as three 21-bit limbs
     int in_union[kMaxExperts];
     int rank_of[kMaxExperts];  // pool rank or -1
@@ -57,10 +62,10 @@ struct Scratch {  // per-batch routing state, one copy per CTA
     int target[kMaxExperts];
     float scale[kMaxExperts];
     float h[kMaxExperts];      // norm table (dynamic pool), staged before the dependency wait
-    int cnt[kFMaxPairs];       // rows of (group, token tile): distinct tokens of the tile that the group serves
-    int goff[kFMaxPairs + 2];  // exclusive prefix of cnt: first compact row of (group, token tile)
-    int pairs[kFMaxPairs];     // the pairs that have rows, in order: group * 2 + token tile
-    int P, n_pairs;
+    int goff[kFMaxPairs + 2];  // exclusive prefix over (group, token tile): first compact row
+    int pairs[kFMaxPairs];     // the pairs that have rows, in order: group * 2 + token tile (before that: the union's experts)
+    int chunk_cnt[kMaxExperts / 32];
+    int P, U, n_pairs;
 };
 constexpr int kFScratchFixed = (int)((sizeof(Scratch) + 15) / 16 * 16);
 
@@ -170,8 +175,10 @@ __global__ void __launch_bounds__(kFThreads, 1) decode_ffn_kernel(const __grid_c
     const int a_bytes = p.a_rows * kFBK * 2;
     const int stage_bytes = a_bytes + kFBBytes;
     Scratch& sc = *reinterpret_cast<Scratch*>(tiles + p.scratch_off);
-    int* ids2 = reinterpret_cast<int*>(tiles + p.scratch_off + kFScratchFixed);
-    float* w2 = reinterpret_cast<float*>(ids2 + p.B * p.K);
+    // one byte per slot (its routed expert, then its target) and, by pool rank, the tokens each group serves as bit masks:
+    // what is not spent here is ring (256 tokens x 8 slots: 20 KB with ids and weights as words, one stage of four)
+    unsigned char* ids8 = tiles + p.scratch_off + kFScratchFixed;
+    uint32_t* tmask = reinterpret_cast<uint32_t*>(ids8 + align16((size_t)p.B * p.K));
 
     // ---- set-up that does not depend on the previous kernel: overlaps its tail under programmatic launch
     if (threadIdx.x == 0) {
@@ -207,7 +214,8 @@ __global__ void __launch_bounds__(kFThreads, 1) decode_ffn_kernel(const __grid_c
         sc.in_union[e] = 0;
         sc.rank_of[e] = -1;
     }
-    for (int i = threadIdx.x; i < kFMaxPairs; i += kFThreads) sc.cnt[i] = 0;
+    const int W = nmt * 4;  // mask words per group
+    for (int i = threadIdx.x; i < (N + 1) * W; i += kFThreads) tmask[i] = 0u;
     if (!is_static) {  // the norm table into shared memory, the loss and scalar tables into L2, while the previous kernel runs
         for (int e = threadIdx.x; e < N; e += kFThreads) sc.h[e] = __ldg(p.h + e);
         const size_t n_el = (size_t)N * N, lines = (n_el * 4 + 127) / 128;
@@ -236,7 +244,7 @@ __global__ void __launch_bounds__(kFThreads, 1) decode_ffn_kernel(const __grid_c
         for (int u = 0; u < 8; ++u) {
             const int s = s0 + u * kFThreads;
             if (id[u] < 0) continue;
-            ids2[s] = id[u];
+            ids8[s] = (unsigned char)id[u];
             if (!is_static) {
                 // The routed weight in 2^-53 fixed point, added as three 21-bit limbs with 32-bit integer atomics (at
                 // most 256 addends per expert, so no limb overflows): exact, and independent of the order of arrival.
@@ -262,41 +270,59 @@ __global__ void __launch_bounds__(kFThreads, 1) decode_ffn_kernel(const __grid_c
         if (threadIdx.x == 0) sc.P = p.M;
         __syncthreads();
     } else {
-        // Eq. 11: score_e = h_e * sum_i w_{i,e} in double; ranked through an order-preserving integer key
-        for (int e = threadIdx.x; e < N; e += kFThreads) {
-            long long key = LLONG_MIN;  // not in the union: never counted, never ranked
-            if (sc.in_union[e]) {
-                const unsigned long long acc = (unsigned long long)sc.acc32[3 * e] +
-                                               ((unsigned long long)sc.acc32[3 * e + 1] << 21) +
-                                               ((unsigned long long)sc.acc32[3 * e + 2] << 42);
-                const double score = (double)acc * (1.0 / 9007199254740992.0) * (double)sc.h[e] + 0.0;
-                key = __double_as_longlong(score);
-                if (key < 0) key ^= 0x7FFFFFFFFFFFFFFFll;  // negative doubles: larger magnitude = smaller
-            }
-            sc.key[e] = key;
+        // Eq. 11: score_e = h_e * sum_i w_{i,e} in double, for the union's experts (in ascending order), ranked through an
+        // order-preserving integer key
+        const int n_chunks = (N + 31) >> 5;
+        for (int c = warp; c < n_chunks; c += kFThreads / 32) {
+            const unsigned m = __ballot_sync(0xffffffffu, c * 32 + lane < N && sc.in_union[c * 32 + lane]);
+            if (lane == 0) sc.chunk_cnt[c] = __popc(m);
         }
         __syncthreads();
-        // pool = best min(M, |U|) experts of the union by (score desc, id asc): rank by counting, a thread per expert
-        // (integer compares on the keys; every lane of a warp reads the same other key: one broadcast load each)
-        for (int e = threadIdx.x; e < N; e += kFThreads) {
-            const long long ke = sc.key[e];
-            if (ke == LLONG_MIN) continue;
+        int* member = sc.pairs;
+        int U = 0;
+        for (int c = 0; c < n_chunks; ++c) U += sc.chunk_cnt[c];
+        for (int c = warp; c < n_chunks; c += kFThreads / 32) {
+            const int e = c * 32 + lane;
+            const bool in = e < N && sc.in_union[e];
+            const unsigned m = __ballot_sync(0xffffffffu, in);
+            if (!in) continue;
+            int pos = __popc(m & ((1u << lane) - 1u));
+            for (int q = 0; q < c; ++q) pos += sc.chunk_cnt[q];
+            const unsigned long long acc = (unsigned long long)sc.acc32[3 * e] +
+                                           ((unsigned long long)sc.acc32[3 * e + 1] << 21) +
+                                           ((unsigned long long)sc.acc32[3 * e + 2] << 42);
+            const double score = (double)acc * (1.0 / 9007199254740992.0) * (double)sc.h[e] + 0.0;
+            long long key = __double_as_longlong(score);
+            if (key < 0) key ^= 0x7FFFFFFFFFFFFFFFll;  // negative doubles: larger magnitude = smaller
+            member[pos] = e;
+            sc.key[pos] = key;
+        }
+        __syncthreads();
+        // pool = best min(M, |U|) experts of the union by (score desc, id asc): rank by counting, several threads per member
+        // (a thread per expert over all N keys took 1.8 us for N = 128)
+        int lanes = 32;
+        while (lanes > 1 && U * lanes > kFThreads) lanes >>= 1;
+        const int sub = threadIdx.x & (lanes - 1);
+        for (int i0 = 0; i0 < U; i0 += kFThreads / lanes) {
+            const int i = i0 + (int)threadIdx.x / lanes;
             int better = 0;
+            if (i < U) {
+                const long long ki = sc.key[i];
 #pragma unroll 4
-            for (int o = 0; o < N; ++o) {
-                const long long ko = sc.key[o];
-                better += (ko > ke || (ko == ke && o < e)) ? 1 : 0;
+                for (int o = sub; o < U; o += lanes) {
+                    const long long ko = sc.key[o];
+                    better += (ko > ki || (ko == ki && o < i)) ? 1 : 0;  // members ascend: position order is id order
+                }
             }
-            if (better < p.M) {
-                sc.rank_of[e] = better;
-                sc.pool[better] = e;
+            for (int o = lanes >> 1; o > 0; o >>= 1) better += __shfl_xor_sync(0xffffffffu, better, o);
+            if (i < U && sub == 0 && better < p.M) {
+                sc.rank_of[member[i]] = better;
+                sc.pool[better] = member[i];
             }
         }
-        if (warp == 0) {
-            int usz = 0;
-            for (int o = lane; o < N; o += 32) usz += sc.in_union[o] ? 1 : 0;
-            usz = __reduce_add_sync(0xffffffffu, usz);
-            if (lane == 0) sc.P = usz < p.M ? usz : p.M;
+        if (threadIdx.x == 0) {
+            sc.P = U < p.M ? U : p.M;
+            sc.U = U;
         }
         __syncthreads();
     }
@@ -308,52 +334,71 @@ __global__ void __launch_bounds__(kFThreads, 1) decode_ffn_kernel(const __grid_c
     };
     if (mine) {
         const int P = sc.P, G = P + (p.n_shared ? 1 : 0);
+        const bool meta = p.pool_ids != nullptr && blockIdx.x == 0;  // the caller asked for the routing metadata
         if (!is_static) {
             // Eq. 12: a source in the pool keeps itself; any other takes its minimum-loss pool expert (ties -> lower
-            // id). Only sources that occur in the batch matter for the execution; CTA 0 fills the whole table.
-            for (int s = tid; s < N; s += nth) {
-                if (blockIdx.x != 0 && !sc.in_union[s]) continue;
-                int bt = s;
-                float scl = 1.0f;
-                if (sc.rank_of[s] < 0) {
-                    const float* row = p.L + (size_t)s * N;
-                    float bl = INFINITY;
-                    bt = 0x7fffffff;
-                    for (int j0 = 0; j0 < P; j0 += 8) {  // eight independent loads in flight
-                        float l[8];
-                        int tt[8];
+            // id). Eight lanes per source, loss and scalar of 32 candidates in one round trip (a thread per source with
+            // its candidates one after the other took 8 us for a pool of 64). Only sources that occur in the batch
+            // matter for the execution; the metadata has the whole table.
+            const int n_src = meta ? N : sc.U, n_grp = nth >> 3, sub = tid & 7;
+            for (int i0 = 0; i0 < n_src; i0 += n_grp) {
+                const int i = i0 + (tid >> 3);
+                const int s = i < n_src ? (meta ? i : sc.pairs[i]) : -1;
+                float bl = INFINITY, bs = 1.0f;
+                int bt = 0x7fffffff;
+                if (s >= 0 && sc.rank_of[s] < 0) {
+                    for (int j0 = sub; j0 < P; j0 += 32) {
+                        float l[4], sv[4];
+                        int tt[4];
 #pragma unroll
-                        for (int u = 0; u < 8; ++u) {
-                            tt[u] = j0 + u < P ? sc.pool[j0 + u] : -1;
-                            l[u] = tt[u] >= 0 ? __ldg(row + tt[u]) : INFINITY;
+                        for (int u = 0; u < 4; ++u) {
+                            tt[u] = j0 + 8 * u < P ? sc.pool[j0 + 8 * u] : -1;
+                            l[u] = tt[u] >= 0 ? __ldg(p.L + (size_t)s * N + tt[u]) : 0.f;
+                            sv[u] = tt[u] >= 0 ? __ldg(p.S + (size_t)s * N + tt[u]) : 0.f;
                         }
 #pragma unroll
-                        for (int u = 0; u < 8; ++u)
-                            if (tt[u] >= 0 && (bt == 0x7fffffff || l[u] < bl || (l[u] == bl && tt[u] < bt))) {
+                        for (int u = 0; u < 4; ++u)
+                            if (tt[u] >= 0 && (l[u] < bl || (l[u] == bl && tt[u] < bt))) {
                                 bl = l[u];
+                                bs = sv[u];
                                 bt = tt[u];
                             }
                     }
-                    scl = __ldg(p.S + (size_t)s * N + bt);
+                } else {
+                    bt = s;  // every lane of the eight alike
                 }
-                sc.target[s] = bt;
-                sc.scale[s] = scl;
+#pragma unroll
+                for (int o = 4; o > 0; o >>= 1) {
+                    const float ol = __shfl_xor_sync(0xffffffffu, bl, o), os = __shfl_xor_sync(0xffffffffu, bs, o);
+                    const int ot = __shfl_xor_sync(0xffffffffu, bt, o);
+                    if (ol < bl || (ol == bl && ot < bt)) {
+                        bl = ol;
+                        bs = os;
+                        bt = ot;
+                    }
+                }
+                if (s >= 0 && sub == 0) {
+                    sc.target[s] = bt;
+                    sc.scale[s] = bs;
+                }
             }
             sync_group();
         }
-        // Eq. 14: every slot in place; [B][K] layout kept
+        // Eq. 14: every slot in place; [B][K] layout kept. A token counts once per distinct target: a bit of its mask
         for (int s = tid; s < BK; s += nth) {
-            const int e = ids2[s];
-            const int t = sc.target[e];
-            const float wv = (float)(p.w64[s] * (double)sc.scale[e]);
-            ids2[s] = t;
-            w2[s] = wv;
-            if (blockIdx.x == 0) {
+            const int e = ids8[s], t = sc.target[e], i = s / K;
+            ids8[s] = (unsigned char)t;
+            atomicOr(&tmask[sc.rank_of[t] * W + (i >> 5)], 1u << (i & 31));
+            if (meta) {
                 p.out_ids[s] = t;
-                p.out_w[s] = wv;
+                p.out_w[s] = (float)(p.w64[s] * (double)sc.scale[e]);
             }
         }
-        if (blockIdx.x == 0) {
+        if (p.n_shared && tid < W) {
+            const int left = B - tid * 32;
+            tmask[P * W + tid] = left >= 32 ? 0xffffffffu : (left > 0 ? (1u << left) - 1u : 0u);
+        }
+        if (meta) {
             for (int e = tid; e < N; e += nth) {
                 p.target[e] = sc.target[e];
                 p.scale[e] = sc.scale[e];
@@ -370,23 +415,16 @@ __global__ void __launch_bounds__(kFThreads, 1) decode_ffn_kernel(const __grid_c
             if (tid == 0) *p.pool_size = P;
         }
         sync_group();
-        // rows per (group, token tile): a token counts once per distinct target among its slots
-        for (int i = tid; i < B; i += nth) {
-            for (int k = 0; k < K; ++k) {
-                const int t = ids2[i * K + k];
-                bool first = true;
-                for (int k2 = 0; k2 < k; ++k2) first = first && ids2[i * K + k2] != t;
-                if (first) atomicAdd(&sc.cnt[sc.rank_of[t] * 2 + (i >> 7)], 1);
-            }
-        }
-        if (p.n_shared && tid < 2) sc.cnt[P * 2 + tid] = tid == 0 ? min(B, 128) : max(B - 128, 0);
-        sync_group();
         // exclusive prefix over (group, tile) = first compact row of each; the pairs that have rows
         if (tid < 32) {
             int carry = 0, n = 0;
             for (int c0 = 0; c0 < 2 * G; c0 += 32) {
                 const int c = c0 + tid;
-                const int v = c < 2 * G ? sc.cnt[c] : 0;
+                int v = 0;
+                if (c < 2 * G && (c & 1) < nmt) {
+                    const uint4 m4 = *reinterpret_cast<const uint4*>(tmask + (c >> 1) * W + (c & 1) * 4);
+                    v = __popc(m4.x) + __popc(m4.y) + __popc(m4.z) + __popc(m4.w);
+                }
                 int incl = v;
 #pragma unroll
                 for (int o = 1; o < 32; o <<= 1) {
@@ -410,16 +448,26 @@ __global__ void __launch_bounds__(kFThreads, 1) decode_ffn_kernel(const __grid_c
                 p.grp_off[g] = sc.goff[2 * g];
                 if (g < G) p.grp_expert[g] = g < P ? sc.pool[g] : N;
             }
-            if (tid == 0) {
-                int tiles = 0;
-                for (int g = 0; g < G; ++g) {
-                    p.grp_tiles[g] = tiles;
-                    tiles += (sc.goff[2 * g + 2] - sc.goff[2 * g] + kTileM - 1) / kTileM;
+            if (tid < 32) {
+                int carry = 0;
+                for (int g0 = 0; g0 < G; g0 += 32) {
+                    const int g = g0 + tid;
+                    const int v = g < G ? (sc.goff[2 * g + 2] - sc.goff[2 * g] + kTileM - 1) / kTileM : 0;
+                    int incl = v;
+#pragma unroll
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const int u = __shfl_up_sync(0xffffffffu, incl, o);
+                        if (tid >= o) incl += u;
+                    }
+                    if (g < G) p.grp_tiles[g] = carry + incl - v;
+                    carry += __shfl_sync(0xffffffffu, incl, 31);
                 }
-                p.grp_tiles[G] = tiles;
-                p.n_groups[0] = G;
-                p.n_groups[1] = sc.goff[2 * G];
-                p.n_groups[2] = sc.goff[2 * P];  // first row of the shared expert's group
+                if (tid == 0) {
+                    p.grp_tiles[G] = carry;
+                    p.n_groups[0] = G;
+                    p.n_groups[1] = sc.goff[2 * G];
+                    p.n_groups[2] = sc.goff[2 * P];  // first row of the shared expert's group
+                }
             }
         }
     }
@@ -517,38 +565,32 @@ __global__ void __launch_bounds__(kFThreads, 1) decode_ffn_kernel(const __grid_c
         for (int w = w_begin; w < total; w += w_stride, ++item) {
             const Item it = decode_item(w, sched, sc, N);
             const int as = item & 1, aphase = (item >> 1) & 1;
-            // Which tokens of the tile does this expert serve? Every warp looks at all four quadrants, so that
-            // it knows how many rows come before its own without talking to the other warps.
+            // Which tokens of the tile does this expert serve? All four quadrants, so that a warp knows how many rows
+            // come before its own
             const bool shared_grp = it.g >= sc.P;
-            unsigned m[4];
-#pragma unroll
-            for (int qq = 0; qq < 4; ++qq) {
-                const int tq = it.mt * 128 + qq * 32 + lane;
-                bool v = false;
-                if (tq < B) {
-                    v = shared_grp;
-                    for (int k = 0; k < K && !v; ++k) v = ids2[tq * K + k] == it.expert;
-                }
-                m[qq] = __ballot_sync(0xffffffffu, v);
-            }
+            const uint4 m4 = *reinterpret_cast<const uint4*>(tmask + it.g * W + it.mt * 4);
+            const unsigned m[4] = {m4.x, m4.y, m4.z, m4.w};
             int before = 0;
 #pragma unroll
             for (int qq = 0; qq < 4; ++qq)
                 if (qq < q) before += __popc(m[qq]);
-            const bool valid = (m[q] >> lane) & 1u;
+            const unsigned mq = q == 0 ? m[0] : (q == 1 ? m[1] : (q == 2 ? m[2] : m[3]));
+            const bool valid = (mq >> lane) & 1u;
             const int tok = it.mt * 128 + row;
-            const int64_t rowpos = sc.goff[it.g * 2 + it.mt] + before + __popc(m[q] & ((1u << lane) - 1u));
+            const int64_t rowpos = sc.goff[it.g * 2 + it.mt] + before + __popc(mq & ((1u << lane) - 1u));
             if (it.j0 == 0 && valid) {
                 // this CTA owns the group's first slice: it writes the group's rows of the execution lists
                 float cw = 1.0f;
                 if (!shared_grp) {
                     bool has = false;
-                    for (int k = 0; k < K; ++k)
-                        if (ids2[tok * K + k] == it.expert) {  // duplicates merged, weights summed in slot order
-                            cw = has ? __fadd_rn(cw, w2[tok * K + k]) : w2[tok * K + k];
-                            p.slot_row[tok * K + k] = has ? -1 : (int32_t)rowpos;
-                            has = true;
-                        }
+                    for (int k = 0; k < K; ++k) {
+                        const int s = tok * K + k;
+                        if (ids8[s] != it.expert) continue;  // duplicates merged, weights summed in slot order
+                        const float wv = (float)(p.w64[s] * (double)sc.scale[p.ids[s]]);
+                        cw = has ? __fadd_rn(cw, wv) : wv;
+                        p.slot_row[s] = has ? -1 : (int32_t)rowpos;
+                        has = true;
+                    }
                 }
                 p.row_tok[rowpos] = tok;
                 p.row_w[rowpos] = cw;
@@ -558,7 +600,7 @@ __global__ void __launch_bounds__(kFThreads, 1) decode_ffn_kernel(const __grid_c
             ok = __shfl_sync(0xffffffffu, ok, 0);
             if (!ok) break;
             ptx::tc_fence_after();
-            if (m[q] != 0u) {  // warp-uniform: some row of this quadrant is stored
+            if (mq != 0u) {  // warp-uniform: some row of this quadrant is stored
                 const uint32_t taddr = tmem_base + as * 256 + ((uint32_t)(q * 32) << 16);
                 const int nch = it.s / 32;
 #pragma unroll 1
@@ -603,12 +645,12 @@ __global__ void __launch_bounds__(kFThreads, 1) decode_ffn_kernel(const __grid_c
 
 }  // namespace
 
-// Shared-memory plan: [ring: stages x (token box + 32 KB of weights)][routing state][ids', w']
+// Shared-memory plan: [ring: stages x (token box + 32 KB of weights)][routing state][ids', token masks]
 size_t decode_ffn_smem_plan(int B, int K, int N, int* stages, int* scratch_off, int* a_rows) {
-    (void)N;
     const int ar = std::min(kTileM, (B + 31) / 32 * 32);
     const int stage_bytes = ar * kFBK * 2 + kFBBytes;
-    const size_t scratch = (kFScratchFixed + (size_t)B * K * 8 + 15) / 16 * 16;
+    const int mask_words = (B + 127) / 128 * 4;
+    const size_t scratch = kFScratchFixed + align16((size_t)B * K) + (size_t)(N + 1) * mask_words * 4;
     const long avail = (long)kFSmemLimit - 1024 - (long)scratch;
     int st = (int)(avail / stage_bytes);
     if (st > kFMaxStages) st = kFMaxStages;
