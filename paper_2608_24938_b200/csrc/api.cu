@@ -959,30 +959,18 @@ static int router_enqueue(const exfold_layer* layer, const void* x, const void* 
     lc.n_shared = 0;
     const Plan pl = make_plan(lc, T, 1);
     if (ws_bytes < pl.total) return EXFOLD_ERR_WORKSPACE_TOO_SMALL;
-    if (clear_status) EXFOLD_CUDA(cudaMemsetAsync(at<char>(ws, pl.status), 0, sizeof(DeviceStatus), s));
-    // fp32 layers, and bf16 batches of at most one row tile (decode): dot products in a fixed order. One 128-row
-    // tile on the tensor cores would walk the whole K loop on a single SM (10-19 us of latency).
+    DeviceStatus* status = at<DeviceStatus>(ws, pl.status);
+    // fp32 layers, and bf16 batches of at most one row tile (decode): dot products in a fixed order
     if (l.dtype == EXFOLD_F32 || (T <= kTileM && aligned16(x) && aligned16(w_router))) {
-        EXFOLD_CUDA(launch_router_simt(x, w_router, l.dtype, T, N, d, logits, s));
+        EXFOLD_CUDA(launch_router_simt(x, w_router, l.dtype, T, N, d, logits, clear_status ? status : nullptr, s));
         return EXFOLD_OK;
     }
-    // bf16: one group of T rows through GEMM-2's instantiation of the grouped kernel (K = d, N output columns in
-    // one 256-column tile, raw fp32 row epilogue); W_r rows past N are zero-filled by the tensor map
     if (!aligned16(x) || !aligned16(w_router)) return EXFOLD_ERR_INVALID_ARG;
-    CUtensorMap tm_x, tm_wr;
-    if (!make_tmap(&tm_x, x, (uint64_t)T, d, 128) || !make_tmap(&tm_wr, w_router, (uint64_t)N, d, 256))
+    RouterGemmParams g{};
+    if (!make_tmap(&g.tm_x, x, (uint64_t)T, d, 128) || !make_tmap(&g.tm_wr, w_router, (uint64_t)N, d, (uint32_t)router_npad(N)))
         return EXFOLD_ERR_CUDA;
-    GroupedGemmParams g{};
-    g.tm_a = tm_x; g.tm_a2 = tm_x; g.tm_b0 = tm_wr; g.tm_b1 = tm_wr;
-    g.offsets = nullptr; g.work_start = nullptr; g.G = 1;  // one group of R = T rows
-    g.n_routed = 1; g.R = (int)T; g.x_rows = (int)T;
-    g.d = N;   // output width
-    g.I = d;   // contraction length
-    g.n_ntiles = 1; g.ksplit = 1; g.a_rows = kTileM;
-    g.row_tok = at<int32_t>(ws, pl.row_tok); g.row_w = at<float>(ws, pl.row_w);  // read, not used, by this epilogue
-    g.o32 = logits; g.status = at<DeviceStatus>(ws, pl.status);
-    const int64_t tiles = (T + kTileM - 1) / kTileM;
-    EXFOLD_CUDA(launch_grouped_gemm2(g, (int)std::min<int64_t>(sm_count(), tiles), s));
+    g.logits = logits; g.T = (int)T; g.N = N; g.nkb = d / kGemmBK; g.clear_status = clear_status ? 1 : 0; g.status = status;
+    EXFOLD_CUDA(launch_router_gemm(g, sm_count(), s));
     return EXFOLD_OK;
 }
 

@@ -66,53 +66,99 @@ __global__ void __launch_bounds__(256) combine_rows_kernel(const __nv_bfloat16* 
     }
 }
 
-// r[i][e] = <W_r[e], x_i>, fp32 accumulation in a fixed order, one warp per (token, expert): fp32 layers, and
-// bf16 batches too small to fill the tensor-core kernel (a single 128-row tile would walk K on one SM)
-template <typename T>
+// r[i][e] = <W_r[e], x_i>, fp32 accumulation in a fixed order: fp32 layers, and bf16 batches too small for the tensor-core
+// kernel. A warp takes EW experts x TW tokens: 1 x 1 spreads a small batch over the most warps; 4 x 4 reads a quarter of
+// the bytes through L2 and converts a quarter as often. The order of a score's sum is the same (lane partition, fused
+// multiply-adds, shuffle tree).
+template <typename T, int EW, int TW>
 __global__ void __launch_bounds__(256) router_simt_kernel(const T* __restrict__ x, const T* __restrict__ wr, int64_t Tn,
-                                                          int N, int d, float* __restrict__ out) {
+                                                          int N, int d, float* __restrict__ out, DeviceStatus* status) {
     const int64_t w = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
     grid_dep_launch();
     grid_dep_wait();  // x may be the output of the previous layer's last kernel
-    if (w >= Tn * N) return;
-    const int64_t i = w / N;
-    const int e = (int)(w % N);
-    const T* xi = x + i * d;
-    const T* we = wr + (size_t)e * d;
-    float acc = 0.f;
+    if (status != nullptr && blockIdx.x == 0 && threadIdx.x < 4) reinterpret_cast<int*>(status)[threadIdx.x] = 0;
+    const int eg = (N + EW - 1) / EW;
+    const int64_t i0 = w / eg * TW;
+    if (i0 >= Tn) return;
+    const int e0 = (int)(w % eg) * EW;
+    const T* xi[TW];
+    const T* we[EW];
+#pragma unroll
+    for (int t = 0; t < TW; ++t) xi[t] = x + (i0 + t < Tn ? i0 + t : Tn - 1) * d;
+#pragma unroll
+    for (int u = 0; u < EW; ++u) we[u] = wr + (size_t)min(e0 + u, N - 1) * d;
+    float acc[EW][TW];
+#pragma unroll
+    for (int u = 0; u < EW; ++u)
+#pragma unroll
+        for (int t = 0; t < TW; ++t) acc[u][t] = 0.f;
     if constexpr (sizeof(T) == 2) {  // bf16: 8 elements (16 bytes) per lane and step; d is a multiple of 64
+#pragma unroll 2
         for (int c = lane * 8; c < d; c += 256) {
-            const uint4 a = *reinterpret_cast<const uint4*>(we + c), b = *reinterpret_cast<const uint4*>(xi + c);
-            const __nv_bfloat162* pa = reinterpret_cast<const __nv_bfloat162*>(&a);
-            const __nv_bfloat162* pb = reinterpret_cast<const __nv_bfloat162*>(&b);
+            uint4 a[EW], b[TW];
+#pragma unroll
+            for (int u = 0; u < EW; ++u) a[u] = *reinterpret_cast<const uint4*>(we[u] + c);
+#pragma unroll
+            for (int t = 0; t < TW; ++t) b[t] = *reinterpret_cast<const uint4*>(xi[t] + c);
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
-                const float2 fa = __bfloat1622float2(pa[j]), fb = __bfloat1622float2(pb[j]);
-                acc = fmaf(fa.x, fb.x, acc);
-                acc = fmaf(fa.y, fb.y, acc);
+                float2 fa[EW];
+#pragma unroll
+                for (int u = 0; u < EW; ++u) fa[u] = __bfloat1622float2(reinterpret_cast<const __nv_bfloat162*>(&a[u])[j]);
+#pragma unroll
+                for (int t = 0; t < TW; ++t) {
+                    const float2 fb = __bfloat1622float2(reinterpret_cast<const __nv_bfloat162*>(&b[t])[j]);
+#pragma unroll
+                    for (int u = 0; u < EW; ++u) {
+                        acc[u][t] = fmaf(fa[u].x, fb.x, acc[u][t]);
+                        acc[u][t] = fmaf(fa[u].y, fb.y, acc[u][t]);
+                    }
+                }
             }
         }
     } else {
-        for (int c = lane; c < d; c += 32) acc = fmaf((float)we[c], (float)xi[c], acc);
+        for (int c = lane; c < d; c += 32) {
+            float fa[EW];
+#pragma unroll
+            for (int u = 0; u < EW; ++u) fa[u] = (float)we[u][c];
+#pragma unroll
+            for (int t = 0; t < TW; ++t) {
+                const float fb = (float)xi[t][c];
+#pragma unroll
+                for (int u = 0; u < EW; ++u) acc[u][t] = fmaf(fa[u], fb, acc[u][t]);
+            }
+        }
     }
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-    if (lane == 0) out[w] = acc;
+    for (int u = 0; u < EW; ++u)
+#pragma unroll
+        for (int t = 0; t < TW; ++t) {
+            float v = acc[u][t];
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+            if (lane == 0 && e0 + u < N && i0 + t < Tn) out[(i0 + t) * N + e0 + u] = v;
+        }
 }
 
+// bf16: 4 x 4 scores per warp once that leaves two warps per SM (Qwen3-shaped prefill of 100 tokens 205.7 -> 202.6 us); fp32 rows
+// are too short for it (150 tokens x 64 experts x 512: 86.0 us, 89.8 with the tile)
+constexpr int kRouterTileWarps = 296;
 }  // namespace
 
 cudaError_t launch_router_simt(const void* x, const void* wr, int dtype, int64_t T, int N, int d, float* out,
-                               cudaStream_t s) {
-    const int64_t warps = T * N;
-    if (warps == 0) return cudaSuccess;
-    const unsigned grid = (unsigned)((warps + 7) / 8);
-    if (dtype == EXFOLD_BF16)
-        return launch_pdl(router_simt_kernel<__nv_bfloat16>, grid, 256, 0, s, reinterpret_cast<const __nv_bfloat16*>(x),
-                          reinterpret_cast<const __nv_bfloat16*>(wr), T, N, d, out);
-    return launch_pdl(router_simt_kernel<float>, grid, 256, 0, s, reinterpret_cast<const float*>(x),
-                      reinterpret_cast<const float*>(wr), T, N, d, out);
+                               DeviceStatus* status, cudaStream_t s) {
+    if (T * N == 0) return cudaSuccess;
+    const unsigned grid = (unsigned)((T * N + 7) / 8);
+    if (dtype != EXFOLD_BF16)
+        return launch_pdl(router_simt_kernel<float, 1, 1>, grid, 256, 0, s, reinterpret_cast<const float*>(x),
+                          reinterpret_cast<const float*>(wr), T, N, d, out, status);
+    const __nv_bfloat16* xb = reinterpret_cast<const __nv_bfloat16*>(x);
+    const __nv_bfloat16* wb = reinterpret_cast<const __nv_bfloat16*>(wr);
+    const int64_t tiles = (T + 3) / 4 * ((N + 3) / 4);
+    if (tiles >= kRouterTileWarps)
+        return launch_pdl(router_simt_kernel<__nv_bfloat16, 4, 4>, (unsigned)((tiles + 7) / 8), 256, 0, s, xb, wb, T, N, d, out, status);
+    return launch_pdl(router_simt_kernel<__nv_bfloat16, 1, 1>, grid, 256, 0, s, xb, wb, T, N, d, out, status);
 }
 
 cudaError_t launch_combine_rows(const __nv_bfloat16* O, const int32_t* inv_pos, int64_t T, int Kr, int d,

@@ -370,8 +370,22 @@ cudaError_t launch_combine_f32(const float* out, const int32_t* inv_pos, const f
                                int n_shared, const int32_t* shared0_dev, float* y, cudaStream_t s);
 
 // ---------------------------------------------------------------- router scores, final sums of the bf16 path
+// Router scores of more than one row tile of tokens, bf16 (router_gemm.cu)
+struct RouterGemmParams {
+    CUtensorMap tm_x;   // x [T][d], box 128 x 64
+    CUtensorMap tm_wr;  // W_r [N][d], box router_npad(N) x 64 (rows past N are zero-filled)
+    float* logits;      // [T][N]
+    int T, N, nkb;      // nkb = d / 64
+    int clear_status;   // the call's first kernel
+    DeviceStatus* status;
+    // set by the launcher
+    int split, npad, part_ld, stages;
+    uint32_t tmem_cols;
+};
+int router_npad(int N);
+cudaError_t launch_router_gemm(RouterGemmParams p, int sms, cudaStream_t s);
 cudaError_t launch_router_simt(const void* x, const void* wr, int dtype, int64_t T, int N, int d, float* out,
-                               cudaStream_t s);
+                               DeviceStatus* status, cudaStream_t s);
 // y[i] = sum_j O[inv_pos[i*Kr+j]] (entries < 0 skipped) (+ O[shared0 + i] for the shared expert), fp32 sum in slot
 // order, bf16 out. shared0 = T*Kr, or *shared0_dev when that is given (decode: known only on the device). A row may
 // be stored as `parts` partial rows (decode's K split), part k at row k * part_rows + row: summed in that order.

@@ -134,9 +134,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1) grouped_gemm_kernel(const __g
     // bound in the same round trip (rows past the device's count are never used)
     const int gd = DEC ? *p.n_groups_dev : G;
     for (int i = threadIdx.x; i <= G; i += kGemmThreads) {
-        // offsets == null: one group of p.R rows (a plain GEMM, e.g. the router scores)
-        s_off[i] = p.offsets != nullptr ? p.offsets[i] : i * p.R;
-        s_ws[i] = p.offsets != nullptr ? p.work_start[i] : i * ((p.R + kTileM - 1) / kTileM);
+        s_off[i] = p.offsets[i];
+        s_ws[i] = p.work_start[i];
         if (DEC) s_exp[i] = i < G ? p.grp_expert[i] : i;  // group -> expert whose weights it uses
     }
     if (DEC) G = gd < G ? gd : G;
@@ -377,7 +376,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) grouped_gemm_kernel(const __g
                             dst[j] = make_uint4(pk[4 * j], pk[4 * j + 1], pk[4 * j + 2], pk[4 * j + 3]);
                     }
                 }
-            } else if (!DEC && p.o32 != nullptr) {  // raw fp32 rows (calibration outputs, router scores)
+            } else if (!DEC && p.o32 != nullptr) {  // raw fp32 rows (calibration outputs)
 #pragma unroll 1
                 for (int c = 0; c < 8; ++c) {
                     const int col0 = it.n_idx * 256 + c * 32;
@@ -385,17 +384,10 @@ __global__ void __launch_bounds__(kGemmThreads, 1) grouped_gemm_kernel(const __g
                     uint32_t v[32];
                     ptx::tmem_ld32(taddr + c * 32, v);
                     ptx::tmem_ld_wait();
-                    if (col0 + 32 <= p.d && (p.d & 3) == 0) {
 #pragma unroll
-                        for (int j = 0; j < 8; ++j)
-                            stage_put(out_buf, lane, j, make_uint4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]));
-                        stage_flush(out_buf, lane, vmask, (int)grow, reinterpret_cast<char*>(p.o32 + col0), (size_t)p.d * 4);
-                    } else if (valid) {  // ragged or unaligned row end (router scores of an odd number of experts)
-                        float* dstf = p.o32 + grow * p.d + col0;
-#pragma unroll
-                        for (int j = 0; j < 32; ++j)
-                            if (col0 + j < p.d) dstf[j] = __uint_as_float(v[j]);
-                    }
+                    for (int j = 0; j < 8; ++j)
+                        stage_put(out_buf, lane, j, make_uint4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]));
+                    stage_flush(out_buf, lane, vmask, (int)grow, reinterpret_cast<char*>(p.o32 + col0), (size_t)p.d * 4);
                 }
             } else {
                 // decode with a K split: part k of a row goes to plane k of the row buffer (p.R rows each)

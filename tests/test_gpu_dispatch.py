@@ -151,3 +151,27 @@ def test_decode_router_scores_by_batch(B, N):
     case.lgd, case.d_lgd = lg.cpu(), lg
     ref = case.oracle_decode(6)
     check_output(y.float().cpu().numpy(), ref["y"], "bf16")
+
+
+@pytest.mark.parametrize("T", [1, 5, 128, 129, 300, 777, 5000])
+@pytest.mark.parametrize("N,d", [(31, 64), (40, 320), (130, 2048), (256, 1088)])
+def test_router_scores_by_prompt_length(T, N, d):
+    """Dot-product kernel up to one row tile (one or 4 x 4 scores per warp), tensor cores with K split over a cluster above
+    (one, two and eight parts, ragged last tile, experts off every multiple) against double sums. Products of bf16 are
+    exact in fp32, so the error is the additions': at most d of them, each within 2^-23 of the partial sum's bound
+    sum |w x|."""
+    from paper_2608_24938_b200 import binding as ex
+    dev = torch.device("cuda:0")
+    g = torch.Generator(device=dev)
+    g.manual_seed(T + N)
+    x = torch.randn((T, d), generator=g, device=dev).to(torch.bfloat16)
+    wr = (torch.randn((N, d), generator=g, device=dev) * d ** -0.5).to(torch.bfloat16)
+    layer = ex.make_layer(N, 0, d, 64, 2, "bf16")
+    ws = ex.alloc_workspace(layer, T, 1)
+    ws.fill_(0xFF)  # also a status record to clear
+    lg = torch.full((T, N), float("nan"), device=dev)
+    assert ex.exfold_router_logits(layer, x, wr, lg, ws) == 0
+    assert ex.exfold_device_status(ws) == 0
+    want = x.double() @ wr.double().T
+    bound = d * 2.0 ** -23 * (x.double().abs() @ wr.double().abs().T)
+    assert bool(((lg.double() - want).abs() <= bound).all())
