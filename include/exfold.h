@@ -26,7 +26,8 @@
  *     three events (large prefill calls run two kernel chains side by side on it) and two copy streams
  *     with ten events (chunked host-buffer prefill). Calls issued by one host thread on
  *     different caller streams share them, so the parts that use them run one after the other;
- *     results do not depend on it. (b) per process: the launch counter, the optional
+ *     results do not depend on it. Also per host thread: for which kernels and devices it has
+ *     raised the shared-memory limit. (b) per process: the launch counter, the optional
  *     per-kernel timing events (exfold_profile_*, off by default, not thread-safe) and the
  *     built-in scratch array of exfold_moe_decode_noalloc. No environment variable is read.
  *   - Calls enqueue work on `cuda_stream` (a cudaStream_t passed as void*, NULL = the

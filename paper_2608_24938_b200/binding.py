@@ -155,7 +155,8 @@ def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
 
 
 def _stream(stream: Optional[torch.cuda.Stream]) -> int:
-    return (stream or torch.cuda.current_stream()).cuda_stream
+    # the raw handle of the current stream: torch.cuda.current_stream() builds a Stream object first, 3.3 us per call
+    return stream.cuda_stream if stream is not None else torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 def make_layer(n_experts: int, n_shared: int, hidden: int, inter: int, top_k: int, dtype) -> exfold_layer:

@@ -197,6 +197,32 @@ ThreadDeviceState* thread_state() {
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return nullptr;
     return &t_state[dev];
 }
+}  // namespace
+
+cudaError_t ensure_smem_bytes(const void* kernel, size_t bytes) {
+    struct Entry {
+        const void* kernel;
+        int dev;
+        size_t limit;
+    };
+    static thread_local Entry cache[256] = {};  // by kernel address; a collision only asks the driver again
+    int dev = 0, optin = 0;
+    cudaError_t err = cudaGetDevice(&dev);
+    if (err != cudaSuccess) return err;
+    Entry& e = cache[(reinterpret_cast<uintptr_t>(kernel) >> 4) & 255];
+    if (e.kernel != kernel || e.dev != dev) {
+        // every thread sets the same value, the most a block may have, so none can lower what another relies on
+        cudaFuncAttributes fa;
+        if ((err = cudaFuncGetAttributes(&fa, kernel)) != cudaSuccess) return err;
+        if ((err = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess) return err;
+        const size_t limit = (size_t)optin - fa.sharedSizeBytes;
+        if ((err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)limit)) != cudaSuccess) return err;
+        e = Entry{kernel, dev, limit};
+    }
+    return bytes <= e.limit ? cudaSuccess : cudaErrorInvalidValue;
+}
+
+namespace {
 bool new_event(cudaEvent_t* e) { return cudaEventCreateWithFlags(e, cudaEventDisableTiming) == cudaSuccess; }
 // second stream (and fork / join events) for the odd-tile passes of a prefill call
 ThreadDeviceState* side_stream() {

@@ -549,7 +549,7 @@ bool decode_small_fits(int B, int K, int d, const void* wg, const void* wu, cons
 
 cudaError_t launch_decode_small(DecodeSmallParams p, int sms, cudaStream_t s) {
     const size_t smem = gateup_bytes(p.B, p.K, p.d);
-    cudaError_t err = cudaFuncSetAttribute(decode_small_gateup_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t err = ensure_smem(decode_small_gateup_kernel, smem);
     if (err != cudaSuccess) return err;
     err = launch_pdl(decode_small_gateup_kernel, std::min(2 * sms, p.max_groups * (p.I / 8)), kThreads, smem, s, p);
     if (err != cudaSuccess) return err;
@@ -560,7 +560,7 @@ cudaError_t launch_decode_small(DecodeSmallParams p, int sms, cudaStream_t s) {
     p.split = 1;
     while (p.split < 8 && items * p.split * 2 <= sms) p.split *= 2;
     const size_t smem2 = (size_t)p.max_groups * (kTB * 8 + 4);
-    err = cudaFuncSetAttribute(decode_small_down_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem2);
+    err = ensure_smem(decode_small_down_kernel, smem2);
     if (err != cudaSuccess) return err;
     if (p.split > 1) return launch_pdl_cluster(decode_small_down_kernel, items * p.split, 32 * warps, smem2, p.split, s, p);
     return launch_pdl(decode_small_down_kernel, items, 32 * warps, smem2, s, p);

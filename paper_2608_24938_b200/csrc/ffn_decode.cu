@@ -664,7 +664,7 @@ cudaError_t launch_decode_ffn(const DecodeFfnParams& p, int sms, cudaStream_t s)
     int stages, scratch_off, a_rows;
     const size_t smem = decode_ffn_smem_plan(p.B, p.K, p.N, &stages, &scratch_off, &a_rows);
     if (stages < 2 || stages != p.stages || scratch_off != p.scratch_off) return cudaErrorInvalidValue;
-    cudaError_t err = cudaFuncSetAttribute(decode_ffn_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t err = ensure_smem(decode_ffn_kernel, smem);
     if (err != cudaSuccess) return err;
     return launch_pdl(decode_ffn_kernel, std::min(sms, kMaxCtas), kFThreads, smem, s, p);
 }

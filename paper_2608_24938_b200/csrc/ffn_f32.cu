@@ -403,7 +403,7 @@ size_t tall_bytes(int tile_rows, int I) {  // two stages of 128 weight rows and 
 
 template <typename K>
 cudaError_t launch_t(K kernel, const FfnF32Params& p, size_t smem, int64_t tiles, cudaStream_t s) {
-    cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t err = ensure_smem(kernel, smem);
     if (err != cudaSuccess) return err;
     return launch_pdl_cluster(kernel, (unsigned)(tiles * kCl), kThreads, smem, kCl, s, p);
 }

@@ -361,8 +361,7 @@ __global__ void __launch_bounds__(kPThreads, 1) grouped_gemm_pair_kernel(const _
 
 template <int MODE>
 cudaError_t launch_pair_t(const GroupedGemmParams& p, int grid, cudaStream_t s) {
-    cudaError_t err = cudaFuncSetAttribute(grouped_gemm_pair_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           kPSmem);
+    cudaError_t err = ensure_smem(grouped_gemm_pair_kernel<MODE>, kPSmem);
     if (err != cudaSuccess) return err;
     grid &= ~1;  // whole pairs
     if (grid < 2) grid = 2;

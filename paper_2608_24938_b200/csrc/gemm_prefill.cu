@@ -448,8 +448,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) grouped_gemm_kernel(const __g
 // time, like the CTA-pair kernel it runs beside, and the two grids cannot leave each other half-filled SM pairs.
 template <int MODE, bool DEC>
 static cudaError_t launch_gemm_t(const GroupedGemmParams& p, int grid, cudaStream_t s, bool whole_tpcs = false) {
-    cudaError_t err = cudaFuncSetAttribute(grouped_gemm_kernel<MODE, DEC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           kGemmSmem);
+    cudaError_t err = ensure_smem(grouped_gemm_kernel<MODE, DEC>, kGemmSmem);
     if (err != cudaSuccess) return err;
     if (whole_tpcs)
         return launch_pdl_cluster(grouped_gemm_kernel<MODE, DEC>, std::max(2, grid & ~1), kGemmThreads, kGemmSmem, 2, s, p);

@@ -505,8 +505,7 @@ cudaError_t launch_decode_route(const DecodeRouteParams& p, cudaStream_t s) {
     const size_t smem = kDecSmemBytes + 2 * (size_t)((p.N + ncl - 1) / ncl) * p.N * sizeof(float);
     cudaError_t err = cudaSuccess;
 #define EXFOLD_DEC_LAUNCH(NPL)                                                                              \
-    err = cudaFuncSetAttribute(decode_route_kernel<NPL>, cudaFuncAttributeMaxDynamicSharedMemorySize,       \
-                               (int)smem);                                                                  \
+    err = ensure_smem(decode_route_kernel<NPL>, smem);                                                                  \
     if (err != cudaSuccess) return err;                                                                     \
     err = launch_pdl_cluster(decode_route_kernel<NPL>, ncl, kDecThreads, smem, ncl, s, p);
     switch (npl) {

@@ -195,7 +195,7 @@ cudaError_t launch_router_gemm(RouterGemmParams p, int sms, cudaStream_t s) {
     const int per = (p.nkb + p.split - 1) / p.split;
     p.stages = std::max(2, std::min(std::min(kRMaxStages, per), 200 * 1024 / stage_bytes));
     const size_t smem = std::max((size_t)p.stages * stage_bytes, (size_t)128 * p.part_ld * sizeof(float)) + 1024;
-    cudaError_t err = cudaFuncSetAttribute(router_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t err = ensure_smem(router_gemm_kernel, smem);
     if (err != cudaSuccess) return err;
     return launch_pdl_cluster(router_gemm_kernel, (unsigned)(tiles * p.split), kRThreads, smem, p.split, s, p);
 }
