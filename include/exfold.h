@@ -23,8 +23,9 @@
  *     workspace must be ordered on one stream.
  *   - What the library keeps between calls, and nothing else: (a) per host thread and device,
  *     created on first use and freed by exfold_thread_release: one extra CUDA stream (highest priority) with
- *     three events (large prefill calls run two kernel chains side by side on it) and two copy streams
- *     with ten events (chunked host-buffer prefill). Calls issued by one host thread on
+ *     three events (large prefill calls run two kernel chains side by side on it), two copy streams
+ *     with ten events (chunked host-buffer prefill) and 1 KiB of pinned host memory (the counts that
+ *     calibrations return). Calls issued by one host thread on
  *     different caller streams share them, so the parts that use them run one after the other;
  *     results do not depend on it. Also per host thread: for which kernels and devices it has
  *     raised the shared-memory limit. (b) per process: the launch counter, the optional

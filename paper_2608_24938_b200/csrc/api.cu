@@ -50,8 +50,8 @@ void prof_reset() {
 // ------------------------------------------------------------------ workspace plan
 struct Plan {
     size_t status, ids, w, omit_src, omit_tgt, block_hist, sb_hist, offsets, work_start, totals, perm, row_tok, row_w,
-        row_exp, pool_ids, pool_size, pool_mask, target, scale, grp_expert, grp_off, n_groups, zeros, calib, big,
-        xs, H, out, grp_tiles, obuf, inv_pos, calib_nrm, calib_warn, w64, total;
+        row_exp, pool_ids, pool_size, pool_mask, target, scale, grp_expert, grp_off, n_groups, calib, big,
+        xs, H, out, grp_tiles, obuf, inv_pos, calib_nrm, w64, total;
 };
 
 bool valid_layer(const exfold_layer* l) {
@@ -78,9 +78,6 @@ Plan make_plan(const exfold_layer& l, int64_t Tm, int Kr) {
         return at;
     };
     p.status = take(sizeof(DeviceStatus));
-    // calibration: unobserved-expert count of each job of a call (ahead of everything whose size depends on the
-    // token count, so that jobs of different lengths share the slots)
-    p.calib_warn = take((size_t)EXFOLD_MAX_CALIB_JOBS * 4);
     p.ids = take(Rm * 4);
     p.w = take(Rm * 4);
     p.omit_src = take((size_t)Tm * l.top_k * 4);
@@ -105,7 +102,6 @@ Plan make_plan(const exfold_layer& l, int64_t Tm, int Kr) {
     p.grp_off = take((G + 2) * 4);
     p.grp_tiles = take((G + 2) * 4);
     p.n_groups = take(16);
-    p.zeros = take((size_t)N * 4);
     p.calib = take((size_t)N * N * (3 * 8 + 4) + (size_t)N * (8 + 4) + 256);
     p.calib_nrm = take(Rm * 8);  // calibration, common-input mode: squared output norms per (token, expert)
     // large buffers: the bf16 pipeline (sorted rows, H, fp32 accumulator) and the SIMT path's
@@ -180,6 +176,7 @@ struct ThreadDeviceState {
     cudaEvent_t fork = nullptr, join = nullptr, mid = nullptr;
     cudaEvent_t start = nullptr, done = nullptr, copied[kMaxHostChunks] = {}, computed[kMaxHostChunks] = {};
     bool side_ok = false, host_ok = false;
+    int* result = nullptr;  // pinned host words that a calibration's last kernels write their counts to
     int sms = 0;
     void release() {
         auto ev = [](cudaEvent_t& e) { if (e) cudaEventDestroy(e); e = nullptr; };
@@ -187,6 +184,8 @@ struct ThreadDeviceState {
         ev(fork); ev(join); ev(mid); ev(start); ev(done);
         for (int c = 0; c < kMaxHostChunks; ++c) { ev(copied[c]); ev(computed[c]); }
         st(side); st(in); st(out);
+        if (result) cudaFreeHost(result);
+        result = nullptr;
         side_ok = host_ok = false;
     }
 };
@@ -248,6 +247,13 @@ ThreadDeviceState* host_helpers() {
         h->host_ok = ok;
     }
     return h && h->host_ok ? h : nullptr;
+}
+// One pinned word per calibration job: read after the stream has drained, without a copy
+int* result_words() {
+    ThreadDeviceState* h = thread_state();
+    if (h && !h->result && cudaHostAlloc(reinterpret_cast<void**>(&h->result), EXFOLD_MAX_CALIB_JOBS * sizeof(int), cudaHostAllocDefault) != cudaSuccess)
+        h->result = nullptr;
+    return h ? h->result : nullptr;
 }
 // Once the side stream has been forked off the caller's stream it is joined again on every way out of the call
 // (also the error returns): later work on the caller's stream, or the end of a stream capture, must not overtake it.
@@ -807,11 +813,11 @@ int exfold_static_pool_build(const exfold_layer* layer, const exfold_tables* tab
     return EXFOLD_OK;
 }
 
-// Enqueues one calibration on the stream (no synchronisation); the number of unobserved experts lands in
-// warn_slot (device memory) when the stream gets there.
+// Enqueues one calibration on the stream (no synchronisation); the number of unobserved experts lands in *unobserved
+// (pinned host memory) when the stream gets there.
 static int calibrate_enqueue(const exfold_layer* layer, const void* x_cal, const float* logits_cal, int64_t m,
                              const void* w_gate, const void* w_up, const void* w_down, const exfold_calib_opts* opts,
-                             exfold_tables* out, void* ws, size_t ws_bytes, void* cuda_stream, int job) {
+                             exfold_tables* out, void* ws, size_t ws_bytes, void* cuda_stream, int* unobserved) {
     if (!valid_layer(layer) || !x_cal || !w_gate || !w_up || !w_down || !opts || !out || !ws)
         return EXFOLD_ERR_INVALID_ARG;
     if (!out->S || !out->L || !out->h || !out->lnh) return EXFOLD_ERR_INVALID_ARG;
@@ -828,28 +834,31 @@ static int calibrate_enqueue(const exfold_layer* layer, const void* x_cal, const
     if (ws_bytes < pl.total) return EXFOLD_ERR_WORKSPACE_TOO_SMALL;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(cuda_stream);
 
-    EXFOLD_CUDA(cudaMemsetAsync(at<char>(ws, pl.status), 0, sizeof(DeviceStatus), s));
+    const bool tensor_path = l.dtype == EXFOLD_BF16;
+    const bool pairs = tensor_path && use_pairs(m * Ke, N, d, I);
+    PdlScope pdl_scope(!pairs);  // as in prefill: a chain of kernels of which most are short
+    DeviceStatus* status = at<DeviceStatus>(ws, pl.status);
     int32_t* ids = at<int32_t>(ws, pl.ids);
     if (opts->mode == 0) {
-        // Top-K in router order: the prefill route kernel with K' = K and a zero ln(h) table
-        EXFOLD_CUDA(cudaMemsetAsync(at<char>(ws, pl.zeros), 0, (size_t)N * 4, s));
+        // Top-K in router order: the prefill route kernel with K' = K and no ln(h) term
         PrefillRouteParams rp{};
-        rp.logits = logits_cal; rp.S = out->S; rp.L = out->L; rp.lnh = at<float>(ws, pl.zeros);
+        rp.logits = logits_cal; rp.S = out->S; rp.L = out->L; rp.lnh = nullptr;
         rp.T = m; rp.N = N; rp.K = K; rp.Kp = K; rp.ids = ids; rp.w = at<float>(ws, pl.w);
         rp.loss_thr = INFINITY;
         rp.omit_src = nullptr; rp.omit_tgt = nullptr; rp.block_hist = at<int32_t>(ws, pl.block_hist);
         rp.sb_hist = at<int32_t>(ws, pl.sb_hist);
-        rp.status = nullptr;
+        rp.status = status;
         EXFOLD_CUDA(launch_prefill_route(rp, s));
     } else {
+        EXFOLD_CUDA(cudaMemsetAsync(status, 0, sizeof(DeviceStatus), s));
         EXFOLD_CUDA(launch_iota_ids(ids, m, N, s));
     }
-    const bool tensor_path = l.dtype == EXFOLD_BF16;
     if (tensor_path && (!aligned16(x_cal) || !aligned16(w_gate) || !aligned16(w_up) || !aligned16(w_down)))
         return EXFOLD_ERR_INVALID_ARG;
     const int64_t Rc = m * Ke;
     if (tensor_path && Rc > (int64_t)1 << 30) return EXFOLD_ERR_UNSUPPORTED;
     CalibStatsParams cs{};
+    const size_t NN = (size_t)N * N, calib_bytes = NN * (3 * 8 + 4) + (size_t)N * (8 + 4);
     // Expert outputs, one fp32 row per (token, expert), sorted by expert. Mode 0 sorts the routed rows like prefill; in
     // mode 1 every expert's rows are the tokens themselves, read from x_cal without a copy.
     int32_t* offsets = at<int32_t>(ws, pl.offsets);
@@ -867,9 +876,11 @@ static int calibrate_enqueue(const exfold_layer* layer, const void* x_cal, const
         cp.perm = at<int32_t>(ws, pl.perm); cp.row_tok = row_tok;
         cp.row_w = at<float>(ws, pl.row_w); cp.row_exp = at<int32_t>(ws, pl.row_exp);
         cp.inv_pos = at<int32_t>(ws, pl.inv_pos);
+        cp.zero = at<int32_t>(ws, pl.calib); cp.zero_words = (int)(calib_bytes / 4);  // the pair sums
         EXFOLD_CUDA(launch_prefill_scatter(cp, s));
         cs.inv_pos = cp.inv_pos;
     } else {
+        EXFOLD_CUDA(cudaMemsetAsync(at<char>(ws, pl.calib), 0, calib_bytes, s));
         EXFOLD_CUDA(launch_calib_common_rows(offsets, work_start, m, N, tile_rows, s));
         cs.inv_pos = nullptr; cs.tok_stride = 1; cs.slot_stride = m;
     }
@@ -893,7 +904,7 @@ static int calibrate_enqueue(const exfold_layer* layer, const void* x_cal, const
         GroupedGemmParams g2 = g;
         g2.tm_a = tm_h; g2.tm_b0 = tm_wd; g2.tm_b1 = tm_wd_half; g2.n_ntiles = (d + 255) / 256;
         g2.o32 = at<float>(ws, pl.xs);  // spans the xs and obuf regions (GEMM-1 is done with xs)
-        const int rc = enqueue_expert_gemms(g, g2, Rc, use_pairs(Rc, N, d, I), 0, s);
+        const int rc = enqueue_expert_gemms(g, g2, Rc, pairs, 0, s);
         if (rc != EXFOLD_OK) return rc;
         cs.out = g2.o32;
     } else {
@@ -906,36 +917,26 @@ static int calibrate_enqueue(const exfold_layer* layer, const void* x_cal, const
     }
 
     char* cb = at<char>(ws, pl.calib);
-    const size_t NN = (size_t)N * N;
-    EXFOLD_CUDA(cudaMemsetAsync(cb, 0, NN * (3 * 8 + 4) + (size_t)N * (8 + 4) + 256, s));
     cs.ids = ids; cs.m = m; cs.Ke = Ke; cs.d = d; cs.N = N;
     cs.A = reinterpret_cast<double*>(cb); cs.Bv = cs.A + NN; cs.C = cs.Bv + NN;
     cs.H = cs.C + NN;
     cs.cnt = reinterpret_cast<int32_t*>(cs.H + N);
     cs.hc = cs.cnt + NN;
-    int32_t* unobs = cs.hc + N;
     if (opts->mode == 1 && Ke >= 32)  // many experts per token: Gram-product form of the same sums
         EXFOLD_CUDA(launch_calib_stats_common(cs, at<double>(ws, pl.calib_nrm), sm_count(), s));
     else
         EXFOLD_CUDA(launch_calib_stats(cs, s));
-    EXFOLD_CUDA(launch_calib_finalize(cs, *opts, out->S, out->L, out->h, out->lnh, out->n_obs, unobs, s));
-    EXFOLD_CUDA(cudaMemcpyAsync(at<int32_t>(ws, pl.calib_warn) + job, unobs, 4, cudaMemcpyDeviceToDevice, s));
+    EXFOLD_CUDA(launch_calib_finalize(cs, *opts, out->S, out->L, out->h, out->lnh, out->n_obs, unobserved, s));
     return EXFOLD_OK;
 }
 
 // The jobs' unobserved-expert counts, after the stream has drained
-static int calibrate_collect(const exfold_layer* layer, int64_t m_max, int Ke, int n_jobs, int32_t* warn, void* ws,
-                             cudaStream_t s) {
-    exfold_layer lc = *layer;
-    lc.n_shared = 0;
-    const Plan pl = make_plan(lc, m_max, Ke);
-    int32_t un[EXFOLD_MAX_CALIB_JOBS];
-    EXFOLD_CUDA(cudaMemcpyAsync(un, at<int32_t>(ws, pl.calib_warn), (size_t)n_jobs * 4, cudaMemcpyDeviceToHost, s));
+static int calibrate_collect(const int* counts, int n_jobs, int32_t* warn, cudaStream_t s) {
     EXFOLD_CUDA(cudaStreamSynchronize(s));
     int any = 0;
     for (int j = 0; j < n_jobs; ++j) {
-        if (warn) warn[j] = un[j];
-        any |= un[j] > 0;
+        if (warn) warn[j] = counts[j];
+        any |= counts[j] > 0;
     }
     return any ? EXFOLD_WARN_UNOBSERVED_EXPERT : EXFOLD_OK;
 }
@@ -943,10 +944,11 @@ static int calibrate_collect(const exfold_layer* layer, int64_t m_max, int Ke, i
 int exfold_calibrate(const exfold_layer* layer, const void* x_cal, const float* logits_cal, int64_t m,
                      const void* w_gate, const void* w_up, const void* w_down, const exfold_calib_opts* opts,
                      exfold_tables* out, void* ws, size_t ws_bytes, void* cuda_stream) {
-    int rc = calibrate_enqueue(layer, x_cal, logits_cal, m, w_gate, w_up, w_down, opts, out, ws, ws_bytes, cuda_stream, 0);
+    int* counts = result_words();
+    if (!counts) return EXFOLD_ERR_CUDA;
+    int rc = calibrate_enqueue(layer, x_cal, logits_cal, m, w_gate, w_up, w_down, opts, out, ws, ws_bytes, cuda_stream, counts);
     if (rc != EXFOLD_OK) return rc;
-    return calibrate_collect(layer, m, opts->mode == 1 ? layer->n_experts : layer->top_k, 1, nullptr, ws,
-                             reinterpret_cast<cudaStream_t>(cuda_stream));
+    return calibrate_collect(counts, 1, nullptr, reinterpret_cast<cudaStream_t>(cuda_stream));
 }
 
 int exfold_calibrate_layers(const exfold_layer* layer, const exfold_calib_job* jobs, int32_t n_jobs,
@@ -959,17 +961,18 @@ int exfold_calibrate_layers(const exfold_layer* layer, const exfold_calib_job* j
         if (!jobs[j].out || jobs[j].m < 1) return EXFOLD_ERR_INVALID_ARG;
         m_max = std::max<int64_t>(m_max, jobs[j].m);
     }
-    // Every job uses the plan of the largest one, so that the jobs' warning slots sit at one place; the jobs run
-    // one after the other on the stream and share the rest of the workspace.
+    // The jobs run one after the other on the stream and share the workspace, sized for the largest one.
     const int Ke = opts->mode == 1 ? layer->n_experts : layer->top_k;
     if (ws_bytes < exfold_workspace_bytes(layer, m_max, Ke)) return EXFOLD_ERR_WORKSPACE_TOO_SMALL;
+    int* counts = result_words();
+    if (!counts) return EXFOLD_ERR_CUDA;
     for (int j = 0; j < n_jobs; ++j) {
         const exfold_calib_job& b = jobs[j];
         int rc = calibrate_enqueue(layer, b.x_cal, b.logits_cal, b.m, b.w_gate, b.w_up, b.w_down, opts, b.out, ws,
-                                   ws_bytes, cuda_stream, j);
+                                   ws_bytes, cuda_stream, counts + j);
         if (rc != EXFOLD_OK) return rc;
     }
-    return calibrate_collect(layer, m_max, Ke, n_jobs, unobserved, ws, reinterpret_cast<cudaStream_t>(cuda_stream));
+    return calibrate_collect(counts, n_jobs, unobserved, reinterpret_cast<cudaStream_t>(cuda_stream));
 }
 
 // Router scores on the stream; `clear_status`: the call stands alone (clears the status record itself)

@@ -79,6 +79,8 @@ __global__ void __launch_bounds__(kStatsThreads) calib_stats_kernel(CalibStatsPa
     constexpr int NV = KE * (KE + 1) / 2;
     __shared__ double s_gram[kStatsThreads / 32][NV];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    grid_dep_launch();
+    grid_dep_wait();
     const int64_t i = (int64_t)blockIdx.x * (kStatsThreads / 32) + warp;
     if (i >= p.m) return;
     const int d = p.d;
@@ -139,6 +141,8 @@ __global__ void __launch_bounds__(kStatsThreads) calib_stats_tiled_kernel(CalibS
     constexpr int NV = 24;  // 16 products, 4 + 4 norms
     __shared__ double s_sum[kStatsThreads / 32][NV];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    grid_dep_launch();
+    grid_dep_wait();
     const int64_t w = (int64_t)blockIdx.x * (kStatsThreads / 32) + warp;
     const int tiles = nb * (nb + 1) / 2;
     const int64_t i = w / tiles;
@@ -211,6 +215,8 @@ __global__ void calib_finalize_kernel(CalibStatsParams p, exfold_calib_opts o, f
                                       float* lnh, int32_t* n_obs, int32_t* unobserved) {
     const int N = p.N;
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+    grid_dep_launch();
+    grid_dep_wait();
     if (idx < N * N) {
         const int s = idx / N, t = idx % N;
         float sv, lv;
@@ -400,30 +406,25 @@ cudaError_t launch_calib_stats(const CalibStatsParams& p, cudaStream_t s) {
     if (p.Ke > kStatsRows) {
         const int nb = (p.Ke + 3) / 4;
         const int64_t warps = p.m * (nb * (nb + 1) / 2);
-        calib_stats_tiled_kernel<<<(unsigned)((warps + kWarps - 1) / kWarps), kStatsThreads, 0, s>>>(p, nb);
-    } else {
-        const unsigned grid = (unsigned)((p.m + kWarps - 1) / kWarps);
-        switch (p.Ke) {
-            case 1: calib_stats_kernel<1><<<grid, kStatsThreads, 0, s>>>(p); break;
-            case 2: calib_stats_kernel<2><<<grid, kStatsThreads, 0, s>>>(p); break;
-            case 3: calib_stats_kernel<3><<<grid, kStatsThreads, 0, s>>>(p); break;
-            case 4: calib_stats_kernel<4><<<grid, kStatsThreads, 0, s>>>(p); break;
-            case 5: calib_stats_kernel<5><<<grid, kStatsThreads, 0, s>>>(p); break;
-            case 6: calib_stats_kernel<6><<<grid, kStatsThreads, 0, s>>>(p); break;
-            case 7: calib_stats_kernel<7><<<grid, kStatsThreads, 0, s>>>(p); break;
-            default: calib_stats_kernel<8><<<grid, kStatsThreads, 0, s>>>(p); break;
-        }
+        return launch_pdl(calib_stats_tiled_kernel, (unsigned)((warps + kWarps - 1) / kWarps), kStatsThreads, 0, s, p, nb);
     }
-    count_launch();
-    return cudaGetLastError();
+    const unsigned grid = (unsigned)((p.m + kWarps - 1) / kWarps);
+    switch (p.Ke) {
+        case 1: return launch_pdl(calib_stats_kernel<1>, grid, kStatsThreads, 0, s, p);
+        case 2: return launch_pdl(calib_stats_kernel<2>, grid, kStatsThreads, 0, s, p);
+        case 3: return launch_pdl(calib_stats_kernel<3>, grid, kStatsThreads, 0, s, p);
+        case 4: return launch_pdl(calib_stats_kernel<4>, grid, kStatsThreads, 0, s, p);
+        case 5: return launch_pdl(calib_stats_kernel<5>, grid, kStatsThreads, 0, s, p);
+        case 6: return launch_pdl(calib_stats_kernel<6>, grid, kStatsThreads, 0, s, p);
+        case 7: return launch_pdl(calib_stats_kernel<7>, grid, kStatsThreads, 0, s, p);
+        default: return launch_pdl(calib_stats_kernel<8>, grid, kStatsThreads, 0, s, p);
+    }
 }
 
 cudaError_t launch_calib_finalize(const CalibStatsParams& p, const exfold_calib_opts& o, float* S, float* L,
                                   float* h, float* lnh, int32_t* n_obs, int32_t* unobserved, cudaStream_t s) {
     const int n = p.N * p.N;
-    calib_finalize_kernel<<<(n + 255) / 256, 256, 0, s>>>(p, o, S, L, h, lnh, n_obs, unobserved);
-    count_launch();
-    return cudaGetLastError();
+    return launch_pdl(calib_finalize_kernel, (n + 255) / 256, 256, 0, s, p, o, S, L, h, lnh, n_obs, unobserved);
 }
 
 cudaError_t launch_iota_ids(int32_t* ids, int64_t m, int N, cudaStream_t s) {

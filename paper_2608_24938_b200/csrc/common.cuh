@@ -177,7 +177,7 @@ struct PrefillRouteParams {
     const float* logits;  // [T][N]
     const float* S;       // [N][N]
     const float* L;       // [N][N]
-    const float* lnh;     // [N]
+    const float* lnh;     // [N], or null: ranked by the scores alone
     int64_t T;
     int N, K, Kp;
     float loss_thr;     // pairs with loss above it are not admissible targets (+inf: off)
@@ -217,6 +217,8 @@ struct PrefillScatterParams {
     float* row_w;       // [R + T*n_shared]
     int32_t* row_exp;   // [R + T*n_shared]
     int32_t* inv_pos;   // [R] sorted row of each route (inverse of perm); may be null
+    int32_t* zero;      // words to clear on the way (calibration: the pair sums); may be null
+    int zero_words;
 };
 
 cudaError_t launch_prefill_route(PrefillRouteParams p, cudaStream_t s);

@@ -95,7 +95,7 @@ __global__ void __launch_bounds__(kRouteMaxThreads) prefill_route_kernel(Prefill
         for (int off = 16; off > 0; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
         const float w = ex / sum;
         // ---- Eq. 10 on log scale: key = logit + ln h (one fp32 add); rank by (key desc, id asc)
-        const float key = has ? __fadd_rn(my_r, p.lnh[my_id]) : -INFINITY;
+        const float key = has ? __fadd_rn(my_r, p.lnh != nullptr ? p.lnh[my_id] : 0.f) : -INFINITY;
         int rank = 0;
         for (int j = 0; j < K; ++j) {
             float kj = __shfl_sync(0xffffffffu, key, j);
@@ -220,6 +220,7 @@ __global__ void __launch_bounds__(kRouteThreads) prefill_scatter_kernel(PrefillS
     __syncthreads();
     grid_dep_launch();
     grid_dep_wait();
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < p.zero_words; i += gridDim.x * blockDim.x) p.zero[i] = 0;
     // Bases of this block: first sorted position of expert e = (rows of experts < e) + (rows of e in
     // earlier blocks). Super-block rows first (nsb of them), then the block rows before this one inside
     // its super-block: nsb + 63 rows of N counters at most, whatever the token count. With a single
