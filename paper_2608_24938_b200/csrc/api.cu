@@ -813,11 +813,11 @@ int exfold_static_pool_build(const exfold_layer* layer, const exfold_tables* tab
     return EXFOLD_OK;
 }
 
-// Enqueues one calibration on the stream (no synchronisation); the number of unobserved experts lands in *unobserved
-// (pinned host memory) when the stream gets there.
+// Enqueues one calibration on the stream (no synchronisation); the number of unobserved experts lands in result_words()[job]
+// when the stream gets there.
 static int calibrate_enqueue(const exfold_layer* layer, const void* x_cal, const float* logits_cal, int64_t m,
                              const void* w_gate, const void* w_up, const void* w_down, const exfold_calib_opts* opts,
-                             exfold_tables* out, void* ws, size_t ws_bytes, void* cuda_stream, int* unobserved) {
+                             exfold_tables* out, void* ws, size_t ws_bytes, void* cuda_stream, int job) {
     if (!valid_layer(layer) || !x_cal || !w_gate || !w_up || !w_down || !opts || !out || !ws)
         return EXFOLD_ERR_INVALID_ARG;
     if (!out->S || !out->L || !out->h || !out->lnh) return EXFOLD_ERR_INVALID_ARG;
@@ -834,6 +834,8 @@ static int calibrate_enqueue(const exfold_layer* layer, const void* x_cal, const
     if (ws_bytes < pl.total) return EXFOLD_ERR_WORKSPACE_TOO_SMALL;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(cuda_stream);
 
+    int* counts = result_words();
+    if (!counts) return EXFOLD_ERR_CUDA;
     const bool tensor_path = l.dtype == EXFOLD_BF16;
     const bool pairs = tensor_path && use_pairs(m * Ke, N, d, I);
     PdlScope pdl_scope(!pairs);  // as in prefill: a chain of kernels of which most are short
@@ -926,12 +928,13 @@ static int calibrate_enqueue(const exfold_layer* layer, const void* x_cal, const
         EXFOLD_CUDA(launch_calib_stats_common(cs, at<double>(ws, pl.calib_nrm), sm_count(), s));
     else
         EXFOLD_CUDA(launch_calib_stats(cs, s));
-    EXFOLD_CUDA(launch_calib_finalize(cs, *opts, out->S, out->L, out->h, out->lnh, out->n_obs, unobserved, s));
+    EXFOLD_CUDA(launch_calib_finalize(cs, *opts, out->S, out->L, out->h, out->lnh, out->n_obs, counts + job, s));
     return EXFOLD_OK;
 }
 
 // The jobs' unobserved-expert counts, after the stream has drained
-static int calibrate_collect(const int* counts, int n_jobs, int32_t* warn, cudaStream_t s) {
+static int calibrate_collect(int n_jobs, int32_t* warn, cudaStream_t s) {
+    const int* counts = result_words();
     EXFOLD_CUDA(cudaStreamSynchronize(s));
     int any = 0;
     for (int j = 0; j < n_jobs; ++j) {
@@ -944,11 +947,9 @@ static int calibrate_collect(const int* counts, int n_jobs, int32_t* warn, cudaS
 int exfold_calibrate(const exfold_layer* layer, const void* x_cal, const float* logits_cal, int64_t m,
                      const void* w_gate, const void* w_up, const void* w_down, const exfold_calib_opts* opts,
                      exfold_tables* out, void* ws, size_t ws_bytes, void* cuda_stream) {
-    int* counts = result_words();
-    if (!counts) return EXFOLD_ERR_CUDA;
-    int rc = calibrate_enqueue(layer, x_cal, logits_cal, m, w_gate, w_up, w_down, opts, out, ws, ws_bytes, cuda_stream, counts);
+    int rc = calibrate_enqueue(layer, x_cal, logits_cal, m, w_gate, w_up, w_down, opts, out, ws, ws_bytes, cuda_stream, 0);
     if (rc != EXFOLD_OK) return rc;
-    return calibrate_collect(counts, 1, nullptr, reinterpret_cast<cudaStream_t>(cuda_stream));
+    return calibrate_collect(1, nullptr, reinterpret_cast<cudaStream_t>(cuda_stream));
 }
 
 int exfold_calibrate_layers(const exfold_layer* layer, const exfold_calib_job* jobs, int32_t n_jobs,
@@ -964,15 +965,13 @@ int exfold_calibrate_layers(const exfold_layer* layer, const exfold_calib_job* j
     // The jobs run one after the other on the stream and share the workspace, sized for the largest one.
     const int Ke = opts->mode == 1 ? layer->n_experts : layer->top_k;
     if (ws_bytes < exfold_workspace_bytes(layer, m_max, Ke)) return EXFOLD_ERR_WORKSPACE_TOO_SMALL;
-    int* counts = result_words();
-    if (!counts) return EXFOLD_ERR_CUDA;
     for (int j = 0; j < n_jobs; ++j) {
         const exfold_calib_job& b = jobs[j];
         int rc = calibrate_enqueue(layer, b.x_cal, b.logits_cal, b.m, b.w_gate, b.w_up, b.w_down, opts, b.out, ws,
-                                   ws_bytes, cuda_stream, counts + j);
+                                   ws_bytes, cuda_stream, j);
         if (rc != EXFOLD_OK) return rc;
     }
-    return calibrate_collect(counts, n_jobs, unobserved, reinterpret_cast<cudaStream_t>(cuda_stream));
+    return calibrate_collect(n_jobs, unobserved, reinterpret_cast<cudaStream_t>(cuda_stream));
 }
 
 // Router scores on the stream; `clear_status`: the call stands alone (clears the status record itself)
