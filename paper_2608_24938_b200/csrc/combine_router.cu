@@ -1,5 +1,7 @@
 // CUDA-core kernels around the expert GEMMs of bf16 layers: the per-token sum of the experts' rows (Eq. 3 / Eq. 4) and
 // the router scores of fp32 layers and small bf16 batches.
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace exfold {
@@ -9,10 +11,8 @@ namespace {
 // Eq. 4's weighted sum for the tensor-core path: GEMM-2 stored w~ * E(x) per route in bf16, sorted by
 // expert; a token's routes are found through the inverse permutation and summed in fp32, slot order
 // (a decode step with a K split: the `parts` planes of a row, in order, inside that).
-// BATCHED: the row indices first, then up to eight row loads in flight together - for the few blocks of a decode
-// step, where the chain index -> row -> next index is all there is (10 -> 3 us for 64 tokens); with thousands of
-// tokens the plain loop is faster (more blocks per SM hide the chain; measured 50 vs 65 us on 8192 tokens).
-template <bool BATCHED>
+// The row indices first, then up to eight row loads in flight together (the chain index -> row -> next index is all
+// there is to a decode step's few blocks: 10 -> 3 us for 64 tokens).
 __global__ void __launch_bounds__(256) combine_rows_kernel(const __nv_bfloat16* __restrict__ O,
                                                            const int32_t* __restrict__ inv_pos, int64_t Tn, int Kr, int d,
                                                            int n_shared, const int32_t* __restrict__ shared0_dev,
@@ -33,29 +33,58 @@ __global__ void __launch_bounds__(256) combine_rows_kernel(const __nv_bfloat16* 
                 acc[2 * q + 1] += f.y;
             }
         };
-        if (BATCHED) {
-            for (int j0 = 0; j0 < n_src; j0 += 8) {
-                int64_t row[8];
+        for (int j0 = 0; j0 < n_src; j0 += 8) {
+            int64_t row[8];
 #pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    const int j = j0 + u;
-                    row[u] = j < Kr ? (int64_t)inv_pos[i * Kr + j] : (j < n_src ? shared0 + i : -1);
-                }
-                for (int part = 0; part < parts; ++part) {
-                    uint4 v[8];
-#pragma unroll
-                    for (int u = 0; u < 8; ++u)
-                        if (row[u] >= 0) v[u] = *reinterpret_cast<const uint4*>(O + (part * part_rows + row[u]) * d + c);
-#pragma unroll
-                    for (int u = 0; u < 8; ++u)  // slot order; a row < 0 is a slot merged into an earlier one
-                        if (row[u] >= 0) add(v[u]);
-                }
+            for (int u = 0; u < 8; ++u) {
+                const int j = j0 + u;
+                row[u] = j < Kr ? (int64_t)inv_pos[i * Kr + j] : (j < n_src ? shared0 + i : -1);
             }
-        } else {  // prefill: every slot has a row of its own and there is one plane
-            for (int j = 0; j <= Kr; ++j) {
-                if (j == Kr && !n_shared) break;
-                const int64_t row = j < Kr ? (int64_t)inv_pos[i * Kr + j] : shared0 + i;
-                add(*reinterpret_cast<const uint4*>(O + row * d + c));
+            for (int part = 0; part < parts; ++part) {
+                uint4 v[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u)
+                    if (row[u] >= 0) v[u] = *reinterpret_cast<const uint4*>(O + (part * part_rows + row[u]) * d + c);
+#pragma unroll
+                for (int u = 0; u < 8; ++u)  // slot order; a row < 0 is a slot merged into an earlier one
+                    if (row[u] >= 0) add(v[u]);
+            }
+        }
+        uint4 o;
+        __nv_bfloat162* o2 = reinterpret_cast<__nv_bfloat162*>(&o);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) o2[u] = __floats2bfloat162_rn(acc[2 * u], acc[2 * u + 1]);
+        *reinterpret_cast<uint4*>(y + i * d + c) = o;
+    }
+}
+
+// The same for prefill, where every slot has a row of its own, with NS rows per token known at compile time: a thread owns
+// eight columns and has all NS row loads in flight, and no registers for what decode needs (8192 tokens x 4 rows x 2048:
+// 35 us with one load at a time and many blocks per SM, 65 with the kernel above, 24 now = 7 TB/s). Rows are read once: not
+// kept in L1.
+template <int NS>
+__global__ void __launch_bounds__(512) combine_rows_exact_kernel(const __nv_bfloat16* __restrict__ O,
+                                                                 const int32_t* __restrict__ inv_pos, int64_t Tn, int Kr, int d,
+                                                                 __nv_bfloat16* __restrict__ y) {
+    const int64_t i = blockIdx.x;
+    grid_dep_launch();
+    grid_dep_wait();
+    int64_t row[NS];
+#pragma unroll
+    for (int j = 0; j < NS; ++j) row[j] = j < Kr ? (int64_t)inv_pos[i * Kr + j] : Tn * Kr + i;
+    for (int c = threadIdx.x * 8; c < d; c += blockDim.x * 8) {
+        uint4 v[NS];
+#pragma unroll
+        for (int j = 0; j < NS; ++j) v[j] = __ldcs(reinterpret_cast<const uint4*>(O + row[j] * d + c));
+        float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int j = 0; j < NS; ++j) {
+            const __nv_bfloat162* h2 = reinterpret_cast<const __nv_bfloat162*>(&v[j]);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const float2 f = __bfloat1622float2(h2[q]);
+                acc[2 * q] += f.x;
+                acc[2 * q + 1] += f.y;
             }
         }
         uint4 o;
@@ -165,11 +194,17 @@ cudaError_t launch_combine_rows(const __nv_bfloat16* O, const int32_t* inv_pos, 
                                 int n_shared, const int32_t* shared0_dev, int parts, int64_t part_rows,
                                 __nv_bfloat16* y, cudaStream_t s) {
     if (T == 0) return cudaSuccess;
-    if (T <= 1024 || parts > 1 || shared0_dev != nullptr)  // decode (merged slots are marked -1, K planes)
-        return launch_pdl(combine_rows_kernel<true>, (unsigned)T, 256, 0, s, O, inv_pos, T, Kr, d, n_shared, shared0_dev,
-                          parts, part_rows, y);
-    return launch_pdl(combine_rows_kernel<false>, (unsigned)T, 256, 0, s, O, inv_pos, T, Kr, d, n_shared, shared0_dev, parts,
-                      part_rows, y);
+    if (parts == 1 && shared0_dev == nullptr) {
+        const int threads = std::min(512, (d / 8 + 31) / 32 * 32);
+        switch (Kr + (n_shared ? 1 : 0)) {
+#define EXFOLD_COMBINE(NS) \
+    case NS: return launch_pdl(combine_rows_exact_kernel<NS>, (unsigned)T, threads, 0, s, O, inv_pos, T, Kr, d, y);
+            EXFOLD_COMBINE(2) EXFOLD_COMBINE(3) EXFOLD_COMBINE(4) EXFOLD_COMBINE(5) EXFOLD_COMBINE(6) EXFOLD_COMBINE(7)
+            EXFOLD_COMBINE(8) EXFOLD_COMBINE(9)
+#undef EXFOLD_COMBINE
+        }
+    }
+    return launch_pdl(combine_rows_kernel, (unsigned)T, 256, 0, s, O, inv_pos, T, Kr, d, n_shared, shared0_dev, parts, part_rows, y);
 }
 
 }  // namespace exfold

@@ -175,3 +175,15 @@ def test_router_scores_by_prompt_length(T, N, d):
     want = x.double() @ wr.double().T
     bound = d * 2.0 ** -23 * (x.double().abs() @ wr.double().abs().T)
     assert bool(((lg.double() - want).abs() <= bound).all())
+
+
+@pytest.mark.parametrize("Kp,ns,d", [(1, 1, 64), (2, 0, 192), (3, 1, 4160), (5, 0, 256), (7, 0, 320), (8, 0, 128), (8, 1, 128),
+                                     (9, 0, 64), (10, 1, 128)])
+def test_rows_summed_per_token(Kp, ns, d):
+    """The per-token sum by number of rows (2 to 9 known at compile time, more in batches of eight) and widths that leave
+    part of a block idle or take two passes."""
+    cfg = si.LayerConfig("sum", 16, ns, d, 64, 10, "bf16", 70, (Kp,), 4, (2,))
+    case = Case(cfg)
+    got, ref = case.run_prefill(Kp), case.oracle_prefill(Kp)
+    check_prefill_meta(got, ref)
+    check_output(got["y"], ref["y"], "bf16")
