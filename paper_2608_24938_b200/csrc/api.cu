@@ -500,6 +500,8 @@ int exfold_moe_prefill_ex(const exfold_layer* layer, const void* x, const float*
     if (k_pre < 1 || k_pre > l.top_k) return EXFOLD_ERR_INVALID_ARG;
     const int N = l.n_experts, K = l.top_k, Kp = k_pre, d = l.hidden, I = l.inter, G = N + l.n_shared;
     const int64_t R = T * Kp, Rtot = R + T * l.n_shared;
+    // A few tokens: the two kernels of a small decode batch on the routes (whatever gemm_path says: same results for all)
+    const bool small = l.dtype == EXFOLD_BF16 && T <= kSmallDecodeBatch && decode_small_fits((int)T, Kp, d, w_gate, w_up, w_down);
     if (Rtot > (int64_t)1 << 30) return EXFOLD_ERR_UNSUPPORTED;
     const Plan pl = make_plan(l, T, Kp);
     if (ws_bytes < pl.total) return EXFOLD_ERR_WORKSPACE_TOO_SMALL;
@@ -509,9 +511,9 @@ int exfold_moe_prefill_ex(const exfold_layer* layer, const void* x, const float*
 
     CUtensorMap tm_xs, tm_x, tm_wg, tm_wu, tm_h, tm_wd, tm_wd_half;
     const int mode = opts == nullptr || opts->gemm_path < 0 || opts->gemm_path > 2 ? 0 : opts->gemm_path;
-    const bool pairs = bf16 && (mode == 2 ? kGemmBK == 64 && Rtot >= 2 * kTileM : mode == 0 && use_pairs(Rtot, G, d, I));
+    const bool pairs = bf16 && !small && (mode == 2 ? kGemmBK == 64 && Rtot >= 2 * kTileM : mode == 0 && use_pairs(Rtot, G, d, I));
     const int sms = sm_count() & ~1;
-    if (bf16) {
+    if (bf16 && !small) {
         const uint64_t E = (uint64_t)G;
         bool ok = make_tmap(&tm_xs, at<char>(ws, pl.xs), (uint64_t)R, d, 128) && make_tmap(&tm_x, x, (uint64_t)T, d, 128) &&
                   make_tmap(&tm_wg, w_gate, E * I, d, 128) && make_tmap(&tm_wu, w_up, E * I, d, 128) &&
@@ -575,9 +577,21 @@ int exfold_moe_prefill_ex(const exfold_layer* layer, const void* x, const float*
     cp.perm = at<int32_t>(ws, pl.perm); cp.row_tok = at<int32_t>(ws, pl.row_tok);
     cp.row_w = at<float>(ws, pl.row_w); cp.row_exp = at<int32_t>(ws, pl.row_exp);
     cp.inv_pos = at<int32_t>(ws, pl.inv_pos);
-    { ProfScope ps(2, s); EXFOLD_CUDA(launch_prefill_scatter(cp, s)); }
+    if (small) cp.xs = nullptr;  // the tokens are read in place; only the metadata needs the permutation
+    if (!small || meta) { ProfScope ps(2, s); EXFOLD_CUDA(launch_prefill_scatter(cp, s)); }
 
-    if (bf16) {
+    if (small) {
+        DecodeSmallParams sp{};
+        sp.x = reinterpret_cast<const __nv_bfloat16*>(x); sp.wg = reinterpret_cast<const __nv_bfloat16*>(w_gate);
+        sp.wu = reinterpret_cast<const __nv_bfloat16*>(w_up); sp.wd = reinterpret_cast<const __nv_bfloat16*>(w_down);
+        sp.y = reinterpret_cast<__nv_bfloat16*>(y); sp.ids = rp.ids; sp.w_in = rp.w;
+        sp.B = (int)T; sp.N = N; sp.K = Kp; sp.M = N; sp.n_shared = l.n_shared; sp.d = d; sp.I = I;
+        sp.max_groups = (int)std::min<int64_t>(N, R) + l.n_shared; sp.max_rows = (int)Rtot;
+        sp.H = at<__nv_bfloat16>(ws, pl.H); sp.row_tok = cp.row_tok; sp.row_w = cp.row_w; sp.row_grp = cp.row_exp;
+        sp.grp_expert = at<int32_t>(ws, pl.grp_expert); sp.n_groups = at<int32_t>(ws, pl.n_groups);
+        ProfScope ps(3, s);
+        EXFOLD_CUDA(launch_decode_small(sp, sm_count(), s));
+    } else if (bf16) {
         GroupedGemmParams g{};
         g.tm_a = tm_xs; g.tm_a2 = tm_x; g.tm_b0 = tm_wg; g.tm_b1 = tm_wu; g.x_rows = (int)T; g.o32 = nullptr;
         g.offsets = cp.offsets; g.work_start = cp.work_start; g.G = G; g.n_routed = N; g.R = (int)R;

@@ -313,7 +313,8 @@ struct DecodeFfnParams {
 };
 cudaError_t launch_decode_ffn(const DecodeFfnParams& p, int sms, cudaStream_t s);
 size_t decode_ffn_smem_plan(int B, int K, int N, int* stages, int* scratch_off, int* a_rows);
-// Decode of at most kSmallDecodeBatch tokens, bf16 layers: two kernels (decode_small.cu)
+// Decode of at most kSmallDecodeBatch tokens, bf16 layers: two kernels (decode_small.cu). Prefill calls that short run the
+// same two after their own routing.
 constexpr int kSmallDecodeBatch = 8;
 struct DecodeSmallParams {
     const __nv_bfloat16* x;
@@ -324,6 +325,7 @@ struct DecodeSmallParams {
     const float* logits;  // [B][N], or null: ids and w64 come from the top-k kernel
     const int32_t* ids;
     const double* w64;
+    const float* w_in;    // prefill: the routes' final weights [B][K]; ids are then executed as they are, no pool, no remap
     const float* S;
     const float* L;
     const float* h;

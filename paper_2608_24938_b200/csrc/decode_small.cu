@@ -1,4 +1,5 @@
-// Decode of small batches (bf16 layers, at most 8 tokens): routing, expert pool and expert FFN in two kernels.
+// Decode of small batches (bf16 layers, at most 8 tokens): routing, expert pool and expert FFN in two kernels. Prefill calls
+// of at most 8 tokens run the same two on the routes that the prefill routing kernel left.
 //
 // A small batch reads the weights of a few experts and does next to no arithmetic on them, so its time is the weights'
 // bytes over HBM plus every fixed cost on the way. The four-kernel chain of larger batches (route_decode.cu,
@@ -21,7 +22,8 @@
 //
 // Measured, four-kernel chain -> this (whole call): Qwen3 shape, 1 token 33.2 -> 21.4 us, 8 tokens with a pool of 32 53.8 -> 44.9;
 // Mixtral shape, 1 token 167 -> 124 (5.7 TB/s); GLM shape, 8 tokens with a pool of 32 213 -> 201. With two 8-column operands,
-// 16 tokens took 57 us against the chain's 42 (the per-CTA routing grows with the tokens), so the line is at 8.
+// Prefill of 1 token 38.7 -> 18.8 (Mixtral shape 220 -> 126), of 8 tokens (Top-6, router) 96 -> 82. With two 8-column operands,
+// a decode of 16 tokens took 57 us against the chain's 42 (the per-CTA routing grows with the tokens), so the line is at 8.
 #include <algorithm>
 
 #include "common.cuh"
@@ -118,6 +120,8 @@ __device__ __forceinline__ int compact_threads(bool flag, int* warp_cnt, int* li
     return all;
 }
 
+// GIVEN: the routes and their weights are final (prefill); else Top-K, pool and remap happen here
+template <bool GIVEN>
 __global__ void __launch_bounds__(kThreads, 2) decode_small_gateup_kernel(DecodeSmallParams p) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ float4 s_red[2][kWarps][32];
@@ -129,10 +133,10 @@ __global__ void __launch_bounds__(kThreads, 2) decode_small_gateup_kernel(Decode
     __nv_bfloat16* xs = reinterpret_cast<__nv_bfloat16*>(smem + kStateBytes + align16((size_t)BK * 16));  // [B][d + pad]
     const int xld = d + kXPad;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const bool is_static = p.st_pool != nullptr;
+    const bool is_static = !GIVEN && p.st_pool != nullptr;
     // the CTA with the fewest work items writes the metadata and the lists
-    const bool scribe = blockIdx.x == gridDim.x - 1, meta = p.pool_ids != nullptr && scribe;
-    const float h_e = !is_static && tid < N ? __ldg(p.h + tid) : 0.f;  // the tables do not depend on earlier kernels
+    const bool scribe = blockIdx.x == gridDim.x - 1, meta = !GIVEN && p.pool_ids != nullptr && scribe;
+    const float h_e = !GIVEN && !is_static && tid < N ? __ldg(p.h + tid) : 0.f;  // the tables do not depend on earlier kernels
     sc.acc32[3 * tid] = sc.acc32[3 * tid + 1] = sc.acc32[3 * tid + 2] = 0u;
     sc.in_union[tid] = 0;
     sc.grp_of[tid] = -1;
@@ -142,7 +146,7 @@ __global__ void __launch_bounds__(kThreads, 2) decode_small_gateup_kernel(Decode
 
     // ---- Eq. 2: a warp per token (or the result of the top-k kernel when that computed the scores)
     float v[8];
-    const bool ranks = p.logits != nullptr && warp < B;
+    const bool ranks = !GIVEN && p.logits != nullptr && warp < B;
     if (ranks) {
 #pragma unroll
         for (int q = 0; q < 8; ++q) v[q] = lane + 32 * q < N ? p.logits[(size_t)warp * N + lane + 32 * q] : -INFINITY;
@@ -158,10 +162,11 @@ __global__ void __launch_bounds__(kThreads, 2) decode_small_gateup_kernel(Decode
             w64[warp * K + lane] = w;
         }
     }
-    if (p.logits == nullptr)
+    if (GIVEN || p.logits == nullptr)
         for (int s = tid; s < BK; s += kThreads) {
             ids[s] = p.ids[s];
-            w64[s] = p.w64[s];
+            if (GIVEN) wrm[s] = p.w_in[s];
+            else w64[s] = p.w64[s];
         }
     __syncthreads();
 
@@ -181,18 +186,19 @@ __global__ void __launch_bounds__(kThreads, 2) decode_small_gateup_kernel(Decode
     } else {
         for (int s = tid; s < BK; s += kThreads) {
             const int e = ids[s];
+            sc.in_union[e] = 1;
+            if (GIVEN) continue;
             const unsigned long long fx = (unsigned long long)(w64[s] * 9007199254740992.0);
             atomicAdd(&sc.acc32[3 * e], (unsigned)(fx & 0x1FFFFFull));
             atomicAdd(&sc.acc32[3 * e + 1], (unsigned)((fx >> 21) & 0x1FFFFFull));
             atomicAdd(&sc.acc32[3 * e + 2], (unsigned)(fx >> 42));
-            sc.in_union[e] = 1;
         }
         __syncthreads();
         const bool is_member = sc.in_union[tid] != 0;
         int mine;
         U = compact_threads(is_member, sc.warp_cnt[0], sc.member, &mine);
         bool pooled = is_member;
-        if (U > p.M || p.pool_ids != nullptr) {
+        if (!GIVEN && (U > p.M || p.pool_ids != nullptr)) {
             // pool = best M experts of the union by (score desc, id asc): rank by counting over the members
             if (is_member) {
                 const unsigned long long acc = (unsigned long long)sc.acc32[3 * tid] +
@@ -255,7 +261,7 @@ __global__ void __launch_bounds__(kThreads, 2) decode_small_gateup_kernel(Decode
     int G = P + p.n_shared;
     if (!is_static && (int)blockIdx.x < G * fblocks) load(blockIdx.x, 0, nxt);
 
-    if (!is_static) {
+    if (!GIVEN && !is_static) {
         // Eq. 12 for the batch's experts outside the pool (all experts for the metadata): a warp per source, loss and
         // scalar of every candidate in one round trip, two sources at a time
         const int n_src = meta ? N : (U > P ? U : 0);
@@ -297,11 +303,12 @@ __global__ void __launch_bounds__(kThreads, 2) decode_small_gateup_kernel(Decode
     }
     // Eq. 14: every slot in place; tokens that each group serves
     for (int s = tid; s < BK; s += kThreads) {
-        const int e = ids[s], t = sc.target[e];
+        const int e = ids[s], t = GIVEN ? e : sc.target[e];
+        atomicOr(&sc.mask[sc.grp_of[t]], 1u << (s / K));
+        if (GIVEN) continue;
         const float wv = (float)(w64[s] * (double)sc.scale[e]);
         ids[s] = t;
         wrm[s] = wv;
-        atomicOr(&sc.mask[sc.grp_of[t]], 1u << (s / K));
         if (meta) {
             p.out_ids[s] = t;
             p.out_w[s] = wv;
@@ -549,9 +556,10 @@ bool decode_small_fits(int B, int K, int d, const void* wg, const void* wu, cons
 
 cudaError_t launch_decode_small(DecodeSmallParams p, int sms, cudaStream_t s) {
     const size_t smem = gateup_bytes(p.B, p.K, p.d);
-    cudaError_t err = ensure_smem(decode_small_gateup_kernel, smem);
+    const auto gateup = p.w_in != nullptr ? decode_small_gateup_kernel<true> : decode_small_gateup_kernel<false>;
+    cudaError_t err = ensure_smem(gateup, smem);
     if (err != cudaSuccess) return err;
-    err = launch_pdl(decode_small_gateup_kernel, std::min(2 * sms, p.max_groups * (p.I / 8)), kThreads, smem, s, p);
+    err = launch_pdl(gateup, std::min(2 * sms, p.max_groups * (p.I / 8)), kThreads, smem, s, p);
     if (err != cudaSuccess) return err;
     // Down kernel, 16 warps per SM: one CTA of 16 warps when there are no more items than SMs (a cluster per item when
     // there are at most half as many), else two CTAs of 8 warps

@@ -187,3 +187,17 @@ def test_rows_summed_per_token(Kp, ns, d):
     got, ref = case.run_prefill(Kp), case.oracle_prefill(Kp)
     check_prefill_meta(got, ref)
     check_output(got["y"], ref["y"], "bf16")
+
+
+@pytest.mark.parametrize("T", [1, 3, 8, 9])
+@pytest.mark.parametrize("N,ns,d,I,K,Kp", [(16, 0, 256, 384, 4, 2), (40, 1, 1088, 192, 6, 6), (256, 1, 128, 64, 32, 32),
+                                            (8, 0, 2432, 128, 2, 1)])
+def test_few_token_prefill(T, N, ns, d, I, K, Kp):
+    """Prefill of at most 8 tokens on the small-batch kernels (9: the grouped GEMMs): metadata bit-exact, outputs to the bf16
+    bound and the same bits with metadata, without, and for every gemm_path."""
+    case = Case(si.LayerConfig("few", N, ns, d, I, K, "bf16", T, (Kp,), 4, (2,)))
+    got, ref = case.run_prefill(Kp), case.oracle_prefill(Kp)
+    check_prefill_meta(got, ref)
+    check_output(got["y"], ref["y"], "bf16")
+    for path in (0, 1, 2):
+        assert np.array_equal(got["y"], case.run_prefill(Kp, with_meta=False, gemm_path=path)["y"])
