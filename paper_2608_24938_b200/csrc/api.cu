@@ -1087,7 +1087,7 @@ int exfold_moe_prefill_host(const exfold_layer* layer, const void* x_host, const
     EXFOLD_CUDA(cudaStreamWaitEvent(h.in, h.start, 0));
     EXFOLD_CUDA(cudaStreamWaitEvent(h.out, h.start, 0));
     const size_t row_x = (size_t)layer->hidden * el, row_l = (size_t)layer->n_experts * 4;
-    const int64_t per = (T / chunks + 127) / 128 * 128;  // whole row tiles per chunk
+    const int64_t per = ((T + chunks - 1) / chunks + 127) / 128 * 128;  // whole row tiles per chunk, all tokens covered
     for (int c = 0; c < chunks; ++c) {
         const int64_t t0 = c * per, n = std::min<int64_t>(per, T - t0);
         if (n <= 0) break;

@@ -21,7 +21,7 @@
 // instruction suffices: at 48 GB/s of weights per SM it is busy a few percent of the time.
 //
 // Measured, four-kernel chain -> this (whole call): Qwen3 shape, 1 token 33.2 -> 21.4 us, 8 tokens with a pool of 32 53.8 -> 44.9;
-// Mixtral shape, 1 token 167 -> 124 (5.7 TB/s); GLM shape, 8 tokens with a pool of 32 213 -> 201. With two 8-column operands,
+// Mixtral shape, 1 token 167 -> 124 (5.7 TB/s); GLM shape, 8 tokens with a pool of 32 213 -> 201.
 // Prefill of 1 token 38.7 -> 18.8 (Mixtral shape 220 -> 126), of 8 tokens (Top-6, router) 96 -> 82. With two 8-column operands,
 // a decode of 16 tokens took 57 us against the chain's 42 (the per-CTA routing grows with the tokens), so the line is at 8.
 #include <algorithm>

@@ -201,3 +201,18 @@ def test_few_token_prefill(T, N, ns, d, I, K, Kp):
     check_output(got["y"], ref["y"], "bf16")
     for path in (0, 1, 2):
         assert np.array_equal(got["y"], case.run_prefill(Kp, with_meta=False, gemm_path=path)["y"])
+
+
+@pytest.mark.parametrize("T", [4095, 4097, 6145, 8192, 8193])
+def test_host_prefill_covers_every_token(T):
+    """Chunked host-buffer prefill around multiples of its chunks (8193 = four chunks of 2048 and one token more): every
+    token computed, bit-identical to the device call."""
+    cfg = si.LayerConfig("chunk", 8, 0, 64, 64, 2, "bf16", T, (1,), 4, (2,))
+    case = Case(cfg)
+    want = case.run_prefill(1, with_meta=False)["y"]
+    ex = case.ex
+    ws = ex.alloc_workspace(case.layer, T, 1, host_staging=True)
+    y = torch.full((T, 64), float("nan"), dtype=torch.bfloat16).pin_memory()
+    ex.exfold_moe_prefill_host(case.layer, case.x.pin_memory(), case.lg.pin_memory(), case.d_wg, case.d_wu, case.d_wd, case.tables, 1, y, ws)
+    assert ex.exfold_device_status(ws) == 0
+    assert np.array_equal(y.float().numpy(), want)
