@@ -133,7 +133,7 @@ size_t exfold_workspace_bytes(const exfold_layer *layer, int64_t max_tokens, int
  * never observed gets S = 0, L = 1e30; an expert never observed gets the mean h of the
  * others and the call returns EXFOLD_WARN_UNOBSERVED_EXPERT after synchronising the
  * stream (this call is off the serving path and does synchronise).
- * Expert outputs: fp32 layers use the fp32 SIMT expert kernel; bf16 layers run the same grouped
+ * Expert outputs: fp32 layers use the fp32 expert kernel; bf16 layers run the same grouped
  * tensor-core GEMMs as prefill (the SwiGLU activation is rounded to bf16 between the two GEMMs, the
  * outputs stay fp32), so the tables of a bf16 layer carry that rounding (~1e-3 relative per token).
  * Workspace: exfold_workspace_bytes(layer, m, K) for mode 0, (layer, m, N) for mode 1 (every expert
@@ -375,7 +375,7 @@ int64_t exfold_launch_count(void);
  * call). Slots: 0 prefill route/fold, 1 prefill scan, 2 prefill scatter+gather, 3 grouped GEMM-1
  * (gate/up + SwiGLU), 4 grouped GEMM-2 (down + scatter-combine), 5 fp32->bf16 conversion,
  * 6 decode pool/remap, 7 decode row gather, 8 decode GEMM-1 (gate/up stream), 9 decode GEMM-2 (down stream),
- * 10 SIMT expert FFN, 11 SIMT combine, 12 / 13 the CTA-pair pass of GEMM-1 / GEMM-2 alone (slots 3 and 4 cover a
+ * 10 fp32 expert FFN, 11 fp32 combine, 12 / 13 the CTA-pair pass of GEMM-1 / GEMM-2 alone (slots 3 and 4 cover a
  * whole GEMM: the pair pass, when it runs, and the one-CTA pass), 14 decode expert FFN of bf16 layers (one kernel:
  * pool / remap prologue + gate and up weight stream, slot 6 is then the per-token Top-K kernel; batches of at most 8
  * tokens: both kernels). Returns EXFOLD_OK or EXFOLD_ERR_CUDA.

@@ -104,7 +104,7 @@ Plan make_plan(const exfold_layer& l, int64_t Tm, int Kr) {
     p.n_groups = take(16);
     p.calib = take((size_t)N * N * (3 * 8 + 4) + (size_t)N * (8 + 4) + 256);
     p.calib_nrm = take(Rm * 8);  // calibration, common-input mode: squared output norms per (token, expert)
-    // large buffers: the bf16 pipeline (sorted rows, H, fp32 accumulator) and the SIMT path's
+    // large buffers: the bf16 pipeline (sorted rows, H, fp32 accumulator) and the fp32 path's
     // per-route outputs are never live at the same time and share one region
     p.big = off;
     size_t a = 0;
