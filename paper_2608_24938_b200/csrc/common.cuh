@@ -276,6 +276,7 @@ cudaError_t launch_decode_topk(const DecodeTopkParams& p, cudaStream_t s);
 // and the execution lists for the grouped down projection (ffn_decode.cu)
 struct DecodeFfnParams {
     CUtensorMap tm_x;     // x [B][d], box a_rows x 64
+    CUtensorMap tm_xg;    // x, box 1 x 64: rows gathered four at a time (more than 128 tokens)
     CUtensorMap tm_wg;    // W_gate as [(E*I)][d], box 128 x 64
     CUtensorMap tm_wu;    // W_up
     CUtensorMap tm_wg64;  // the same with 64-row boxes (half-width items)

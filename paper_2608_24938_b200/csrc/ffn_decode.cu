@@ -10,7 +10,8 @@
 //
 // Tokens are the 128-row M operand, read from x IN PLACE (all B tokens of the tile: no gathered copy; a token the
 // expert does not serve costs nothing extra and is simply not stored), weights the N = 256 operand, which is the
-// orientation in which a tcgen05.mma consumes weight bytes fastest (its cost follows M, not N). The two halves of
+// orientation in which a tcgen05.mma consumes weight bytes fastest (its cost follows M, not N). Above 128 tokens a
+// group of few rows is one item with its rows gathered instead (kGatherRows below). The two halves of
 // tensor memory alternate between items, so the SwiGLU epilogue of one item overlaps the MMAs of the next.
 // H is compact: one row per distinct (token, pool expert) pair, grouped by pool rank, tokens ascending. The down
 // projection then runs on the grouped GEMM-2 kernel with the whole intermediate dimension as K, which keeps the
@@ -29,7 +30,7 @@
 // Routing prologue, dependency wait -> pool known -> first weights multiplied -> row lists done: 64 tokens 3.2 -> 5.9 -> 12 us
 // before the members-only ranking, the eight-lane target search and the token masks; 256 tokens 4.5, 19 (nothing streams
 // before the lists there), 17 us. Whole call then -> now: Qwen3 shape 64 tokens, pool 16 43.4 -> 42.4 us; 256 tokens with the
-// router, pool 64 192 -> 180, pool 16 74 -> 66 (also a fourth ring stage, from the slot tables' bytes).
+// router, pool 64 192 -> 180 (dense items), pool 16 74 -> 66 (also a fourth ring stage, from the slot tables' bytes).
 //
 // Item sizes: full slices of 128 features; the last partial round of full items is cut into halves (s = 64) when
 // that lets more SMs share it, and a trailing 64-wide slice of I is a half by itself.
@@ -47,6 +48,13 @@ constexpr int kFThreads = 224;   // warp 0 and 6: TMA producers, warp 1: MMA iss
 constexpr int kFBK = 64;         // K elements per ring stage (one 128-byte swizzle row)
 constexpr int kFBBytes = 256 * kFBK * 2;   // weight part of a stage: 128 gate rows + 128 up rows
 constexpr int kFMaxStages = 8;
+// Above 128 tokens a group of at most kGatherRows rows is one item whose rows are gathered from x (TMA gather4, ~60-85
+// cycles of the SM's copy engine per four rows, so 64 rows fit the ~1200 cycles in which an SM's share of HBM brings a stage
+// of weights); a larger group runs as one dense item per token tile that it touches, which pulls its weights through the SM
+// twice. 256 tokens with the router, Qwen3 shape, pool 64 (some 32 rows per group): kernel 116 -> 96 us, call 187 -> 151 us;
+// with the limit at 32 rows 161 us, at 96 152.4, at 128 152.8.
+constexpr int kGatherRows = 64;
+constexpr int kGather = 2;
 constexpr int kFTmemCols = 512;
 constexpr int kFMaxPairs = 2 * kMaxGroups;      // (group, token tile) pairs: B <= 256 is at most two tiles
 constexpr int kFSmemLimit = 227 * 1024 - 2048;  // dynamic shared memory the kernel may ask for
@@ -63,14 +71,14 @@ struct Scratch {  // per-batch routing state, one copy per CTA
     float scale[kMaxExperts];
     float h[kMaxExperts];      // norm table (dynamic pool), staged before the dependency wait
     int goff[kFMaxPairs + 2];  // exclusive prefix over (group, token tile): first compact row
-    int pairs[kFMaxPairs];     // the pairs that have rows, in order: group * 2 + token tile (before that: the union's experts)
+    int pairs[kFMaxPairs];     // the work list's rows: group * 4 + token tile, or + kGather (before that: the union's experts)
     int chunk_cnt[kMaxExperts / 32];
     int P, U, n_pairs;
 };
 constexpr int kFScratchFixed = (int)((sizeof(Scratch) + 15) / 16 * 16);
 
 struct Item {
-    int expert, g, mt, j0, s;
+    int expert, g, mt, j0, s;  // mt: token tile, or kGather: all rows of the group, gathered
 };
 
 struct Sched {  // the same in every role of a CTA
@@ -147,9 +155,9 @@ __device__ __forceinline__ Item decode_item(int w, const Sched& sc, const Scratc
         it.j0 = sc.nfull * 128;
         it.s = 64;
     }
-    const int code = sc.identity ? pair * 2 : s.pairs[pair];
-    it.g = code >> 1;
-    it.mt = code & 1;
+    const int code = sc.identity ? pair * 4 : s.pairs[pair];
+    it.g = code >> 2;
+    it.mt = code & 3;
     it.expert = it.g < s.P ? s.pool[it.g] : N;  // group P is the shared expert
     return it;
 }
@@ -159,6 +167,8 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float a, float b) {
     return *reinterpret_cast<uint32_t*>(&v);
 }
 
+// NMT: token tiles of 128 (one kernel for both: 64 tokens 0.5 % slower, from the gathers' code)
+template <int NMT>
 __global__ void __launch_bounds__(kFThreads, 1) decode_ffn_kernel(const __grid_constant__ DecodeFfnParams p) {
     extern __shared__ unsigned char smem_raw[];
     __shared__ __align__(8) uint64_t full_bar[kFMaxStages];
@@ -167,6 +177,7 @@ __global__ void __launch_bounds__(kFThreads, 1) decode_ffn_kernel(const __grid_c
     __shared__ __align__(8) uint64_t tempty_bar[2];
     __shared__ uint32_t tmem_base_s;
     __shared__ int abort_s;
+    __shared__ __align__(16) int s_rows[2][NMT == 2 ? kGatherRows : 4];  // per producer: the tokens of a gathered item
 
     unsigned char* tiles =
         reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -183,6 +194,7 @@ __global__ void __launch_bounds__(kFThreads, 1) decode_ffn_kernel(const __grid_c
     // ---- set-up that does not depend on the previous kernel: overlaps its tail under programmatic launch
     if (threadIdx.x == 0) {
         ptx::prefetch_tmap(&p.tm_x);
+        if (NMT == 2) ptx::prefetch_tmap(&p.tm_xg);
         ptx::prefetch_tmap(&p.tm_wg);
         ptx::prefetch_tmap(&p.tm_wu);
         ptx::prefetch_tmap(&p.tm_wg96);
@@ -204,7 +216,7 @@ __global__ void __launch_bounds__(kFThreads, 1) decode_ffn_kernel(const __grid_c
     }
     const int B = p.B, N = p.N, K = p.K, BK = B * K;
     const bool is_static = p.st_pool != nullptr;
-    const int nmt = (B + 127) >> 7;
+    const int nmt = NMT == 2 ? 2 : (B + 127) >> 7;  // 1 as a run-time value: as a constant 0.4 % slower (64 tokens)
     // With the dynamic pool and one token tile every pool expert has a row (it is in the union), so the work list
     // is known as soon as the pool is: the producer and MMA warps leave for their roles then, and the epilogue
     // warps finish the routing (targets, remap, row lists, metadata) while the first weights stream in.
@@ -415,27 +427,42 @@ __global__ void __launch_bounds__(kFThreads, 1) decode_ffn_kernel(const __grid_c
             if (tid == 0) *p.pool_size = P;
         }
         sync_group();
-        // exclusive prefix over (group, tile) = first compact row of each; the pairs that have rows
+        // exclusive prefix over (group, tile) = first compact row of each; the work list's rows
         if (tid < 32) {
             int carry = 0, n = 0;
-            for (int c0 = 0; c0 < 2 * G; c0 += 32) {
-                const int c = c0 + tid;
-                int v = 0;
-                if (c < 2 * G && (c & 1) < nmt) {
-                    const uint4 m4 = *reinterpret_cast<const uint4*>(tmask + (c >> 1) * W + (c & 1) * 4);
-                    v = __popc(m4.x) + __popc(m4.y) + __popc(m4.z) + __popc(m4.w);
-                }
-                int incl = v;
+            for (int g0 = 0; g0 < G; g0 += 32) {
+                const int g = g0 + tid;
+                int v[2] = {0, 0};
+#pragma unroll
+                for (int mt = 0; mt < 2; ++mt)
+                    if (g < G && mt < nmt) {
+                        const uint4 m4 = *reinterpret_cast<const uint4*>(tmask + g * W + mt * 4);
+                        v[mt] = __popc(m4.x) + __popc(m4.y) + __popc(m4.z) + __popc(m4.w);
+                    }
+                const int rows = v[0] + v[1];
+                const bool gather = nmt == 2 && rows > 0 && rows <= kGatherRows;
+                const int entries = gather ? 1 : (v[0] > 0) + (v[1] > 0);
+                int incl = rows;
 #pragma unroll
                 for (int o = 1; o < 32; o <<= 1) {
                     const int u = __shfl_up_sync(0xffffffffu, incl, o);
                     if (tid >= o) incl += u;
                 }
-                if (c < 2 * G) sc.goff[c] = carry + incl - v;
+                const unsigned one = __ballot_sync(0xffffffffu, entries > 0), two = __ballot_sync(0xffffffffu, entries > 1);
+                const unsigned below = (1u << tid) - 1u;
+                if (g < G) {
+                    sc.goff[2 * g] = carry + incl - rows;
+                    sc.goff[2 * g + 1] = carry + incl - v[1];
+                    int q = n + __popc(one & below) + __popc(two & below);
+                    if (gather) {
+                        sc.pairs[q] = g * 4 + kGather;
+                    } else {
+                        if (v[0] > 0) sc.pairs[q++] = g * 4;
+                        if (v[1] > 0) sc.pairs[q] = g * 4 + 1;
+                    }
+                }
                 carry += __shfl_sync(0xffffffffu, incl, 31);
-                const unsigned m = __ballot_sync(0xffffffffu, v > 0);
-                if (v > 0) sc.pairs[n + __popc(m & ((1u << tid) - 1u))] = c;
-                n += __popc(m);
+                n += __popc(one) + __popc(two);
             }
             if (tid == 0) {
                 sc.goff[2 * G] = carry;
@@ -483,42 +510,63 @@ __global__ void __launch_bounds__(kFThreads, 1) decode_ffn_kernel(const __grid_c
 
     if (warp == 0 || warp == 6) {
         // ------------------------------------------------ TMA producers (k-block c belongs to producer c % 2)
-        if (lane == 0) {
-            const int me = warp == 0 ? 0 : 1;
-            int stage = 0, phase = 0, turn = 0;
-            bool ok = true;
+        const int me = warp == 0 ? 0 : 1;
+        int stage = 0, phase = 0, turn = 0;
+        int ok = 1;
+        if (NMT == 2 || lane == 0) {  // a whole warp where rows are gathered
             for (int w = w_begin; w < total && ok; w += w_stride) {
                 const Item it = decode_item(w, sched, sc, N);
-                const int xrow = it.mt * 128;
-                const int wrow = it.expert * p.I + it.j0;
-                const uint32_t tx = (uint32_t)(a_bytes + 2 * it.s * kFBK * 2);
-                for (int kb = 0; kb < nkb; ++kb) {
-                    if (turn == me) {
-                        if (!ptx::mbar_wait(&empty_bar[stage], phase ^ 1, abort_flag, p.status, 1)) {
-                            ok = false;
-                            break;
-                        }
-                        unsigned char* a_dst = tiles + stage * stage_bytes;
-                        unsigned char* b_dst = a_dst + a_bytes;
-                        ptx::mbar_expect_tx(&full_bar[stage], tx);
-                        ptx::tma_load_2d(a_dst, &p.tm_x, &full_bar[stage], kb * kFBK, xrow);
-                        if (it.s == 128) {
-                            ptx::tma_load_2d(b_dst, &p.tm_wg, &full_bar[stage], kb * kFBK, wrow);
-                            ptx::tma_load_2d(b_dst + 128 * kFBK * 2, &p.tm_wu, &full_bar[stage], kb * kFBK, wrow);
-                        } else if (it.s == 96) {
-                            ptx::tma_load_2d(b_dst, &p.tm_wg96, &full_bar[stage], kb * kFBK, wrow);
-                            ptx::tma_load_2d(b_dst + 96 * kFBK * 2, &p.tm_wu96, &full_bar[stage], kb * kFBK, wrow);
-                        } else {
-                            ptx::tma_load_2d(b_dst, &p.tm_wg64, &full_bar[stage], kb * kFBK, wrow);
-                            ptx::tma_load_2d(b_dst + 64 * kFBK * 2, &p.tm_wu64, &full_bar[stage], kb * kFBK, wrow);
-                        }
+                int n4 = 0;  // groups of four rows to gather
+                if (NMT == 2 && it.mt == kGather) {
+                    int n = 0;
+                    __syncwarp();
+                    for (int q = 0; q < W; ++q) {
+                        const uint32_t m = tmask[it.g * W + q];
+                        if ((m >> lane) & 1u) s_rows[me][n + __popc(m & ((1u << lane) - 1u))] = q * 32 + lane;
+                        n += __popc(m);
                     }
-                    turn ^= 1;
-                    if (++stage == stages) {
-                        stage = 0;
-                        phase ^= 1;
+                    __syncwarp();
+                    n4 = (n + 3) >> 2;
+                    if (lane < 4 * n4 - n) s_rows[me][n + lane] = s_rows[me][0];  // the last four filled up
+                    __syncwarp();
+                }
+                if (lane == 0) {
+                    const int xrow = NMT == 2 && it.mt == 1 ? 128 : 0;
+                    const int wrow = it.expert * p.I + it.j0;
+                    const uint32_t tx = (uint32_t)((n4 > 0 ? n4 * 512 : a_bytes) + 2 * it.s * kFBK * 2);
+                    for (int kb = 0; kb < nkb; ++kb) {
+                        if (turn == me) {
+                            if (!ptx::mbar_wait(&empty_bar[stage], phase ^ 1, abort_flag, p.status, 1)) {
+                                ok = 0;
+                                break;
+                            }
+                            unsigned char* a_dst = tiles + stage * stage_bytes;
+                            unsigned char* b_dst = a_dst + a_bytes;
+                            ptx::mbar_expect_tx(&full_bar[stage], tx);
+                            if (n4 == 0) ptx::tma_load_2d(a_dst, &p.tm_x, &full_bar[stage], kb * kFBK, xrow);
+                            if (it.s == 128) {
+                                ptx::tma_load_2d(b_dst, &p.tm_wg, &full_bar[stage], kb * kFBK, wrow);
+                                ptx::tma_load_2d(b_dst + 128 * kFBK * 2, &p.tm_wu, &full_bar[stage], kb * kFBK, wrow);
+                            } else if (it.s == 96) {
+                                ptx::tma_load_2d(b_dst, &p.tm_wg96, &full_bar[stage], kb * kFBK, wrow);
+                                ptx::tma_load_2d(b_dst + 96 * kFBK * 2, &p.tm_wu96, &full_bar[stage], kb * kFBK, wrow);
+                            } else {
+                                ptx::tma_load_2d(b_dst, &p.tm_wg64, &full_bar[stage], kb * kFBK, wrow);
+                                ptx::tma_load_2d(b_dst + 64 * kFBK * 2, &p.tm_wu64, &full_bar[stage], kb * kFBK, wrow);
+                            }
+                            for (int q = 0; q < n4; ++q) {
+                                const int4 r = *reinterpret_cast<const int4*>(&s_rows[me][4 * q]);
+                                ptx::tma_gather4(a_dst + q * 512, &p.tm_xg, &full_bar[stage], kb * kFBK, r.x, r.y, r.z, r.w);
+                            }
+                        }
+                        turn ^= 1;
+                        if (++stage == stages) {
+                            stage = 0;
+                            phase ^= 1;
+                        }
                     }
                 }
+                if (NMT == 2) ok = __shfl_sync(0xffffffffu, ok, 0);
             }
         }
         __syncwarp();
@@ -565,19 +613,39 @@ __global__ void __launch_bounds__(kFThreads, 1) decode_ffn_kernel(const __grid_c
         for (int w = w_begin; w < total; w += w_stride, ++item) {
             const Item it = decode_item(w, sched, sc, N);
             const int as = item & 1, aphase = (item >> 1) & 1;
-            // Which tokens of the tile does this expert serve? All four quadrants, so that a warp knows how many rows
-            // come before its own
             const bool shared_grp = it.g >= sc.P;
-            const uint4 m4 = *reinterpret_cast<const uint4*>(tmask + it.g * W + it.mt * 4);
-            const unsigned m[4] = {m4.x, m4.y, m4.z, m4.w};
-            int before = 0;
+            bool valid;
+            unsigned mq;  // this quadrant's rows that are stored
+            int tok;
+            int64_t rowpos;
+            if (NMT == 2 && it.mt == kGather) {  // the group's rows in order
+                valid = row < sc.goff[2 * it.g + 2] - sc.goff[2 * it.g];
+                mq = __ballot_sync(0xffffffffu, valid);
+                rowpos = sc.goff[2 * it.g] + row;
+                tok = 0;
+                if (it.j0 == 0 && valid) {  // the row-th token of the mask
+                    int left = row, q8 = 0;
+                    uint32_t m = tmask[it.g * W];
+                    while (left >= __popc(m)) {
+                        left -= __popc(m);
+                        m = tmask[it.g * W + ++q8];
+                    }
+                    tok = q8 * 32 + (int)__fns(m, 0, left + 1);
+                }
+            } else {
+                // Which tokens of the tile does this expert serve? All four quadrants, so that a warp knows how many rows
+                // come before its own
+                const uint4 m4 = *reinterpret_cast<const uint4*>(tmask + it.g * W + it.mt * 4);
+                const unsigned m[4] = {m4.x, m4.y, m4.z, m4.w};
+                int before = 0;
 #pragma unroll
-            for (int qq = 0; qq < 4; ++qq)
-                if (qq < q) before += __popc(m[qq]);
-            const unsigned mq = q == 0 ? m[0] : (q == 1 ? m[1] : (q == 2 ? m[2] : m[3]));
-            const bool valid = (mq >> lane) & 1u;
-            const int tok = it.mt * 128 + row;
-            const int64_t rowpos = sc.goff[it.g * 2 + it.mt] + before + __popc(mq & ((1u << lane) - 1u));
+                for (int qq = 0; qq < 4; ++qq)
+                    if (qq < q) before += __popc(m[qq]);
+                mq = q == 0 ? m[0] : (q == 1 ? m[1] : (q == 2 ? m[2] : m[3]));
+                valid = (mq >> lane) & 1u;
+                tok = it.mt * 128 + row;
+                rowpos = sc.goff[it.g * 2 + it.mt] + before + __popc(mq & ((1u << lane) - 1u));
+            }
             if (it.j0 == 0 && valid) {
                 // this CTA owns the group's first slice: it writes the group's rows of the execution lists
                 float cw = 1.0f;
@@ -664,9 +732,10 @@ cudaError_t launch_decode_ffn(const DecodeFfnParams& p, int sms, cudaStream_t s)
     int stages, scratch_off, a_rows;
     const size_t smem = decode_ffn_smem_plan(p.B, p.K, p.N, &stages, &scratch_off, &a_rows);
     if (stages < 2 || stages != p.stages || scratch_off != p.scratch_off) return cudaErrorInvalidValue;
-    cudaError_t err = ensure_smem(decode_ffn_kernel, smem);
+    auto kernel = p.B > 128 ? decode_ffn_kernel<2> : decode_ffn_kernel<1>;
+    cudaError_t err = ensure_smem(kernel, smem);
     if (err != cudaSuccess) return err;
-    return launch_pdl(decode_ffn_kernel, std::min(sms, kMaxCtas), kFThreads, smem, s, p);
+    return launch_pdl(kernel, std::min(sms, kMaxCtas), kFThreads, smem, s, p);
 }
 
 }  // namespace exfold

@@ -153,6 +153,32 @@ def test_decode_router_scores_by_batch(B, N):
     check_output(y.float().cpu().numpy(), ref["y"], "bf16")
 
 
+@pytest.mark.parametrize("rows,ns,d,I", [
+    ([1, 3, 4, 5, 63, 64, 65, 51], 0, 256, 384),     # 256 tokens: gathered up to 64 rows, dense above
+    ([64, 65], 1, 64, 64),                           # 129 tokens, one K chunk, half-width items, the shared expert dense
+    ([64, 64, 1], 0, 1088, 192),                     # every group gathered, 17 chunks
+    ([130, 126], 0, 128, 192),                       # none
+    ([2] * 100, 0, 128, 128),                        # many small groups
+])
+@pytest.mark.parametrize("place", ["mixed", "sorted"])
+def test_decode_group_sizes_above_128_tokens(rows, ns, d, I, place):
+    """More than 128 tokens: the gate/up items of small groups gather their rows, larger groups run per token tile. Each
+    token's one expert is given; "sorted" puts a group's tokens next to one another (a group then touches one tile or two)."""
+    B, N = sum(rows), len(rows)
+    case = Case(si.LayerConfig("groups", N, ns, d, I, 1, "bf16", 8, (1,), B, (N,)))
+    owner = np.repeat(np.arange(N), rows)
+    if place == "mixed":
+        owner = np.random.default_rng(5).permutation(owner)
+    case.lgd[torch.arange(B), torch.from_numpy(owner)] = 20.0
+    case.d_lgd = case.lgd.to(case.dev)
+    got, ref = case.run_decode(N), case.oracle_decode(N)
+    check_decode_meta(got, ref, N)
+    assert np.array_equal(got["ids"].reshape(-1), owner)
+    check_output(got["y"], ref["y"], "bf16")
+    plain = case.run_decode(N, with_meta=False)
+    assert np.array_equal(got["y"], plain["y"])
+
+
 @pytest.mark.parametrize("T", [1, 5, 128, 129, 300, 777, 5000])
 @pytest.mark.parametrize("N,d", [(31, 64), (40, 320), (130, 2048), (256, 1088)])
 def test_router_scores_by_prompt_length(T, N, d):
