@@ -31,6 +31,9 @@
 // before the members-only ranking, the eight-lane target search and the token masks; 256 tokens 4.5, 19 (nothing streams
 // before the lists there), 17 us. Whole call then -> now: Qwen3 shape 64 tokens, pool 16 43.4 -> 42.4 us; 256 tokens with the
 // router, pool 64 192 -> 180 (dense items), pool 16 74 -> 66 (also a fourth ring stage, from the slot tables' bytes).
+// Then slots four to a load, ranks on the keys' upper halves, a list of the sources outside the pool with 64 candidates per
+// round trip, no integer division per slot, and the schedule ahead of the dependency wait: 256 tokens 14.5 -> 9.7 us from the
+// wait to the first item (call 149 -> 146.5 us), 120 tokens with the router, pool 16 53.9 -> 52.6, 32 tokens 48.5 -> 48.1.
 //
 // Item sizes: full slices of 128 features; the last partial round of full items is cut into halves (s = 64) when
 // that lets more SMs share it, and a trailing 64-wide slice of I is a half by itself.
@@ -72,7 +75,6 @@ struct Scratch {  // per-batch routing state, one copy per CTA
     float h[kMaxExperts];      // norm table (dynamic pool), staged before the dependency wait
     int goff[kFMaxPairs + 2];  // exclusive prefix over (group, token tile): first compact row
     int pairs[kFMaxPairs];     // the work list's rows: group * 4 + token tile, or + kGather (before that: the union's experts)
-    int chunk_cnt[kMaxExperts / 32];
     int P, U, n_pairs;
 };
 constexpr int kFScratchFixed = (int)((sizeof(Scratch) + 15) / 16 * 16);
@@ -177,6 +179,7 @@ __global__ void __launch_bounds__(kFThreads, 1) decode_ffn_kernel(const __grid_c
     __shared__ __align__(8) uint64_t tempty_bar[2];
     __shared__ uint32_t tmem_base_s;
     __shared__ int abort_s;
+    __shared__ Sched sched_s;  // for the expected number of list entries
     __shared__ __align__(16) int s_rows[2][NMT == 2 ? kGatherRows : 4];  // per producer: the tokens of a gathered item
 
     unsigned char* tiles =
@@ -237,36 +240,56 @@ __global__ void __launch_bounds__(kFThreads, 1) decode_ffn_kernel(const __grid_c
             ptx::prefetch_l2(p.S + el);
         }
     }
+    // The schedule of the list that is expected (every group one entry, the pool full): its divisions take a microsecond
+    if (threadIdx.x == 96) sched_s = make_sched(min(p.M, min(N, BK)) + (p.n_shared ? 1 : 0), p.I, (int)gridDim.x, early ? 1 : 0);
     ptx::tc_fence_before();
     __syncthreads();
     grid_dep_wait();  // the per-token Top-K of the previous kernel; the previous call's readers of the workspace
 
     // ---- routing, batch level (Eq. 11, 12, 14), the same in every CTA
-    // (a thread's loads first, eight slots at a time: independent L2 round trips instead of one per slot)
-    for (int s0 = threadIdx.x; s0 < BK; s0 += kFThreads * 8) {
-        int id[8];
-        double wv[8];
+    // (four slots to a load, a thread's loads first: one L2 round trip for 256 tokens x 8)
+    auto add_slot = [&](int id, double wv) {
+        // The routed weight in 2^-53 fixed point, added as three 21-bit limbs with 32-bit integer atomics (at most 256
+        // addends per expert, so no limb overflows): exact, and independent of the order of arrival.
+        const unsigned long long fx = (unsigned long long)(wv * 9007199254740992.0);
+        atomicAdd(&sc.acc32[3 * id], (unsigned)(fx & 0x1FFFFFull));
+        atomicAdd(&sc.acc32[3 * id + 1], (unsigned)((fx >> 21) & 0x1FFFFFull));
+        atomicAdd(&sc.acc32[3 * id + 2], (unsigned)(fx >> 42));
+        sc.in_union[id] = 1;
+    };
+    const int BK4 = BK >> 2;
+    for (int s0 = threadIdx.x; s0 < BK4; s0 += kFThreads * 3) {
+        int4 id[3];
+        double2 wv[3][2];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
+        for (int u = 0; u < 3; ++u) {
             const int s = s0 + u * kFThreads;
-            id[u] = s < BK ? p.ids[s] : -1;
-            wv[u] = s < BK && !is_static ? p.w64[s] : 0.0;
-        }
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const int s = s0 + u * kFThreads;
-            if (id[u] < 0) continue;
-            ids8[s] = (unsigned char)id[u];
+            if (s >= BK4) break;
+            id[u] = reinterpret_cast<const int4*>(p.ids)[s];
             if (!is_static) {
-                // The routed weight in 2^-53 fixed point, added as three 21-bit limbs with 32-bit integer atomics (at
-                // most 256 addends per expert, so no limb overflows): exact, and independent of the order of arrival.
-                const unsigned long long fx = (unsigned long long)(wv[u] * 9007199254740992.0);
-                atomicAdd(&sc.acc32[3 * id[u]], (unsigned)(fx & 0x1FFFFFull));
-                atomicAdd(&sc.acc32[3 * id[u] + 1], (unsigned)((fx >> 21) & 0x1FFFFFull));
-                atomicAdd(&sc.acc32[3 * id[u] + 2], (unsigned)(fx >> 42));
-                sc.in_union[id[u]] = 1;
+                wv[u][0] = reinterpret_cast<const double2*>(p.w64)[2 * s];
+                wv[u][1] = reinterpret_cast<const double2*>(p.w64)[2 * s + 1];
             }
         }
+#pragma unroll
+        for (int u = 0; u < 3; ++u) {
+            const int s = s0 + u * kFThreads;
+            if (s >= BK4) break;
+            reinterpret_cast<uchar4*>(ids8)[s] =
+                make_uchar4((unsigned char)id[u].x, (unsigned char)id[u].y, (unsigned char)id[u].z, (unsigned char)id[u].w);
+            if (!is_static) {
+                add_slot(id[u].x, wv[u][0].x);
+                add_slot(id[u].y, wv[u][0].y);
+                add_slot(id[u].z, wv[u][1].x);
+                add_slot(id[u].w, wv[u][1].y);
+            }
+        }
+    }
+    if (threadIdx.x < (BK & 3)) {
+        const int s = BK4 * 4 + threadIdx.x;
+        const int id = p.ids[s];
+        ids8[s] = (unsigned char)id;
+        if (!is_static) add_slot(id, p.w64[s]);
     }
     __syncthreads();
     if (is_static) {
@@ -285,51 +308,67 @@ __global__ void __launch_bounds__(kFThreads, 1) decode_ffn_kernel(const __grid_c
         // Eq. 11: score_e = h_e * sum_i w_{i,e} in double, for the union's experts (in ascending order), ranked through an
         // order-preserving integer key
         const int n_chunks = (N + 31) >> 5;
-        for (int c = warp; c < n_chunks; c += kFThreads / 32) {
-            const unsigned m = __ballot_sync(0xffffffffu, c * 32 + lane < N && sc.in_union[c * 32 + lane]);
-            if (lane == 0) sc.chunk_cnt[c] = __popc(m);
-        }
-        __syncthreads();
         int* member = sc.pairs;
+        int* khi = reinterpret_cast<int*>(sc.scale);  // the keys' upper halves
         int U = 0;
-        for (int c = 0; c < n_chunks; ++c) U += sc.chunk_cnt[c];
-        for (int c = warp; c < n_chunks; c += kFThreads / 32) {
+        for (int c = 0; c < n_chunks; ++c) {
             const int e = c * 32 + lane;
             const bool in = e < N && sc.in_union[e];
             const unsigned m = __ballot_sync(0xffffffffu, in);
-            if (!in) continue;
-            int pos = __popc(m & ((1u << lane) - 1u));
-            for (int q = 0; q < c; ++q) pos += sc.chunk_cnt[q];
-            const unsigned long long acc = (unsigned long long)sc.acc32[3 * e] +
-                                           ((unsigned long long)sc.acc32[3 * e + 1] << 21) +
-                                           ((unsigned long long)sc.acc32[3 * e + 2] << 42);
-            const double score = (double)acc * (1.0 / 9007199254740992.0) * (double)sc.h[e] + 0.0;
-            long long key = __double_as_longlong(score);
-            if (key < 0) key ^= 0x7FFFFFFFFFFFFFFFll;  // negative doubles: larger magnitude = smaller
-            member[pos] = e;
-            sc.key[pos] = key;
+            if (in && c % (kFThreads / 32) == warp) {
+                const int pos = U + __popc(m & ((1u << lane) - 1u));
+                const unsigned long long acc = (unsigned long long)sc.acc32[3 * e] +
+                                               ((unsigned long long)sc.acc32[3 * e + 1] << 21) +
+                                               ((unsigned long long)sc.acc32[3 * e + 2] << 42);
+                const double score = (double)acc * (1.0 / 9007199254740992.0) * (double)sc.h[e] + 0.0;
+                long long key = __double_as_longlong(score);
+                if (key < 0) key ^= 0x7FFFFFFFFFFFFFFFll;  // negative doubles: larger magnitude = smaller
+                member[pos] = e;
+                sc.key[pos] = key;
+                khi[pos] = (int)(key >> 32);
+            }
+            U += __popc(m);
         }
+        if (threadIdx.x < (-U & 3)) khi[U + threadIdx.x] = INT_MIN;
         __syncthreads();
-        // pool = best min(M, |U|) experts of the union by (score desc, id asc): rank by counting, several threads per member
-        // (a thread per expert over all N keys took 1.8 us for N = 128)
+        // pool = best min(M, |U|) experts of the union by (score desc, id asc): rank by counting, several threads per
+        // member, on the keys' upper halves four to a load; only a member whose half another one shares counts whole keys.
+        // A member outside the pool is a source; rank - M is its place in the list.
         int lanes = 32;
         while (lanes > 1 && U * lanes > kFThreads) lanes >>= 1;
         const int sub = threadIdx.x & (lanes - 1);
+        int* src = reinterpret_cast<int*>(sc.acc32);
         for (int i0 = 0; i0 < U; i0 += kFThreads / lanes) {
             const int i = i0 + (int)threadIdx.x / lanes;
-            int better = 0;
+            int better = 0, same = 0;
             if (i < U) {
-                const long long ki = sc.key[i];
+                const int ki = khi[i];
 #pragma unroll 4
-                for (int o = sub; o < U; o += lanes) {
-                    const long long ko = sc.key[o];
-                    better += (ko > ki || (ko == ki && o < i)) ? 1 : 0;  // members ascend: position order is id order
+                for (int o = sub; 4 * o < U; o += lanes) {
+                    const int4 ko = reinterpret_cast<const int4*>(khi)[o];
+                    better += (ko.x > ki) + (ko.y > ki) + (ko.z > ki) + (ko.w > ki);
+                    same += (ko.x == ki) + (ko.y == ki) + (ko.z == ki) + (ko.w == ki);
                 }
             }
-            for (int o = lanes >> 1; o > 0; o >>= 1) better += __shfl_xor_sync(0xffffffffu, better, o);
-            if (i < U && sub == 0 && better < p.M) {
-                sc.rank_of[member[i]] = better;
-                sc.pool[better] = member[i];
+            for (int o = lanes >> 1; o > 0; o >>= 1) {
+                better += __shfl_xor_sync(0xffffffffu, better, o);
+                same += __shfl_xor_sync(0xffffffffu, same, o);
+            }
+            if (i < U && sub == 0) {
+                if (same > 1) {
+                    const long long ki = sc.key[i];
+                    better = 0;
+                    for (int o = 0; o < U; ++o) {
+                        const long long ko = sc.key[o];
+                        better += (ko > ki || (ko == ki && o < i)) ? 1 : 0;  // members ascend: position order is id order
+                    }
+                }
+                if (better < p.M) {
+                    sc.rank_of[member[i]] = better;
+                    sc.pool[better] = member[i];
+                } else {
+                    src[better - p.M] = member[i];
+                }
             }
         }
         if (threadIdx.x == 0) {
@@ -349,27 +388,32 @@ __global__ void __launch_bounds__(kFThreads, 1) decode_ffn_kernel(const __grid_c
         const bool meta = p.pool_ids != nullptr && blockIdx.x == 0;  // the caller asked for the routing metadata
         if (!is_static) {
             // Eq. 12: a source in the pool keeps itself; any other takes its minimum-loss pool expert (ties -> lower
-            // id). Eight lanes per source, loss and scalar of 32 candidates in one round trip (a thread per source with
+            // id). Eight lanes per source, loss and scalar of 64 candidates in one round trip (a thread per source with
             // its candidates one after the other took 8 us for a pool of 64). Only sources that occur in the batch
             // matter for the execution; the metadata has the whole table.
-            const int n_src = meta ? N : sc.U, n_grp = nth >> 3, sub = tid & 7;
+            for (int j = tid; j < P; j += nth) {
+                sc.target[sc.pool[j]] = sc.pool[j];
+                sc.scale[sc.pool[j]] = 1.0f;
+            }
+            const int* src = reinterpret_cast<const int*>(sc.acc32);
+            const int n_src = meta ? N : sc.U - P, n_grp = nth >> 3, sub = tid & 7;
             for (int i0 = 0; i0 < n_src; i0 += n_grp) {
                 const int i = i0 + (tid >> 3);
-                const int s = i < n_src ? (meta ? i : sc.pairs[i]) : -1;
+                const int s = i < n_src ? (meta ? i : src[i]) : -1;
                 float bl = INFINITY, bs = 1.0f;
                 int bt = 0x7fffffff;
                 if (s >= 0 && sc.rank_of[s] < 0) {
-                    for (int j0 = sub; j0 < P; j0 += 32) {
-                        float l[4], sv[4];
-                        int tt[4];
+                    for (int j0 = sub; j0 < P; j0 += 64) {
+                        float l[8], sv[8];
+                        int tt[8];
 #pragma unroll
-                        for (int u = 0; u < 4; ++u) {
+                        for (int u = 0; u < 8; ++u) {
                             tt[u] = j0 + 8 * u < P ? sc.pool[j0 + 8 * u] : -1;
                             l[u] = tt[u] >= 0 ? __ldg(p.L + (size_t)s * N + tt[u]) : 0.f;
                             sv[u] = tt[u] >= 0 ? __ldg(p.S + (size_t)s * N + tt[u]) : 0.f;
                         }
 #pragma unroll
-                        for (int u = 0; u < 4; ++u)
+                        for (int u = 0; u < 8; ++u)
                             if (tt[u] >= 0 && (l[u] < bl || (l[u] == bl && tt[u] < bt))) {
                                 bl = l[u];
                                 bs = sv[u];
@@ -397,13 +441,25 @@ __global__ void __launch_bounds__(kFThreads, 1) decode_ffn_kernel(const __grid_c
             sync_group();
         }
         // Eq. 14: every slot in place; [B][K] layout kept. A token counts once per distinct target: a bit of its mask
-        for (int s = tid; s < BK; s += nth) {
-            const int e = ids8[s], t = sc.target[e], i = s / K;
-            ids8[s] = (unsigned char)t;
-            atomicOr(&tmask[sc.rank_of[t] * W + (i >> 5)], 1u << (i & 31));
-            if (meta) {
-                p.out_ids[s] = t;
-                p.out_w[s] = (float)(p.w64[s] * (double)sc.scale[e]);
+        const unsigned inv_k = ((1u << 18) + K - 1) / K;  // s / K = s * inv_k >> 18: s * K < 2^17
+        for (int s0 = tid; s0 < BK; s0 += 4 * nth) {
+            int e[4], t[4], r[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) e[u] = s0 + u * nth < BK ? ids8[s0 + u * nth] : -1;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) t[u] = e[u] >= 0 ? sc.target[e[u]] : 0;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) r[u] = e[u] >= 0 ? sc.rank_of[t[u]] : 0;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                if (e[u] < 0) continue;
+                const int s = s0 + u * nth, i = (int)(((unsigned)s * inv_k) >> 18);
+                ids8[s] = (unsigned char)t[u];
+                atomicOr(&tmask[r[u] * W + (i >> 5)], 1u << (i & 31));
+                if (meta) {
+                    p.out_ids[s] = t[u];
+                    p.out_w[s] = (float)(p.w64[s] * (double)sc.scale[e[u]]);
+                }
             }
         }
         if (p.n_shared && tid < W) {
@@ -501,7 +557,9 @@ __global__ void __launch_bounds__(kFThreads, 1) decode_ffn_kernel(const __grid_c
     if (!early) __syncthreads();
     ptx::tc_fence_after();
 
-    const Sched sched = make_sched(early ? sc.P + (p.n_shared ? 1 : 0) : sc.n_pairs, p.I, (int)gridDim.x, early ? 1 : 0);
+    const int n_list = early ? sc.P + (p.n_shared ? 1 : 0) : sc.n_pairs;
+    Sched sched = sched_s;
+    if (n_list != sched.n_pairs) sched = make_sched(n_list, p.I, (int)gridDim.x, early ? 1 : 0);
     const int total = sched.total;
     const int w_begin = (int)blockIdx.x < sched.ctas ? (int)blockIdx.x : total, w_stride = sched.ctas;
     const uint32_t tmem_base = tmem_base_s;

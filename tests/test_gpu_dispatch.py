@@ -179,6 +179,31 @@ def test_decode_group_sizes_above_128_tokens(rows, ns, d, I, place):
     assert np.array_equal(got["y"], plain["y"])
 
 
+@pytest.mark.parametrize("B,N,K,M", [
+    (9, 16, 5, 4),       # slots not a multiple of four, more members than pool places
+    (33, 40, 3, 40),     # the pool is the batch's union
+    (129, 40, 3, 16),    # two token tiles, ragged
+    (64, 256, 8, 200),   # more candidates than one round trip holds
+    (256, 128, 16, 70),  # the most slots
+    (256, 130, 8, 1),
+])
+@pytest.mark.parametrize("h_step", [0.0, 2.0 ** -23])
+def test_decode_pool_of_near_ties(B, N, K, M, h_step):
+    """Experts in pairs of equal router scores and (almost) equal norms: pool scores that agree in their upper halves (equal,
+    or apart by one unit of the norm's last place) are ranked by the whole score, then by id."""
+    case = Case(si.LayerConfig("ties", N, 0, 64, 64, K, "bf16", 8, (1,), B, (M,)))
+    case.lgd[:, 1::2] = case.lgd[:, 0:N - N % 2:2]
+    case.d_lgd = case.lgd.to(case.dev)
+    S, L, h, lnh = case.tables_host
+    h = 1.0 + h_step * (torch.arange(N) % 2).to(h.dtype)
+    case.set_tables((S, L, h, torch.log(h)))
+    got, ref = case.run_decode(M), case.oracle_decode(M)
+    check_decode_meta(got, ref, M)
+    check_output(got["y"], ref["y"], "bf16")
+    plain = case.run_decode(M, with_meta=False)
+    assert np.array_equal(got["y"], plain["y"])
+
+
 @pytest.mark.parametrize("T", [1, 5, 128, 129, 300, 777, 5000])
 @pytest.mark.parametrize("N,d", [(31, 64), (40, 320), (130, 2048), (256, 1088)])
 def test_router_scores_by_prompt_length(T, N, d):
