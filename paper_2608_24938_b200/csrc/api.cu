@@ -725,18 +725,18 @@ static int decode_impl(const exfold_layer* layer, const void* x, const float* lo
             // routing in its prologue and streams the pool's gate and up weights against x in place -> grouped down
             // projection over the compact rows -> per-token sum of the rows.
             int stages = 0, scratch_off = 0, ar = 0;
-            decode_ffn_smem_plan((int)B, K, N, &stages, &scratch_off, &ar);
+            const int max_groups = std::min(pool_m, N) + l.n_shared, sms = std::min(sm_count(), kMaxCtas);
+            const int alt = decode_ffn_alt((int)B, max_groups, I, sms);
+            decode_ffn_smem_plan((int)B, K, N, alt, &stages, &scratch_off, &ar);
             if (stages < 2) return EXFOLD_ERR_UNSUPPORTED;
-            CUtensorMap tm_x, tm_xg{}, tm_wg64, tm_wu64, tm_wg96, tm_wu96;
             const uint64_t E = (uint64_t)G;
-            if (!make_tmap(&tm_x, x, (uint64_t)B, d, ar) || (B > 128 && !make_tmap(&tm_xg, x, (uint64_t)B, d, 1)) ||
-                !make_tmap(&tm_wg64, w_gate, E * I, d, 64) ||
-                !make_tmap(&tm_wu64, w_up, E * I, d, 64) || !make_tmap(&tm_wg96, w_gate, E * I, d, 96) ||
-                !make_tmap(&tm_wu96, w_up, E * I, d, 96))
+            DecodeFfnParams fp{};
+            fp.alt = alt; fp.tm_wg = tm_wg; fp.tm_wu = tm_wu;
+            if (!make_tmap(&fp.tm_x, x, (uint64_t)B, d, ar) || (B > 128 && !make_tmap(&fp.tm_xg, x, (uint64_t)B, d, 1)) ||
+                !make_tmap(&fp.tm_wg64, w_gate, E * I, d, 64) || !make_tmap(&fp.tm_wu64, w_up, E * I, d, 64) ||
+                (alt && (!make_tmap(&fp.tm_wg_alt, w_gate, E * I, d, alt) || !make_tmap(&fp.tm_wu_alt, w_up, E * I, d, alt))))
                 return EXFOLD_ERR_CUDA;
             { ProfScope ps(6, s); EXFOLD_CUDA(launch_decode_topk(tp, s)); }
-            DecodeFfnParams fp{};
-            fp.tm_x = tm_x; fp.tm_xg = tm_xg; fp.tm_wg = tm_wg; fp.tm_wu = tm_wu; fp.tm_wg64 = tm_wg64; fp.tm_wu64 = tm_wu64; fp.tm_wg96 = tm_wg96; fp.tm_wu96 = tm_wu96;
             fp.ids = rp.ids; fp.w64 = tp.w64; fp.S = tables->S; fp.L = tables->L; fp.h = tables->h;
             fp.st_pool = rp.st_pool; fp.st_target = rp.st_target; fp.st_scale = rp.st_scale;
             fp.B = (int)B; fp.N = N; fp.K = K; fp.M = pool_m; fp.n_shared = l.n_shared; fp.d = d; fp.I = I; fp.a_rows = ar;
@@ -753,9 +753,7 @@ static int decode_impl(const exfold_layer* layer, const void* x, const float* lo
             // Down projection on the grouped GEMM-2 kernel over the compact rows (the whole intermediate dimension is
             // its K, so no partial outputs meet in memory); each row's weighted output is stored once, in bf16, and a
             // token's rows are then summed in slot order: no atomics, so a decode step is reproducible bit for bit.
-            const int max_groups = std::min(pool_m, N) + l.n_shared;
             const int tiles_per_group = (int)((B + kTileM - 1) / kTileM);
-            const int sms = std::min(sm_count(), kMaxCtas);
             GroupedGemmParams g{};
             g.tm_a = tm_h; g.tm_a2 = tm_h; g.tm_b0 = tm_wd; g.tm_b1 = tm_wd; g.x_rows = 1; g.o32 = nullptr;
             g.offsets = rp.grp_off; g.work_start = rp.grp_tiles; g.G = max_groups; g.n_routed = 0x7fffffff;

@@ -284,8 +284,9 @@ struct DecodeFfnParams {
     CUtensorMap tm_wu;    // W_up
     CUtensorMap tm_wg64;  // the same with 64-row boxes (half-width items)
     CUtensorMap tm_wu64;
-    CUtensorMap tm_wg96;  // and with 96-row boxes (a single round of 96-wide items)
-    CUtensorMap tm_wu96;
+    CUtensorMap tm_wg_alt;  // and with boxes of alt rows
+    CUtensorMap tm_wu_alt;
+    int alt;                // 96, 32 or 0: decode_ffn_alt
     const int32_t* ids;   // [B][K] from the top-k kernel
     const double* w64;    // [B][K]
     const float* S;       // tables (dynamic pool)
@@ -316,7 +317,8 @@ struct DecodeFfnParams {
     DeviceStatus* status;
 };
 cudaError_t launch_decode_ffn(const DecodeFfnParams& p, int sms, cudaStream_t s);
-size_t decode_ffn_smem_plan(int B, int K, int N, int* stages, int* scratch_off, int* a_rows);
+int decode_ffn_alt(int B, int max_groups, int I, int sms);
+size_t decode_ffn_smem_plan(int B, int K, int N, int alt, int* stages, int* scratch_off, int* a_rows);
 // Decode of at most kSmallDecodeBatch tokens, bf16 layers: two kernels (decode_small.cu). Prefill calls that short run the
 // same two after their own routing.
 constexpr int kSmallDecodeBatch = 8;

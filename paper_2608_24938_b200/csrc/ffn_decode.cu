@@ -36,7 +36,7 @@
 // wait to the first item (call 149 -> 146.5 us), 120 tokens with the router, pool 16 53.9 -> 52.6, 32 tokens 48.5 -> 48.1.
 //
 // Item sizes: full slices of 128 features; the last partial round of full items is cut into halves (s = 64) when
-// that lets more SMs share it, and a trailing 64-wide slice of I is a half by itself.
+// that lets more SMs share it, and a trailing 64-wide slice of I is a half by itself. Single rounds: 96- or 32-wide slices.
 #include <algorithm>
 #include <climits>
 
@@ -50,7 +50,7 @@ namespace {
 constexpr int kFThreads = 224;   // warp 0 and 6: TMA producers, warp 1: MMA issuer, warps 2-5: epilogue
 constexpr int kFBK = 64;         // K elements per ring stage (one 128-byte swizzle row)
 constexpr int kFBBytes = 256 * kFBK * 2;   // weight part of a stage: 128 gate rows + 128 up rows
-constexpr int kFMaxStages = 8;
+constexpr int kFMaxStages = 16;
 // Above 128 tokens a group of at most kGatherRows rows is one item whose rows are gathered from x (TMA gather4, ~60-85
 // cycles of the SM's copy engine per four rows, so 64 rows fit the ~1200 cycles in which an SM's share of HBM brings a stage
 // of weights); a larger group runs as one dense item per token tile that it touches, which pulls its weights through the SM
@@ -63,6 +63,10 @@ constexpr int kFMaxPairs = 2 * kMaxGroups;      // (group, token tile) pairs: B 
 constexpr int kFSmemLimit = 227 * 1024 - 2048;  // dynamic shared memory the kernel may ask for
 static_assert(kGemmBK == 64, "the decode FFN kernel stages 64 K elements per k-block");
 static_assert(kMaxDecodeBatch <= 256, "two token tiles per group at most");
+
+__host__ __device__ constexpr int decode_ffn_stage_bytes(int a_rows, int alt) {
+    return a_rows * kFBK * 2 + (alt == 32 ? kFBBytes / 4 : kFBBytes);
+}
 
 struct Scratch {  // per-batch routing state, one copy per CTA
     long long key[kMaxExperts];        // by union member: order-preserving integer image of score_e
@@ -85,7 +89,7 @@ struct Item {
 
 struct Sched {  // the same in every role of a CTA
     int n_pairs, nfull, has_half, f_keep, split, total;
-    int n96;       // > 0: every item is a 96-wide slice, n96 per pair (see make_sched)
+    int alt, n_alt;  // n_alt > 0: every item is an alt-wide slice (96 or 32), n_alt per pair (see make_sched)
     int identity;  // pair p is (group p, token tile 0): no list needed
     int ctas;      // CTAs that take work: item w belongs to CTA w % ctas
 };
@@ -96,7 +100,7 @@ struct Sched {  // the same in every role of a CTA
 // In units of the time one SM needs for a full item alone, a phase of n SMs working at once takes z * max(1, n / c)
 // for items of size z: about c = 110 SMs of this kernel saturate HBM (measured: it streams ~55 GB/s per SM, ~6 TB/s together).
 // (b) wins when the remainder would leave a few SMs working alone (448 items: 112 x 4 rather than 148 x 3 + 8 halves).
-__device__ __forceinline__ Sched make_sched(int n_pairs, int I, int grid, int identity) {
+__device__ __forceinline__ Sched make_sched(int n_pairs, int I, int grid, int identity, int alt) {
     Sched sc;
     sc.identity = identity;
     sc.n_pairs = n_pairs;
@@ -109,13 +113,15 @@ __device__ __forceinline__ Sched make_sched(int n_pairs, int I, int grid, int id
     // Less than one round of full items, too many to halve: 96-wide slices when they divide I and still fit one round.
     // What an SM streams is bounded by the bytes its ring keeps in flight over the loaded HBM latency (~60 GB/s), so a
     // single round goes faster on more SMs with smaller items (16 experts x 768: 128 items of 0.75 MB, not 96 of 1 MB).
-    sc.n96 = 0;
-    if (q == 0 && r > 0 && !can_split && H == 0 && I % 96 == 0 && n_pairs * (I / 96) <= grid && I / 96 > sc.nfull) {
-        sc.n96 = I / 96;
+    // Few groups, so that even 32-wide slices all have an SM to themselves (decided by the host, decode_ffn_alt): those.
+    sc.alt = alt;
+    sc.n_alt = 0;
+    if (alt == 32 || (alt == 96 && q == 0 && r > 0 && !can_split && H == 0 && n_pairs * (I / 96) <= grid && I / 96 > sc.nfull)) {
+        sc.n_alt = I / alt;
         sc.split = 0;
         sc.ctas = grid;
         sc.f_keep = 0;
-        sc.total = n_pairs * sc.n96;
+        sc.total = n_pairs * sc.n_alt;
         return sc;
     }
     float ta = (float)q * fmaxf(1.0f, (float)grid / c);
@@ -139,10 +145,10 @@ __device__ __forceinline__ Sched make_sched(int n_pairs, int I, int grid, int id
 __device__ __forceinline__ Item decode_item(int w, const Sched& sc, const Scratch& s, int N) {
     Item it;
     int pair;
-    if (sc.n96 > 0) {
-        pair = w / sc.n96;
-        it.j0 = (w - pair * sc.n96) * 96;
-        it.s = 96;
+    if (sc.n_alt > 0) {
+        pair = w / sc.n_alt;
+        it.j0 = (w - pair * sc.n_alt) * sc.alt;
+        it.s = sc.alt;
     } else if (w < sc.f_keep) {
         pair = w / sc.nfull;
         it.j0 = (w - pair * sc.nfull) * 128;
@@ -187,7 +193,7 @@ __global__ void __launch_bounds__(kFThreads, 1) decode_ffn_kernel(const __grid_c
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int stages = p.stages;
     const int a_bytes = p.a_rows * kFBK * 2;
-    const int stage_bytes = a_bytes + kFBBytes;
+    const int stage_bytes = decode_ffn_stage_bytes(p.a_rows, p.alt);
     Scratch& sc = *reinterpret_cast<Scratch*>(tiles + p.scratch_off);
     // one byte per slot (its routed expert, then its target) and, by pool rank, the tokens each group serves as bit masks:
     // what is not spent here is ring (256 tokens x 8 slots: 20 KB with ids and weights as words, one stage of four)
@@ -200,8 +206,10 @@ __global__ void __launch_bounds__(kFThreads, 1) decode_ffn_kernel(const __grid_c
         if (NMT == 2) ptx::prefetch_tmap(&p.tm_xg);
         ptx::prefetch_tmap(&p.tm_wg);
         ptx::prefetch_tmap(&p.tm_wu);
-        ptx::prefetch_tmap(&p.tm_wg96);
-        ptx::prefetch_tmap(&p.tm_wu96);
+        if (p.alt) {
+            ptx::prefetch_tmap(&p.tm_wg_alt);
+            ptx::prefetch_tmap(&p.tm_wu_alt);
+        }
         for (int s = 0; s < kFMaxStages; ++s) {
             ptx::mbar_init(&full_bar[s], 1);
             ptx::mbar_init(&empty_bar[s], 1);
@@ -241,7 +249,7 @@ __global__ void __launch_bounds__(kFThreads, 1) decode_ffn_kernel(const __grid_c
         }
     }
     // The schedule of the list that is expected (every group one entry, the pool full): its divisions take a microsecond
-    if (threadIdx.x == 96) sched_s = make_sched(min(p.M, min(N, BK)) + (p.n_shared ? 1 : 0), p.I, (int)gridDim.x, early ? 1 : 0);
+    if (threadIdx.x == 96) sched_s = make_sched(min(p.M, min(N, BK)) + (p.n_shared ? 1 : 0), p.I, (int)gridDim.x, early ? 1 : 0, p.alt);
     ptx::tc_fence_before();
     __syncthreads();
     grid_dep_wait();  // the per-token Top-K of the previous kernel; the previous call's readers of the workspace
@@ -559,7 +567,7 @@ __global__ void __launch_bounds__(kFThreads, 1) decode_ffn_kernel(const __grid_c
 
     const int n_list = early ? sc.P + (p.n_shared ? 1 : 0) : sc.n_pairs;
     Sched sched = sched_s;
-    if (n_list != sched.n_pairs) sched = make_sched(n_list, p.I, (int)gridDim.x, early ? 1 : 0);
+    if (n_list != sched.n_pairs) sched = make_sched(n_list, p.I, (int)gridDim.x, early ? 1 : 0, p.alt);
     const int total = sched.total;
     const int w_begin = (int)blockIdx.x < sched.ctas ? (int)blockIdx.x : total, w_stride = sched.ctas;
     const uint32_t tmem_base = tmem_base_s;
@@ -605,12 +613,12 @@ __global__ void __launch_bounds__(kFThreads, 1) decode_ffn_kernel(const __grid_c
                             if (it.s == 128) {
                                 ptx::tma_load_2d(b_dst, &p.tm_wg, &full_bar[stage], kb * kFBK, wrow);
                                 ptx::tma_load_2d(b_dst + 128 * kFBK * 2, &p.tm_wu, &full_bar[stage], kb * kFBK, wrow);
-                            } else if (it.s == 96) {
-                                ptx::tma_load_2d(b_dst, &p.tm_wg96, &full_bar[stage], kb * kFBK, wrow);
-                                ptx::tma_load_2d(b_dst + 96 * kFBK * 2, &p.tm_wu96, &full_bar[stage], kb * kFBK, wrow);
-                            } else {
+                            } else if (it.s == 64) {
                                 ptx::tma_load_2d(b_dst, &p.tm_wg64, &full_bar[stage], kb * kFBK, wrow);
                                 ptx::tma_load_2d(b_dst + 64 * kFBK * 2, &p.tm_wu64, &full_bar[stage], kb * kFBK, wrow);
+                            } else {
+                                ptx::tma_load_2d(b_dst, &p.tm_wg_alt, &full_bar[stage], kb * kFBK, wrow);
+                                ptx::tma_load_2d(b_dst + it.s * kFBK * 2, &p.tm_wu_alt, &full_bar[stage], kb * kFBK, wrow);
                             }
                             for (int q = 0; q < n4; ++q) {
                                 const int4 r = *reinterpret_cast<const int4*>(&s_rows[me][4 * q]);
@@ -635,7 +643,7 @@ __global__ void __launch_bounds__(kFThreads, 1) decode_ffn_kernel(const __grid_c
             const uint32_t lo_step = (uint32_t)stage_bytes >> 4, lo_b = (uint32_t)a_bytes >> 4;
             const uint32_t desc_hi32 = (uint32_t)(ptx::make_kmajor_sw128_desc(0) >> 32);
             constexpr uint32_t idesc256 = ptx::make_idesc_bf16(128, 256), idesc128 = ptx::make_idesc_bf16(128, 128),
-                               idesc192 = ptx::make_idesc_bf16(128, 192);
+                               idesc192 = ptx::make_idesc_bf16(128, 192), idesc64 = ptx::make_idesc_bf16(128, 64);
             int stage = 0, phase = 0, item = 0;
             uint32_t a_lo = lo0;
             bool ok = true, ready = false;
@@ -645,7 +653,7 @@ __global__ void __launch_bounds__(kFThreads, 1) decode_ffn_kernel(const __grid_c
                 if (!ptx::mbar_wait(&tempty_bar[as], aphase ^ 1, abort_flag, p.status, 2)) break;
                 ptx::tc_fence_after();
                 const uint32_t d_tmem = tmem_base + as * 256;
-                const uint32_t idesc = it.s == 128 ? idesc256 : (it.s == 96 ? idesc192 : idesc128);
+                const uint32_t idesc = it.s == 128 ? idesc256 : (it.s == 64 ? idesc128 : (it.s == 96 ? idesc192 : idesc64));
                 for (int kb = 0; kb < nkb; ++kb) {
                     if (!ready && !ptx::mbar_wait(&full_bar[stage], phase, abort_flag, p.status, 3)) {
                         ok = false;
@@ -771,10 +779,20 @@ __global__ void __launch_bounds__(kFThreads, 1) decode_ffn_kernel(const __grid_c
 
 }  // namespace
 
-// Shared-memory plan: [ring: stages x (token box + 32 KB of weights)][routing state][ids', token masks]
-size_t decode_ffn_smem_plan(int B, int K, int N, int* stages, int* scratch_off, int* a_rows) {
+// Width of the slices beside 128 and 64 that a call may use (make_sched). 32 where every (group, 32 features) of the largest
+// pool has an SM to itself: a group of I = 768 then streams on 24 SMs, not on 12 with halves.
+// Whole call without / with: Qwen3 shape 16 tokens, pool 4 28.9 / 28.2 us, 128 tokens, pool 2 31.1 / 30.0, 200 tokens, pool 3
+// 37.5 / 35.9; GLM shape 100 tokens, pool 1 50.5 / 47.3.
+int decode_ffn_alt(int B, int max_groups, int I, int sms) {
+    if (I % 32 == 0 && (int64_t)((B + 127) / 128) * max_groups * (I / 32) <= std::min(sms, kMaxCtas)) return 32;
+    return I % 96 == 0 ? 96 : 0;
+}
+
+// Shared-memory plan: [ring: stages x (token box + 32 KB of weights, 8 KB when all slices are 32 wide)][routing state][ids',
+// token masks]
+size_t decode_ffn_smem_plan(int B, int K, int N, int alt, int* stages, int* scratch_off, int* a_rows) {
     const int ar = std::min(kTileM, (B + 31) / 32 * 32);
-    const int stage_bytes = ar * kFBK * 2 + kFBBytes;
+    const int stage_bytes = decode_ffn_stage_bytes(ar, alt);
     const int mask_words = (B + 127) / 128 * 4;
     const size_t scratch = kFScratchFixed + align16((size_t)B * K) + (size_t)(N + 1) * mask_words * 4;
     const long avail = (long)kFSmemLimit - 1024 - (long)scratch;
@@ -788,7 +806,7 @@ size_t decode_ffn_smem_plan(int B, int K, int N, int* stages, int* scratch_off, 
 
 cudaError_t launch_decode_ffn(const DecodeFfnParams& p, int sms, cudaStream_t s) {
     int stages, scratch_off, a_rows;
-    const size_t smem = decode_ffn_smem_plan(p.B, p.K, p.N, &stages, &scratch_off, &a_rows);
+    const size_t smem = decode_ffn_smem_plan(p.B, p.K, p.N, p.alt, &stages, &scratch_off, &a_rows);
     if (stages < 2 || stages != p.stages || scratch_off != p.scratch_off) return cudaErrorInvalidValue;
     auto kernel = p.B > 128 ? decode_ffn_kernel<2> : decode_ffn_kernel<1>;
     cudaError_t err = ensure_smem(kernel, smem);
