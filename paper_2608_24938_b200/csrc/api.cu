@@ -669,12 +669,11 @@ static int decode_impl(const exfold_layer* layer, const void* x, const float* lo
     // a group has at most B rows: the token box of the GEMMs needs only that many (multiple of 32, <= 128)
     const int a_rows = (int)std::min<int64_t>(kTileM, (B + 31) / 32 * 32);
 
-    CUtensorMap tm_wg, tm_wu, tm_h, tm_wd;
+    CUtensorMap tm_wg, tm_wu, tm_h;
     if (bf16) {
         const uint64_t E = (uint64_t)G;
         bool ok = make_tmap(&tm_wg, w_gate, E * I, d, 128) && make_tmap(&tm_wu, w_up, E * I, d, 128) &&
-                  make_tmap(&tm_h, at<char>(ws, pl.H), (uint64_t)max_rows, I, a_rows) &&
-                  make_tmap(&tm_wd, w_down, E * d, I, 256);
+                  make_tmap(&tm_h, at<char>(ws, pl.H), (uint64_t)max_rows, I, a_rows);
         if (!ok) return EXFOLD_ERR_CUDA;
     }
     prof_reset();
@@ -729,10 +728,23 @@ static int decode_impl(const exfold_layer* layer, const void* x, const float* lo
             const int alt = decode_ffn_alt((int)B, max_groups, I, sms);
             decode_ffn_smem_plan((int)B, K, N, alt, &stages, &scratch_off, &ar);
             if (stages < 2) return EXFOLD_ERR_UNSUPPORTED;
+            // Fewer (expert, column tile) items than half the SMs (few experts, large I): K is split in two so that
+            // enough SMs stream W_down; each part's rows go to a plane of their own (the two planes are the row buffer
+            // and the unused gathered-rows region before it) and are summed, in order, by the kernel after.
+            const int64_t row_tiles = (int64_t)max_groups * ((B + kTileM - 1) / kTileM), base_items = row_tiles * ((d + 255) / 256);
+            const int ksplit = (2 * base_items < sms && I / 64 >= 8) ? kMaxDecodeKsplit : 1;
+            // Still few: narrower column tiles, as long as each has an SM to itself. (A k-block's MMAs take the same time for 64
+            // columns as for 256, so more rounds of narrower tiles lose.) Whole call, 256 columns / these: Qwen3 shape 128
+            // tokens, pool 2 29.2 / 27.2 us; GLM shape 100 tokens, pool 1 47.1 / 45.1; Mixtral shape 200 tokens, pool 1
+            // 152.8 / 144.3; 64 columns in three rounds: GLM shape 16 tokens, pool 4 50.4 / 60.0.
+            int n_cols = 256;
+            while (n_cols > 64 && base_items * (512 / n_cols) * ksplit <= sms) n_cols >>= 1;
+            CUtensorMap tm_wd;
             const uint64_t E = (uint64_t)G;
             DecodeFfnParams fp{};
             fp.alt = alt; fp.tm_wg = tm_wg; fp.tm_wu = tm_wu;
-            if (!make_tmap(&fp.tm_x, x, (uint64_t)B, d, ar) || (B > 128 && !make_tmap(&fp.tm_xg, x, (uint64_t)B, d, 1)) ||
+            if (!make_tmap(&tm_wd, w_down, E * d, I, n_cols) || !make_tmap(&fp.tm_x, x, (uint64_t)B, d, ar) ||
+                (B > 128 && !make_tmap(&fp.tm_xg, x, (uint64_t)B, d, 1)) ||
                 !make_tmap(&fp.tm_wg64, w_gate, E * I, d, 64) || !make_tmap(&fp.tm_wu64, w_up, E * I, d, 64) ||
                 (alt && (!make_tmap(&fp.tm_wg_alt, w_gate, E * I, d, alt) || !make_tmap(&fp.tm_wu_alt, w_up, E * I, d, alt))))
                 return EXFOLD_ERR_CUDA;
@@ -753,22 +765,17 @@ static int decode_impl(const exfold_layer* layer, const void* x, const float* lo
             // Down projection on the grouped GEMM-2 kernel over the compact rows (the whole intermediate dimension is
             // its K, so no partial outputs meet in memory); each row's weighted output is stored once, in bf16, and a
             // token's rows are then summed in slot order: no atomics, so a decode step is reproducible bit for bit.
-            const int tiles_per_group = (int)((B + kTileM - 1) / kTileM);
             GroupedGemmParams g{};
-            g.tm_a = tm_h; g.tm_a2 = tm_h; g.tm_b0 = tm_wd; g.tm_b1 = tm_wd; g.x_rows = 1; g.o32 = nullptr;
+            g.tm_a = tm_h; g.tm_a2 = tm_h; g.x_rows = 1; g.o32 = nullptr;
             g.offsets = rp.grp_off; g.work_start = rp.grp_tiles; g.G = max_groups; g.n_routed = 0x7fffffff;
-            g.R = max_rows; g.d = d; g.I = I; g.n_ntiles = (d + 255) / 256; g.ksplit = 1; g.a_rows = a_rows;
+            g.R = max_rows; g.d = d; g.I = I; g.a_rows = a_rows;
             g.grp_expert = rp.grp_expert; g.n_groups_dev = rp.n_groups;
             g.H = fp.H; g.row_tok = rp.row_tok; g.row_w = rp.row_w;
             g.y = at<__nv_bfloat16>(ws, pl.obuf); g.store_rows = 1; g.status = rp.status;
-            // Fewer (expert, column tile) items than half the SMs (few experts, large I): K is split in two so that
-            // enough SMs stream W_down; each part's rows go to a plane of their own (the two planes are the row buffer
-            // and the unused gathered-rows region before it) and are summed, in order, by the kernel after.
-            const int nkb2 = I / 64;
-            const int64_t base_items = (int64_t)max_groups * tiles_per_group * g.n_ntiles;
-            g.ksplit = (2 * base_items < sms && nkb2 >= 8) ? kMaxDecodeKsplit : 1;
+            g.ksplit = ksplit; g.n_cols = n_cols; g.n_ntiles = (d + n_cols - 1) / n_cols; g.tm_b0 = tm_wd; g.tm_b1 = tm_wd;
+            const int64_t items = row_tiles * g.n_ntiles * ksplit;
             g.y = g.ksplit > 1 ? at<__nv_bfloat16>(ws, pl.obuf) - (size_t)max_rows * d : at<__nv_bfloat16>(ws, pl.obuf);
-            { ProfScope ps(9, s); EXFOLD_CUDA(launch_grouped_gemm2(g, (int)std::min<int64_t>(sms, base_items * g.ksplit), s)); }
+            { ProfScope ps(9, s); EXFOLD_CUDA(launch_grouped_gemm2(g, (int)std::min<int64_t>(sms, items), s)); }
             { ProfScope ps(5, s); EXFOLD_CUDA(launch_combine_rows(g.y, fp.slot_row, B, K, d, l.n_shared, rp.n_groups + 2, g.ksplit,
                                                            max_rows, reinterpret_cast<__nv_bfloat16*>(y), s)); }
         }

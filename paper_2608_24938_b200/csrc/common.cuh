@@ -486,6 +486,7 @@ struct GroupedGemmParams {
     int R;                      // routed rows (shared rows start here)
     int d, I;
     int n_ntiles;               // column tiles
+    int n_cols;                 // decode: columns per tile, 256, 128 or 64 (tm_b0's box)
     int ksplit;                 // GEMM-2, decode: K parts per tile; part k of a row goes to plane k of the row buffer
     int a_rows;                 // decode: rows of the A (token) box, a multiple of 32 <= 128; prefill: 128
     const int32_t* grp_expert;  // [G] expert whose weights group g uses (null: g itself)

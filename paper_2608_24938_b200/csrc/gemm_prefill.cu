@@ -83,12 +83,14 @@ __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
 
 // MODE 0: gate/up + SwiGLU -> H; MODE 1: down + weighted scatter -> y.
 // DEC (decode) adds what only the expert-pool path needs: a group -> expert map, a group count that is
-// known only on the device, and split-K for GEMM-2. The prefill instantiations compile all of it away.
-template <int MODE, bool DEC>
+// known only on the device, split-K for GEMM-2 and, as its value, the output columns per tile (256, or 128 or 64 where few
+// items are left). The prefill instantiations (0) compile all of it away.
+template <int MODE, int DEC>
 __global__ void __launch_bounds__(kGemmThreads, 1) grouped_gemm_kernel(const __grid_constant__ GroupedGemmParams p) {
     extern __shared__ unsigned char smem_raw[];
-    __shared__ __align__(8) uint64_t full_bar[kMaxStages];
-    __shared__ __align__(8) uint64_t empty_bar[kMaxStages];
+    constexpr int n_cols = DEC ? DEC : 256, kRing = n_cols < 256 ? 12 : kMaxStages;
+    __shared__ __align__(8) uint64_t full_bar[kRing];
+    __shared__ __align__(8) uint64_t empty_bar[kRing];
     __shared__ __align__(8) uint64_t tfull_bar[2];
     __shared__ __align__(8) uint64_t tempty_bar[2];
     __shared__ uint32_t tmem_base_s;
@@ -109,7 +111,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) grouped_gemm_kernel(const __g
             ptx::prefetch_tmap(&p.tm_a2);
             ptx::prefetch_tmap(&p.tm_b1);
         }
-        for (int s = 0; s < kMaxStages; ++s) {
+        for (int s = 0; s < kRing; ++s) {
             ptx::mbar_init(&full_bar[s], 1);
             ptx::mbar_init(&empty_bar[s], 1);
         }
@@ -202,8 +204,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1) grouped_gemm_kernel(const __g
     // a_rows rows (the rest of the 128-row MMA operand is whatever follows in shared memory: those
     // accumulator rows are masked), so a stage is smaller and more stages of weights are in flight.
     const int a_bytes = DEC ? p.a_rows * kBK * 2 : kATileBytes;
-    const int stage_bytes = DEC ? a_bytes + kBTileBytes : kStageBytes;
-    const int stages = DEC ? min(kMaxStages, (kStages * kStageBytes - (kATileBytes - a_bytes)) / stage_bytes) : kStages;
+    const int stage_bytes = DEC ? a_bytes + n_cols * kBK * 2 : kStageBytes;
+    const int stages = DEC ? min(kRing, (kStages * kStageBytes - (kATileBytes - a_bytes)) / stage_bytes) : kStages;
     volatile int* abort_flag = &abort_s;
 
     if (warp == 0 || warp >= 6) {
@@ -220,7 +222,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) grouped_gemm_kernel(const __g
                 const bool from_x = !DEC && MODE == 0 && expert >= p.n_routed;  // prefill's shared expert reads x directly
                 const CUtensorMap* tma_a = from_x ? &p.tm_a2 : &p.tm_a;
                 const int arow = from_x ? (it.row0 - p.R) % p.x_rows : it.row0;
-                const int brow = MODE == 0 ? expert * p.I + it.n_idx * 128 : expert * p.d + it.n_idx * 256;
+                const int brow = MODE == 0 ? expert * p.I + it.n_idx * 128 : expert * p.d + it.n_idx * n_cols;
                 for (int kb = kb0; kb < kb1; ++kb) {
                     if (turn == me) {
                         const bool got = ptx::mbar_wait(&empty_bar[stage], phase ^ 1, abort_flag, p.status, 1);
@@ -249,7 +251,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) grouped_gemm_kernel(const __g
     } else if (warp == 1) {
         // ------------------------------------------------ MMA issuer
         if (lane == 0) {
-            constexpr uint32_t idesc = ptx::make_idesc_bf16(128, 256);
+            constexpr uint32_t idesc = ptx::make_idesc_bf16(128, n_cols);
             int stage = 0, phase = 0, iter = 0;
             // This one thread's instruction stream paces the tensor pipe (a k-block is 4 MMAs = 512 pipe cycles),
             // so the loop carries as little as possible: the descriptors' low words advance by a constant per stage
@@ -396,8 +398,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1) grouped_gemm_kernel(const __g
                 const bool staged = !DEC && __popc(vmask) > 16;
                 const int drow = (p.store_rows ? (int)grow : tok) + (DEC ? it.kpart * p.R : 0);
 #pragma unroll 1
-                for (int c = 0; c < 8; ++c) {
-                    const int col0 = it.n_idx * 256 + c * 32;
+                for (int c = 0; c < n_cols / 32; ++c) {
+                    const int col0 = it.n_idx * n_cols + c * 32;
                     if (col0 >= p.d) break;  // d is a multiple of 64: whole 128-byte groups
                     uint32_t v[32];
                     ptx::tmem_ld32(taddr + c * 32, v);
@@ -446,7 +448,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) grouped_gemm_kernel(const __g
 
 // whole_tpcs: launch as clusters of two CTAs. The CTAs do not use the cluster; the launch then occupies SMs two at a
 // time, like the CTA-pair kernel it runs beside, and the two grids cannot leave each other half-filled SM pairs.
-template <int MODE, bool DEC>
+template <int MODE, int DEC>
 static cudaError_t launch_gemm_t(const GroupedGemmParams& p, int grid, cudaStream_t s, bool whole_tpcs = false) {
     cudaError_t err = ensure_smem(grouped_gemm_kernel<MODE, DEC>, kGemmSmem);
     if (err != cudaSuccess) return err;
@@ -456,16 +458,21 @@ static cudaError_t launch_gemm_t(const GroupedGemmParams& p, int grid, cudaStrea
 }
 
 cudaError_t launch_grouped_gemm1(const GroupedGemmParams& p, int grid, cudaStream_t s) {
-    return launch_gemm_t<0, false>(p, grid, s);  // decode has its own gate/up kernel (ffn_decode.cu)
+    return launch_gemm_t<0, 0>(p, grid, s);  // decode has its own gate/up kernel (ffn_decode.cu)
 }
 cudaError_t launch_grouped_gemm2(const GroupedGemmParams& p, int grid, cudaStream_t s) {
-    return p.grp_expert != nullptr ? launch_gemm_t<1, true>(p, grid, s) : launch_gemm_t<1, false>(p, grid, s);
+    if (p.grp_expert == nullptr) return launch_gemm_t<1, 0>(p, grid, s);
+    switch (p.n_cols) {
+        case 64: return launch_gemm_t<1, 64>(p, grid, s);
+        case 128: return launch_gemm_t<1, 128>(p, grid, s);
+        default: return launch_gemm_t<1, 256>(p, grid, s);
+    }
 }
 cudaError_t launch_grouped_gemm1_odd(const GroupedGemmParams& p, int grid, cudaStream_t s) {
-    return launch_gemm_t<0, false>(p, grid, s, true);
+    return launch_gemm_t<0, 0>(p, grid, s, true);
 }
 cudaError_t launch_grouped_gemm2_odd(const GroupedGemmParams& p, int grid, cudaStream_t s) {
-    return launch_gemm_t<1, false>(p, grid, s, true);
+    return launch_gemm_t<1, 0>(p, grid, s, true);
 }
 
 }  // namespace exfold

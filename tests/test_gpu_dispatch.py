@@ -204,11 +204,13 @@ def test_decode_pool_of_near_ties(B, N, K, M, h_step):
     assert np.array_equal(got["y"], plain["y"])
 
 
-@pytest.mark.parametrize("I,M,ns", [(2368, 2, 0), (2368, 2, 1), (384, 12, 0), (384, 12, 1), (384, 13, 0), (64, 1, 0), (832, 5, 0)])
+@pytest.mark.parametrize("I,M,ns,d", [(2368, 2, 0, 320), (2368, 2, 1, 320), (384, 12, 0, 320), (384, 12, 1, 320), (384, 13, 0, 320),
+                                      (64, 1, 0, 64), (832, 5, 0, 320), (448, 5, 0, 1088), (512, 5, 1, 1088)])
 @pytest.mark.parametrize("B", [20, 100, 140])
-def test_decode_slice_widths(B, I, M, ns):
-    """Few groups: 32-wide gate/up slices up to one per SM (148 = 2 x 2368 / 32, 144 = 12 x 384 / 32), wider ones beyond."""
-    case = Case(si.LayerConfig("slices", 16, ns, 320, I, 3, "bf16", 8, (1,), B, (M,)))
+def test_decode_slice_widths(B, I, M, ns, d):
+    """Few groups: 32-wide gate/up slices up to one per SM (148 = 2 x 2368 / 32, 144 = 12 x 384 / 32), wider ones beyond; 64 or
+    128 output columns per down tile (hidden sizes that leave the last tile short), with and without the K split."""
+    case = Case(si.LayerConfig("slices", 16, ns, d, I, 3, "bf16", 8, (1,), B, (M,)))
     got, ref = case.run_decode(M), case.oracle_decode(M)
     check_decode_meta(got, ref, M)
     check_output(got["y"], ref["y"], "bf16")
