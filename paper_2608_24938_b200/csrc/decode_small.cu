@@ -263,11 +263,13 @@ __global__ void __launch_bounds__(kThreads, 2) decode_small_gateup_kernel(Decode
 
     if (!GIVEN && !is_static) {
         // Eq. 12 for the batch's experts outside the pool (all experts for the metadata): a warp per source, loss and
-        // scalar of every candidate in one round trip, two sources at a time
+        // scalar of every candidate in one round trip, two sources at a time. A NaN loss is never smaller, but the
+        // best-ranked expert's is where the search starts and stays.
         const int n_src = meta ? N : (U > P ? U : 0);
         for (int i0 = warp; i0 < n_src; i0 += 2 * kWarps) {
             int s2[2], bj[2];
             float bl[2], bs[2];
+            unsigned nan = 0;
 #pragma unroll
             for (int u = 0; u < 2; ++u) {
                 const int i = i0 + u * kWarps;
@@ -280,7 +282,8 @@ __global__ void __launch_bounds__(kThreads, 2) decode_small_gateup_kernel(Decode
                     for (int j = lane; j < P; j += 32) {
                         const int t = sc.grp[j];
                         const float l = __ldg(p.L + (size_t)s2[u] * N + t), sv = __ldg(p.S + (size_t)s2[u] * N + t);
-                        if (bj[u] == 0x7fffffff || l < bl[u] || (l == bl[u] && t < bj[u])) {
+                        nan |= isnan(l) ? 1u << u : 0u;
+                        if (l < bl[u] || (l == bl[u] && t < bj[u])) {
                             bl[u] = l;
                             bs[u] = sv;
                             bj[u] = t;
@@ -290,9 +293,18 @@ __global__ void __launch_bounds__(kThreads, 2) decode_small_gateup_kernel(Decode
 #pragma unroll
             for (int u = 0; u < 2; ++u) {
                 if (s2[u] < 0) continue;  // warp-uniform
-                const int bt = warp_argmin(bj[u] != 0x7fffffff, float_order_key(bl[u]), bj[u]);
+                int bt = warp_argmin(bj[u] != 0x7fffffff, float_order_key(bl[u]), bj[u]);
                 const unsigned who = __ballot_sync(0xffffffffu, bj[u] == bt);
-                const float scl = __shfl_sync(0xffffffffu, bs[u], __ffs(who) - 1);
+                float scl = __shfl_sync(0xffffffffu, bs[u], __ffs(who) - 1);
+                if (__any_sync(0xffffffffu, (nan >> u) & 1u)) {
+                    int first = 0;
+                    while (sc.rank[first] != 0) ++first;
+                    first = sc.member[first];
+                    if (isnan(__ldg(p.L + (size_t)s2[u] * N + first))) {
+                        bt = first;
+                        scl = __ldg(p.S + (size_t)s2[u] * N + first);
+                    }
+                }
                 if (lane == 0) {
                     sc.target[s2[u]] = bt;
                     sc.scale[s2[u]] = scl;
