@@ -396,7 +396,8 @@ __global__ void __launch_bounds__(kFThreads, 1) decode_ffn_kernel(const __grid_c
         const bool meta = p.pool_ids != nullptr && blockIdx.x == 0;  // the caller asked for the routing metadata
         if (!is_static) {
             // Eq. 12: a source in the pool keeps itself; any other takes its minimum-loss pool expert (ties -> lower
-            // id). Eight lanes per source, loss and scalar of 64 candidates in one round trip (a thread per source with
+            // id; a NaN loss is never smaller, but the best-ranked expert's is where the search starts and stays).
+            // Eight lanes per source, loss and scalar of 64 candidates in one round trip (a thread per source with
             // its candidates one after the other took 8 us for a pool of 64). Only sources that occur in the batch
             // matter for the execution; the metadata has the whole table.
             for (int j = tid; j < P; j += nth) {
@@ -408,7 +409,7 @@ __global__ void __launch_bounds__(kFThreads, 1) decode_ffn_kernel(const __grid_c
             for (int i0 = 0; i0 < n_src; i0 += n_grp) {
                 const int i = i0 + (tid >> 3);
                 const int s = i < n_src ? (meta ? i : src[i]) : -1;
-                float bl = INFINITY, bs = 1.0f;
+                float bl = INFINITY, bs = 1.0f, l_first = 0.f, s_first = 1.0f;
                 int bt = 0x7fffffff;
                 if (s >= 0 && sc.rank_of[s] < 0) {
                     for (int j0 = sub; j0 < P; j0 += 64) {
@@ -419,6 +420,10 @@ __global__ void __launch_bounds__(kFThreads, 1) decode_ffn_kernel(const __grid_c
                             tt[u] = j0 + 8 * u < P ? sc.pool[j0 + 8 * u] : -1;
                             l[u] = tt[u] >= 0 ? __ldg(p.L + (size_t)s * N + tt[u]) : 0.f;
                             sv[u] = tt[u] >= 0 ? __ldg(p.S + (size_t)s * N + tt[u]) : 0.f;
+                        }
+                        if (j0 == 0) {
+                            l_first = l[0];
+                            s_first = sv[0];
                         }
 #pragma unroll
                         for (int u = 0; u < 8; ++u)
@@ -442,8 +447,9 @@ __global__ void __launch_bounds__(kFThreads, 1) decode_ffn_kernel(const __grid_c
                     }
                 }
                 if (s >= 0 && sub == 0) {
-                    sc.target[s] = bt;
-                    sc.scale[s] = bs;
+                    const bool stays = isnan(l_first);
+                    sc.target[s] = stays ? sc.pool[0] : bt;
+                    sc.scale[s] = stays ? s_first : bs;
                 }
             }
             sync_group();

@@ -9,7 +9,7 @@ from harness import Case, check_decode_meta, check_output
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("B", [3, 8])
+@pytest.mark.parametrize("B", [3, 8, 20, 140])
 @pytest.mark.parametrize("N,M", [(16, 1), (40, 3), (40, 12), (200, 70)])
 def test_decode_targets_of_nan_losses(B, N, M):
     """Eq. 12 over losses of which a third are NaN or infinite, some sources' all: a NaN is never smaller, and one at the
