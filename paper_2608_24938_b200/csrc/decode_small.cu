@@ -457,15 +457,12 @@ __global__ void __launch_bounds__(32 * kMaxDownWarps, 1) decode_small_down_kerne
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ float4 s_red[kMaxDownWarps][32];
     const int B = p.B, d = p.d, I = p.I, split = p.split;
-    int* s_row = reinterpret_cast<int*>(smem);                          // [max_groups][8] compact row, -1: not served
-    float* s_w = reinterpret_cast<float*>(s_row + p.max_groups * kTB);  // [max_groups][8] weight
-    int* s_exp = reinterpret_cast<int*>(s_w + p.max_groups * kTB);      // [max_groups]
+    // [max_groups][8 / 2]: compact rows of two tokens (-1: not served) in .x and .y, their weights in .z and .w
+    int4* s_rw = reinterpret_cast<int4*>(smem);
+    int* s_exp = reinterpret_cast<int*>(s_rw + p.max_groups * (kTB / 2));  // [max_groups]
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, n_thr = (int)blockDim.x, n_warps = n_thr >> 5;
     const int part = (int)blockIdx.x % split, c0 = (int)blockIdx.x / split * 16;
-    for (int i = tid; i < p.max_groups * kTB; i += n_thr) {
-        s_row[i] = -1;
-        s_w[i] = 0.f;
-    }
+    for (int i = tid; i < p.max_groups * (kTB / 2); i += n_thr) s_rw[i] = make_int4(-1, -1, 0, 0);
     __syncthreads();
     grid_dep_wait();
     const int G = p.n_groups[0], rows = p.n_groups[1];
@@ -473,8 +470,9 @@ __global__ void __launch_bounds__(32 * kMaxDownWarps, 1) decode_small_down_kerne
         const int t = p.row_tok[r], g = p.row_grp[r];
         const float w = p.row_w[r];
         if (r < rows) {
-            s_row[g * kTB + t] = r;
-            s_w[g * kTB + t] = w;
+            int* at = reinterpret_cast<int*>(s_rw + g * (kTB / 2) + (t >> 1)) + (t & 1);
+            at[0] = r;
+            at[2] = __float_as_int(w);
         }
     }
     for (int g = tid; g < p.max_groups; g += n_thr) {
@@ -495,7 +493,7 @@ __global__ void __launch_bounds__(32 * kMaxDownWarps, 1) decode_small_down_kerne
             const __nv_bfloat16* w = p.wd + ((size_t)s_exp[g] * d + c0 + lr) * I + kc;
             ld_stream(an[u][0], w);
             ld_stream(an[u][1], w + (size_t)8 * I);
-            const int row = s_row[g * kTB + lr];
+            const int row = reinterpret_cast<const int*>(s_rw + g * (kTB / 2) + (lr >> 1))[lr & 1];
             if (row >= 0) ld_rows(hn[u], p.H + (size_t)row * I + kc);
             else zero8(hn[u]);
         }
@@ -518,11 +516,15 @@ __global__ void __launch_bounds__(32 * kMaxDownWarps, 1) decode_small_down_kerne
             if (j >= nch) break;  // warp-uniform
             float c[4] = {0.f, 0.f, 0.f, 0.f};
             mma_chunk(c, a[u][0], a[u][1], hb[u]);
-            const float2 w = *reinterpret_cast<const float2*>(s_w + j / per * kTB + (lane & 3) * 2);
-            acc[0] = fmaf(w.x, c[0], acc[0]);
-            acc[1] = fmaf(w.y, c[1], acc[1]);
-            acc[2] = fmaf(w.x, c[2], acc[2]);
-            acc[3] = fmaf(w.y, c[3], acc[3]);
+            const int4 rw = s_rw[j / per * (kTB / 2) + (lane & 3)];
+            if (rw.x >= 0) {  // not for a token that the group does not serve: its zeros make NaN of infinite weights
+                acc[0] = fmaf(__int_as_float(rw.z), c[0], acc[0]);
+                acc[2] = fmaf(__int_as_float(rw.z), c[2], acc[2]);
+            }
+            if (rw.y >= 0) {
+                acc[1] = fmaf(__int_as_float(rw.w), c[1], acc[1]);
+                acc[3] = fmaf(__int_as_float(rw.w), c[3], acc[3]);
+            }
         }
     }
     s_red[warp][lane] = make_float4(acc[0], acc[1], acc[2], acc[3]);

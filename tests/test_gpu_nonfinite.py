@@ -28,3 +28,39 @@ def test_decode_targets_of_nan_losses(B, N, M):
     check_output(got["y"], ref["y"], "bf16")
     plain = case.run_decode(M, with_meta=False)  # without metadata only the batch's experts get targets
     assert np.array_equal(got["y"], plain["y"])
+
+
+@pytest.mark.parametrize("T", [1, 2, 5, 8, 9, 40, 130])
+@pytest.mark.parametrize("dtype,ns", [("bf16", 0), ("bf16", 1), ("f32", 0)])
+@pytest.mark.parametrize("bad", [float("inf"), float("nan")])
+def test_a_broken_expert_touches_its_own_tokens_only(T, dtype, ns, bad):
+    """One non-finite weight in one expert: the outputs of tokens that are not routed to it keep their bits, those of its
+    own tokens are not finite. Prefill, decode with the dynamic and the static pool; gate, up and down weights in turn."""
+    N, K, d, I = 12, 2, 192, 320
+    case = Case(si.LayerConfig("broken", N, ns, d, I, K, dtype, T, (K,), T, (N,)))
+    ex, dev = case.ex, case.dev
+    for lg in (case.lg, case.lgd):  # expert 3 serves every third token, the first among them
+        lg[:, 3] = torch.where(torch.arange(T) % 3 == 0, 9.0, -9.0)
+    case.d_lg, case.d_lgd = case.lg.to(dev), case.lgd.to(dev)
+    case.d_x, case.d_xd = case.d_x.abs() + 0.5, case.d_xd.abs() + 0.5  # no zero meets the bad weight
+    pool = [torch.empty(N, dtype=torch.int32, device=dev), torch.empty(N, dtype=torch.int32, device=dev), torch.empty(N, device=dev)]
+    sp = ex.exfold_static_pool_build(case.layer, case.tables, N, *pool)
+
+    def static():
+        y = torch.full((T, d), float("nan"), dtype=case.d_wg.dtype, device=dev)
+        ws = case.workspace(T, K)
+        ex.exfold_moe_decode_static(case.layer, case.d_xd, case.d_lgd, case.d_wg, case.d_wu, case.d_wd, sp, y, ws)
+        return y.float().cpu().numpy()
+
+    runs = [lambda: case.run_prefill(K, with_meta=False)["y"], lambda: case.run_decode(N, with_meta=False)["y"], static]
+    clean = [run() for run in runs]
+    mine = np.arange(T) % 3 == 0
+    for w in (case.d_wg, case.d_wu, case.d_wd):
+        keep = w[3, 5, 7].clone()
+        w[3, 5, 7] = bad
+        for run, want in zip(runs, clean):
+            got = run()
+            assert np.array_equal(got[~mine], want[~mine])
+            if bad != bad or w is not case.d_wg:  # (an infinite gate may be silu(-inf) = 0 or x - inf)
+                assert not np.isfinite(got[mine]).all(axis=1).any()
+        w[3, 5, 7] = keep
