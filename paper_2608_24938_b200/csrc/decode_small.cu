@@ -136,7 +136,6 @@ __global__ void __launch_bounds__(kThreads, 2) decode_small_gateup_kernel(Decode
     const bool is_static = !GIVEN && p.st_pool != nullptr;
     // the CTA with the fewest work items writes the metadata and the lists
     const bool scribe = blockIdx.x == gridDim.x - 1, meta = !GIVEN && p.pool_ids != nullptr && scribe;
-    const float h_e = !GIVEN && !is_static && tid < N ? __ldg(p.h + tid) : 0.f;  // the tables do not depend on earlier kernels
     sc.acc32[3 * tid] = sc.acc32[3 * tid + 1] = sc.acc32[3 * tid + 2] = 0u;
     sc.in_union[tid] = 0;
     sc.grp_of[tid] = -1;
@@ -151,6 +150,8 @@ __global__ void __launch_bounds__(kThreads, 2) decode_small_gateup_kernel(Decode
 #pragma unroll
         for (int q = 0; q < 8; ++q) v[q] = lane + 32 * q < N ? p.logits[(size_t)warp * N + lane + 32 * q] : -INFINITY;
     }
+    // not before the wait: the caller may have written the table on this stream right before the call
+    const float h_e = !GIVEN && !is_static && tid < N ? __ldg(p.h + tid) : 0.f;
     for (int t = 0; t < B; ++t)  // lands while the routing below runs
         for (int c = tid * 8; c < d; c += kThreads * 8) cp_async16(xs + t * xld + c, p.x + (size_t)t * d + c);
     asm volatile("cp.async.commit_group;" ::: "memory");

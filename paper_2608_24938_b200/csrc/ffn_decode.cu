@@ -76,7 +76,6 @@ struct Scratch {  // per-batch routing state, one copy per CTA
     int pool[kMaxExperts];     // pool experts by rank
     int target[kMaxExperts];
     float scale[kMaxExperts];
-    float h[kMaxExperts];      // norm table (dynamic pool), staged before the dependency wait
     int goff[kFMaxPairs + 2];  // exclusive prefix over (group, token tile): first compact row
     int pairs[kFMaxPairs];     // the work list's rows: group * 4 + token tile, or + kGather (before that: the union's experts)
     int P, U, n_pairs;
@@ -239,8 +238,8 @@ __global__ void __launch_bounds__(kFThreads, 1) decode_ffn_kernel(const __grid_c
     }
     const int W = nmt * 4;  // mask words per group
     for (int i = threadIdx.x; i < (N + 1) * W; i += kFThreads) tmask[i] = 0u;
-    if (!is_static) {  // the norm table into shared memory, the loss and scalar tables into L2, while the previous kernel runs
-        for (int e = threadIdx.x; e < N; e += kFThreads) sc.h[e] = __ldg(p.h + e);
+    if (!is_static) {  // the tables into L2 while the previous kernel runs (only a hint: they are read after the wait)
+        if (warp == 5 && lane * 32 < N) ptx::prefetch_l2(p.h + lane * 32);
         const size_t n_el = (size_t)N * N, lines = (n_el * 4 + 127) / 128;
         for (size_t i = (size_t)blockIdx.x * kFThreads + threadIdx.x; i < lines; i += (size_t)gridDim.x * kFThreads) {
             const size_t el = i * 32 < n_el ? i * 32 : n_el - 1;
@@ -265,6 +264,15 @@ __global__ void __launch_bounds__(kFThreads, 1) decode_ffn_kernel(const __grid_c
         atomicAdd(&sc.acc32[3 * id + 2], (unsigned)(fx >> 42));
         sc.in_union[id] = 1;
     };
+    // The norms that this thread scores below, in the slots' round trip. Not before the wait: the caller may have written
+    // the table on this stream right before the call.
+    static_assert(kMaxExperts <= 2 * kFThreads, "two norms per thread");
+    float h_e[2];
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+        const int e = threadIdx.x + u * kFThreads;
+        h_e[u] = !is_static && e < N ? __ldg(p.h + e) : 0.f;
+    }
     const int BK4 = BK >> 2;
     for (int s0 = threadIdx.x; s0 < BK4; s0 += kFThreads * 3) {
         int4 id[3];
@@ -328,7 +336,7 @@ __global__ void __launch_bounds__(kFThreads, 1) decode_ffn_kernel(const __grid_c
                 const unsigned long long acc = (unsigned long long)sc.acc32[3 * e] +
                                                ((unsigned long long)sc.acc32[3 * e + 1] << 21) +
                                                ((unsigned long long)sc.acc32[3 * e + 2] << 42);
-                const double score = (double)acc * (1.0 / 9007199254740992.0) * (double)sc.h[e] + 0.0;
+                const double score = (double)acc * (1.0 / 9007199254740992.0) * (double)(c < kFThreads / 32 ? h_e[0] : h_e[1]) + 0.0;
                 long long key = __double_as_longlong(score);
                 if (key < 0) key ^= 0x7FFFFFFFFFFFFFFFll;  // negative doubles: larger magnitude = smaller
                 member[pos] = e;
