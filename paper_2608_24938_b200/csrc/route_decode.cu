@@ -365,6 +365,7 @@ __global__ void __launch_bounds__(256) decode_topk_kernel(DecodeTopkParams p) {
     const int N = p.N, K = p.K, d = p.d;
     const int i0 = (ROUTER ? (int)blockIdx.x / kTopkCluster : (int)blockIdx.x) * TT;
     grid_dep_launch();
+    if (ROUTER) cg::this_cluster().barrier_arrive();  // waited for before the first remote write: the first CTA has started
     grid_dep_wait();  // x may be the previous layer's output; the workspace may still be read by the previous call
     if (blockIdx.x == 0 && threadIdx.x < 4) reinterpret_cast<int*>(p.status)[threadIdx.x] = 0;
     if (ROUTER) {
@@ -379,6 +380,7 @@ __global__ void __launch_bounds__(256) decode_topk_kernel(DecodeTopkParams p) {
         const __nv_bfloat16* xi[TW];
 #pragma unroll
         for (int t = 0; t < TW; ++t) xi[t] = p.x + (size_t)min(i0 + t0 + t, p.B - 1) * d;
+        bool started = false;
         for (int e0 = e_lo + warp % kExpGroups * EW; e0 < e_hi; e0 += kExpGroups * EW) {
             const __nv_bfloat16* we[EW];
 #pragma unroll
@@ -411,6 +413,10 @@ __global__ void __launch_bounds__(256) decode_topk_kernel(DecodeTopkParams p) {
                     }
                 }
             }
+            if (!started) {  // warp-uniform
+                cluster.barrier_wait();
+                started = true;
+            }
 #pragma unroll
             for (int u = 0; u < EW; ++u)
 #pragma unroll
@@ -425,6 +431,7 @@ __global__ void __launch_bounds__(256) decode_topk_kernel(DecodeTopkParams p) {
                     }
                 }
         }
+        if (!started) cluster.barrier_wait();  // warps without an expert
         cluster.sync();  // every score of the tokens is in the first CTA's shared memory
         if (rank != 0) return;
     }

@@ -153,6 +153,32 @@ def test_decode_router_scores_by_batch(B, N):
     check_output(y.float().cpu().numpy(), ref["y"], "bf16")
 
 
+@pytest.mark.parametrize("B", [1, 9, 80, 81, 128, 129, 256])
+@pytest.mark.parametrize("N", [5, 40, 256])
+def test_decode_router_scores_of_short_rows(B, N):
+    """Rows of 64: the shortest dot products, whose scores the cluster's CTAs write to the first one soonest after its
+    start; CTAs and warps without experts. Against double sums (the bound of test_router_scores_by_prompt_length), the
+    call on them against the oracle, the same bits every time."""
+    d, K = 64, 4
+    case = Case(si.LayerConfig("short", N, 0, d, 64, K, "bf16", 8, (1,), B, (3,)))
+    ex, dev = case.ex, case.dev
+    wr = si.router_weights(case.cfg).to(dev)
+    x64, w64 = case.d_xd.double(), wr.double()
+    want, bound = x64 @ w64.T, d * 2.0 ** -23 * (x64.abs() @ w64.abs().T)
+    y, first = torch.empty((B, d), dtype=torch.bfloat16, device=dev), None
+    ws = case.workspace(B, K)
+    for _ in range(20):
+        lg = torch.full((B, N), float("nan"), device=dev)
+        ex.exfold_moe_decode_layer(case.layer, case.d_xd, wr, case.d_wg, case.d_wu, case.d_wd, case.tables, 3, y, ws, lg)
+        got = (lg, y.clone())
+        first = first or got
+        assert torch.equal(got[0], first[0]) and torch.equal(got[1], first[1])
+    assert ex.exfold_device_status(ws) == 0
+    assert bool(((first[0].double() - want).abs() <= bound).all())
+    case.lgd, case.d_lgd = first[0].cpu(), first[0]
+    check_output(first[1].float().cpu().numpy(), case.oracle_decode(3)["y"], "bf16")
+
+
 @pytest.mark.parametrize("rows,ns,d,I", [
     ([1, 3, 4, 5, 63, 64, 65, 51], 0, 256, 384),     # 256 tokens: gathered up to 64 rows, dense above
     ([64, 65], 1, 64, 64),                           # 129 tokens, one K chunk, half-width items, the shared expert dense
