@@ -833,11 +833,10 @@ int exfold_static_pool_build(const exfold_layer* layer, const exfold_tables* tab
     return EXFOLD_OK;
 }
 
-// Enqueues one calibration on the stream (no synchronisation); the number of unobserved experts lands in result_words()[job]
-// when the stream gets there.
-static int calibrate_enqueue(const exfold_layer* layer, const void* x_cal, const float* logits_cal, int64_t m,
-                             const void* w_gate, const void* w_up, const void* w_down, const exfold_calib_opts* opts,
-                             exfold_tables* out, void* ws, size_t ws_bytes, void* cuda_stream, int job) {
+// The arguments of one calibration, before anything is launched. m * Ke <= 2^30 rows follow from m <= 2^22, Ke <= 256.
+static int calibrate_check(const exfold_layer* layer, const void* x_cal, const float* logits_cal, int64_t m,
+                           const void* w_gate, const void* w_up, const void* w_down, const exfold_calib_opts* opts,
+                           const exfold_tables* out, const void* ws, size_t ws_bytes) {
     if (!valid_layer(layer) || !x_cal || !w_gate || !w_up || !w_down || !opts || !out || !ws)
         return EXFOLD_ERR_INVALID_ARG;
     if (!out->S || !out->L || !out->h || !out->lnh) return EXFOLD_ERR_INVALID_ARG;
@@ -845,13 +844,25 @@ static int calibrate_enqueue(const exfold_layer* layer, const void* x_cal, const
     if (opts->mode != 0 && opts->mode != 1) return EXFOLD_ERR_INVALID_ARG;
     if (opts->mode == 0 && !logits_cal) return EXFOLD_ERR_INVALID_ARG;
     if ((reinterpret_cast<uintptr_t>(ws) & 255) != 0) return EXFOLD_ERR_INVALID_ARG;
+    exfold_layer lc = *layer;
+    lc.n_shared = 0;  // the shared expert is never folded, so it is not calibrated
+    if (ws_bytes < make_plan(lc, m, opts->mode == 1 ? lc.n_experts : lc.top_k).total) return EXFOLD_ERR_WORKSPACE_TOO_SMALL;
+    if (layer->dtype == EXFOLD_BF16 && (!aligned16(x_cal) || !aligned16(w_gate) || !aligned16(w_up) || !aligned16(w_down)))
+        return EXFOLD_ERR_INVALID_ARG;
+    return EXFOLD_OK;
+}
+
+// Enqueues one calibration of checked arguments on the stream (no synchronisation); the number of unobserved experts lands in
+// result_words()[job] when the stream gets there.
+static int calibrate_enqueue(const exfold_layer* layer, const void* x_cal, const float* logits_cal, int64_t m,
+                             const void* w_gate, const void* w_up, const void* w_down, const exfold_calib_opts* opts,
+                             exfold_tables* out, void* ws, void* cuda_stream, int job) {
     const exfold_layer& l = *layer;
     const int N = l.n_experts, K = l.top_k, d = l.hidden, I = l.inter;
     const int Ke = opts->mode == 1 ? N : K;
     exfold_layer lc = l;
-    lc.n_shared = 0;  // the shared expert is never folded, so it is not calibrated
+    lc.n_shared = 0;
     const Plan pl = make_plan(lc, m, Ke);
-    if (ws_bytes < pl.total) return EXFOLD_ERR_WORKSPACE_TOO_SMALL;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(cuda_stream);
 
     int* counts = result_words();
@@ -875,10 +886,7 @@ static int calibrate_enqueue(const exfold_layer* layer, const void* x_cal, const
         EXFOLD_CUDA(cudaMemsetAsync(status, 0, sizeof(DeviceStatus), s));
         EXFOLD_CUDA(launch_iota_ids(ids, m, N, s));
     }
-    if (tensor_path && (!aligned16(x_cal) || !aligned16(w_gate) || !aligned16(w_up) || !aligned16(w_down)))
-        return EXFOLD_ERR_INVALID_ARG;
     const int64_t Rc = m * Ke;
-    if (tensor_path && Rc > (int64_t)1 << 30) return EXFOLD_ERR_UNSUPPORTED;
     CalibStatsParams cs{};
     const size_t NN = (size_t)N * N, calib_bytes = NN * (3 * 8 + 4) + (size_t)N * (8 + 4);
     // Expert outputs, one fp32 row per (token, expert), sorted by expert. Mode 0 sorts the routed rows like prefill; in
@@ -967,7 +975,8 @@ static int calibrate_collect(int n_jobs, int32_t* warn, cudaStream_t s) {
 int exfold_calibrate(const exfold_layer* layer, const void* x_cal, const float* logits_cal, int64_t m,
                      const void* w_gate, const void* w_up, const void* w_down, const exfold_calib_opts* opts,
                      exfold_tables* out, void* ws, size_t ws_bytes, void* cuda_stream) {
-    int rc = calibrate_enqueue(layer, x_cal, logits_cal, m, w_gate, w_up, w_down, opts, out, ws, ws_bytes, cuda_stream, 0);
+    int rc = calibrate_check(layer, x_cal, logits_cal, m, w_gate, w_up, w_down, opts, out, ws, ws_bytes);
+    if (rc == EXFOLD_OK) rc = calibrate_enqueue(layer, x_cal, logits_cal, m, w_gate, w_up, w_down, opts, out, ws, cuda_stream, 0);
     if (rc != EXFOLD_OK) return rc;
     return calibrate_collect(1, nullptr, reinterpret_cast<cudaStream_t>(cuda_stream));
 }
@@ -987,9 +996,16 @@ int exfold_calibrate_layers(const exfold_layer* layer, const exfold_calib_job* j
     if (ws_bytes < exfold_workspace_bytes(layer, m_max, Ke)) return EXFOLD_ERR_WORKSPACE_TOO_SMALL;
     for (int j = 0; j < n_jobs; ++j) {
         const exfold_calib_job& b = jobs[j];
-        int rc = calibrate_enqueue(layer, b.x_cal, b.logits_cal, b.m, b.w_gate, b.w_up, b.w_down, opts, b.out, ws,
-                                   ws_bytes, cuda_stream, j);
+        int rc = calibrate_check(layer, b.x_cal, b.logits_cal, b.m, b.w_gate, b.w_up, b.w_down, opts, b.out, ws, ws_bytes);
         if (rc != EXFOLD_OK) return rc;
+    }
+    for (int j = 0; j < n_jobs; ++j) {
+        const exfold_calib_job& b = jobs[j];
+        int rc = calibrate_enqueue(layer, b.x_cal, b.logits_cal, b.m, b.w_gate, b.w_up, b.w_down, opts, b.out, ws, cuda_stream, j);
+        if (rc != EXFOLD_OK) {  // the jobs before this one still write their tables and their counts
+            cudaStreamSynchronize(reinterpret_cast<cudaStream_t>(cuda_stream));
+            return rc;
+        }
     }
     return calibrate_collect(n_jobs, unobserved, reinterpret_cast<cudaStream_t>(cuda_stream));
 }

@@ -124,6 +124,29 @@ def test_bad_arguments_are_rejected_before_launch(ex):
     assert ex.lib.exfold_static_scratch_address(None) == ex.EXFOLD_ERR_INVALID_ARG
 
 
+def test_calibration_is_refused_before_anything_is_launched(ex):
+    """Every argument of every job is checked before the first launch, the first allocation and the first CUDA call."""
+    layer = ex.make_layer(8, 0, 128, 256, 2, "bf16")
+    p, big = 0x10000, 1 << 40  # fake, aligned, never dereferenced
+    out = ex.exfold_tables(p, p, p, p, None)
+    opts = ex.exfold_calib_opts(1e-3, -4, 4, 1e-12, 0)
+    before = ex.exfold_launch_count()
+
+    def job(x=p, lg=p, m=16, wg=p, wu=p, wd=p, tables=out):
+        return ex.exfold_calib_job(x, lg, m, wg, wu, wd, C.pointer(tables))
+
+    no_h = ex.exfold_tables(p, p, None, p, None)
+    for bad in (job(x=p + 8), job(wg=p + 2), job(wu=p + 8), job(wd=p + 8), job(x=None), job(lg=None), job(m=(1 << 22) + 1),
+                job(tables=no_h)):
+        assert ex.lib.exfold_calibrate(C.byref(layer), bad.x_cal, bad.logits_cal, bad.m, bad.w_gate, bad.w_up, bad.w_down,
+                                       C.byref(opts), bad.out, p, big, None) == ex.EXFOLD_ERR_INVALID_ARG
+        for jobs in ([bad], [job(), bad], [job(), job(), bad, job()]):
+            arr = (ex.exfold_calib_job * len(jobs))(*jobs)
+            assert ex.lib.exfold_calibrate_layers(C.byref(layer), arr, len(jobs), C.byref(opts), None, p, big,
+                                                  None) == ex.EXFOLD_ERR_INVALID_ARG
+    assert ex.exfold_launch_count() == before
+
+
 def test_product_package_does_not_touch_the_oracle():
     """The CUDA path and the oracle share no code and neither imports the other."""
     pkg = os.path.join(ROOT, "paper_2608_24938_b200")
