@@ -272,11 +272,11 @@ int exfold_router_logits(const exfold_layer *layer, const void *x, const void *w
  * layer's output, captured in one CUDA graph). w_router [N][d] in the layer dtype; `logits` [T][N] fp32 is a
  * caller-owned device buffer that receives the scores (16-byte aligned; the layer needs them as scratch and
  * the caller may want them). Everything else as in exfold_moe_prefill / exfold_moe_decode, including the
- * workspace size. The scores are those of exfold_router_logits, bit for bit: decode batches (and prefill calls of
- * at most 128 tokens) take the fixed-order dot-product kernel, which joins the decode call's chain of programmatic
- * dependent launches; longer prefill calls compute the scores with a separate tensor-core launch (a Top-K taken
- * inside a tensor-core epilogue could not be reproduced bit for bit by another summation order, so the two
- * steps stay separate kernels there).
+ * workspace size. Decode batches take the fixed-order dot products, in the decode call's chain of programmatic
+ * dependent launches; prefill calls run exfold_router_logits (above 128 tokens a tensor-core launch of its own: a
+ * Top-K taken inside a tensor-core epilogue could not be reproduced bit for bit by another summation order). So the
+ * scores are those of exfold_router_logits bit for bit, except in decode batches of more than 128 tokens, where that
+ * call accumulates in another order (~1e-6 relative).
  */
 int exfold_moe_prefill_layer(const exfold_layer *layer, const void *x, const void *w_router, int64_t T,
                              const void *w_gate, const void *w_up, const void *w_down,
