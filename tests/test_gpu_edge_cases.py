@@ -164,29 +164,32 @@ def test_host_buffer_calls_with_metadata():
 
 # ------------------------------------------------------------------ one host thread, two streams
 def test_two_prefill_calls_on_two_streams_of_one_thread():
-    """Calls of >= 24 row tiles run part of their work on a second stream that the library keeps per host
+    """Calls on the CTA pairs run part of their work on a second stream that the library keeps per host
     thread; two caller streams used from one thread share it. Each call has its own workspace and output;
-    both must equal the single-stream result bit for bit, and the oracle within tolerance."""
+    both must equal the one-stream, one-CTA-kernel result bit for bit, and the oracle within tolerance."""
     cfg = small_bf16(n_experts=4, hidden=256, inter=256, top_k=2, prefill_tokens=2048, logits="normal")  # 32 row tiles
     case = Case(cfg)
     ex, T, dev = case.ex, cfg.prefill_tokens, case.dev
-    y_ref = case.run_prefill(2, with_meta=False)["y"]
+    y_ref = case.run_prefill(2, with_meta=False, gemm_path=1)["y"]
     need = ex.exfold_workspace_bytes(case.layer, T, 2)
     wss = [torch.full((need,), 0xFF, dtype=torch.uint8, device=dev) for _ in range(2)]
     ys = [torch.full((T, cfg.hidden), float("nan"), dtype=torch.bfloat16, device=dev) for _ in range(2)]
     streams = [torch.cuda.Stream(), torch.cuda.Stream()]
     torch.cuda.synchronize()
+    launches = ex.exfold_launch_count()
     for rep in range(3):
         for i in (0, 1):
-            ex.exfold_moe_prefill(case.layer, case.d_x, case.d_lg, case.d_wg, case.d_wu, case.d_wd, case.tables, 2,
-                                  ys[i], wss[i], stream=streams[i])
+            ex.exfold_moe_prefill_ex(case.layer, case.d_x, case.d_lg, case.d_wg, case.d_wu, case.d_wd, case.tables, 2,
+                                     ys[i], wss[i], gemm_path=2, stream=streams[i])
+    # route, scatter, the two passes of either GEMM, the sum: the odd-tile passes ran on the second stream
+    assert ex.exfold_launch_count() - launches == 6 * 7
     for i in (0, 1):
         assert ex.exfold_device_status(wss[i], streams[i]) == 0
         assert np.array_equal(ys[i].float().cpu().numpy(), y_ref)
     check_output(y_ref, case.oracle_prefill(2)["y"], "bf16")
     assert ex.exfold_thread_release() == 0      # and the per-thread objects come back on the next call
-    ex.exfold_moe_prefill(case.layer, case.d_x, case.d_lg, case.d_wg, case.d_wu, case.d_wd, case.tables, 2, ys[0],
-                          wss[0])
+    ex.exfold_moe_prefill_ex(case.layer, case.d_x, case.d_lg, case.d_wg, case.d_wu, case.d_wd, case.tables, 2, ys[0],
+                             wss[0], gemm_path=2)
     assert ex.exfold_device_status(wss[0]) == 0
     assert np.array_equal(ys[0].float().cpu().numpy(), y_ref)
 
@@ -252,26 +255,28 @@ def test_long_prompt_sorted_routes(T, kw):
 
 # ------------------------------------------------------------------ shared expert beside the scatter kernel, under capture
 def test_shared_expert_pairs_under_graph_capture():
-    """With a shared expert and enough rows for the CTA-pair kernels, the shared expert's gate/up pairs run on the
+    """With a shared expert, on the CTA-pair kernels, the shared expert's gate/up pairs run on the
     library's second stream beside the scatter kernel, and the odd-tile passes fork there a second time. The same
     call captured into a CUDA graph (both forks and joins become graph edges) and replayed gives the bits of the
     plain stream call; outputs against the oracle on a token sample."""
     case = Case(small_bf16(n_shared=1, prefill_tokens=3001, hidden=256, inter=384, logits="normal"), std=0.1)
     cfg, ex, dev = case.cfg, case.ex, case.dev
     T, Kp = case.T, 2
-    ref = case.run_prefill(Kp, with_meta=False)["y"]
+    ref = case.run_prefill(Kp, with_meta=False, gemm_path=1)["y"]
     ws = case.workspace(T, Kp)
     y = torch.full((T, cfg.hidden), float("nan"), dtype=torch.bfloat16, device=dev)
     stream = torch.cuda.Stream()
     with torch.cuda.stream(stream):
-        ex.exfold_moe_prefill(case.layer, case.d_x, case.d_lg, case.d_wg, case.d_wu, case.d_wd, case.tables, Kp, y, ws,
-                              stream=stream)   # warm-up outside the capture: the second stream is created here
+        ex.exfold_moe_prefill_ex(case.layer, case.d_x, case.d_lg, case.d_wg, case.d_wu, case.d_wd, case.tables, Kp, y, ws,
+                                 gemm_path=2, stream=stream)   # warm-up outside the capture: the second stream is created here
         stream.synchronize()
         y.fill_(float("nan"))
         graph = torch.cuda.CUDAGraph()
+        launches = ex.exfold_launch_count()
         with torch.cuda.graph(graph, stream=stream):
-            ex.exfold_moe_prefill(case.layer, case.d_x, case.d_lg, case.d_wg, case.d_wu, case.d_wd, case.tables, Kp, y,
-                                  ws, stream=stream)
+            ex.exfold_moe_prefill_ex(case.layer, case.d_x, case.d_lg, case.d_wg, case.d_wu, case.d_wd, case.tables, Kp, y,
+                                     ws, gemm_path=2, stream=stream)
+        assert ex.exfold_launch_count() - launches == 8  # the shared expert's pairs, then two passes of either GEMM
         for _ in range(3):
             graph.replay()
         stream.synchronize()
@@ -302,17 +307,21 @@ def test_decode_slicing_variants(N, K, B, M, inter):
 def test_chunked_host_prefill_with_a_shared_expert():
     """A host-buffer prefill call long enough to run in chunks, on a layer with a shared expert: every chunk forks
     the second stream twice (the shared expert's gate/up pairs beside the scatter kernel, then the odd-tile passes)
-    while the copy streams bring the next chunk in and the previous one out. Same bits as the call on device buffers."""
-    cfg = small_bf16(prefill_tokens=8500, n_experts=8, n_shared=1, hidden=128, inter=128, top_k=2, logits="normal")
+    while the copy streams bring the next chunk in and the previous one out. Same bits as the call on device buffers,
+    there on the one-CTA kernel. (Three chunks of 2176 tokens and one of 1972, three rows each: 46 row tiles or more x 1344
+    k-blocks, enough for the CTA pairs, which cannot be asked for here.)"""
+    cfg = small_bf16(prefill_tokens=8500, n_experts=4, n_shared=1, hidden=1024, inter=7168, top_k=2, logits="normal")
     case = Case(cfg)
-    ex, T, K, Kp = case.ex, case.T, cfg.top_k, 1
-    ref = case.run_prefill(Kp, with_meta=False)["y"]
+    ex, T, K, Kp = case.ex, case.T, cfg.top_k, 2
+    ref = case.run_prefill(Kp, with_meta=False, gemm_path=1)["y"]
     ws = ex.alloc_workspace(case.layer, T, K, host_staging=True)
     ws.fill_(0xFF)
     xh, lh = case.x.pin_memory(), case.lg.pin_memory()
     for _ in range(2):
         yh = torch.full((T, cfg.hidden), float("nan"), dtype=torch.bfloat16).pin_memory()
+        launches = ex.exfold_launch_count()
         ex.exfold_moe_prefill_host(case.layer, xh, lh, case.d_wg, case.d_wu, case.d_wd, case.tables, Kp, yh, ws)
+        assert ex.exfold_launch_count() - launches == 4 * 8
         assert ex.exfold_device_status(ws) == 0
         assert np.array_equal(yh.float().numpy(), ref)
     idx = sample_tokens(T, 40)

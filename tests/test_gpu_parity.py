@@ -257,13 +257,15 @@ def test_prefill_with_side_by_side_passes_replays_from_a_cuda_graph():
     stream = torch.cuda.Stream()
     with torch.cuda.stream(stream):
         for y in (y_direct, y_direct):   # the second call runs with every lazily created object in place
-            ex.exfold_moe_prefill(case.layer, case.d_x, case.d_lg, case.d_wg, case.d_wu, case.d_wd, case.tables, 2, y, ws,
-                                  stream=stream)
+            ex.exfold_moe_prefill_ex(case.layer, case.d_x, case.d_lg, case.d_wg, case.d_wu, case.d_wd, case.tables, 2, y, ws,
+                                     gemm_path=2, stream=stream)
         stream.synchronize()
         graph = torch.cuda.CUDAGraph()
+        launches = ex.exfold_launch_count()
         with torch.cuda.graph(graph, stream=stream):
-            ex.exfold_moe_prefill(case.layer, case.d_x, case.d_lg, case.d_wg, case.d_wu, case.d_wd, case.tables, 2, y_graph,
-                                  ws, stream=stream)
+            ex.exfold_moe_prefill_ex(case.layer, case.d_x, case.d_lg, case.d_wg, case.d_wu, case.d_wd, case.tables, 2, y_graph,
+                                     ws, gemm_path=2, stream=stream)
+        assert ex.exfold_launch_count() - launches == 7  # two passes of either GEMM
         for _ in range(3):
             graph.replay()
         stream.synchronize()
