@@ -169,6 +169,49 @@ def test_calibrate_bf16_on_tensor_cores(mode, N):
     assert (np.diag(Sg) == 1).all() and (np.diag(Lg) == 0).all()
 
 
+@pytest.mark.parametrize("mode,m", [(0, 6001), (1, 2817), (1, 3001)])
+def test_calibrate_on_cta_pairs(mode, m):
+    """Calibrations with 60 000 tile x k-blocks or more run their GEMMs on the CTA pairs, the odd last tiles beside them, with
+    GEMM-2's fp32 rows over the rows that GEMM-1 reads (mode 1, 2817 tokens: 11 pairs and a one-row tile per expert;
+    3001: 12 pairs with a ragged second tile). Eq. 6-9 written out in double on the GPU; tolerances as above."""
+    N, K, d, I = 8, 4, 1024, 2048
+    case = Case(small_bf16(n_experts=N, top_k=K, hidden=d, inter=I, logits="normal"), std=0.03, correlated=0.8)
+    ex, dev = case.ex, case.dev
+    xc, lc = si.hidden_states(case.cfg, m, "x_cal"), si.router_logits(case.cfg, m, "logits_cal")
+    x64 = xc.to(dev).double()
+    outs = torch.empty((m, N, d), dtype=torch.float64, device=dev)
+    for e in range(N):
+        h = torch.nn.functional.silu(x64 @ case.d_wg[e].double().T) * (x64 @ case.d_wu[e].double().T)
+        outs[:, e] = h @ case.d_wd[e].double().T
+    seen = torch.zeros((m, N), dtype=torch.float64, device=dev)
+    seen.scatter_(1, lc.to(dev).topk(K, dim=1).indices if mode == 0 else torch.arange(N, device=dev).expand(m, N), 1.0)
+    gram = outs @ outs.transpose(1, 2)
+    nrm = torch.diagonal(gram, dim1=1, dim2=2) * seen
+    w = nrm.sqrt()
+    a = torch.einsum("is,ist,it->st", w, gram, seen)
+    b, c = w.T @ nrm, (w * nrm).T @ seen
+    eye = torch.eye(N, dtype=torch.bool, device=dev)
+    scl = (a / (b + 1e-3)).clamp(-4.0, 4.0)
+    loss = ((c - 2.0 * scl * a + scl * scl * b).clamp_min(0.0) / (c + 1e-12)).masked_fill(eye, 0.0)
+    scl = scl.masked_fill(eye, 1.0)
+
+    S, L = torch.full((N, N), float("nan"), device=dev), torch.full((N, N), float("nan"), device=dev)
+    h, lnh = torch.full((N,), float("nan"), device=dev), torch.empty(N, device=dev)
+    n_obs = torch.full((N, N), -1, dtype=torch.int32, device=dev)
+    ws = ex.alloc_workspace(case.layer, m, N if mode else K)
+    ws.fill_(0xFF)
+    launches = ex.exfold_launch_count()
+    rc = ex.exfold_calibrate(case.layer, xc.to(dev), lc.to(dev), case.d_wg, case.d_wu, case.d_wd,
+                             ex.make_tables(S, L, h, lnh, n_obs), ws, mode=mode)
+    assert ex.exfold_launch_count() - launches == 8  # two passes of either GEMM, four kernels around them
+    assert rc == 0 and ex.exfold_device_status(ws) == 0
+    assert torch.equal(n_obs.double(), (seen.T @ seen).masked_fill(eye, 0.0))
+    assert float(scl[~eye].abs().mean()) > 0.1
+    np.testing.assert_allclose(S.cpu().numpy(), scl.cpu().numpy(), rtol=5e-3, atol=5e-3)
+    np.testing.assert_allclose(L.cpu().numpy(), loss.cpu().numpy(), rtol=5e-3, atol=5e-3)
+    np.testing.assert_allclose(h.cpu().numpy(), (w.sum(0) / seen.sum(0)).cpu().numpy(), rtol=3e-3)
+
+
 # ------------------------------------------------------------------ bf16 tensor-core path
 @pytest.mark.parametrize("Kp", [2, 1, 4])
 def test_bf16_prefill_small(Kp):
