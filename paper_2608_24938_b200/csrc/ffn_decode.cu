@@ -56,6 +56,12 @@ constexpr int kFMaxStages = 16;
 // of weights); a larger group runs as one dense item per token tile that it touches, which pulls its weights through the SM
 // twice. 256 tokens with the router, Qwen3 shape, pool 64 (some 32 rows per group): kernel 116 -> 96 us, call 187 -> 151 us;
 // with the limit at 32 rows 161 us, at 96 152.4, at 128 152.8.
+// Where one item per (group, slice) leaves SMs idle, the two dense items of a group run at the same time on those, and the
+// gathers only lengthen the one: the limit falls with the square of the share of SMs that gathered items would fill. Whole
+// call dense / limit of 64 / this: 32 experts of 2048 x 512, 160 tokens, pool of 8 35.3 / 41.9 / 34.8 us, pool of 32 58.7 /
+// 49.9 / 50.0; 13 + 1 experts of 832 x 768, 130 tokens, pool of 4 27.9 / 30.3 / 28.0; 16 + 1 of 3648 x 1664, 130 tokens,
+// pool of 8 95.3 / 102.9 / 97.9; Qwen3 shape, 130 tokens, pool of 8 45.0 / 49.4 / 42.1 (pool of 16, all SMs but a third: 62.1 /
+// 52.3 / 58.8).
 constexpr int kGatherRows = 64;
 constexpr int kGather = 2;
 constexpr int kFTmemCols = 512;
@@ -504,6 +510,8 @@ __global__ void __launch_bounds__(kFThreads, 1) decode_ffn_kernel(const __grid_c
         sync_group();
         // exclusive prefix over (group, tile) = first compact row of each; the work list's rows
         if (tid < 32) {
+            const float fill = fminf(1.0f, (float)(G * ((p.I + 127) / 128)) / (float)gridDim.x);
+            const int gather_limit = (int)(kGatherRows * fill * fill);
             int carry = 0, n = 0;
             for (int g0 = 0; g0 < G; g0 += 32) {
                 const int g = g0 + tid;
@@ -515,7 +523,7 @@ __global__ void __launch_bounds__(kFThreads, 1) decode_ffn_kernel(const __grid_c
                         v[mt] = __popc(m4.x) + __popc(m4.y) + __popc(m4.z) + __popc(m4.w);
                     }
                 const int rows = v[0] + v[1];
-                const bool gather = nmt == 2 && rows > 0 && rows <= kGatherRows;
+                const bool gather = nmt == 2 && rows > 0 && rows <= gather_limit;
                 const int entries = gather ? 1 : (v[0] > 0) + (v[1] > 0);
                 int incl = rows;
 #pragma unroll

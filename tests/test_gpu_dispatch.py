@@ -185,6 +185,11 @@ def test_decode_router_scores_of_short_rows(B, N):
     ([64, 64, 1], 0, 1088, 192),                     # every group gathered, 17 chunks
     ([130, 126], 0, 128, 192),                       # none
     ([2] * 100, 0, 128, 128),                        # many small groups
+    # the lists above leave SMs idle (the last aside), so that few rows or none are gathered; these fill them, or nearly
+    ([1, 3, 4, 5, 63, 64, 65, 51], 0, 256, 2432),
+    ([64, 65], 1, 64, 6336),
+    ([64, 64, 1], 0, 1088, 6336),
+    ([42, 43, 41] + [3] * 37, 0, 128, 384),          # 120 of 148 SMs: up to 42 rows
 ])
 @pytest.mark.parametrize("place", ["mixed", "sorted"])
 def test_decode_group_sizes_above_128_tokens(rows, ns, d, I, place):
