@@ -353,7 +353,8 @@ __global__ void __launch_bounds__(kDecThreads) decode_route_kernel(DecodeRoutePa
 // Without the router: one CTA per token. With it: a cluster of 8 CTAs per TT tokens, each taking an eighth of the
 // experts (one CTA alone would walk the whole router matrix with a handful of loads in flight); the scores meet
 // in the shared memory of the cluster's first CTA, which then ranks them. TT = 1 spreads a small batch over the most SMs: a
-// warp takes two experts at a time. TT = 8: a warp takes 4 experts x 4 tokens, so that a conversion serves four products
+// warp takes two experts at a time, or one where that gives all eight warps work (at most 64 experts: 8 of 4096 x 2048, 96
+// tokens 60.6 us per call with two, 49.1 with one; 32 of 2048 x 512, 16 tokens 33.2 and 31.1). TT = 8: a warp takes 4 experts x 4 tokens, so that a conversion serves four products
 // and the router matrix is read through L2 once per 8 tokens. CTA 0 also clears the status record.
 // The batch-level half (pool, targets, remap) runs in the prologue of the gate/up kernel (ffn_decode.cu).
 constexpr int kTopkCluster = 8;
@@ -369,7 +370,8 @@ __global__ void __launch_bounds__(256) decode_topk_kernel(DecodeTopkParams p) {
     grid_dep_wait();  // x may be the previous layer's output; the workspace may still be read by the previous call
     if (blockIdx.x == 0 && threadIdx.x < 4) reinterpret_cast<int*>(p.status)[threadIdx.x] = 0;
     if (ROUTER) {
-        constexpr int EW = TT == 1 ? 2 : 4, TW = TT == 1 ? 1 : 4;  // experts and tokens of a warp
+        constexpr int EW = TT == 1 ? (NPL <= 2 ? 1 : 2) : 4, TW = TT == 1 ? 1 : 4;  // experts and tokens of a warp
+        constexpr int kSteps = EW == 1 ? 4 : 2;  // in flight
         constexpr int kTokGroups = TT / TW, kExpGroups = 8 / kTokGroups;
         cg::cluster_group cluster = cg::this_cluster();
         const int rank = (int)cluster.block_rank();
@@ -390,7 +392,7 @@ __global__ void __launch_bounds__(256) decode_topk_kernel(DecodeTopkParams p) {
             for (int u = 0; u < EW; ++u)
 #pragma unroll
                 for (int t = 0; t < TW; ++t) acc[u][t] = 0.f;
-#pragma unroll 2
+#pragma unroll kSteps
             for (int c = lane * 8; c < d; c += 256) {
                 uint4 a[EW], b[TW];
 #pragma unroll
