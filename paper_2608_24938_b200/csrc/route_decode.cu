@@ -527,18 +527,21 @@ cudaError_t launch_decode_route(const DecodeRouteParams& p, cudaStream_t s) {
     return err;
 }
 
-// From this batch on (and with enough experts to fill the tiles) clusters take 8 tokens. Whole decode call with the router,
-// TT = 1 / 8: Qwen3 shape 40 tokens 50.5 / 51.8 us, 64 tokens 51.2 / 52.6, 120 tokens 58.3 / 54.2, 256 tokens 207 / 199; GLM
-// shape 40 tokens 139 / 141, 128 tokens 251 / 244.
-constexpr int kTopkTileBatch = 81;
+// From this batch on clusters take 8 tokens, with more than 64 experts. About 100 one-token clusters are resident at once, so
+// that their time steps up behind 96 tokens. Whole decode call with the router, TT = 1 / 8, 96, 104, 128 and 256 tokens: Qwen3
+// shape 51.1 / 53.4 us, 55.8 / 53.7, 56.6 / 53.5, 81.8 / 72.2; GLM shape (pool of 8) 86.3 / 90.2, 94.3 / 90.6, 96.1 / 90.8,
+// 135.5 / 122.7; 256 experts of 2048 x 512 55.9 / 59.1, 61.9 / 59.3, 65.0 / 59.8, 87.4 / 76.6. With few experts the 32 x 8 tiles
+// leave warps idle: 40 experts of 4096 x 256, 128 and 256 tokens 49.7 / 52.9, 63.0 / 65.3; 64 of 1024 x 512 31.5 / 31.6, 40.4 / 37.1.
+constexpr int kTopkTileBatch = 97;
 template <int NPL>
 static cudaError_t launch_topk_t(const DecodeTopkParams& p, cudaStream_t s) {
     // max_smem: the gate/up kernel's CTAs start beside these (64 tokens, Qwen3 shape, pool 16: whole call 0.5 % faster; the
     // same for the per-token sum of the previous call cost the Mixtral shape 2 %)
     if (p.w_router == nullptr) return launch_pdl_as(decode_topk_kernel<NPL, false, 1>, p.B, 256, 0, 1, true, s, p);
-    if (p.B < kTopkTileBatch || p.N < 32)
-        return launch_pdl_as(decode_topk_kernel<NPL, true, 1>, (unsigned)p.B * kTopkCluster, 256, 0, kTopkCluster, true, s, p);
-    return launch_pdl_as(decode_topk_kernel<NPL, true, 8>, (unsigned)(p.B + 7) / 8 * kTopkCluster, 256, 0, kTopkCluster, true, s, p);
+    if constexpr (NPL > 2)
+        if (p.B >= kTopkTileBatch)
+            return launch_pdl_as(decode_topk_kernel<NPL, true, 8>, (unsigned)(p.B + 7) / 8 * kTopkCluster, 256, 0, kTopkCluster, true, s, p);
+    return launch_pdl_as(decode_topk_kernel<NPL, true, 1>, (unsigned)p.B * kTopkCluster, 256, 0, kTopkCluster, true, s, p);
 }
 
 cudaError_t launch_decode_topk(const DecodeTopkParams& p, cudaStream_t s) {

@@ -133,11 +133,12 @@ def test_small_decode_batches(shape, mode):
     assert np.array_equal(got["y"], plain["y"])
 
 
-@pytest.mark.parametrize("B", [80, 81, 87, 128])
-@pytest.mark.parametrize("N", [31, 32, 100, 256])
+@pytest.mark.parametrize("B", [80, 81, 87, 96, 97, 103, 128])
+@pytest.mark.parametrize("N", [31, 32, 64, 65, 100, 256])
 def test_decode_router_scores_by_batch(B, N):
-    """Router scores inside the decode call, a token per cluster or eight (from 81 tokens and 32 experts on; ragged last
-    cluster, experts not a multiple of the tiles): the bits of exfold_router_logits."""
+    """Router scores inside the decode call, a token per cluster (a warp takes one expert, above 64 experts two) or eight
+    (from 97 tokens and 65 experts on; ragged last cluster, experts not a multiple of the tiles): the bits of
+    exfold_router_logits."""
     case = Case(si.LayerConfig("rt", N, 0, 320, 64, 4, "bf16", 8, (1,), B, (6,)))
     ex, dev = case.ex, case.dev
     wr = si.router_weights(case.cfg).to(dev)
