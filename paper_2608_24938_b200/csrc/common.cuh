@@ -129,28 +129,22 @@ __device__ __forceinline__ double warp_topk_softmax(const float (&v)[NPL], int N
     return ex / sum;
 }
 
-// Programmatic launch; cluster > 1: the grid split into thread-block clusters (distributed shared memory); max_smem: the SM's
-// L1 given to shared memory as far as it goes, so that CTAs of a successor that needs it start beside this kernel's (an SM
-// changes the split only when it is idle)
+// Programmatic launch; cluster > 1: the grid split into thread-block clusters (distributed shared memory)
 template <typename... KArgs, typename... Args>
-cudaError_t launch_pdl_as(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, unsigned cluster, bool max_smem,
-                          cudaStream_t s, Args... args) {
+cudaError_t launch_pdl_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, unsigned cluster,
+                               cudaStream_t s, Args... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
-    cudaLaunchAttribute attr[3];
+    cudaLaunchAttribute attr[2];
     unsigned n = 0;
     if (cluster > 1) {
         attr[n].id = cudaLaunchAttributeClusterDimension;
         attr[n].val.clusterDim.x = cluster;
         attr[n].val.clusterDim.y = 1;
         attr[n++].val.clusterDim.z = 1;
-    }
-    if (max_smem) {
-        attr[n].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
-        attr[n++].val.sharedMemCarveout = 100;
     }
     if (pdl_enabled()) {
         attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -164,12 +158,7 @@ cudaError_t launch_pdl_as(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_
 }
 template <typename... KArgs, typename... Args>
 cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Args... args) {
-    return launch_pdl_as(kernel, grid, block, smem, 1, false, s, args...);
-}
-template <typename... KArgs, typename... Args>
-cudaError_t launch_pdl_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, unsigned cluster,
-                               cudaStream_t s, Args... args) {
-    return launch_pdl_as(kernel, grid, block, smem, cluster, false, s, args...);
+    return launch_pdl_cluster(kernel, grid, block, smem, 1, s, args...);
 }
 
 __host__ __device__ inline size_t align16(size_t v) { return (v + 15) / 16 * 16; }

@@ -535,13 +535,11 @@ cudaError_t launch_decode_route(const DecodeRouteParams& p, cudaStream_t s) {
 constexpr int kTopkTileBatch = 97;
 template <int NPL>
 static cudaError_t launch_topk_t(const DecodeTopkParams& p, cudaStream_t s) {
-    // max_smem: the gate/up kernel's CTAs start beside these (64 tokens, Qwen3 shape, pool 16: whole call 0.5 % faster; the
-    // same for the per-token sum of the previous call cost the Mixtral shape 2 %)
-    if (p.w_router == nullptr) return launch_pdl_as(decode_topk_kernel<NPL, false, 1>, p.B, 256, 0, 1, true, s, p);
+    if (p.w_router == nullptr) return launch_pdl(decode_topk_kernel<NPL, false, 1>, p.B, 256, 0, s, p);
     if constexpr (NPL > 2)
         if (p.B >= kTopkTileBatch)
-            return launch_pdl_as(decode_topk_kernel<NPL, true, 8>, (unsigned)(p.B + 7) / 8 * kTopkCluster, 256, 0, kTopkCluster, true, s, p);
-    return launch_pdl_as(decode_topk_kernel<NPL, true, 1>, (unsigned)p.B * kTopkCluster, 256, 0, kTopkCluster, true, s, p);
+            return launch_pdl_cluster(decode_topk_kernel<NPL, true, 8>, (unsigned)(p.B + 7) / 8 * kTopkCluster, 256, 0, kTopkCluster, s, p);
+    return launch_pdl_cluster(decode_topk_kernel<NPL, true, 1>, (unsigned)p.B * kTopkCluster, 256, 0, kTopkCluster, s, p);
 }
 
 cudaError_t launch_decode_topk(const DecodeTopkParams& p, cudaStream_t s) {
