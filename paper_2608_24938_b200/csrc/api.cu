@@ -621,7 +621,7 @@ int exfold_moe_prefill_ex(const exfold_layer* layer, const void* x, const float*
         fp.offsets = cp.offsets; fp.tile_start = cp.work_start; fp.row_tok = cp.row_tok; fp.row_w = cp.row_w;
         if (direct) fp.y = reinterpret_cast<float*>(y);
         else fp.out = at<float>(ws, pl.out);
-        { ProfScope ps(10, s); EXFOLD_CUDA(launch_ffn_f32(fp, Rtot, s)); }
+        { ProfScope ps(10, s); EXFOLD_CUDA(launch_ffn_f32(fp, Rtot, sm_count(), s)); }
         if (!direct) {
             ProfScope ps(11, s);
             EXFOLD_CUDA(launch_combine_f32(fp.out, cp.inv_pos, cp.row_w, T, Kp, d, l.n_shared, nullptr,
@@ -791,7 +791,9 @@ static int decode_impl(const exfold_layer* layer, const void* x, const float* lo
         FfnF32Params fp = f32_params(x, w_gate, w_up, w_down, d, I, max_groups, rp.tile_rows);
         fp.offsets = rp.grp_off; fp.tile_start = rp.grp_tiles; fp.grp_expert = rp.grp_expert; fp.n_groups_dev = rp.n_groups;
         fp.row_tok = rp.row_tok; fp.row_w = rp.row_w; fp.out = at<float>(ws, pl.out);
-        { ProfScope ps(10, s); EXFOLD_CUDA(launch_ffn_f32(fp, max_rows, s)); }
+        // a token has at most as many rows as the pool has experts
+        const int64_t rows = B * std::min(K, (int)pool_m) + B * l.n_shared;
+        { ProfScope ps(10, s); EXFOLD_CUDA(launch_ffn_f32(fp, rows, sm_count(), s)); }
         { ProfScope ps(11, s); EXFOLD_CUDA(launch_combine_f32(fp.out, rp.slot_row, rp.row_w, B, K, d, l.n_shared, rp.n_groups + 2,
                                                               reinterpret_cast<float*>(y), s)); }
     }
@@ -942,7 +944,7 @@ static int calibrate_enqueue(const exfold_layer* layer, const void* x_cal, const
         fp.offsets = offsets; fp.tile_start = work_start; fp.x_rows = m;
         fp.row_tok = opts->mode == 0 ? row_tok : nullptr;
         fp.out = at<float>(ws, pl.out);
-        EXFOLD_CUDA(launch_ffn_f32(fp, Rc, s));
+        EXFOLD_CUDA(launch_ffn_f32(fp, Rc, sm_count(), s));
         cs.out = fp.out;
     }
 

@@ -372,7 +372,7 @@ struct FfnF32Params {
     float* y;                     // [tokens][d]: every token has one row, stored weighted (out unused)
 };
 int ffn_f32_tile_rows(int64_t rows, int G, int d, int I);
-cudaError_t launch_ffn_f32(FfnF32Params p, int64_t rows, cudaStream_t s);
+cudaError_t launch_ffn_f32(const FfnF32Params& p, int64_t rows, int sms, cudaStream_t s);
 cudaError_t launch_combine_f32(const float* out, const int32_t* inv_pos, const float* row_w, int64_t T, int Kr, int d,
                                int n_shared, const int32_t* shared0_dev, float* y, cudaStream_t s);
 

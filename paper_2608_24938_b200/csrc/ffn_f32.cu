@@ -1,8 +1,8 @@
 // Expert FFN of fp32 layers (Eq. 1) on the CUDA cores: tensor cores would round fp32 inputs.
 //
-// A cluster of 8 CTAs per row tile (up to tile_rows sorted rows of one expert). Phase 0: CTA r computes its eighth of the
-// intermediate features, gate and up, for all rows of the tile, and leaves silu(gate) * up in shared memory. Phase 1,
-// after a cluster barrier: CTA r computes its eighth of the output features with all of I as K. The activation crosses the
+// A cluster of 8 CTAs (4 or 2 where there are many tiles of a small layer) per row tile (up to tile_rows sorted rows of one
+// expert). Phase 0: CTA r computes its share of the intermediate features, gate and up, for all rows of the tile, and leaves silu(gate) * up in shared memory. Phase 1,
+// after a cluster barrier: CTA r computes its share of the output features with all of I as K. The activation crosses the
 // cluster through distributed shared memory and never goes to memory; one launch does the whole FFN, and a tile's weights
 // are read once per tile instead of once per row. Two kernels:
 //
@@ -25,6 +25,7 @@
 // of 768 x 1024 750 -> 158 -> 149 us (12.7 TFLOP/s); 2048 rows of 256 x 512 270 -> 130 -> 123. What bounds the tall form now
 // is shared-memory reads (a 16-byte read costs a wavefront per quarter warp, so 32 for the 64 multiply-adds they feed).
 #include <algorithm>
+#include <cmath>
 
 #include "common.cuh"
 #include "ptx.cuh"
@@ -37,7 +38,7 @@ namespace {
 
 namespace cg = cooperative_groups;
 
-constexpr int kCl = 8;         // CTAs per row tile
+constexpr int kMaxCl = 8;  // CTAs per row tile, at most
 constexpr int kThreads = 256;  // 8 warps
 constexpr int kKC = 32;        // tall tiles: K elements per stage
 constexpr int kLd = kKC + 4;   // row pitch in floats: 16-byte aligned, the rows of a warp's read hit distinct banks
@@ -100,7 +101,7 @@ __device__ __forceinline__ void lane_sums(float* v, int lane) {
     }
 }
 
-template <bool VEC>
+template <int CL, bool VEC>
 __global__ void __launch_bounds__(kThreads) ffn_f32_short_kernel(FfnF32Params p) {
     extern __shared__ __align__(16) float smem[];
     __shared__ Tile s_tile;
@@ -112,12 +113,12 @@ __global__ void __launch_bounds__(kThreads) ffn_f32_short_kernel(FfnF32Params p)
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     constexpr int kWarps = kThreads / 32;
     grid_dep_wait();
-    if (!find_tile(p, (int)(blockIdx.x / kCl), &s_tile)) return;  // the whole cluster
+    if (!find_tile(p, (int)(blockIdx.x / CL), &s_tile)) return;  // the whole cluster
     cluster.barrier_arrive();  // waited for before the first remote write: all CTAs of the cluster have started
     const int rows = s_tile.rows;
     const int64_t row0 = s_tile.row0;
     const size_t e = s_tile.expert;
-    const int per0 = (I + kCl - 1) / kCl, per1 = (d + kCl - 1) / kCl;
+    const int per0 = (I + CL - 1) / CL, per1 = (d + CL - 1) / CL;
 
     // Lane's elements of K chunk c: VEC 4 consecutive ones, else 4 that are 32 apart
     auto load_w = [&](const float* row, bool in, int c, int K) {
@@ -206,14 +207,14 @@ __global__ void __launch_bounds__(kThreads) ffn_f32_short_kernel(FfnF32Params p)
                     cluster.barrier_wait();
                     started = true;
                 }
-                // lanes 0-15 hold gate, 16-31 up of the same (feature, token): both compute, each writes to four CTAs
+                // lanes 0-15 hold gate, 16-31 up of the same (feature, token): both compute, each writes to half of the CTAs
                 const float other = __shfl_xor_sync(0xffffffffu, acc[0], 16);
                 const float h = lane < 16 ? swiglu(acc[0], other) : swiglu(other, acc[0]);
                 const int fl = gi * 2 + (q & 1);
                 if (fl < n0)
 #pragma unroll
-                    for (int c = 0; c < kCl / 2; ++c)
-                        cluster.map_shared_rank(hs, c + (lane < 16 ? 0 : kCl / 2))[t * hld + rank * per0 + fl] = h;
+                    for (int c = 0; c < CL / 2; ++c)
+                        cluster.map_shared_rank(hs, c + (lane < 16 ? 0 : CL / 2))[t * hld + rank * per0 + fl] = h;
             } else if (gi * kSW + q < n1 && t < rows) {
                 const int col = rank * per1 + gi * kSW + q;
                 if (p.y != nullptr) p.y[(int64_t)p.row_tok[row0 + t] * d + col] = p.row_w[row0 + t] * acc[0];
@@ -256,7 +257,7 @@ __device__ __forceinline__ void mac_chunk(const float* ws, const float* xs, int 
         for (int q = 0; q < NW; ++q) acc[r][q] += part[r][q];
 }
 
-template <int TM, int NW, int RW, bool VEC>
+template <int CL, int TM, int NW, int RW, bool VEC>
 __global__ void __launch_bounds__(kThreads, 2) ffn_f32_tall_kernel(FfnF32Params p) {
     constexpr int BM = 4 * TM * RW;              // rows of the tile
     constexpr int kAcross = 8 / RW;              // warps along the features and along K
@@ -274,7 +275,7 @@ __global__ void __launch_bounds__(kThreads, 2) ffn_f32_tall_kernel(FfnF32Params 
     const int lr = lane >> 3, lf = lane & 7, wr = warp / kAcross, wa = warp % kAcross;
     const int d = p.d, I = p.I, fpc = p.fpc, hld = p.hld;
     grid_dep_wait();
-    if (!find_tile(p, (int)(blockIdx.x / kCl), &s_tile)) return;  // the whole cluster
+    if (!find_tile(p, (int)(blockIdx.x / CL), &s_tile)) return;  // the whole cluster
     const int rows = s_tile.rows;
     const int64_t row0 = s_tile.row0;
     const size_t e = s_tile.expert;
@@ -295,7 +296,7 @@ __global__ void __launch_bounds__(kThreads, 2) ffn_f32_tall_kernel(FfnF32Params 
             cluster.sync();     // every slice of H is in place
         }
         // phase 0: H[:, rank's features] = silu(x W_gate^T) * (x W_up^T); phase 1: out[:, rank's columns] = H W_down^T
-        const int K = phase == 0 ? d : I, per = phase == 0 ? fpc : (d + kCl - 1) / kCl;
+        const int K = phase == 0 ? d : I, per = phase == 0 ? fpc : (d + CL - 1) / CL;
         const int lo = rank * per, hi = min(phase == 0 ? I : d, lo + per);
         // A power of two of warps (n_wf) lies along the stage's weight rows, the others split K; afterwards the warps with
         // wk == 0 hold the sums of token rows wr * 4 TM + 4 r + lr and stage rows wf * 8 NW + 8 q + lf.
@@ -394,18 +395,36 @@ __global__ void __launch_bounds__(kThreads, 2) ffn_f32_tall_kernel(FfnF32Params 
 }
 
 constexpr size_t kSmemLimit = 227 * 1024 - 1024;
-int features_per_cta(int I) { return ((I + kCl - 1) / kCl + kKC - 1) / kKC * kKC; }
+int features_per_cta(int I, int cl) { return ((I + cl - 1) / cl + kKC - 1) / kKC * kKC; }
 size_t short_bytes(int d, int I) { return (size_t)kSR * ((d + 127) / 128 * 128 + (I + 127) / 128 * 128 + 4) * sizeof(float); }
-size_t tall_bytes(int tile_rows, int I) {  // two stages of 128 weight rows and the form's token rows, then the slice of H
+size_t tall_bytes(int tile_rows, int I, int cl) {  // two stages of 128 weight rows and the form's token rows, then the slice of H
     const int form_rows = tile_rows > 16 ? 32 : 16;
-    return ((size_t)2 * (128 + form_rows) * kLd + (size_t)tile_rows * (features_per_cta(I) + 4)) * sizeof(float);
+    return ((size_t)2 * (128 + form_rows) * kLd + (size_t)tile_rows * (features_per_cta(I, cl) + 4)) * sizeof(float);
 }
 
-template <typename K>
+template <int CL, typename K>
 cudaError_t launch_t(K kernel, const FfnF32Params& p, size_t smem, int64_t tiles, cudaStream_t s) {
     cudaError_t err = ensure_smem(kernel, smem);
     if (err != cudaSuccess) return err;
-    return launch_pdl_cluster(kernel, (unsigned)(tiles * kCl), kThreads, smem, kCl, s, p);
+    return launch_pdl_cluster(kernel, (unsigned)(tiles * CL), kThreads, smem, CL, s, p);
+}
+template <int CL, bool VEC>
+cudaError_t launch_form(FfnF32Params p, int64_t tiles, cudaStream_t s) {
+    if (p.tile_rows == kSR && short_bytes(p.d, p.I) <= kSmemLimit) {
+        p.hld = (p.I + 127) / 128 * 128 + 4;
+        return launch_t<CL>(ffn_f32_short_kernel<CL, VEC>, p, short_bytes(p.d, p.I), tiles, s);
+    }
+    p.fpc = features_per_cta(p.I, CL);
+    p.hld = p.fpc + 4;
+    const size_t smem = tall_bytes(p.tile_rows, p.I, CL);
+    if (p.tile_rows > 16) return launch_t<CL>(ffn_f32_tall_kernel<CL, 4, 4, 2, VEC>, p, smem, tiles, s);
+    return launch_t<CL>(ffn_f32_tall_kernel<CL, 4, 2, 1, VEC>, p, smem, tiles, s);
+}
+template <int CL>
+cudaError_t launch_cl(const FfnF32Params& p, int64_t tiles, cudaStream_t s) {
+    auto a16 = [](const void* q) { return (reinterpret_cast<uintptr_t>(q) & 15) == 0; };
+    const bool vec = p.I % 4 == 0 && a16(p.x) && a16(p.wg) && a16(p.wu) && a16(p.wd);
+    return vec ? launch_form<CL, true>(p, tiles, s) : launch_form<CL, false>(p, tiles, s);
 }
 
 // y[i][c] = sum_j w(row) out[row][c] over the token's rows in slot order (row = inv_pos[i][j], -1: merged into an earlier
@@ -449,28 +468,40 @@ __global__ void __launch_bounds__(128) combine_f32_kernel(const float* __restric
 int ffn_f32_tile_rows(int64_t rows, int G, int d, int I) {
     if (rows <= (int64_t)kSR * G && short_bytes(d, I) <= kSmemLimit) return kSR;
     int tile_rows = rows > (int64_t)48 * G ? 32 : 16;
-    while (tile_rows > 1 && tall_bytes(tile_rows, I) > kSmemLimit) tile_rows /= 2;
+    while (tile_rows > 1 && tall_bytes(tile_rows, I, kMaxCl) > kSmemLimit) tile_rows /= 2;
     return tile_rows;
 }
 
-cudaError_t launch_ffn_f32(FfnF32Params p, int64_t rows, cudaStream_t s) {
+// CTAs per row tile. Two CTAs share an SM, so that clusters run in waves (fragmented by the chip's partitions to some nine
+// tenths; a last wave that is nearly empty costs half of one), each of which takes a fixed 8 us and, in proportion to a CTA's
+// share of the layer, 0.28 + 0.037 per row and weight row of 1000: few tiles want eight CTAs each, many tiles of a small
+// layer fewer, in fewer waves. The tiles are estimated from the rows (over as many groups as random rows meet). Whole prefill
+// call with 8, 4 and 2 CTAs, and with one CTA per route before there were row tiles: 195 experts of 64 x 64, 943 tokens x 3
+// 78.4, 46.7, 32.5, 67.8 us; 60 of 128 x 256, 500 x 4 85.9, 64.7, 52.4, 123.3; 60 of 512 x 512 255.8, 260.9, 283.1, 795.8; 16 of
+// 128 x 256, 64 x 2 17.1, 18.9, 23.1, 42.1. Over 90 shapes of 64 x 64 to 1024 x 2048 and 12 to 371 tiles the choice is 3.1 %
+// above the best of the three, 11 % below eight CTAs always.
+static int cluster_ctas(int64_t rows, int64_t tiles, const FfnF32Params& p, int sms) {
+    const double r = (double)rows, used = p.G * (1.0 - std::exp(-r / p.G));  // groups with a row
+    const double est = std::min((double)tiles, std::max(used, r / p.tile_rows + used / 2));
+    const double share = (double)p.d * p.I * (0.28 + 0.037 * p.tile_rows) / 1000.0;
+    int best = kMaxCl;
+    double best_t = 1e30;
+    for (int cl = kMaxCl; cl >= 2; cl /= 2) {
+        if (cl < kMaxCl && tall_bytes(p.tile_rows, p.I, cl) > kSmemLimit) break;
+        const double x = est * cl / (1.84 * sms), t = (x <= 1.0 ? 1.0 : 0.5 * (std::ceil(x) + x + 0.3)) * (8.0 + share / cl);
+        if (t < 0.9 * best_t) {  // fewer only for a clear gain
+            best_t = t;
+            best = cl;
+        }
+    }
+    return best;
+}
+
+cudaError_t launch_ffn_f32(const FfnF32Params& p, int64_t rows, int sms, cudaStream_t s) {
     if (rows == 0) return cudaSuccess;
     const int64_t tiles = std::min<int64_t>(rows, rows / p.tile_rows + p.G);
-    auto a16 = [](const void* q) { return (reinterpret_cast<uintptr_t>(q) & 15) == 0; };
-    const bool vec = p.I % 4 == 0 && a16(p.x) && a16(p.wg) && a16(p.wu) && a16(p.wd);
-    if (p.tile_rows == kSR && short_bytes(p.d, p.I) <= kSmemLimit) {
-        p.hld = (p.I + 127) / 128 * 128 + 4;
-        const size_t smem = short_bytes(p.d, p.I);
-        return vec ? launch_t(ffn_f32_short_kernel<true>, p, smem, tiles, s) : launch_t(ffn_f32_short_kernel<false>, p, smem, tiles, s);
-    }
-    p.fpc = features_per_cta(p.I);
-    p.hld = p.fpc + 4;
-    const size_t smem = tall_bytes(p.tile_rows, p.I);
-    if (p.tile_rows > 16)
-        return vec ? launch_t(ffn_f32_tall_kernel<4, 4, 2, true>, p, smem, tiles, s)
-                   : launch_t(ffn_f32_tall_kernel<4, 4, 2, false>, p, smem, tiles, s);
-    return vec ? launch_t(ffn_f32_tall_kernel<4, 2, 1, true>, p, smem, tiles, s)
-               : launch_t(ffn_f32_tall_kernel<4, 2, 1, false>, p, smem, tiles, s);
+    const int cl = cluster_ctas(rows, tiles, p, sms);
+    return cl == 8 ? launch_cl<8>(p, tiles, s) : (cl == 4 ? launch_cl<4>(p, tiles, s) : launch_cl<2>(p, tiles, s));
 }
 
 cudaError_t launch_combine_f32(const float* out, const int32_t* inv_pos, const float* row_w, int64_t T, int Kr, int d,

@@ -48,9 +48,16 @@ def test_calibration_sums_by_top_k(K):
     (5, 0, 256, 390, 3, 257, 3, 256, 2),    # 32-row tiles, element-wise staging, merged decode slots
     (40, 0, 36, 1100, 5, 130, 4, 33, 17),   # 16-row tiles, several feature passes per CTA
     (16, 0, 384, 640, 2, 50, 2, 40, 5),     # 8-row tiles, two feature passes
+    # many tiles: 4 or 2 CTAs per cluster, of 8-, 16- and 32-row tiles, vector and element-wise
+    (180, 1, 64, 96, 2, 200, 2, 109, 180),
+    (90, 0, 68, 33, 3, 150, 3, 100, 90),
+    (60, 0, 128, 256, 4, 500, 4, 128, 60),
+    (60, 1, 36, 1100, 4, 400, 3, 70, 40),
+    (8, 0, 64, 64, 2, 3000, 2, 256, 8),
+    (9, 1, 132, 390, 3, 2000, 2, 256, 9),
 ])
 def test_f32_layer_shapes(shape):
-    """fp32 layers: row-tile sizes, vector and element-wise staging, ragged widths, shared expert; routing bit-exact,
+    """fp32 layers: row-tile sizes, CTAs per cluster, vector and element-wise staging, ragged widths, shared expert; routing bit-exact,
     outputs to fp32 rounding (two-level sums of at most ~1100 terms: 2e-6 of the norm; seen ~3e-7)."""
     N, ns, d, I, K, T, Kp, B, M = shape
     case = Case(si.LayerConfig("f32s", N, ns, d, I, K, "f32", T, (Kp,), B, (M,)))
