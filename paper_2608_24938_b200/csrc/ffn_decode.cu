@@ -200,10 +200,11 @@ __global__ void __launch_bounds__(kFThreads, 1) decode_ffn_kernel(const __grid_c
     const int a_bytes = p.a_rows * kFBK * 2;
     const int stage_bytes = decode_ffn_stage_bytes(p.a_rows, p.alt);
     Scratch& sc = *reinterpret_cast<Scratch*>(tiles + p.scratch_off);
-    // one byte per slot (its routed expert, then its target) and, by pool rank, the tokens each group serves as bit masks:
-    // what is not spent here is ring (256 tokens x 8 slots: 20 KB with ids and weights as words, one stage of four)
-    unsigned char* ids8 = tiles + p.scratch_off + kFScratchFixed;
-    uint32_t* tmask = reinterpret_cast<uint32_t*>(ids8 + align16((size_t)p.B * p.K));
+    // two bytes per slot (its routed expert in the upper, the expert that runs it in the lower one) and, by pool rank, the
+    // tokens each group serves as bit masks: what is not spent here is ring (256 tokens x 8 slots: 20 KB with ids and weights
+    // as words, one stage of four)
+    unsigned short* slots = reinterpret_cast<unsigned short*>(tiles + p.scratch_off + kFScratchFixed);
+    uint32_t* tmask = reinterpret_cast<uint32_t*>(tiles + p.scratch_off + kFScratchFixed + align16((size_t)p.B * p.K * 2));
 
     // ---- set-up that does not depend on the previous kernel: overlaps its tail under programmatic launch
     if (threadIdx.x == 0) {
@@ -297,8 +298,8 @@ __global__ void __launch_bounds__(kFThreads, 1) decode_ffn_kernel(const __grid_c
         for (int u = 0; u < 3; ++u) {
             const int s = s0 + u * kFThreads;
             if (s >= BK4) break;
-            reinterpret_cast<uchar4*>(ids8)[s] =
-                make_uchar4((unsigned char)id[u].x, (unsigned char)id[u].y, (unsigned char)id[u].z, (unsigned char)id[u].w);
+            reinterpret_cast<uint2*>(slots)[s] = make_uint2((unsigned)id[u].x << 8 | (unsigned)id[u].y << 24,
+                                                            (unsigned)id[u].z << 8 | (unsigned)id[u].w << 24);
             if (!is_static) {
                 add_slot(id[u].x, wv[u][0].x);
                 add_slot(id[u].y, wv[u][0].y);
@@ -310,7 +311,7 @@ __global__ void __launch_bounds__(kFThreads, 1) decode_ffn_kernel(const __grid_c
     if (threadIdx.x < (BK & 3)) {
         const int s = BK4 * 4 + threadIdx.x;
         const int id = p.ids[s];
-        ids8[s] = (unsigned char)id;
+        slots[s] = (unsigned short)(id << 8);
         if (!is_static) add_slot(id, p.w64[s]);
     }
     __syncthreads();
@@ -470,7 +471,7 @@ __global__ void __launch_bounds__(kFThreads, 1) decode_ffn_kernel(const __grid_c
         for (int s0 = tid; s0 < BK; s0 += 4 * nth) {
             int e[4], t[4], r[4];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) e[u] = s0 + u * nth < BK ? ids8[s0 + u * nth] : -1;
+            for (int u = 0; u < 4; ++u) e[u] = s0 + u * nth < BK ? slots[s0 + u * nth] >> 8 : -1;
 #pragma unroll
             for (int u = 0; u < 4; ++u) t[u] = e[u] >= 0 ? sc.target[e[u]] : 0;
 #pragma unroll
@@ -479,7 +480,7 @@ __global__ void __launch_bounds__(kFThreads, 1) decode_ffn_kernel(const __grid_c
             for (int u = 0; u < 4; ++u) {
                 if (e[u] < 0) continue;
                 const int s = s0 + u * nth, i = (int)(((unsigned)s * inv_k) >> 18);
-                ids8[s] = (unsigned char)t[u];
+                slots[s] = (unsigned short)(e[u] << 8 | t[u]);
                 atomicOr(&tmask[r[u] * W + (i >> 5)], 1u << (i & 31));
                 if (meta) {
                     p.out_ids[s] = t[u];
@@ -738,8 +739,8 @@ __global__ void __launch_bounds__(kFThreads, 1) decode_ffn_kernel(const __grid_c
                     bool has = false;
                     for (int k = 0; k < K; ++k) {
                         const int s = tok * K + k;
-                        if (ids8[s] != it.expert) continue;  // duplicates merged, weights summed in slot order
-                        const int id = p.ids[s];
+                        const int id = slots[s] >> 8;
+                        if ((slots[s] & 255) != it.expert) continue;  // duplicates merged, weights summed in slot order
                         const float scl = is_static ? sc.scale[id] : (id == it.expert ? 1.0f : __ldg(p.S + (size_t)id * N + it.expert));
                         const float wv = (float)(p.w64[s] * (double)scl);
                         cw = has ? __fadd_rn(cw, wv) : wv;
@@ -809,13 +810,13 @@ int decode_ffn_alt(int B, int max_groups, int I, int sms) {
     return I % 96 == 0 ? 96 : 0;
 }
 
-// Shared-memory plan: [ring: stages x (token box + 32 KB of weights, 8 KB when all slices are 32 wide)][routing state][ids',
+// Shared-memory plan: [ring: stages x (token box + 32 KB of weights, 8 KB when all slices are 32 wide)][routing state][slots,
 // token masks]
 size_t decode_ffn_smem_plan(int B, int K, int N, int alt, int* stages, int* scratch_off, int* a_rows) {
     const int ar = std::min(kTileM, (B + 31) / 32 * 32);
     const int stage_bytes = decode_ffn_stage_bytes(ar, alt);
     const int mask_words = (B + 127) / 128 * 4;
-    const size_t scratch = kFScratchFixed + align16((size_t)B * K) + (size_t)(N + 1) * mask_words * 4;
+    const size_t scratch = kFScratchFixed + align16((size_t)B * K * 2) + (size_t)(N + 1) * mask_words * 4;
     const long avail = (long)kFSmemLimit - 1024 - (long)scratch;
     int st = (int)(avail / stage_bytes);
     if (st > kFMaxStages) st = kFMaxStages;
