@@ -148,7 +148,7 @@ EncodeTiledFn encode_fn() {
 
 constexpr int kMaxHostChunks = 4;  // host-buffer prefill: chunks of >= 2048 tokens in flight
 
-// bf16 matrix [rows][cols] row-major; box = box_rows x kGemmBK columns, swizzle as wide as a box row
+// bf16 matrix [rows][cols] row-major; box = box_rows x kGemmBK columns, 128-byte swizzle (a box row)
 bool make_tmap(CUtensorMap* m, const void* base, uint64_t rows, uint64_t cols, uint32_t box_rows) {
     EncodeTiledFn fn = encode_fn();
     if (!fn) return false;
@@ -157,7 +157,7 @@ bool make_tmap(CUtensorMap* m, const void* base, uint64_t rows, uint64_t cols, u
     cuuint32_t box[2] = {(cuuint32_t)kGemmBK, box_rows};
     cuuint32_t estr[2] = {1, 1};
     CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
-                    CU_TENSOR_MAP_INTERLEAVE_NONE, kGemmBK == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
+                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                     CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS;
@@ -305,7 +305,7 @@ int64_t expected_tiles(int64_t rows, int G) { return rows / kTileM + G / 2; }
 bool use_pairs(int64_t rows, int G, int d, int I) {
     const int64_t tiles = rows / kTileM;
     const int64_t kblocks = (int64_t)((I + 127) / 128) * (d / kGemmBK) + (int64_t)((d + 255) / 256) * (I / kGemmBK);
-    return kGemmBK == 64 && tiles >= G && expected_tiles(rows, G) >= 24 && tiles * kblocks >= (int64_t)400 * sm_count();
+    return tiles >= G && expected_tiles(rows, G) >= 24 && tiles * kblocks >= (int64_t)400 * sm_count();
 }
 
 // The two grouped GEMMs of bf16 expert rows (prefill, calibration): g = GEMM-1, g2 = GEMM-2 on `rows` sorted rows.
@@ -511,7 +511,7 @@ int exfold_moe_prefill_ex(const exfold_layer* layer, const void* x, const float*
 
     CUtensorMap tm_xs, tm_x, tm_wg, tm_wu, tm_h, tm_wd, tm_wd_half;
     const int mode = opts == nullptr || opts->gemm_path < 0 || opts->gemm_path > 2 ? 0 : opts->gemm_path;
-    const bool pairs = bf16 && !small && (mode == 2 ? kGemmBK == 64 && Rtot >= 2 * kTileM : mode == 0 && use_pairs(Rtot, G, d, I));
+    const bool pairs = bf16 && !small && (mode == 2 ? Rtot >= 2 * kTileM : mode == 0 && use_pairs(Rtot, G, d, I));
     const int sms = sm_count() & ~1;
     if (bf16 && !small) {
         const uint64_t E = (uint64_t)G;

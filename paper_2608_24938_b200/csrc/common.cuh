@@ -22,12 +22,7 @@ constexpr int kMaxExperts = 256;  // routed experts
 constexpr int kMaxTopK = 32;
 constexpr int kMaxGroups = kMaxExperts + 1;  // + shared expert
 constexpr int kTileM = 128;                  // token rows per prefill GEMM tile
-#ifndef EXFOLD_BK
-#define EXFOLD_BK 64
-#endif
-// K elements per pipeline stage of the tensor-core GEMMs: 64 (128-byte rows, 128-byte swizzle) or 32 (64-byte rows,
-// 64-byte swizzle: half the bytes per stage, so twice as many stages fit in shared memory)
-constexpr int kGemmBK = EXFOLD_BK;
+constexpr int kGemmBK = 64;  // K elements per pipeline stage of the tensor-core GEMMs: 128-byte rows, 128-byte swizzle
 constexpr int kMaxDecodeBatch = 256;
 constexpr int kMaxCtas = 160;                // persistent grids never exceed this (148 SMs on B200)
 
@@ -59,8 +54,8 @@ cudaError_t ensure_smem(void (*kernel)(KArgs...), size_t bytes) {
     return ensure_smem_bytes(reinterpret_cast<const void*>(kernel), bytes);
 }
 
-// Programmatic launch is requested per call chain: it pays for the short, latency-bound decode chain and
-// measured slower for prefill (early-resident successors compete with the running kernel).
+// Programmatic launch is requested per call chain: it pays for chains of short, latency-bound kernels and measured slower
+// where prefill runs CTA pairs (early-resident successors compete with the running kernel).
 void set_pdl(bool on);
 bool pdl_enabled();
 
@@ -500,7 +495,7 @@ struct GroupedGemmParams {
 cudaError_t launch_grouped_gemm1(const GroupedGemmParams& p, int grid, cudaStream_t s);
 cudaError_t launch_grouped_gemm2(const GroupedGemmParams& p, int grid, cudaStream_t s);
 // Prefill on CTA pairs: every group's row tiles two at a time (a last odd tile is left to the kernels above with
-// odd_only = 1). GEMM-2 needs tm_b1 = W_down with 128-row boxes. No grp_expert, no K split, o32 = null.
+// odd_only = 1). GEMM-2 needs tm_b1 = W_down with 128-row boxes. No grp_expert, no K split.
 cudaError_t launch_grouped_gemm1_pair(const GroupedGemmParams& p, int grid, cudaStream_t s);
 cudaError_t launch_grouped_gemm2_pair(const GroupedGemmParams& p, int grid, cudaStream_t s);
 // The odd-tile pass beside them (p.odd_only = 1; prefill instantiation), launched two CTAs at a time so that the two

@@ -67,7 +67,6 @@ constexpr int kGather = 2;
 constexpr int kFTmemCols = 512;
 constexpr int kFMaxPairs = 2 * kMaxGroups;      // (group, token tile) pairs: B <= 256 is at most two tiles
 constexpr int kFSmemLimit = 227 * 1024 - 2048;  // dynamic shared memory the kernel may ask for
-static_assert(kGemmBK == 64, "the decode FFN kernel stages 64 K elements per k-block");
 static_assert(kMaxDecodeBatch <= 256, "two token tiles per group at most");
 
 __host__ __device__ constexpr int decode_ffn_stage_bytes(int a_rows, int alt) {

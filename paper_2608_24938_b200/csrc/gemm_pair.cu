@@ -32,7 +32,6 @@ constexpr int kPSmem = kPStages * kPStageBytes + 4 * kStageOutBytes + 1024;
 constexpr int kPProducers = 2;
 constexpr int kPThreads = 192 + 32 * (kPProducers - 1);
 constexpr int kPTmemCols = 512;
-static_assert(kGemmBK == 64, "the pair kernel stages 64 K elements (one 128-byte swizzle row) per k-block");
 
 struct PairItem {
     int g, row0, rows1, n_idx;  // rows1: valid rows of the second tile (the first is always full)

@@ -23,23 +23,17 @@ namespace exfold {
 
 namespace {
 
-constexpr int kBK = kGemmBK;                  // K elements per stage: one swizzle row (128 or 64 bytes)
-#ifndef EXFOLD_STAGES
-#define EXFOLD_STAGES (EXFOLD_BK == 64 ? 4 : 9)
-#endif
-constexpr int kStages = EXFOLD_STAGES;
-constexpr int kMaxStages = kBK == 64 ? 6 : 12;  // decode loads a shorter A box per stage and fits more stages
+constexpr int kBK = kGemmBK;                  // K elements per stage: one swizzle row (128 bytes)
+constexpr int kStages = 4;
+constexpr int kMaxStages = 6;  // decode loads a shorter A box per stage and fits more stages
 constexpr int kATileBytes = kTileM * kBK * 2;  // 16 KB
 constexpr int kBTileBytes = 256 * kBK * 2;     // 32 KB
 constexpr int kStageBytes = kATileBytes + kBTileBytes;
 constexpr int kGemmSmem = kStages * kStageBytes + 4 * kStageOutBytes + 1024;
-#ifndef EXFOLD_PRODUCERS
-#define EXFOLD_PRODUCERS (EXFOLD_BK == 64 ? 2 : 3)
-#endif
 // One thread's loop {wait for the stage, expect_tx, 2-3 TMA issues} takes ~600-700 cycles: longer than the 512
 // cycles the tensor pipe needs for a k-block. The k-blocks are therefore dealt round-robin over kProducers
 // one-thread producers in warps of their own (warp 0 and the warps after the epilogue warps).
-constexpr int kProducers = EXFOLD_PRODUCERS;
+constexpr int kProducers = 2;
 constexpr int kGemmThreads = 192 + 32 * (kProducers - 1);
 constexpr int kTmemCols = 512;
 
@@ -243,8 +237,6 @@ __global__ void __launch_bounds__(kGemmThreads, 1) grouped_gemm_kernel(const __g
                         phase ^= 1;
                     }
                 }
-            }
-            if (me == 0) {
             }
         }
         __syncwarp();

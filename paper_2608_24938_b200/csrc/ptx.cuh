@@ -115,7 +115,7 @@ __device__ __forceinline__ void tc_fence_before() {
 __device__ __forceinline__ void tc_fence_after() {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 }
-// One k-block of the main loop in a single instruction sequence: issue kGemmBK/16 K=16 MMAs on this stage's operands,
+// One k-block of the main loop in a single instruction sequence: issue four K=16 MMAs on this stage's operands,
 // with a poll of `next_full` (the NEXT stage's operands) before the last of them (descriptor low words advance by 32 bytes = 2 per MMA;
 // `desc_hi` is the shared high word), commit to `empty`, and only then read the poll's predicate, so that the
 // poll's round trip overlaps the MMA issue. Returns whether the next stage was already complete.
@@ -136,11 +136,7 @@ __device__ __forceinline__ bool umma_kblock_bf16(uint32_t tmem_d, uint32_t a_lo,
         "add.u32 lb, %3, 2;\n"
         "mov.b64 da, {la, %4};\n"
         "mov.b64 db, {lb, %4};\n"
-#if EXFOLD_BK != 64
-        "mbarrier.try_wait.parity.shared::cta.b64 pr, [%8], %9;\n"
-#endif
         "tcgen05.mma.cta_group::1.kind::f16 [%1], da, db, %5, 1;\n"
-#if EXFOLD_BK == 64
         "add.u32 la, %2, 4;\n"
         "add.u32 lb, %3, 4;\n"
         "mov.b64 da, {la, %4};\n"
@@ -152,7 +148,6 @@ __device__ __forceinline__ bool umma_kblock_bf16(uint32_t tmem_d, uint32_t a_lo,
         "mov.b64 db, {lb, %4};\n"
         "mbarrier.try_wait.parity.shared::cta.b64 pr, [%8], %9;\n"
         "tcgen05.mma.cta_group::1.kind::f16 [%1], da, db, %5, 1;\n"
-#endif
         "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%7];\n"
         "selp.b32 %0, 1, 0, pr;\n"
         "}\n"
@@ -267,8 +262,8 @@ __device__ __forceinline__ void tmem_ld_wait() {
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
-// Shared-memory matrix descriptor for a K-major bf16 tile stored as rows of kGemmBK elements (128 or 64 bytes)
-// with the swizzle TMA applies (SWIZZLE_128B / SWIZZLE_64B): 8-row groups are 8 rows apart (1024 / 512 bytes).
+// Shared-memory matrix descriptor for a K-major bf16 tile stored as rows of kGemmBK elements (128 bytes)
+// with the swizzle TMA applies (SWIZZLE_128B): 8-row groups are 1024 bytes apart.
 // The tile base must be aligned to that group size. Advancing by 16 elements along K adds 32 bytes (>>4 = 2)
 // to the start-address field.
 __device__ __forceinline__ uint64_t make_kmajor_sw128_desc(uint32_t smem_addr) {
@@ -278,7 +273,7 @@ __device__ __forceinline__ uint64_t make_kmajor_sw128_desc(uint32_t smem_addr) {
     desc |= (uint64_t)0 << 16;                         // leading byte offset: unused for swizzled K-major
     desc |= (uint64_t)(group_bytes >> 4) << 32;        // stride byte offset between 8-row groups
     desc |= (uint64_t)1 << 46;                         // descriptor version for sm_100
-    desc |= (uint64_t)(kGemmBK == 64 ? 2 : 4) << 61;   // layout type: SWIZZLE_128B = 2, SWIZZLE_64B = 4
+    desc |= (uint64_t)2 << 61;                         // layout type: SWIZZLE_128B
     return desc;
 }
 

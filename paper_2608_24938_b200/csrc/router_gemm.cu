@@ -26,7 +26,6 @@ namespace cg = cooperative_groups;
 constexpr int kRThreads = 192;  // warp 0: TMA producer, warp 1: MMA issuer, warps 2-5: accumulator rows
 constexpr int kRMaxStages = 6;
 constexpr int kRBK = 64;
-static_assert(kGemmBK == 64, "the router kernel stages 64 K elements per k-block");
 
 // Bounded wait that looks at the CTA's own abort flag only
 __device__ __forceinline__ bool wait_local(uint64_t* bar, uint32_t parity, volatile int* abort_flag, DeviceStatus* st, int where) {
