@@ -338,11 +338,11 @@ def prefill_roofline(wl, Kp, kern, peaks, peak_src, touched):
                                 if ratio else "no ncu capture of this shape",
                 "peak_source": f"{peak_src} burst bf16 matmul", "launch_ms": r4(kern["gemm1_gateup_swiglu"]),
                 "flop_per_launch": f1, "algorithmic_bytes_per_launch": b1}
-    if "simt_ffn" in kern:
+    if "ffn_f32" in kern:
         flop = rows * 6.0 * d * I
-        ach = flop / (kern["simt_ffn"] * 1e-3) / 1e12
-        return {"kernel": "SIMT fp32 expert FFN", "bound": "alu", "achieved": r4(ach), "peak": 72.0,
-                "unit": "TFLOP/s", "frac": r4(ach / 72.0), "traffic": None, "launch_ms": r4(kern["simt_ffn"]),
+        ach = flop / (kern["ffn_f32"] * 1e-3) / 1e12
+        return {"kernel": "fp32 expert FFN (CUDA cores, clusters of 2 to 8 CTAs per row tile)", "bound": "alu", "achieved": r4(ach), "peak": 72.0,
+                "unit": "TFLOP/s", "frac": r4(ach / 72.0), "traffic": None, "launch_ms": r4(kern["ffn_f32"]),
                 "flop_per_launch": flop, "peak_source": "148 SMs x 128 fp32 lanes x 2 flop x 1.9 GHz"}
     return None
 
@@ -380,19 +380,6 @@ def decode_roofline(wl, kern, peaks, pool):
         if td > 0:
             out["down_gbs"] = r4(byts / 3.0 / td / 1e9)
             out["ffn_gbs"] = r4(byts / (t + td) / 1e9)
-        return out
-    if "decode_gateup" in kern:
-        gu = byts * 2.0 / 3.0
-        tg = kern["decode_gateup"] * 1e-3
-        ratio = NCU_TRAFFIC_RATIO.get(name, {}).get("decode_gateup")
-        out = {"kernel": "decode GEMM-1 (gate/up weight stream over the pool), tcgen05", "bound": "hbm",
-               "achieved": r4(gu / tg / 1e9), "peak": peaks["hbm_gbs"], "unit": "GB/s",
-               "frac": r4(gu / tg / 1e9 / peaks["hbm_gbs"]), "traffic": None if ratio is None else gu * ratio,
-               "bytes_per_launch": gu, "launch_ms": r4(kern["decode_gateup"])}
-        td = kern.get("decode_down", 0.0) * 1e-3
-        if td > 0:
-            out["down_gbs"] = r4(byts / 3.0 / td / 1e9)
-            out["ffn_gbs"] = r4(byts / (tg + td) / 1e9)
         return out
     return None
 

@@ -50,7 +50,7 @@ void prof_reset() {
 // ------------------------------------------------------------------ workspace plan
 struct Plan {
     size_t status, ids, w, omit_src, omit_tgt, block_hist, sb_hist, offsets, work_start, totals, perm, row_tok, row_w,
-        row_exp, pool_ids, pool_size, pool_mask, target, scale, grp_expert, grp_off, n_groups, calib, big,
+        row_grp, pool_ids, pool_size, pool_mask, target, scale, grp_expert, grp_off, n_groups, calib, big,
         xs, H, out, grp_tiles, obuf, inv_pos, calib_nrm, w64, total;
 };
 
@@ -91,7 +91,7 @@ Plan make_plan(const exfold_layer& l, int64_t Tm, int Kr) {
     p.inv_pos = take(Rm * 4);
     p.row_tok = take(Rtot * 4);
     p.row_w = take(Rtot * 4);
-    p.row_exp = take(Rtot * 4);
+    p.row_grp = take(Rtot * 4);  // small batches: group of each row
     p.w64 = take((size_t)std::min<int64_t>(Tm, kMaxDecodeBatch) * l.top_k * 8);  // decode: routed weights in double
     p.pool_ids = take((size_t)N * 4);
     p.pool_size = take(16);
@@ -575,7 +575,7 @@ int exfold_moe_prefill_ex(const exfold_layer* layer, const void* x, const float*
     cp.offsets = at<int32_t>(ws, pl.offsets); cp.work_start = at<int32_t>(ws, pl.work_start);
     cp.x = x; cp.xs = bf16 ? at<char>(ws, pl.xs) : nullptr;
     cp.perm = at<int32_t>(ws, pl.perm); cp.row_tok = at<int32_t>(ws, pl.row_tok);
-    cp.row_w = at<float>(ws, pl.row_w); cp.row_exp = at<int32_t>(ws, pl.row_exp);
+    cp.row_w = at<float>(ws, pl.row_w);
     cp.inv_pos = at<int32_t>(ws, pl.inv_pos);
     if (small) cp.xs = nullptr;  // the tokens are read in place; only the metadata needs the permutation
     if (!small || meta) { ProfScope ps(2, s); EXFOLD_CUDA(launch_prefill_scatter(cp, s)); }
@@ -587,7 +587,7 @@ int exfold_moe_prefill_ex(const exfold_layer* layer, const void* x, const float*
         sp.y = reinterpret_cast<__nv_bfloat16*>(y); sp.ids = rp.ids; sp.w_in = rp.w;
         sp.B = (int)T; sp.N = N; sp.K = Kp; sp.M = N; sp.n_shared = l.n_shared; sp.d = d; sp.I = I;
         sp.max_groups = (int)std::min<int64_t>(N, R) + l.n_shared; sp.max_rows = (int)Rtot;
-        sp.H = at<__nv_bfloat16>(ws, pl.H); sp.row_tok = cp.row_tok; sp.row_w = cp.row_w; sp.row_grp = cp.row_exp;
+        sp.H = at<__nv_bfloat16>(ws, pl.H); sp.row_tok = cp.row_tok; sp.row_w = cp.row_w; sp.row_grp = at<int32_t>(ws, pl.row_grp);
         sp.grp_expert = at<int32_t>(ws, pl.grp_expert); sp.n_groups = at<int32_t>(ws, pl.n_groups);
         ProfScope ps(3, s);
         EXFOLD_CUDA(launch_decode_small(sp, sm_count(), s));
@@ -716,7 +716,7 @@ static int decode_impl(const exfold_layer* layer, const void* x, const float* lo
                 sp.out_ids = out_ids; sp.out_w = rp.w; sp.target = rp.target; sp.scale = rp.scale;
             }
             sp.H = at<__nv_bfloat16>(ws, pl.H); sp.row_tok = rp.row_tok; sp.row_w = rp.row_w;
-            sp.row_grp = at<int32_t>(ws, pl.row_exp); sp.grp_expert = rp.grp_expert; sp.n_groups = rp.n_groups;
+            sp.row_grp = at<int32_t>(ws, pl.row_grp); sp.grp_expert = rp.grp_expert; sp.n_groups = rp.n_groups;
             sp.status = w_router == nullptr ? rp.status : nullptr;
             { ProfScope ps(14, s); EXFOLD_CUDA(launch_decode_small(sp, sm_count(), s)); }
         } else {
@@ -906,7 +906,7 @@ static int calibrate_enqueue(const exfold_layer* layer, const void* x_cal, const
         cp.offsets = offsets; cp.work_start = work_start;
         cp.x = x_cal; cp.xs = tensor_path ? at<char>(ws, pl.xs) : nullptr;
         cp.perm = at<int32_t>(ws, pl.perm); cp.row_tok = row_tok;
-        cp.row_w = at<float>(ws, pl.row_w); cp.row_exp = at<int32_t>(ws, pl.row_exp);
+        cp.row_w = at<float>(ws, pl.row_w);
         cp.inv_pos = at<int32_t>(ws, pl.inv_pos);
         cp.zero = at<int32_t>(ws, pl.calib); cp.zero_words = (int)(calib_bytes / 4);  // the pair sums
         EXFOLD_CUDA(launch_prefill_scatter(cp, s));

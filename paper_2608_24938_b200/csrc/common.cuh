@@ -202,7 +202,6 @@ struct PrefillScatterParams {
     int32_t* perm;      // [R]
     int32_t* row_tok;   // [R + T*n_shared]
     float* row_w;       // [R + T*n_shared]
-    int32_t* row_exp;   // [R + T*n_shared]
     int32_t* inv_pos;   // [R] sorted row of each route (inverse of perm); may be null
     int32_t* zero;      // words to clear on the way (calibration: the pair sums); may be null
     int zero_words;

@@ -299,14 +299,12 @@ __global__ void __launch_bounds__(kRouteThreads) prefill_scatter_kernel(PrefillS
         if (p.inv_pos != nullptr) p.inv_pos[route] = q;
         p.row_tok[q] = (int32_t)(route / Kp);
         p.row_w[q] = p.w[route];
-        p.row_exp[q] = p.ids[route];
     }
     if (p.n_shared && part == 0) {  // shared-expert rows follow the routed rows, identity order, weight 1
         const int64_t R = p.T * Kp;
         for (int t = threadIdx.x; t < ntok; t += blockDim.x) {
             p.row_tok[R + tok0 + t] = (int32_t)(tok0 + t);
             p.row_w[R + tok0 + t] = 1.0f;
-            p.row_exp[R + tok0 + t] = N;
         }
     }
     if (p.xs != nullptr && p.d_bytes > 0) {
