@@ -322,8 +322,8 @@ int exfold_moe_decode_host(const exfold_layer *layer, const void *x_host, const 
  * Limits and rules:
  *   - the call needs exfold_workspace_bytes(layer, B, layer->top_k) bytes of scratch; if that
  *     exceeds EXFOLD_STATIC_SCRATCH_BYTES it returns EXFOLD_ERR_EXCEEDS_STATIC_SCRATCH and launches
- *     nothing (e.g. Qwen3- and Mixtral-shaped layers fit up to B = 64, the GLM-4.5-Air-shaped
- *     one up to B = 32);
+ *     nothing (e.g. a Qwen3-shaped layer fits up to B = 101, a Mixtral-shaped one up to 92, the GLM-4.5-Air-shaped
+ *     one up to 45);
  *   - it calls no cudaMalloc, cudaFree or any allocating library routine;
  *   - the first call on each device looks up the array's device address (with that device
  *     current); make that first call outside any stream capture;
