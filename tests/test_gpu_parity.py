@@ -27,7 +27,7 @@ def calibrated_tables(case, cfg, lam=1e-3):
     return xc, lc, cal
 
 
-# ------------------------------------------------------------------ fp32 tiny layer 
+# ------------------------------------------------------------------ fp32 tiny layer
 @pytest.mark.parametrize("correlated", [0.0, 0.8])
 def test_tiny_fp32_layer(correlated):
     cfg = TINY
