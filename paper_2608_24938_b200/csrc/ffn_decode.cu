@@ -194,7 +194,7 @@ __global__ void __launch_bounds__(kFThreads, 1) decode_ffn_kernel(const __grid_c
 
     unsigned char* tiles =
         reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = ptx::warp_index(), lane = threadIdx.x & 31;
     const int stages = p.stages;
     const int a_bytes = p.a_rows * kFBK * 2;
     const int stage_bytes = decode_ffn_stage_bytes(p.a_rows, p.alt);
@@ -598,7 +598,7 @@ __global__ void __launch_bounds__(kFThreads, 1) decode_ffn_kernel(const __grid_c
         const int me = warp == 0 ? 0 : 1;
         int stage = 0, phase = 0, turn = 0;
         int ok = 1;
-        if (NMT == 2 || lane == 0) {  // a whole warp where rows are gathered
+        if (NMT == 2 || ptx::elect_one()) {  // a whole warp where rows are gathered
             for (int w = w_begin; w < total && ok; w += w_stride) {
                 const Item it = decode_item(w, sched, sc, N);
                 int n4 = 0;  // groups of four rows to gather
@@ -615,7 +615,7 @@ __global__ void __launch_bounds__(kFThreads, 1) decode_ffn_kernel(const __grid_c
                     if (lane < 4 * n4 - n) s_rows[me][n + lane] = s_rows[me][0];  // the last four filled up
                     __syncwarp();
                 }
-                if (lane == 0) {
+                if (NMT == 1 || ptx::elect_one()) {
                     const int xrow = NMT == 2 && it.mt == 1 ? 128 : 0;
                     const int wrow = it.expert * p.I + it.j0;
                     const uint32_t tx = (uint32_t)((n4 > 0 ? n4 * 512 : a_bytes) + 2 * it.s * kFBK * 2);
@@ -657,7 +657,7 @@ __global__ void __launch_bounds__(kFThreads, 1) decode_ffn_kernel(const __grid_c
         __syncwarp();
     } else if (warp == 1) {
         // ------------------------------------------------ MMA issuer
-        if (lane == 0) {
+        if (ptx::elect_one()) {
             const uint32_t lo0 = (ptx::smem_u32(tiles) & 0x3FFFFu) >> 4;
             const uint32_t lo_step = (uint32_t)stage_bytes >> 4, lo_b = (uint32_t)a_bytes >> 4;
             const uint32_t desc_hi32 = (uint32_t)(ptx::make_kmajor_sw128_desc(0) >> 32);

@@ -83,7 +83,7 @@ __global__ void __launch_bounds__(kPThreads, 1) grouped_gemm_pair_kernel(const _
 
     unsigned char* tiles =
         reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = ptx::warp_index(), lane = threadIdx.x & 31;
     const int rank = (int)ptx::cluster_ctarank();  // 0 = leader
     const int pair_id = (int)blockIdx.x >> 1, n_launched = (int)gridDim.x >> 1;
     // GEMM-1: the leader stages W_gate rows, its peer W_up rows; GEMM-2: both halves come from W_down (tm_b1: 128-row box)
@@ -173,7 +173,7 @@ __global__ void __launch_bounds__(kPThreads, 1) grouped_gemm_pair_kernel(const _
 
     if (warp == 0 || warp == 6) {
         // ------------------------------------------------ TMA producers (both CTAs; k-block c belongs to producer c % 2)
-        if (lane == 0) {
+        if (ptx::elect_one()) {
             const int me = warp == 0 ? 0 : 1;
             int stage = 0, phase = 0, turn = 0;
             bool ok = true;
@@ -206,7 +206,7 @@ __global__ void __launch_bounds__(kPThreads, 1) grouped_gemm_pair_kernel(const _
         __syncwarp();
     } else if (warp == 1) {
         // ------------------------------------------------ MMA issuer (leader CTA only)
-        if (lane == 0 && rank == 0) {
+        if (rank == 0 && ptx::elect_one()) {
             constexpr uint32_t idesc = ptx::make_idesc_bf16(256, 256);
             const uint32_t lo0 = (ptx::smem_u32(tiles) & 0x3FFFFu) >> 4;
             constexpr uint32_t lo_step = (uint32_t)kPStageBytes >> 4, lo_b = (uint32_t)kPATileBytes >> 4;

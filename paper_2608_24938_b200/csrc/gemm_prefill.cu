@@ -96,7 +96,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) grouped_gemm_kernel(const __g
 
     unsigned char* tiles =
         reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = ptx::warp_index(), lane = threadIdx.x & 31;
     // ---- prologue that does not depend on earlier kernels: overlaps their tail under programmatic launch
     if (threadIdx.x == 0) {
         ptx::prefetch_tmap(&p.tm_a);
@@ -204,7 +204,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) grouped_gemm_kernel(const __g
 
     if (warp == 0 || warp >= 6) {
         // ------------------------------------------------ TMA producers (k-block c belongs to producer c % kProducers)
-        if (lane == 0) {
+        if (ptx::elect_one()) {
             const int me = warp == 0 ? 0 : warp - 5;
             int stage = 0, phase = 0, turn = 0;
             bool ok = true;
@@ -242,7 +242,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) grouped_gemm_kernel(const __g
         __syncwarp();
     } else if (warp == 1) {
         // ------------------------------------------------ MMA issuer
-        if (lane == 0) {
+        if (ptx::elect_one()) {
             constexpr uint32_t idesc = ptx::make_idesc_bf16(128, n_cols);
             int stage = 0, phase = 0, iter = 0;
             // This one thread's instruction stream paces the tensor pipe (a k-block is 4 MMAs = 512 pipe cycles),

@@ -53,7 +53,7 @@ __global__ void __launch_bounds__(kRThreads, 1) router_gemm_kernel(const __grid_
     __shared__ int abort_s;
     unsigned char* tiles =
         reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = ptx::warp_index(), lane = threadIdx.x & 31;
     cg::cluster_group cluster = cg::this_cluster();
     const int split = p.split, rank = (int)cluster.block_rank();
     const int row0 = (int)blockIdx.x / split * 128;
@@ -83,7 +83,7 @@ __global__ void __launch_bounds__(kRThreads, 1) router_gemm_kernel(const __grid_
     const int a_bytes = 128 * kRBK * 2, stage_bytes = a_bytes + p.npad * kRBK * 2;
 
     if (warp == 0) {
-        if (lane == 0) {
+        if (ptx::elect_one()) {
             int stage = 0, phase = 0;
             for (int kb = kb0; kb < kb1; ++kb) {
                 if (!wait_local(&empty_bar[stage], phase ^ 1, abort_flag, p.status, 1)) break;
@@ -99,7 +99,7 @@ __global__ void __launch_bounds__(kRThreads, 1) router_gemm_kernel(const __grid_
         }
         __syncwarp();
     } else if (warp == 1) {
-        if (lane == 0) {
+        if (ptx::elect_one()) {
             const uint32_t idesc = ptx::make_idesc_bf16(128, p.npad);
             const uint32_t lo0 = (ptx::smem_u32(tiles) & 0x3FFFFu) >> 4;
             const uint32_t hi = (uint32_t)(ptx::make_kmajor_sw128_desc(0) >> 32);
