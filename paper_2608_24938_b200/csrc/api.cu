@@ -365,6 +365,39 @@ int enqueue_expert_gemms(GroupedGemmParams& g, GroupedGemmParams& g2, int64_t ro
     return EXFOLD_OK;
 }
 
+// The same GEMMs on the mixed kernel (gemm_mixed.cu): one launch each on the caller's stream. x, w_gate, w_up: the matrices
+// behind g.tm_a2, tm_b0 and tm_b1; `experts` of them.
+int enqueue_mixed_gemms(const GroupedGemmParams& g, const GroupedGemmParams& g2, const void* xs, int64_t R, int64_t rows,
+                        const void* x, const void* w_gate, const void* w_up, int experts, cudaStream_t s) {
+    MixedGemmParams m1{}, m2{};
+    m1.g = g;
+    m2.g = g2;
+    const uint64_t wrows = (uint64_t)experts * g.I;
+    if (!make_tmap(&m1.tm_b0_half, w_gate, wrows, g.d, 64) || !make_tmap(&m1.tm_b1_half, w_up, wrows, g.d, 64)) return EXFOLD_ERR_CUDA;
+    for (int i = 0; i < 3; ++i)
+        if (!make_tmap(&m1.tm_a_part[i], xs, (uint64_t)R, g.d, 64 >> i) || !make_tmap(&m1.tm_x_part[i], x, (uint64_t)g.x_rows, g.d, 64 >> i) ||
+            !make_tmap(&m2.tm_a_part[i], g.H, (uint64_t)rows, g.I, 64 >> i))
+            return EXFOLD_ERR_CUDA;
+    m1.queue = &g.status->queue[0];
+    m2.queue = &g.status->queue[1];
+    { ProfScope ps(3, s); EXFOLD_CUDA(launch_grouped_gemm1_mixed(m1, sm_count(), s)); }
+    { ProfScope ps(4, s); EXFOLD_CUDA(launch_grouped_gemm2_mixed(m2, sm_count(), s)); }
+    return EXFOLD_OK;
+}
+
+// Whether they do. The mixed kernel computes and loads what a group's rows need, where row tiles of 128 rows waste half a tile
+// per group, and reads a weight tile once; but it has half as many workers (CTA pairs), and an item costs a pair more to hand over.
+// So it wants a few rounds of items, and long ones (48 k-blocks of GEMM-1 and more) or groups of most of a row tile and more.
+// With eight row tiles per group and more, the waste is small and the passes side by side on their own SMs are as fast.
+// Measured, whole prefill call on row tiles / mixed: GLM shape (K' = 4) 48 tokens 502 / 478 us, 768 768 / 727, 3072 972 / 863,
+// 12288 2391 / 2222; Mixtral shape (K' = 1) 192 tokens 466 / 443, 1536 750 / 567, 3072 1301 / 1231; Qwen3 shape (K' = 4) 384
+// tokens 110 / 123, 1536 164 / 167, 3072 225 / 216, 6144 351 / 326; 64 experts of 1024 x 512 (K' = 4) 768 tokens 64 / 71, 6144
+// 142 / 140; 16 of 2048 x 2048 (K' = 2) 384 tokens 90 / 96, 3072 194 / 172; 11 of 2688 x 512 (K' = 3) 768 tokens 58 / 65.
+bool use_mixed(int64_t rows, int G, int d, int I) {
+    const int64_t items = (int64_t)G * ((I + 127) / 128) * std::max<int64_t>(1, rows / (256 * (int64_t)G));
+    return rows / kTileM < (int64_t)8 * G && items >= (int64_t)3 * sm_count() && (d >= 48 * kGemmBK || rows >= (int64_t)96 * G);
+}
+
 struct PdlScope {  // programmatic dependent launch for the launches of this scope
     explicit PdlScope(bool on) { set_pdl(on); }
     ~PdlScope() { set_pdl(false); }
@@ -512,6 +545,7 @@ int exfold_moe_prefill_ex(const exfold_layer* layer, const void* x, const float*
     CUtensorMap tm_xs, tm_x, tm_wg, tm_wu, tm_h, tm_wd, tm_wd_half;
     const int mode = opts == nullptr || opts->gemm_path < 0 || opts->gemm_path > 2 ? 0 : opts->gemm_path;
     const bool pairs = bf16 && !small && (mode == 2 ? Rtot >= 2 * kTileM : mode == 0 && use_pairs(Rtot, G, d, I));
+    const bool mixed = bf16 && !small && mode == 0 && use_mixed(Rtot, G, d, I);
     const int sms = sm_count() & ~1;
     if (bf16 && !small) {
         const uint64_t E = (uint64_t)G;
@@ -527,7 +561,7 @@ int exfold_moe_prefill_ex(const exfold_layer* layer, const void* x, const float*
     // programmatic dependent launch hides their launches and set-up (Qwen3 shape 20 tokens 66.8 -> 56.5 us, 777 tokens 279
     // -> 270; Mixtral shape 200 tokens 532 -> 514). The large calls launch plainly: early-resident successors compete with
     // the running kernels (19-32 us slower).
-    PdlScope pdl_scope(!pairs);
+    PdlScope pdl_scope(!pairs || mixed);
 
     PrefillRouteParams rp{};
     rp.logits = logits; rp.S = tables->S; rp.L = tables->L; rp.lnh = tables->lnh;
@@ -541,6 +575,7 @@ int exfold_moe_prefill_ex(const exfold_layer* layer, const void* x, const float*
     rp.sb_hist = at<int32_t>(ws, pl.sb_hist);
     // the first kernel of the call clears the status record (not for the later chunks of a chunked host call)
     rp.status = t_keep_status ? nullptr : at<DeviceStatus>(ws, pl.status);
+    rp.queue = mixed ? at<DeviceStatus>(ws, pl.status)->queue : nullptr;
     { ProfScope ps(0, s); EXFOLD_CUDA(launch_prefill_route(rp, s)); }
 
     // The shared expert's gate/up projection needs nothing the routing kernels produce (its rows are x itself, its
@@ -569,7 +604,7 @@ int exfold_moe_prefill_ex(const exfold_layer* layer, const void* x, const float*
 
     PrefillScatterParams cp{};
     cp.T = T; cp.N = N; cp.n_shared = l.n_shared; cp.Kp = Kp; cp.d_bytes = bf16 ? d * 2 : 0;
-    cp.tile_rows = bf16 ? kTileM : ffn_f32_tile_rows(Rtot, G, d, I);
+    cp.tile_rows = mixed ? kMixedTiles : bf16 ? kTileM : ffn_f32_tile_rows(Rtot, G, d, I);
     cp.nblk = (int)((T + kRouteTokensPerBlock - 1) / kRouteTokensPerBlock);
     cp.ids = rp.ids; cp.w = rp.w; cp.block_hist = rp.block_hist; cp.sb_hist = rp.sb_hist;
     cp.offsets = at<int32_t>(ws, pl.offsets); cp.work_start = at<int32_t>(ws, pl.work_start);
@@ -609,7 +644,9 @@ int exfold_moe_prefill_ex(const exfold_layer* layer, const void* x, const float*
             g.shared_split = 2;
             EXFOLD_CUDA(cudaStreamWaitEvent(s, early_side->mid, 0));
         }
-        if ((rc = enqueue_expert_gemms(g, g2, Rtot, pairs, shared_pairs, s)) != EXFOLD_OK) return rc;
+        rc = mixed ? enqueue_mixed_gemms(g, g2, at<char>(ws, pl.xs), R, Rtot, x, w_gate, w_up, G, s)
+                   : enqueue_expert_gemms(g, g2, Rtot, pairs, shared_pairs, s);
+        if (rc != EXFOLD_OK) return rc;
         early_join.armed = false;  // the passes above have joined the second stream
         if (!direct) {
             ProfScope ps(5, s);
@@ -871,7 +908,8 @@ static int calibrate_enqueue(const exfold_layer* layer, const void* x_cal, const
     if (!counts) return EXFOLD_ERR_CUDA;
     const bool tensor_path = l.dtype == EXFOLD_BF16;
     const bool pairs = tensor_path && use_pairs(m * Ke, N, d, I);
-    PdlScope pdl_scope(!pairs);  // as in prefill: a chain of kernels of which most are short
+    const bool mixed = tensor_path && use_mixed(m * Ke, N, d, I);
+    PdlScope pdl_scope(!pairs || mixed);  // as in prefill: a chain of kernels of which most are short
     DeviceStatus* status = at<DeviceStatus>(ws, pl.status);
     int32_t* ids = at<int32_t>(ws, pl.ids);
     if (opts->mode == 0) {
@@ -883,6 +921,7 @@ static int calibrate_enqueue(const exfold_layer* layer, const void* x_cal, const
         rp.omit_src = nullptr; rp.omit_tgt = nullptr; rp.block_hist = at<int32_t>(ws, pl.block_hist);
         rp.sb_hist = at<int32_t>(ws, pl.sb_hist);
         rp.status = status;
+        rp.queue = mixed ? status->queue : nullptr;
         EXFOLD_CUDA(launch_prefill_route(rp, s));
     } else {
         EXFOLD_CUDA(cudaMemsetAsync(status, 0, sizeof(DeviceStatus), s));
@@ -896,7 +935,7 @@ static int calibrate_enqueue(const exfold_layer* layer, const void* x_cal, const
     int32_t* offsets = at<int32_t>(ws, pl.offsets);
     int32_t* work_start = at<int32_t>(ws, pl.work_start);
     int32_t* row_tok = at<int32_t>(ws, pl.row_tok);
-    const int tile_rows = tensor_path ? kTileM : ffn_f32_tile_rows(Rc, N, d, I);
+    const int tile_rows = mixed ? kMixedTiles : tensor_path ? kTileM : ffn_f32_tile_rows(Rc, N, d, I);
     if (opts->mode == 0) {
         PrefillScatterParams cp{};
         cp.T = m; cp.N = N; cp.n_shared = 0; cp.Kp = K; cp.d_bytes = tensor_path ? d * 2 : 0; cp.tile_rows = tile_rows;
@@ -936,7 +975,8 @@ static int calibrate_enqueue(const exfold_layer* layer, const void* x_cal, const
         GroupedGemmParams g2 = g;
         g2.tm_a = tm_h; g2.tm_b0 = tm_wd; g2.tm_b1 = tm_wd_half; g2.n_ntiles = (d + 255) / 256;
         g2.o32 = at<float>(ws, pl.xs);  // spans the xs and obuf regions (GEMM-1 is done with xs)
-        const int rc = enqueue_expert_gemms(g, g2, Rc, pairs, 0, s);
+        const int rc = mixed ? enqueue_mixed_gemms(g, g2, at<char>(ws, pl.xs), Rc, Rc, x_cal, w_gate, w_up, N, s)
+                             : enqueue_expert_gemms(g, g2, Rc, pairs, 0, s);
         if (rc != EXFOLD_OK) return rc;
         cs.out = g2.o32;
     } else {

@@ -376,7 +376,7 @@ __global__ void calib_common_rows_kernel(int32_t* offsets, int32_t* work_start, 
     const int g = blockIdx.x * blockDim.x + threadIdx.x;
     if (g <= N) {
         offsets[g] = (int32_t)(g * m);
-        work_start[g] = (int32_t)(g * ((m + tile_rows - 1) / tile_rows));
+        work_start[g] = (int32_t)(g * row_tiles((int)m, tile_rows));
     }
 }
 

@@ -14,7 +14,9 @@ struct DeviceStatus {
     int code;    // 0 or EXFOLD_ERR_DEVICE_TIMEOUT
     int where;   // which wait gave up (kernel-specific tag)
     int detail;  // block index
-    int pad[61];
+    int pad0;
+    int queue[2];  // work counters of the mixed GEMMs, cleared by the call's routing kernel
+    int pad[58];
 };
 static_assert(sizeof(DeviceStatus) == 256, "status record is 256 bytes");
 
@@ -178,6 +180,7 @@ struct PrefillRouteParams {
     int32_t* sb_hist;     // [ceil(nblk / kRouteSuperBlock)][N] retained routes per (super-block, expert); the
                           //   launcher clears it, the blocks add to it (not with a single super-block)
     DeviceStatus* status; // cleared by block 0 (first kernel of a call); may be null
+    int* queue;           // DeviceStatus::queue, cleared by block 0; may be null
 };
 constexpr int kRouteTokensPerBlock = 32;
 constexpr int kRouteThreads = 512;
@@ -185,11 +188,21 @@ constexpr int kRouteMaxThreads = 1024;  // a warp per token of the block
 constexpr int kRouteFewBlocks = 148;    // up to this many blocks the kernels spread them over more threads or blocks
 constexpr int kRouteSuperBlock = 64;  // blocks per super-block of the two-level histogram
 
+// Row tiles of a group for the mixed GEMMs (gemm_mixed.cu): whole 256-row items, and one ragged item of the rest. A rest above
+// kRaggedMax rows takes a whole item's time as it is: masked rows of a whole item.
+constexpr int kRaggedMax = 224;
+constexpr int kMixedTiles = 0;  // as tile_rows: the work list counts these
+__host__ __device__ inline int whole_items(int rows) { return rows / 256 + (rows % 256 > kRaggedMax ? 1 : 0); }
+__host__ __device__ inline int ragged_rows(int rows) { return rows % 256 > kRaggedMax ? 0 : rows % 256; }
+__host__ __device__ inline int row_tiles(int rows, int tile_rows) {
+    return tile_rows == kMixedTiles ? whole_items(rows) + (ragged_rows(rows) > 0 ? 1 : 0) : (rows + tile_rows - 1) / tile_rows;
+}
+
 struct PrefillScatterParams {
     int64_t T;
     int N, n_shared, Kp, d_bytes;  // d_bytes: bytes of one x row (0: no gather)
     int nblk;                   // blocks of the route kernel (= blocks of this kernel)
-    int tile_rows;              // rows per tile of the work list (kTileM, or the fp32 FFN's)
+    int tile_rows;              // rows per tile of the work list (kTileM, the fp32 FFN's, or kMixedTiles)
     int split;                  // blocks per token block (set by the launcher)
     const int32_t* ids;         // [T][Kp]
     const float* w;             // [T][Kp]
@@ -501,5 +514,17 @@ cudaError_t launch_grouped_gemm2_pair(const GroupedGemmParams& p, int grid, cuda
 // grids share the GPU by whole SM pairs
 cudaError_t launch_grouped_gemm1_odd(const GroupedGemmParams& p, int grid, cudaStream_t s);
 cudaError_t launch_grouped_gemm2_odd(const GroupedGemmParams& p, int grid, cudaStream_t s);
+
+// Whole 256-row tiles and ragged remainders of every group in one dynamically scheduled pass over CTA pairs (gemm_mixed.cu)
+struct MixedGemmParams {
+    GroupedGemmParams g;       // work_start counts kMixedTiles; tm_b1: W_down with 128-row boxes (GEMM-2)
+    CUtensorMap tm_a_part[3];  // tm_a's matrix with boxes of 64, 32 and 16 rows
+    CUtensorMap tm_x_part[3];  // tm_a2's (GEMM-1)
+    CUtensorMap tm_b0_half;    // W_gate and W_up with 64-row boxes (GEMM-1)
+    CUtensorMap tm_b1_half;
+    int* queue;                // work counter, zero at the start
+};
+cudaError_t launch_grouped_gemm1_mixed(const MixedGemmParams& p, int grid, cudaStream_t s);
+cudaError_t launch_grouped_gemm2_mixed(const MixedGemmParams& p, int grid, cudaStream_t s);
 
 }  // namespace exfold

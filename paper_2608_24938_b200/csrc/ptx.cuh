@@ -48,15 +48,32 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
     return ok != 0;
 }
 
+// The same with cluster scope: what a thread of another CTA read or wrote before it arrived is done
+__device__ __forceinline__ bool mbar_try_wait_cluster(uint64_t* bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n"
+        ".reg .pred p;\n"
+        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
+        "selp.b32 %0, 1, 0, p;\n"
+        "}\n"
+        : "=r"(ok)
+        : "r"(smem_u32(bar)), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+
 constexpr uint64_t kWaitLimitNs = 2000000000ull;  // 2 s per wait, far above any legitimate wait here
 
 // Bounded wait. `abort_flag` is a CTA-local shared word set by whoever gives up first.
+template <bool CLUSTER = false>
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
                                           DeviceStatus* st, int where) {
-    if (mbar_try_wait(bar, parity)) return true;
+    auto poll = [&]() { return CLUSTER ? mbar_try_wait_cluster(bar, parity) : mbar_try_wait(bar, parity); };
+    if (poll()) return true;
     uint64_t t0 = 0;
     for (uint32_t it = 1;; ++it) {
-        if (mbar_try_wait(bar, parity)) return true;
+        if (poll()) return true;
         if ((it & 255u) == 0u) {
             if (*abort_flag) return false;
             if (((volatile int*)&st->code)[0] != 0) {
@@ -206,9 +223,28 @@ __device__ __forceinline__ void umma_commit_pair(uint64_t* bar, uint16_t cta_mas
         ::"r"(smem_u32(bar)), "h"(cta_mask)
         : "memory");
 }
-// Arrive on the leader CTA's barrier at `bar`'s offset (from either CTA of the pair)
+// Arrive on the leader CTA's barrier at `bar`'s offset (from either CTA of the pair). Relaxed: it hands over accumulators whose
+// loads are complete, no memory; a release would wait for the thread's global stores.
 __device__ __forceinline__ void mbar_arrive_leader(uint64_t* bar) {
-    asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(smem_u32(bar) & kPeerBitMask) : "memory");
+    asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(smem_u32(bar) & kPeerBitMask) : "memory");
+}
+// The same as a release: what this thread read or wrote before is done
+__device__ __forceinline__ void mbar_arrive_leader_cluster(uint64_t* bar) {
+    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(smem_u32(bar) & kPeerBitMask) : "memory");
+}
+// Address of this CTA's shared-memory offset in CTA `rank` of the cluster
+__device__ __forceinline__ uint32_t mapa(const void* p, uint32_t rank) {
+    uint32_t a;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
+    return a;
+}
+// 16 bytes to this CTA's shared-memory offset in CTA `rank` of the cluster; `bar` there counts one arrival and the bytes
+__device__ __forceinline__ void st_async(void* dst, const int4& v, uint64_t* bar, uint32_t rank) {
+    const uint32_t b = mapa(bar, rank);
+    asm volatile("mbarrier.arrive.expect_tx.release.cluster.shared::cluster.b64 _, [%0], 16;" ::"r"(b) : "memory");
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(mapa(dst, rank)),
+                 "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w), "r"(b)
+                 : "memory");
 }
 // The pair form of umma_kblock_bf16 (K = 64 per stage): four M256 MMAs over both CTAs, the commit frees the stage in
 // both CTAs (`empty` at the same offset in each).
@@ -273,6 +309,17 @@ __device__ __forceinline__ void tmem_ld_wait() {
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
+// The same wait, for loads that are in flight while other work is done: what uses v comes after it
+__device__ __forceinline__ void tmem_ld_wait(uint32_t (&v)[32]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7]), "+r"(v[8]),
+                   "+r"(v[9]), "+r"(v[10]), "+r"(v[11]), "+r"(v[12]), "+r"(v[13]), "+r"(v[14]), "+r"(v[15]), "+r"(v[16]),
+                   "+r"(v[17]), "+r"(v[18]), "+r"(v[19]), "+r"(v[20]), "+r"(v[21]), "+r"(v[22]), "+r"(v[23]), "+r"(v[24]),
+                   "+r"(v[25]), "+r"(v[26]), "+r"(v[27]), "+r"(v[28]), "+r"(v[29]), "+r"(v[30]), "+r"(v[31])
+                 :
+                 : "memory");
+}
+
 // Shared-memory matrix descriptor for a K-major bf16 tile stored as rows of kGemmBK elements (128 bytes)
 // with the swizzle TMA applies (SWIZZLE_128B): 8-row groups are 1024 bytes apart.
 // The tile base must be aligned to that group size. Advancing by 16 elements along K adds 32 bytes (>>4 = 2)
@@ -311,14 +358,34 @@ __device__ __forceinline__ void stage_flush(const unsigned char* buf, int lane, 
                                             size_t row_bytes) {
     __syncwarp();
     const int c = lane & 7;
+    uint4 v[8];  // all of them read before the first store: the compiler cannot tell shared memory from dst
+#pragma unroll
+    for (int it = 0; it < 8; ++it) {
+        const int r = it * 4 + (lane >> 3);
+        v[it] = *reinterpret_cast<const uint4*>(buf + r * 128 + ((c ^ (r & 7)) << 4));
+    }
 #pragma unroll
     for (int it = 0; it < 8; ++it) {
         const int r = it * 4 + (lane >> 3);
         const int target = __shfl_sync(0xffffffffu, row, r);
-        if ((valid >> r) & 1u)
-            *reinterpret_cast<uint4*>(dst + (size_t)target * row_bytes + c * 16) =
-                *reinterpret_cast<const uint4*>(buf + r * 128 + ((c ^ (r & 7)) << 4));
+        if ((valid >> r) & 1u) *reinterpret_cast<uint4*>(dst + (size_t)target * row_bytes + c * 16) = v[it];
     }
+    __syncwarp();
+}
+// The same with the lanes' rows one after another: row r of the warp goes to dst + r * row_bytes
+__device__ __forceinline__ void stage_flush_rows(const unsigned char* buf, int lane, unsigned valid, char* dst, size_t row_bytes) {
+    __syncwarp();
+    const int c = lane & 7;
+    dst += (size_t)(lane >> 3) * row_bytes + c * 16;
+    uint4 v[8];
+#pragma unroll
+    for (int it = 0; it < 8; ++it) {
+        const int r = it * 4 + (lane >> 3);
+        v[it] = *reinterpret_cast<const uint4*>(buf + r * 128 + ((c ^ (r & 7)) << 4));
+    }
+#pragma unroll
+    for (int it = 0; it < 8; ++it)
+        if ((valid >> (it * 4 + (lane >> 3))) & 1u) *reinterpret_cast<uint4*>(dst + (size_t)(it * 4) * row_bytes) = v[it];
     __syncwarp();
 }
 

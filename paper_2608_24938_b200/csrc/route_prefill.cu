@@ -32,6 +32,7 @@ __global__ void __launch_bounds__(kRouteMaxThreads) prefill_route_kernel(Prefill
     __syncthreads();
     grid_dep_wait();
     if (p.status != nullptr && blockIdx.x == 0 && threadIdx.x < 4) reinterpret_cast<int*>(p.status)[threadIdx.x] = 0;
+    if (p.queue != nullptr && blockIdx.x == 0 && threadIdx.x < 2) p.queue[threadIdx.x] = 0;
 
     const int N = p.N, K = p.K, Kp = p.Kp, Ko = p.K - p.Kp;
     const int64_t tok0 = (int64_t)blockIdx.x * kRouteTokensPerBlock;
@@ -258,7 +259,7 @@ __global__ void __launch_bounds__(kRouteThreads) prefill_scatter_kernel(PrefillS
         const int off = block_prefix(rows, N, warp_tot, &all_rows);
         if (e < N) cnt[e] = off + pre[e];
         if (blockIdx.x == 0) {  // group offsets and the row-tile prefix for the GEMM work list
-            const int tiles = (rows + p.tile_rows - 1) / p.tile_rows;
+            const int tiles = row_tiles(rows, p.tile_rows);
             const int tile0 = block_prefix(tiles, N, warp_tot, &all_tiles);
             if (e < N) {
                 p.offsets[e] = off;
@@ -269,7 +270,7 @@ __global__ void __launch_bounds__(kRouteThreads) prefill_scatter_kernel(PrefillS
                 p.work_start[N] = all_tiles;
                 if (p.n_shared) {
                     p.offsets[N + 1] = all_rows + (int)p.T;
-                    p.work_start[N + 1] = all_tiles + (int)((p.T + p.tile_rows - 1) / p.tile_rows);
+                    p.work_start[N + 1] = all_tiles + row_tiles((int)p.T, p.tile_rows);
                 }
             }
         }
