@@ -387,15 +387,16 @@ int enqueue_mixed_gemms(const GroupedGemmParams& g, const GroupedGemmParams& g2,
 
 // Whether they do. The mixed kernel computes and loads what a group's rows need, where row tiles of 128 rows waste half a tile
 // per group, and reads a weight tile once; but it has half as many workers (CTA pairs), and an item costs a pair more to hand over.
-// So it wants a few rounds of items, and long ones (48 k-blocks of GEMM-1 and more) or groups of most of a row tile and more.
+// So it wants a few rounds of items, and long ones (48 k-blocks of GEMM-1 and more) or groups of a few rows and more.
 // With eight row tiles per group and more, the waste is small and the passes side by side on their own SMs are as fast.
 // Measured, whole prefill call on row tiles / mixed: GLM shape (K' = 4) 48 tokens 502 / 478 us, 768 768 / 727, 3072 972 / 863,
-// 12288 2391 / 2222; Mixtral shape (K' = 1) 192 tokens 466 / 443, 1536 750 / 567, 3072 1301 / 1231; Qwen3 shape (K' = 4) 384
-// tokens 110 / 123, 1536 164 / 167, 3072 225 / 216, 6144 351 / 326; 64 experts of 1024 x 512 (K' = 4) 768 tokens 64 / 71, 6144
-// 142 / 140; 16 of 2048 x 2048 (K' = 2) 384 tokens 90 / 96, 3072 194 / 172; 11 of 2688 x 512 (K' = 3) 768 tokens 58 / 65.
+// 12288 2391 / 2222; Mixtral shape (K' = 1) 192 tokens 466 / 443, 1536 750 / 567, 3072 1301 / 1231; Qwen3 shape, even / skewed
+// scores, 777 tokens (K' = 4) 228 / 221, 132 / 133, (K' = 6) 237 / 227, 182 / 178, 1536 tokens 253 / 249, 235 / 218; 64 experts of
+// 2048 x 1408 (K' = 3) 384 tokens 197 / 200, 1536 225 / 218; 160 of 1536 x 1024 200 tokens 229 / 231, 1536 285 / 273. Few items:
+// 64 experts of 1024 x 512 (K' = 4) 768 tokens 64 / 71; 11 of 2688 x 512 (K' = 3) 58 / 65.
 bool use_mixed(int64_t rows, int G, int d, int I) {
     const int64_t items = (int64_t)G * ((I + 127) / 128) * std::max<int64_t>(1, rows / (256 * (int64_t)G));
-    return rows / kTileM < (int64_t)8 * G && items >= (int64_t)3 * sm_count() && (d >= 48 * kGemmBK || rows >= (int64_t)96 * G);
+    return rows / kTileM < (int64_t)8 * G && items >= (int64_t)3 * sm_count() && (d >= 48 * kGemmBK || rows >= (int64_t)24 * G);
 }
 
 struct PdlScope {  // programmatic dependent launch for the launches of this scope

@@ -1,0 +1,77 @@
+"""Whole row tiles and ragged remainders in one pass (gemm_mixed.cu), at the group sizes where it can go wrong: against the
+one-CTA kernel bit for bit (the same products accumulated in the same order) and against the CPU oracle."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import synth_inputs as si
+from harness import A, Case, check_output, check_prefill_meta
+
+pytestmark = pytest.mark.gpu
+
+EDGES = [0, 1, 2, 31, 32, 33, 63, 64, 65, 96, 97, 127, 128, 129, 160, 161, 192, 193, 223, 224, 225, 255, 256, 257, 288, 289, 383, 384,
+         480, 481, 511, 512, 513, 767, 768, 769]
+
+
+@pytest.mark.parametrize("d,I", [(64, 896), (320, 832), (1088, 64 * 13)])
+def test_group_sizes_at_the_edges_of_tiles(d, I):
+    """One route per token, dealt so that the experts own exactly the sizes above: one k-block, K and N tails, column tiles of
+    which the second CTA has none, groups without rows."""
+    sizes = (EDGES * 2)[:64]
+    T, N = sum(sizes), len(sizes)
+    case = Case(si.LayerConfig("edges", N, 0, d, I, 2, "bf16", T, (1,), 4, (2,)))
+    owner = np.repeat(np.arange(N), sizes)[np.random.default_rng(3).permutation(T)]
+    lg = torch.full((T, N), -4.0)
+    lg[torch.arange(T), torch.from_numpy(owner)] = 4.0
+    lg[torch.arange(T), torch.from_numpy((owner + 1) % N)] = -3.0
+    case.lg, case.d_lg = lg, lg.to(case.dev)
+    case.set_tables((case.tables_host[0], case.tables_host[1], torch.ones(N), torch.zeros(N)))
+    got, one = case.run_prefill(1), case.run_prefill(1, with_meta=False, gemm_path=1)["y"]
+    assert np.array_equal(np.diff(got["offsets"]), sizes)
+    assert np.array_equal(got["y"], one)
+    idx = np.random.default_rng(4).choice(T, 300, replace=False)
+    check_output(got["y"][idx], case.oracle_prefill(1, tok_idx=idx)["y"], "bf16")
+
+
+@pytest.mark.parametrize("T", [2000, 2048, 2049, 2170])
+def test_shared_expert_beside_the_scatter_kernel(T):
+    """A shared expert whose gate/up pairs run on the second stream: the pass takes what is left of its group (an odd last row
+    tile, or nothing), and all of it in the down projection."""
+    case = Case(si.LayerConfig("shared", 8, 1, 1024, 7168, 3, "bf16", T, (2,), 4, (2,)))
+    got, one = case.run_prefill(2), case.run_prefill(2, with_meta=False, gemm_path=1)["y"]
+    assert np.array_equal(got["y"], one)
+    idx = np.random.default_rng(5).choice(T, 24, replace=False)
+    check_output(got["y"][idx], case.oracle_prefill(2, tok_idx=idx)["y"], "bf16")
+
+
+@pytest.mark.parametrize("Kp,ns,T,d", [(2, 0, 4000, 192), (3, 1, 2500, 128), (3, 0, 40, 3136)])
+def test_rows_of_several_routes(Kp, ns, T, d):
+    """Several routes per token through the per-route buffer; few rows of a wide layer."""
+    case = Case(si.LayerConfig("routes", 64, ns, d, 896, 4, "bf16", T, (Kp,), 4, (2,), logits="zipf"))
+    got, ref = case.run_prefill(Kp), case.oracle_prefill(Kp, tok_idx=np.arange(min(T, 200)))
+    check_prefill_meta(got, ref)
+    check_output(got["y"][:200], ref["y"], "bf16")
+    assert np.array_equal(got["y"], case.run_prefill(Kp, with_meta=False, gemm_path=1)["y"])
+
+
+@pytest.mark.parametrize("mode,m", [(0, 2000), (1, 130), (1, 225)])
+def test_calibration(mode, m):
+    """fp32 rows of whole and ragged items: the oracle's tables, tolerances as in test_calibrate_bf16_on_tensor_cores."""
+    cfg = si.LayerConfig("calib", 64, 0, 128, 896, 4, "bf16", 64, (2,), 4, (2,))
+    case = Case(cfg, correlated=0.8)
+    ex, dev, N = case.ex, case.dev, cfg.n_experts
+    xc, lc = si.hidden_states(cfg, m, "x_cal"), si.router_logits(cfg, m, "logits_cal")
+    ref = oracle.calibrate(A(xc), lc.numpy(), A(case.wg), A(case.wu), A(case.wd), N, cfg.top_k, mode=mode)
+    S = torch.full((N, N), float("nan"), device=dev)
+    L, h, lnh = torch.full_like(S, float("nan")), torch.full((N,), float("nan"), device=dev), torch.empty(N, device=dev)
+    n_obs = torch.full((N, N), -1, dtype=torch.int32, device=dev)
+    ws = ex.alloc_workspace(case.layer, m, N if mode else cfg.top_k)
+    ws.fill_(0xFF)
+    ex.exfold_calibrate(case.layer, xc.to(dev), lc.to(dev), case.d_wg, case.d_wu, case.d_wd, ex.make_tables(S, L, h, lnh, n_obs), ws, mode=mode)
+    assert ex.exfold_device_status(ws) == 0
+    assert np.array_equal(n_obs.cpu().numpy(), ref["n_obs"])
+    np.testing.assert_allclose(S.cpu().numpy(), ref["S"], rtol=5e-3, atol=5e-3)
+    seen = (ref["n_obs"] > 0) | np.eye(N, dtype=bool)
+    np.testing.assert_allclose(L.cpu().numpy()[seen], ref["L"][seen], rtol=5e-3, atol=5e-3)
+    np.testing.assert_allclose(h.cpu().numpy(), ref["h"], rtol=3e-3)
