@@ -577,7 +577,10 @@ int exfold_moe_prefill_ex(const exfold_layer* layer, const void* x, const float*
     // the first kernel of the call clears the status record (not for the later chunks of a chunked host call)
     rp.status = t_keep_status ? nullptr : at<DeviceStatus>(ws, pl.status);
     rp.queue = mixed ? at<DeviceStatus>(ws, pl.status)->queue : nullptr;
-    { ProfScope ps(0, s); EXFOLD_CUDA(launch_prefill_route(rp, s)); }
+    // few tokens of an fp32 layer: its FFN kernel routes them itself
+    const int tile_rows = mixed ? kMixedTiles : bf16 ? kTileM : ffn_f32_tile_rows(Rtot, G, d, I);
+    const bool routed = !bf16 && ffn_f32_routes(T, N, Kp, l.n_shared, d, I, tile_rows, sm_count());
+    if (!routed) { ProfScope ps(0, s); EXFOLD_CUDA(launch_prefill_route(rp, s)); }
 
     // The shared expert's gate/up projection needs nothing the routing kernels produce (its rows are x itself, its
     // rows of H lie behind the routed ones): its whole row-tile pairs run on the second stream beside the scatter
@@ -605,7 +608,7 @@ int exfold_moe_prefill_ex(const exfold_layer* layer, const void* x, const float*
 
     PrefillScatterParams cp{};
     cp.T = T; cp.N = N; cp.n_shared = l.n_shared; cp.Kp = Kp; cp.d_bytes = bf16 ? d * 2 : 0;
-    cp.tile_rows = mixed ? kMixedTiles : bf16 ? kTileM : ffn_f32_tile_rows(Rtot, G, d, I);
+    cp.tile_rows = tile_rows;
     cp.nblk = (int)((T + kRouteTokensPerBlock - 1) / kRouteTokensPerBlock);
     cp.ids = rp.ids; cp.w = rp.w; cp.block_hist = rp.block_hist; cp.sb_hist = rp.sb_hist;
     cp.offsets = at<int32_t>(ws, pl.offsets); cp.work_start = at<int32_t>(ws, pl.work_start);
@@ -614,7 +617,7 @@ int exfold_moe_prefill_ex(const exfold_layer* layer, const void* x, const float*
     cp.row_w = at<float>(ws, pl.row_w);
     cp.inv_pos = at<int32_t>(ws, pl.inv_pos);
     if (small) cp.xs = nullptr;  // the tokens are read in place; only the metadata needs the permutation
-    if (!small || meta) { ProfScope ps(2, s); EXFOLD_CUDA(launch_prefill_scatter(cp, s)); }
+    if (!routed && (!small || meta)) { ProfScope ps(2, s); EXFOLD_CUDA(launch_prefill_scatter(cp, s)); }
 
     if (small) {
         DecodeSmallParams sp{};
@@ -659,7 +662,14 @@ int exfold_moe_prefill_ex(const exfold_layer* layer, const void* x, const float*
         fp.offsets = cp.offsets; fp.tile_start = cp.work_start; fp.row_tok = cp.row_tok; fp.row_w = cp.row_w;
         if (direct) fp.y = reinterpret_cast<float*>(y);
         else fp.out = at<float>(ws, pl.out);
-        { ProfScope ps(10, s); EXFOLD_CUDA(launch_ffn_f32(fp, Rtot, sm_count(), s)); }
+        if (routed) {
+            const FfnF32Route rt{rp, l.n_shared, cp.offsets, cp.perm, cp.inv_pos, cp.row_tok, cp.row_w};
+            ProfScope ps(10, s);
+            EXFOLD_CUDA(launch_ffn_f32_routed(fp, rt, Rtot, s));
+        } else {
+            ProfScope ps(10, s);
+            EXFOLD_CUDA(launch_ffn_f32(fp, Rtot, sm_count(), s));
+        }
         if (!direct) {
             ProfScope ps(11, s);
             EXFOLD_CUDA(launch_combine_f32(fp.out, cp.inv_pos, cp.row_w, T, Kp, d, l.n_shared, nullptr,

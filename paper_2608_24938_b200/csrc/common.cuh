@@ -379,6 +379,19 @@ struct FfnF32Params {
     float* y;                     // [tokens][d]: every token has one row, stored weighted (out unused)
 };
 int ffn_f32_tile_rows(int64_t rows, int G, int d, int I);
+// Prefill of few tokens: the FFN kernel routes the tokens itself and writes the permutation (p.offsets, tile_start, row_tok,
+// row_w unused)
+struct FfnF32Route {
+    PrefillRouteParams r;  // block_hist, sb_hist unused
+    int n_shared;
+    int32_t* offsets;      // as PrefillScatterParams
+    int32_t* perm;
+    int32_t* inv_pos;
+    int32_t* row_tok;
+    float* row_w;
+};
+bool ffn_f32_routes(int64_t T, int N, int Kp, int n_shared, int d, int I, int tile_rows, int sms);
+cudaError_t launch_ffn_f32_routed(const FfnF32Params& p, const FfnF32Route& rt, int64_t rows, cudaStream_t s);
 cudaError_t launch_ffn_f32(const FfnF32Params& p, int64_t rows, int sms, cudaStream_t s);
 cudaError_t launch_combine_f32(const float* out, const int32_t* inv_pos, const float* row_w, int64_t T, int Kr, int d,
                                int n_shared, const int32_t* shared0_dev, float* y, cudaStream_t s);

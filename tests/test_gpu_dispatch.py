@@ -318,3 +318,17 @@ def test_host_prefill_covers_every_token(T):
     ex.exfold_moe_prefill_host(case.layer, case.x.pin_memory(), case.lg.pin_memory(), case.d_wg, case.d_wu, case.d_wd, case.tables, 1, y, ws)
     assert ex.exfold_device_status(ws) == 0
     assert np.array_equal(y.float().numpy(), want)
+
+
+@pytest.mark.parametrize("T,N,ns,d,I,K,Kp", [
+    (1, 8, 0, 128, 256, 2, 1), (7, 8, 1, 128, 256, 2, 2), (64, 8, 0, 128, 256, 2, 1), (65, 8, 0, 128, 250, 2, 2), (128, 8, 0, 64, 96, 3, 1),
+    (127, 16, 0, 64, 96, 4, 2), (129, 16, 0, 64, 96, 4, 1), (9, 33, 1, 132, 64, 5, 3), (20, 128, 0, 64, 64, 8, 2), (16, 2, 0, 64, 64, 2, 1),
+    (3, 100, 1, 96, 64, 32, 16), (20, 129, 0, 64, 64, 3, 1), (2, 8, 0, 3584, 3584, 2, 2)])
+def test_fp32_prefill_that_routes_in_its_ffn_kernel(T, N, ns, d, I, K, Kp):
+    """Few tokens of an fp32 layer: routing inside the FFN kernel (up to 128 tokens, 128 experts, one wave of clusters) and the
+    kernels of its own beyond; metadata bit-exact, safeguards included, outputs to fp32 rounding."""
+    case = Case(si.LayerConfig("f32r", N, ns, d, I, K, "f32", T, (Kp,), 4, (2,)))
+    got, ref = case.run_prefill(Kp), case.oracle_prefill(Kp)
+    check_prefill_meta(got, ref)
+    assert check_output(got["y"], ref["y"], "f32")[1] < 2e-6
+    assert np.array_equal(got["y"], case.run_prefill(Kp, with_meta=False)["y"])
