@@ -578,7 +578,7 @@ int exfold_moe_prefill_ex(const exfold_layer* layer, const void* x, const float*
     rp.status = t_keep_status ? nullptr : at<DeviceStatus>(ws, pl.status);
     rp.queue = mixed ? at<DeviceStatus>(ws, pl.status)->queue : nullptr;
     // few tokens of an fp32 layer: its FFN kernel routes them itself
-    const int tile_rows = mixed ? kMixedTiles : bf16 ? kTileM : ffn_f32_tile_rows(Rtot, G, d, I);
+    const int tile_rows = mixed ? kMixedTiles : bf16 ? kTileM : ffn_f32_tile_rows(Rtot, G, d, I, sm_count());
     const bool routed = !bf16 && ffn_f32_routes(T, N, Kp, l.n_shared, d, I, tile_rows, sm_count());
     if (!routed) { ProfScope ps(0, s); EXFOLD_CUDA(launch_prefill_route(rp, s)); }
 
@@ -834,13 +834,13 @@ static int decode_impl(const exfold_layer* layer, const void* x, const float* lo
             if (rc != EXFOLD_OK) return rc;
         }
         const int max_groups = std::min(pool_m, N) + l.n_shared;
-        rp.tile_rows = ffn_f32_tile_rows(max_rows, max_groups, d, I);
+        // a token has at most as many rows as the pool has experts
+        const int64_t rows = B * std::min(K, (int)pool_m) + B * l.n_shared;
+        rp.tile_rows = ffn_f32_tile_rows(rows, max_groups, d, I, sm_count());
         { ProfScope ps(6, s); EXFOLD_CUDA(launch_decode_route(rp, s)); }
         FfnF32Params fp = f32_params(x, w_gate, w_up, w_down, d, I, max_groups, rp.tile_rows);
         fp.offsets = rp.grp_off; fp.tile_start = rp.grp_tiles; fp.grp_expert = rp.grp_expert; fp.n_groups_dev = rp.n_groups;
         fp.row_tok = rp.row_tok; fp.row_w = rp.row_w; fp.out = at<float>(ws, pl.out);
-        // a token has at most as many rows as the pool has experts
-        const int64_t rows = B * std::min(K, (int)pool_m) + B * l.n_shared;
         { ProfScope ps(10, s); EXFOLD_CUDA(launch_ffn_f32(fp, rows, sm_count(), s)); }
         { ProfScope ps(11, s); EXFOLD_CUDA(launch_combine_f32(fp.out, rp.slot_row, rp.row_w, B, K, d, l.n_shared, rp.n_groups + 2,
                                                               reinterpret_cast<float*>(y), s)); }
@@ -946,7 +946,7 @@ static int calibrate_enqueue(const exfold_layer* layer, const void* x_cal, const
     int32_t* offsets = at<int32_t>(ws, pl.offsets);
     int32_t* work_start = at<int32_t>(ws, pl.work_start);
     int32_t* row_tok = at<int32_t>(ws, pl.row_tok);
-    const int tile_rows = mixed ? kMixedTiles : tensor_path ? kTileM : ffn_f32_tile_rows(Rc, N, d, I);
+    const int tile_rows = mixed ? kMixedTiles : tensor_path ? kTileM : ffn_f32_tile_rows(Rc, N, d, I, sm_count());
     if (opts->mode == 0) {
         PrefillScatterParams cp{};
         cp.T = m; cp.N = N; cp.n_shared = 0; cp.Kp = K; cp.d_bytes = tensor_path ? d * 2 : 0; cp.tile_rows = tile_rows;

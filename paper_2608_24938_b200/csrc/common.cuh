@@ -378,7 +378,7 @@ struct FfnF32Params {
     float* out;                   // [rows][d] unweighted expert outputs, or
     float* y;                     // [tokens][d]: every token has one row, stored weighted (out unused)
 };
-int ffn_f32_tile_rows(int64_t rows, int G, int d, int I);
+int ffn_f32_tile_rows(int64_t rows, int G, int d, int I, int sms);
 // Prefill of few tokens: the FFN kernel routes the tokens itself and writes the permutation (p.offsets, tile_start, row_tok,
 // row_w unused)
 struct FfnF32Route {

@@ -602,11 +602,18 @@ __global__ void __launch_bounds__(128) combine_f32_kernel(const float* __restric
 
 }  // namespace
 
+static int64_t short_tiles(int64_t rows, int G) { return std::min<int64_t>(rows, rows / kSR + G); }  // at most
+
 // Rows per tile: a tile computes all of its rows, so short groups want short tiles (and more of them to fill the SMs); a
-// tile's weights are read once per tile, so long groups want long ones. Short tiles need the tokens and H in shared memory
+// tile's weights are read once per tile, so long groups want long ones. The short form is the faster one for as long as its
+// tiles are kShortWaves waves of clusters at most. Whole call with tall / short tiles: tiny layer prefill (K' = 1) 75 tokens
+// 20.3 / 12.0 us, 342 23.5 / 19.4, 509 35.0 / 22.8, (K' = 2) 456 40.4 / 28.3, 770 (6 waves) 34.6 / 39.2; decode of 116 tokens, pool
+// of 3 35.2 / 21.9; 28 experts of 320 x 960, 41 tokens, pool of 8 85 / 53; 9 of 384 x 736, 79 tokens 85 / 60; 30 + 1 of 96 x 128,
+// 871 tokens (K' = 3, 13 waves) 39 / 56. Short tiles need the tokens and H in shared memory
 // whole (d + I up to ~7000); tall ones are halved while the slice of H does not fit (32 rows: I above ~11 000).
-int ffn_f32_tile_rows(int64_t rows, int G, int d, int I) {
-    if (rows <= (int64_t)kSR * G && short_bytes(d, I) <= kSmemLimit) return kSR;
+constexpr int kShortWaves = 5;
+int ffn_f32_tile_rows(int64_t rows, int G, int d, int I, int sms) {
+    if ((rows <= (int64_t)kSR * G || short_tiles(rows, G) * kMaxCl * 100 <= (int64_t)184 * kShortWaves * sms) && short_bytes(d, I) <= kSmemLimit) return kSR;
     int tile_rows = rows > (int64_t)48 * G ? 32 : 16;
     while (tile_rows > 1 && tall_bytes(tile_rows, I, kMaxCl) > kSmemLimit) tile_rows /= 2;
     return tile_rows;
@@ -645,13 +652,12 @@ cudaError_t launch_ffn_f32(const FfnF32Params& p, int64_t rows, int sms, cudaStr
 }
 
 // One wave of clusters (each repeats the routing), and the routes of all tokens in shared memory
-static int64_t routed_tiles(int64_t rows, int G) { return std::min<int64_t>(rows, rows / kSR + G); }
 bool ffn_f32_routes(int64_t T, int N, int Kp, int n_shared, int d, int I, int tile_rows, int sms) {
     return tile_rows == kSR && short_bytes(d, I) + sizeof(RouteSmem) + 256 <= kSmemLimit && T <= kRoutedTokens && T * Kp <= kRoutedSlots && N <= 128 &&
-           routed_tiles(T * (Kp + n_shared), N + n_shared) * kMaxCl * 100 <= (int64_t)184 * sms;
+           short_tiles(T * (Kp + n_shared), N + n_shared) * kMaxCl * 100 <= (int64_t)184 * sms;
 }
 cudaError_t launch_ffn_f32_routed(const FfnF32Params& p, const FfnF32Route& rt, int64_t rows, cudaStream_t s) {
-    const int64_t tiles = routed_tiles(rows, p.G);
+    const int64_t tiles = short_tiles(rows, p.G);
     return vec_loads(p) ? launch_routed<true>(p, rt, tiles, s) : launch_routed<false>(p, rt, tiles, s);
 }
 

@@ -332,3 +332,15 @@ def test_fp32_prefill_that_routes_in_its_ffn_kernel(T, N, ns, d, I, K, Kp):
     check_prefill_meta(got, ref)
     assert check_output(got["y"], ref["y"], "f32")[1] < 2e-6
     assert np.array_equal(got["y"], case.run_prefill(Kp, with_meta=False)["y"])
+
+
+@pytest.mark.parametrize("T,B,N,ns,d,I,K,Kp,M", [(456, 116, 8, 0, 128, 256, 2, 2, 3), (600, 230, 8, 0, 64, 96, 2, 2, 2), (700, 33, 7, 1, 68, 90, 5, 5, 1)])
+def test_fp32_short_tiles_of_long_groups(T, B, N, ns, d, I, K, Kp, M):
+    """Groups of many short tiles (a few waves of clusters, four or two CTAs each) and, last, the tall tiles beyond."""
+    case = Case(si.LayerConfig("f32t", N, ns, d, I, K, "f32", T, (Kp,), B, (M,)))
+    got, ref = case.run_prefill(Kp), case.oracle_prefill(Kp)
+    check_prefill_meta(got, ref)
+    assert check_output(got["y"], ref["y"], "f32")[1] < 2e-6
+    got, ref = case.run_decode(M), case.oracle_decode(M)
+    check_decode_meta(got, ref, M)
+    assert check_output(got["y"], ref["y"], "f32")[1] < 2e-6
