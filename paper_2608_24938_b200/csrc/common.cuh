@@ -390,8 +390,11 @@ struct FfnF32Route {
     int32_t* row_tok;
     float* row_w;
 };
-bool ffn_f32_routes(int64_t T, int N, int Kp, int n_shared, int d, int I, int tile_rows, int sms);
+// rows: of all groups, at most; slots: routes per token that the kernel holds
+bool ffn_f32_routes(int64_t T, int64_t rows, int G, int N, int slots, int d, int I, int tile_rows, int sms);
 cudaError_t launch_ffn_f32_routed(const FfnF32Params& p, const FfnF32Route& rt, int64_t rows, cudaStream_t s);
+// Decode of few tokens, likewise (the group tables of rt are not written)
+cudaError_t launch_ffn_f32_routed(const FfnF32Params& p, const DecodeRouteParams& rt, int64_t rows, cudaStream_t s);
 cudaError_t launch_ffn_f32(const FfnF32Params& p, int64_t rows, int sms, cudaStream_t s);
 cudaError_t launch_combine_f32(const float* out, const int32_t* inv_pos, const float* row_w, int64_t T, int Kr, int d,
                                int n_shared, const int32_t* shared0_dev, float* y, cudaStream_t s);

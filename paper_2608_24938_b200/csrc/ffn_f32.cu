@@ -109,7 +109,8 @@ __device__ __forceinline__ void lane_sums(float* v, int lane) {
 // 12.3 -> 8.9, with the router before it 16.0 -> 12.3.
 constexpr int kRoutedTokens = 128;
 constexpr int kRoutedSlots = 512;  // routes, at most
-struct RouteSmem {
+constexpr int kRoutedExperts = 128;
+struct PrefillRouteSmem {
     short id[kRoutedSlots];
     float w[kRoutedSlots];
     int cnt[kMaxExperts];
@@ -120,7 +121,7 @@ struct RouteSmem {
 };
 
 template <int CL, int NPL>
-__device__ __forceinline__ bool route_tile(const FfnF32Route& rt, cg::cluster_group& cluster, int tile, RouteSmem& sm, Tile* st) {
+__device__ __forceinline__ bool route_tile(const FfnF32Route& rt, cg::cluster_group& cluster, int tile, PrefillRouteSmem& sm, Tile* st) {
     const PrefillRouteParams& p = rt.r;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, rank = (int)cluster.block_rank();
     const int T = (int)p.T, N = p.N, Kp = p.Kp, Ko = p.K - p.Kp, n = T * Kp;
@@ -227,12 +228,257 @@ __device__ __forceinline__ bool route_tile(const FfnF32Route& rt, cg::cluster_gr
     return true;
 }
 
-// NPL > 0: the kernel routes the tokens itself (scores per lane); 0: the tiles' rows come from the lists
-template <int CL, bool VEC, int NPL>
-__global__ void __launch_bounds__(kThreads) ffn_f32_short_kernel(FfnF32Params p, const __grid_constant__ FfnF32Route rt) {
+// Decode on a grid of one wave, likewise: every cluster takes the Top-K of all tokens (a token per warp at a time), sums the
+// routed weights, ranks the pool, finds the targets (an expert per warp at a time), remaps the slots and picks the rows of its
+// tile; the first cluster writes the metadata, each tile its part of the lists that the sum after it reads. The arithmetic is
+// decode_route_kernel's. Whole call before / now: tiny layer 16 tokens 16.1 / 12.7 us, one 15.5 / 12.3, 74 19.9 / 15.0.
+struct DecodeRouteSmem {
+    double w64[kRoutedSlots];
+    double score[kRoutedExperts];
+    unsigned long long acc[kRoutedExperts];  // sum_i w_{i,e} in 2^-53 units: exact, order-independent
+    short id[kRoutedSlots];
+    float wrm[kRoutedSlots];  // remapped weights
+    int in_union[kRoutedExperts];
+    int rank_of[kRoutedExperts];  // pool rank or -1
+    int pool[kRoutedExperts];
+    int target[kRoutedExperts];
+    float scale[kRoutedExperts];
+    unsigned mask[kRoutedExperts][kRoutedTokens / 32];  // by pool rank: the tokens with a row
+    int warp_sum[kThreads / 32];
+    int skip, P;
+    int tok[kSR];
+    float rw[kSR];
+};
+
+template <int CL, int NPL>
+__device__ __forceinline__ bool route_tile(const DecodeRouteParams& p, cg::cluster_group& cluster, int tile, DecodeRouteSmem& sm, Tile* st) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, rank = (int)cluster.block_rank();
+    const int B = p.B, N = p.N, K = p.K, M = p.M, n = B * K;
+    const bool first = blockIdx.x < CL, meta = first && rank == 0;
+    const bool is_static = p.st_pool != nullptr;
+    constexpr int kWarps = kThreads / 32;
+    for (int e = tid; e < N; e += kThreads) {
+        sm.acc[e] = 0ull;
+        sm.in_union[e] = 0;
+        sm.rank_of[e] = -1;
+        sm.pool[e] = 0;  // (a NaN norm leaves ranks that no expert has)
+    }
+    for (int i = tid; i < kRoutedExperts * (kRoutedTokens / 32); i += kThreads) (&sm.mask[0][0])[i] = 0u;
+    if (tid == 0) st->g = -1;
+    cluster.barrier_arrive();
+    grid_dep_wait();
+    if (p.status != nullptr && blockIdx.x == 0 && tid < 4) reinterpret_cast<int*>(p.status)[tid] = 0;
+    bool started = false;
+    for (int i = warp * CL + rank; i < B; i += CL * kWarps) {  // Eq. 2
+        float v[NPL];
+#pragma unroll
+        for (int q = 0; q < NPL; ++q) v[q] = lane + 32 * q < N ? p.logits[(size_t)i * N + lane + 32 * q] : -INFINITY;
+        int id;
+        const double w = warp_topk_softmax<NPL>(v, N, K, lane, &id);
+        if (!started) cluster.barrier_wait();  // before the first remote write: all CTAs of the cluster have started
+        started = true;
+        if (lane < K) {
+#pragma unroll
+            for (int c = 0; c < CL; ++c) {
+                cluster.map_shared_rank(sm.id, c)[i * K + lane] = (short)id;
+                cluster.map_shared_rank(sm.w64, c)[i * K + lane] = w;
+            }
+        }
+    }
+    if (!started) cluster.barrier_wait();
+    cluster.sync();  // every copy of the routes is complete
+    if (is_static) {
+        for (int e = tid; e < N; e += kThreads) {
+            sm.target[e] = p.st_target[e];
+            sm.scale[e] = p.st_scale[e];
+        }
+        for (int j = tid; j < M; j += kThreads) {
+            const int e = p.st_pool[j];
+            sm.pool[j] = e;
+            sm.rank_of[e] = j;
+        }
+        if (tid == 0) sm.P = M;
+        __syncthreads();
+    } else {
+        for (int s = tid; s < n; s += kThreads) {
+            const int e = sm.id[s];
+            atomicAdd(&sm.acc[e], (unsigned long long)(sm.w64[s] * 9007199254740992.0));
+            sm.in_union[e] = 1;
+        }
+        __syncthreads();
+        // Eq. 11: score_e = h_e * sum_i w_{i,e}; a thread per expert counts the better ones (score desc, id asc)
+        int in = 0;
+        if (tid < N) {
+            in = sm.in_union[tid];
+            sm.score[tid] = (double)sm.acc[tid] * (1.0 / 9007199254740992.0) * (double)p.h[tid];
+        }
+        const int usz = __syncthreads_count(in);
+        if (in) {
+            const double se = sm.score[tid];
+            int better = 0;
+            for (int o = 0; o < N; ++o)
+                better += sm.in_union[o] && (sm.score[o] > se || (sm.score[o] == se && o < tid)) ? 1 : 0;
+            if (better < M) {
+                sm.rank_of[tid] = better;
+                sm.pool[better] = tid;
+            }
+        }
+        if (tid == 0) sm.P = usz < M ? usz : M;
+        __syncthreads();
+        // Eq. 12, a warp of the cluster per source expert: itself if in the pool, else its minimum-loss pool expert
+        const int P = sm.P;
+        for (int s = warp * CL + rank; s < N; s += CL * kWarps) {
+            int bt = s;
+            float sc = 1.0f;
+            if (sm.rank_of[s] < 0) {  // warp-uniform
+                const float* row = p.L + (size_t)s * N;
+                float bl = INFINITY;
+                int bj = 0x7fffffff;
+                for (int j = lane; j < P; j += 32) {
+                    const int t = sm.pool[j];
+                    const float l = __ldg(row + t);
+                    if (bj == 0x7fffffff || l < bl || (l == bl && t < bj)) {
+                        bl = l;
+                        bj = t;
+                    }
+                }
+                bt = warp_argmin(bj != 0x7fffffff, float_order_key(bl), bj);
+                sc = __ldg(p.S + (size_t)s * N + bt);
+            }
+            if (lane < CL) {
+                cluster.map_shared_rank(sm.target, lane)[s] = bt;
+                cluster.map_shared_rank(sm.scale, lane)[s] = sc;
+            }
+        }
+        cluster.sync();  // the targets are in every copy
+    }
+    const int P = sm.P;
+    for (int s = tid; s < n; s += kThreads) {  // Eq. 14
+        const int e = sm.id[s], t = sm.target[e], i = s / K;
+        const float wv = (float)(sm.w64[s] * (double)sm.scale[e]);
+        sm.id[s] = (short)t;
+        sm.wrm[s] = wv;
+        if (sm.rank_of[t] >= 0) atomicOr(&sm.mask[sm.rank_of[t]][i >> 5], 1u << (i & 31));
+        if (meta) {
+            p.ids[s] = t;
+            p.w[s] = wv;
+        }
+    }
+    if (meta) {
+        for (int e = tid; e < N; e += kThreads) {
+            p.target[e] = sm.target[e];
+            p.scale[e] = sm.scale[e];
+            p.pool_ids[e] = e < P ? sm.pool[e] : -1;
+        }
+        if (tid < 8) {
+            uint32_t m = 0;
+            for (int b = 0; b < 32; ++b) {
+                const int e = tid * 32 + b;
+                if (e < N && sm.rank_of[e] >= 0) m |= 1u << b;
+            }
+            p.pool_mask[tid] = m;
+        }
+        if (tid == 0) *p.pool_size = P;
+    }
+    __syncthreads();
+    // a thread per group: its rows and tiles, prefixes of both in one word
+    int mine = 0;
+    if (tid < P)
+#pragma unroll
+        for (int q = 0; q < kRoutedTokens / 32; ++q) mine += __popc(sm.mask[tid][q]);
+    const int packed = mine | (mine + kSR - 1) / kSR << 16;
+    int incl = packed;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int u = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += u;
+    }
+    if (lane == 31) sm.warp_sum[warp] = incl;
+    __syncthreads();
+    int before = incl - packed, all = 0;
+#pragma unroll
+    for (int w = 0; w < kWarps; ++w) {
+        if (w < warp) before += sm.warp_sum[w];
+        all += sm.warp_sum[w];
+    }
+    const int off = before & 0xffff, t0 = before >> 16, rows = all & 0xffff, pool_tiles = all >> 16;
+    if (meta && tid == 0) {
+        p.n_groups[0] = P + (p.n_shared ? 1 : 0);
+        p.n_groups[1] = rows + (p.n_shared ? B : 0);
+        p.n_groups[2] = rows;  // first row of the shared expert's group
+    }
+    if (tile >= pool_tiles) {  // the shared expert's rows: the tokens in order, weight 1
+        const int j0 = (tile - pool_tiles) * kSR;
+        if (!p.n_shared || j0 >= B) return false;
+        if (tid == 0) *st = Tile{P, rows + j0, min(kSR, B - j0), N};
+        if (tid < kSR && j0 + tid < B) {
+            sm.tok[tid] = j0 + tid;
+            if (rank == 0) {
+                p.row_tok[rows + j0 + tid] = j0 + tid;
+                p.row_w[rows + j0 + tid] = 1.0f;
+            }
+        }
+        __syncthreads();
+        return true;
+    }
+    if (tile >= t0 && tile < t0 + (packed >> 16)) {
+        const int k = (tile - t0) * kSR;
+        *st = Tile{tid, off + k, min(kSR, mine - k), sm.pool[tid]};
+        sm.skip = k;
+    }
+    __syncthreads();
+    if (warp == 0) {  // the group's tokens in order
+        const int g = st->g, e = st->expert, k = sm.skip, row0 = st->row0;
+        for (int q = 0, seen = 0; q < kRoutedTokens / 32; ++q) {
+            const unsigned m = sm.mask[g][q];
+            const int i = q * 32 + lane, at = seen + __popc(m & ((1u << lane) - 1u)) - k;
+            if (((m >> lane) & 1u) && at >= 0 && at < kSR) {
+                float ws = 0.f;
+                int slot = -1;  // a token's first slot with this target has the row, the others are merged into it
+                for (int a = 0; a < K; ++a)
+                    if (sm.id[i * K + a] == e) {
+                        ws = slot >= 0 ? __fadd_rn(ws, sm.wrm[i * K + a]) : sm.wrm[i * K + a];
+                        if (rank == 0) p.slot_row[i * K + a] = slot >= 0 ? -1 : row0 + at;
+                        if (slot < 0) slot = a;
+                    }
+                sm.tok[at] = i;
+                if (rank == 0) {
+                    p.row_tok[row0 + at] = i;
+                    p.row_w[row0 + at] = ws;
+                }
+            }
+            seen += __popc(m);
+        }
+    }
+    __syncthreads();
+    return true;
+}
+
+struct NoRoute {};  // the tiles' rows come from lists that kernels before it wrote
+struct NoRouteSmem {
+    int tok[1];
+    float rw[1];
+};
+template <typename R>
+struct RouteSmemOf {
+    using type = NoRouteSmem;
+};
+template <>
+struct RouteSmemOf<FfnF32Route> {
+    using type = PrefillRouteSmem;
+};
+template <>
+struct RouteSmemOf<DecodeRouteParams> {
+    using type = DecodeRouteSmem;
+};
+
+// R: who routes the tokens; NPL: their scores per lane
+template <int CL, bool VEC, typename R, int NPL>
+__global__ void __launch_bounds__(kThreads) ffn_f32_short_kernel(FfnF32Params p, const __grid_constant__ R rt) {
     extern __shared__ __align__(16) float smem[];
     __shared__ Tile s_tile;
-    __shared__ RouteSmem rs;
+    __shared__ typename RouteSmemOf<R>::type rs;
+    constexpr bool kRoutes = NPL > 0;
     const int d = p.d, I = p.I, xld = (d + 127) / 128 * 128, hld = p.hld;  // whole 128-wide K chunks
     float* xs = smem;             // [8][xld]
     float* hs = smem + kSR * xld;  // [8][hld]
@@ -240,7 +486,7 @@ __global__ void __launch_bounds__(kThreads) ffn_f32_short_kernel(FfnF32Params p,
     const int rank = (int)cluster.block_rank();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     constexpr int kWarps = kThreads / 32;
-    if constexpr (NPL > 0) {
+    if constexpr (kRoutes) {
         if (!route_tile<CL, NPL>(rt, cluster, (int)(blockIdx.x / CL), rs, &s_tile)) return;  // the whole cluster
     } else {
         grid_dep_wait();
@@ -287,14 +533,14 @@ __global__ void __launch_bounds__(kThreads) ffn_f32_short_kernel(FfnF32Params p,
     const int n0 = max(0, min(I, (rank + 1) * per0) - rank * per0), n1 = max(0, min(d, (rank + 1) * per1) - rank * per1);
     if (warp * 2 < n0) load_item(0, warp, 0, nxt);  // the first weights before the tokens, whose addresses take a round trip
     for (int t = warp; t < kSR; t += kWarps) {
-        const float* src = p.x + (t < rows ? (NPL > 0 ? (int64_t)rs.tok[t] : token_of(p, row0 + t)) : 0) * d;
+        const float* src = p.x + (t < rows ? (kRoutes ? (int64_t)rs.tok[t] : token_of(p, row0 + t)) : 0) * d;
         for (int k = lane * 4; k < xld; k += 128)
             *reinterpret_cast<float4*>(xs + t * xld + k) = load4<VEC>(src + k, t < rows ? d - k : 0);
     }
     for (int i = threadIdx.x; i < kSR * (hld - I); i += kThreads)  // columns past I: read by the last chunk
         hs[i / (hld - I) * hld + I + i % (hld - I)] = 0.f;
     __syncthreads();
-    bool started = NPL > 0;
+    bool started = kRoutes;
 
 #pragma unroll 1
     for (int phase = 0; phase < 2; ++phase) {
@@ -349,7 +595,7 @@ __global__ void __launch_bounds__(kThreads) ffn_f32_short_kernel(FfnF32Params p,
                         cluster.map_shared_rank(hs, c + (lane < 16 ? 0 : CL / 2))[t * hld + rank * per0 + fl] = h;
             } else if (gi * kSW + q < n1 && t < rows) {
                 const int col = rank * per1 + gi * kSW + q;
-                if (p.y != nullptr) p.y[(int64_t)(NPL > 0 ? rs.tok[t] : p.row_tok[row0 + t]) * d + col] = (NPL > 0 ? rs.rw[t] : p.row_w[row0 + t]) * acc[0];
+                if (p.y != nullptr) p.y[(int64_t)(kRoutes ? rs.tok[t] : p.row_tok[row0 + t]) * d + col] = (kRoutes ? rs.rw[t] : p.row_w[row0 + t]) * acc[0];
                 else p.out[(row0 + t) * d + col] = acc[0];
             }
         }
@@ -544,7 +790,7 @@ template <int CL, bool VEC>
 cudaError_t launch_form(FfnF32Params p, int64_t tiles, cudaStream_t s) {
     if (p.tile_rows == kSR && short_bytes(p.d, p.I) <= kSmemLimit) {
         p.hld = (p.I + 127) / 128 * 128 + 4;
-        return launch_t<CL>(ffn_f32_short_kernel<CL, VEC, 0>, short_bytes(p.d, p.I), tiles, s, p, FfnF32Route{});
+        return launch_t<CL>(ffn_f32_short_kernel<CL, VEC, NoRoute, 0>, short_bytes(p.d, p.I), tiles, s, p, NoRoute{});
     }
     p.fpc = features_per_cta(p.I, CL);
     p.hld = p.fpc + 4;
@@ -556,11 +802,11 @@ bool vec_loads(const FfnF32Params& p) {
     auto a16 = [](const void* q) { return (reinterpret_cast<uintptr_t>(q) & 15) == 0; };
     return p.I % 4 == 0 && a16(p.x) && a16(p.wg) && a16(p.wu) && a16(p.wd);
 }
-template <bool VEC>
-cudaError_t launch_routed(FfnF32Params p, const FfnF32Route& rt, int64_t tiles, cudaStream_t s) {
+template <bool VEC, typename R>
+cudaError_t launch_routed(FfnF32Params p, const R& rt, int N, int64_t tiles, cudaStream_t s) {
     p.hld = (p.I + 127) / 128 * 128 + 4;
-    if (rt.r.N <= 32) return launch_t<kMaxCl>(ffn_f32_short_kernel<kMaxCl, VEC, 1>, short_bytes(p.d, p.I), tiles, s, p, rt);
-    return launch_t<kMaxCl>(ffn_f32_short_kernel<kMaxCl, VEC, 4>, short_bytes(p.d, p.I), tiles, s, p, rt);
+    if (N <= 32) return launch_t<kMaxCl>(ffn_f32_short_kernel<kMaxCl, VEC, R, 1>, short_bytes(p.d, p.I), tiles, s, p, rt);
+    return launch_t<kMaxCl>(ffn_f32_short_kernel<kMaxCl, VEC, R, 4>, short_bytes(p.d, p.I), tiles, s, p, rt);
 }
 template <int CL>
 cudaError_t launch_cl(const FfnF32Params& p, int64_t tiles, cudaStream_t s) {
@@ -606,14 +852,14 @@ static int64_t short_tiles(int64_t rows, int G) { return std::min<int64_t>(rows,
 
 // Rows per tile: a tile computes all of its rows, so short groups want short tiles (and more of them to fill the SMs); a
 // tile's weights are read once per tile, so long groups want long ones. The short form is the faster one for as long as its
-// tiles are kShortWaves waves of clusters at most. Whole call with tall / short tiles: tiny layer prefill (K' = 1) 75 tokens
+// tiles are a few waves of clusters at most: five where the alternative is 16-row tiles or the layer is small, else three. Whole call with tall / short tiles: tiny layer prefill (K' = 1) 75 tokens
 // 20.3 / 12.0 us, 342 23.5 / 19.4, 509 35.0 / 22.8, (K' = 2) 456 40.4 / 28.3, 770 (6 waves) 34.6 / 39.2; decode of 116 tokens, pool
 // of 3 35.2 / 21.9; 28 experts of 320 x 960, 41 tokens, pool of 8 85 / 53; 9 of 384 x 736, 79 tokens 85 / 60; 30 + 1 of 96 x 128,
-// 871 tokens (K' = 3, 13 waves) 39 / 56. Short tiles need the tokens and H in shared memory
+// 871 tokens (K' = 3, 13 waves) 39 / 56; 83 + 1 of 160 x 480, decode of 159 tokens, pool of 6 (4.3 waves) 66 / 76. Short tiles need the tokens and H in shared memory
 // whole (d + I up to ~7000); tall ones are halved while the slice of H does not fit (32 rows: I above ~11 000).
-constexpr int kShortWaves = 5;
 int ffn_f32_tile_rows(int64_t rows, int G, int d, int I, int sms) {
-    if ((rows <= (int64_t)kSR * G || short_tiles(rows, G) * kMaxCl * 100 <= (int64_t)184 * kShortWaves * sms) && short_bytes(d, I) <= kSmemLimit) return kSR;
+    const int waves = rows <= (int64_t)48 * G || (int64_t)d * I <= 48 * 1024 ? 5 : 3;
+    if ((rows <= (int64_t)kSR * G || short_tiles(rows, G) * kMaxCl * 100 <= (int64_t)184 * waves * sms) && short_bytes(d, I) <= kSmemLimit) return kSR;
     int tile_rows = rows > (int64_t)48 * G ? 32 : 16;
     while (tile_rows > 1 && tall_bytes(tile_rows, I, kMaxCl) > kSmemLimit) tile_rows /= 2;
     return tile_rows;
@@ -652,13 +898,18 @@ cudaError_t launch_ffn_f32(const FfnF32Params& p, int64_t rows, int sms, cudaStr
 }
 
 // One wave of clusters (each repeats the routing), and the routes of all tokens in shared memory
-bool ffn_f32_routes(int64_t T, int N, int Kp, int n_shared, int d, int I, int tile_rows, int sms) {
-    return tile_rows == kSR && short_bytes(d, I) + sizeof(RouteSmem) + 256 <= kSmemLimit && T <= kRoutedTokens && T * Kp <= kRoutedSlots && N <= 128 &&
-           short_tiles(T * (Kp + n_shared), N + n_shared) * kMaxCl * 100 <= (int64_t)184 * sms;
+bool ffn_f32_routes(int64_t T, int64_t rows, int G, int N, int slots, int d, int I, int tile_rows, int sms) {
+    constexpr size_t route_bytes = std::max(sizeof(PrefillRouteSmem), sizeof(DecodeRouteSmem)) + 256;
+    return tile_rows == kSR && short_bytes(d, I) + route_bytes <= kSmemLimit && T <= kRoutedTokens && T * slots <= kRoutedSlots &&
+           N <= kRoutedExperts && short_tiles(rows, G) * kMaxCl * 100 <= (int64_t)184 * sms;
 }
 cudaError_t launch_ffn_f32_routed(const FfnF32Params& p, const FfnF32Route& rt, int64_t rows, cudaStream_t s) {
     const int64_t tiles = short_tiles(rows, p.G);
-    return vec_loads(p) ? launch_routed<true>(p, rt, tiles, s) : launch_routed<false>(p, rt, tiles, s);
+    return vec_loads(p) ? launch_routed<true>(p, rt, rt.r.N, tiles, s) : launch_routed<false>(p, rt, rt.r.N, tiles, s);
+}
+cudaError_t launch_ffn_f32_routed(const FfnF32Params& p, const DecodeRouteParams& rt, int64_t rows, cudaStream_t s) {
+    const int64_t tiles = short_tiles(rows, p.G);
+    return vec_loads(p) ? launch_routed<true>(p, rt, rt.N, tiles, s) : launch_routed<false>(p, rt, rt.N, tiles, s);
 }
 
 cudaError_t launch_combine_f32(const float* out, const int32_t* inv_pos, const float* row_w, int64_t T, int Kr, int d,

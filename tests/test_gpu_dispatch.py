@@ -344,3 +344,29 @@ def test_fp32_short_tiles_of_long_groups(T, B, N, ns, d, I, K, Kp, M):
     got, ref = case.run_decode(M), case.oracle_decode(M)
     check_decode_meta(got, ref, M)
     assert check_output(got["y"], ref["y"], "f32")[1] < 2e-6
+
+
+@pytest.mark.parametrize("B,N,ns,d,I,K,M", [
+    (1, 8, 0, 128, 256, 2, 2), (16, 8, 0, 128, 256, 2, 4), (31, 8, 1, 128, 250, 2, 8), (32, 8, 0, 64, 96, 3, 1), (33, 16, 0, 64, 96, 4, 6),
+    (64, 33, 0, 132, 64, 5, 3), (128, 8, 0, 64, 64, 2, 2), (129, 8, 0, 64, 64, 2, 2), (9, 128, 1, 64, 64, 9, 100), (9, 129, 0, 64, 64, 4, 5),
+    (16, 40, 0, 64, 64, 32, 7)])
+def test_fp32_decode_that_routes_in_its_ffn_kernel(B, N, ns, d, I, K, M):
+    """Few tokens of an fp32 layer: pool, targets and lists inside the FFN kernel (up to 128 tokens, 128 experts, one wave of
+    clusters) and the kernels of its own beyond, dynamic and static pool: metadata bit-exact, outputs to fp32 rounding."""
+    case = Case(si.LayerConfig("f32d", N, ns, d, I, K, "f32", 8, (1,), B, (M,)))
+    got, ref = case.run_decode(M), case.oracle_decode(M)
+    check_decode_meta(got, ref, M)
+    assert check_output(got["y"], ref["y"], "f32")[1] < 2e-6
+    ex, dev = case.ex, case.dev
+    pool_ids, target = torch.empty(M, dtype=torch.int32, device=dev), torch.empty(N, dtype=torch.int32, device=dev)
+    scale = torch.empty(N, device=dev)
+    pool = ex.exfold_static_pool_build(case.layer, case.tables, M, pool_ids, target, scale)
+    ws, y = case.workspace(B, K), torch.full((B, d), float("nan"), device=dev)
+    ids = torch.empty((B, K), dtype=torch.int32, device=dev)
+    w = torch.empty((B, K), device=dev)
+    ex.exfold_moe_decode_static(case.layer, case.d_xd, case.d_lgd, case.d_wg, case.d_wu, case.d_wd, pool, y, ws, meta=dict(ids=ids, w=w))
+    assert ex.exfold_device_status(ws) == 0
+    routed = case.lgd.topk(K, dim=1).indices
+    assert np.array_equal(ids.cpu().numpy(), target.cpu().numpy()[routed.numpy()])
+    yr = oracle.moe_apply(A(case.xd), A(case.wg), A(case.wu), A(case.wd), ids.cpu().numpy(), w.cpu().numpy(), N, ns)
+    assert check_output(y.cpu().numpy(), yr, "f32")[1] < 2e-6
