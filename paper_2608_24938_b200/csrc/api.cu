@@ -580,7 +580,9 @@ int exfold_moe_prefill_ex(const exfold_layer* layer, const void* x, const float*
     // few tokens of an fp32 layer: its FFN kernel routes them itself
     const int tile_rows = mixed ? kMixedTiles : bf16 ? kTileM : ffn_f32_tile_rows(Rtot, G, d, I, sm_count());
     const bool routed = !bf16 && ffn_f32_routes(T, Rtot, G, N, Kp, d, I, tile_rows, sm_count());
-    if (!routed) { ProfScope ps(0, s); EXFOLD_CUDA(launch_prefill_route(rp, s)); }
+    // (so do the small-batch kernels, unless the caller asks for the metadata, of which the scatter kernel writes a part)
+    const bool small_routed = small && meta == nullptr;
+    if (!routed && !small_routed) { ProfScope ps(0, s); EXFOLD_CUDA(launch_prefill_route(rp, s)); }
 
     // The shared expert's gate/up projection needs nothing the routing kernels produce (its rows are x itself, its
     // rows of H lie behind the routed ones): its whole row-tile pairs run on the second stream beside the scatter
@@ -624,6 +626,10 @@ int exfold_moe_prefill_ex(const exfold_layer* layer, const void* x, const float*
         sp.x = reinterpret_cast<const __nv_bfloat16*>(x); sp.wg = reinterpret_cast<const __nv_bfloat16*>(w_gate);
         sp.wu = reinterpret_cast<const __nv_bfloat16*>(w_up); sp.wd = reinterpret_cast<const __nv_bfloat16*>(w_down);
         sp.y = reinterpret_cast<__nv_bfloat16*>(y); sp.ids = rp.ids; sp.w_in = rp.w;
+        if (small_routed) {
+            sp.route = rp;
+            sp.status = rp.status;
+        }
         sp.B = (int)T; sp.N = N; sp.K = Kp; sp.M = N; sp.n_shared = l.n_shared; sp.d = d; sp.I = I;
         sp.max_groups = (int)std::min<int64_t>(N, R) + l.n_shared; sp.max_rows = (int)Rtot;
         sp.H = at<__nv_bfloat16>(ws, pl.H); sp.row_tok = cp.row_tok; sp.row_w = cp.row_w; sp.row_grp = at<int32_t>(ws, pl.row_grp);

@@ -327,7 +327,8 @@ struct DecodeSmallParams {
     const float* logits;  // [B][N], or null: ids and w64 come from the top-k kernel
     const int32_t* ids;
     const double* w64;
-    const float* w_in;    // prefill: the routes' final weights [B][K]; ids are then executed as they are, no pool, no remap
+    const float* w_in;    // prefill: the routes' final weights [B][K]; ids are then executed as they are, no pool, no remap,
+    PrefillRouteParams route;  // or, with route.logits set, the kernel routes the tokens itself (no metadata)
     const float* S;
     const float* L;
     const float* h;

@@ -28,6 +28,7 @@
 
 #include "common.cuh"
 #include "ptx.cuh"
+#include "route_token.cuh"
 
 #include <cooperative_groups.h>
 
@@ -120,7 +121,8 @@ __device__ __forceinline__ int compact_threads(bool flag, int* warp_cnt, int* li
     return all;
 }
 
-// GIVEN: the routes and their weights are final (prefill); else Top-K, pool and remap happen here
+// GIVEN: prefill, the routes and their weights are final (or found here, a token per warp, as prefill does); else Top-K, pool and
+// remap happen here
 template <bool GIVEN>
 __global__ void __launch_bounds__(kThreads, 2) decode_small_gateup_kernel(DecodeSmallParams p) {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -145,17 +147,24 @@ __global__ void __launch_bounds__(kThreads, 2) decode_small_gateup_kernel(Decode
 
     // ---- Eq. 2: a warp per token (or the result of the top-k kernel when that computed the scores)
     float v[8];
-    const bool ranks = !GIVEN && p.logits != nullptr && warp < B;
+    const float* logits = GIVEN ? p.route.logits : p.logits;
+    const bool ranks = logits != nullptr && warp < B;
     if (ranks) {
 #pragma unroll
-        for (int q = 0; q < 8; ++q) v[q] = lane + 32 * q < N ? p.logits[(size_t)warp * N + lane + 32 * q] : -INFINITY;
+        for (int q = 0; q < 8; ++q) v[q] = lane + 32 * q < N ? logits[(size_t)warp * N + lane + 32 * q] : -INFINITY;
     }
     // not before the wait: the caller may have written the table on this stream right before the call
     const float h_e = !GIVEN && !is_static && tid < N ? __ldg(p.h + tid) : 0.f;
     for (int t = 0; t < B; ++t)  // lands while the routing below runs
         for (int c = tid * 8; c < d; c += kThreads * 8) cp_async16(xs + t * xld + c, p.x + (size_t)t * d + c);
     asm volatile("cp.async.commit_group;" ::: "memory");
-    if (ranks) {
+    if (GIVEN && ranks) {
+        const TokenRoute r = route_token<8>(p.route, v, lane);
+        if (r.kept) {
+            ids[warp * K + r.rank] = r.id;
+            wrm[warp * K + r.rank] = r.w;
+        }
+    } else if (ranks) {
         int id;
         const double w = warp_topk_softmax<8>(v, N, K, lane, &id);
         if (lane < K) {
@@ -163,7 +172,7 @@ __global__ void __launch_bounds__(kThreads, 2) decode_small_gateup_kernel(Decode
             w64[warp * K + lane] = w;
         }
     }
-    if (GIVEN || p.logits == nullptr)
+    if (logits == nullptr)
         for (int s = tid; s < BK; s += kThreads) {
             ids[s] = p.ids[s];
             if (GIVEN) wrm[s] = p.w_in[s];
