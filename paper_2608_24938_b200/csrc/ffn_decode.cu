@@ -774,10 +774,9 @@ __global__ void __launch_bounds__(kFThreads, 1) decode_ffn_kernel(const __grid_c
                             const float h1 = __fdividef(g1, 1.0f + __expf(-g1)) * u1;
                             pk[j] = pack_bf16x2(h0, h1);
                         }
-                        uint4* dst = reinterpret_cast<uint4*>(p.H + rowpos * p.I + it.j0 + c * 32);
-#pragma unroll
-                        for (int j = 0; j < 4; ++j)
-                            dst[j] = make_uint4(pk[4 * j], pk[4 * j + 1], pk[4 * j + 2], pk[4 * j + 3]);
+                        __nv_bfloat16* dst = p.H + rowpos * p.I + it.j0 + c * 32;
+                        ptx::st_global32(dst, pk);
+                        ptx::st_global32(dst + 16, pk + 8);
                     }
                 }
             }

@@ -382,10 +382,9 @@ __global__ void __launch_bounds__(kXThreads, 1) grouped_gemm_mixed_kernel(const 
                             pk[j] = pack_bf16x2(__fdividef(g0, 1.0f + __expf(-g0)) * u0, __fdividef(g1, 1.0f + __expf(-g1)) * u1);
                         }
                         if (valid) {
-                            uint4* dst = reinterpret_cast<uint4*>(p.g.H + (size_t)grow * p.g.I + col0);
-#pragma unroll
-                            for (int j = 0; j < 4; ++j)
-                                dst[j] = make_uint4(pk[4 * j], pk[4 * j + 1], pk[4 * j + 2], pk[4 * j + 3]);
+                            __nv_bfloat16* dst = p.g.H + (size_t)grow * p.g.I + col0;
+                            ptx::st_global32(dst, pk);
+                            ptx::st_global32(dst + 16, pk + 8);
                         }
                     }
                 } else {

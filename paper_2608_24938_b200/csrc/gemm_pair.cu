@@ -301,10 +301,8 @@ __global__ void __launch_bounds__(kPThreads, 1) grouped_gemm_pair_kernel(const _
                         pk[j] = pack2_bf16(h0, h1);
                     }
                     if (valid) {
-                        uint4* dst = reinterpret_cast<uint4*>(p.H + grow * p.I + col0);
-#pragma unroll
-                        for (int j = 0; j < 4; ++j)
-                            dst[j] = make_uint4(pk[4 * j], pk[4 * j + 1], pk[4 * j + 2], pk[4 * j + 3]);
+                        ptx::st_global32(p.H + grow * p.I + col0, pk);
+                        ptx::st_global32(p.H + grow * p.I + col0 + 16, pk + 8);
                     }
                 }
             } else if (p.o32 != nullptr) {  // raw fp32 rows (calibration outputs)
