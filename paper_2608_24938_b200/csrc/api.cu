@@ -1007,7 +1007,7 @@ static int calibrate_enqueue(const exfold_layer* layer, const void* x_cal, const
     }
 
     char* cb = at<char>(ws, pl.calib);
-    cs.ids = ids; cs.m = m; cs.Ke = Ke; cs.d = d; cs.N = N;
+    cs.ids = ids; cs.status = status; cs.m = m; cs.Ke = Ke; cs.d = d; cs.N = N;
     cs.A = reinterpret_cast<double*>(cb); cs.Bv = cs.A + NN; cs.C = cs.Bv + NN;
     cs.H = cs.C + NN;
     cs.cnt = reinterpret_cast<int32_t*>(cs.H + N);
@@ -1015,7 +1015,7 @@ static int calibrate_enqueue(const exfold_layer* layer, const void* x_cal, const
     if (opts->mode == 1 && Ke >= 32)  // many experts per token: Gram-product form of the same sums
         EXFOLD_CUDA(launch_calib_stats_common(cs, at<double>(ws, pl.calib_nrm), sm_count(), s));
     else
-        EXFOLD_CUDA(launch_calib_stats(cs, s));
+        EXFOLD_CUDA(launch_calib_stats(cs, sm_count(), s));
     EXFOLD_CUDA(launch_calib_finalize(cs, *opts, out->S, out->L, out->h, out->lnh, out->n_obs, counts + job, s));
     return EXFOLD_OK;
 }

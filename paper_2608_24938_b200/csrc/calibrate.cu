@@ -3,6 +3,7 @@
 // weight w = |u|, accumulate A = sum w<v,u>, B = sum w|v|^2, C = sum w|u|^2 in double;
 // then S = clip(A / (B + lambda)), L = max(0, C - 2 S A + S^2 B) / (C + eps).
 #include "common.cuh"
+#include "ptx.cuh"
 
 #include <algorithm>
 
@@ -70,68 +71,117 @@ __device__ __forceinline__ void add_pair(const CalibStatsParams& p, int s, int t
     atomicAdd(&p.cnt[pq], 1);
 }
 
-// Pair sums of one token per warp, KE = Top-K <= 8: the token's KE output rows are read once, 16 bytes per lane and
-// row with the next chunk in flight, converted to double once, and all KE (KE + 1) / 2 inner products accumulate in
-// registers. Bound by reading the rows (4 KE d bytes per token). Before, a warp per ordered pair re-read both rows and
-// took three sums each: 8192 tokens x 8 rows x 2048 columns 619 us, now 137 (3.9 TB/s).
+// Pair sums of a token per warp, KE = Top-K <= 8: the token's KE output rows are read once, converted to double once, and all
+// KE (KE + 1) / 2 inner products accumulate in registers. Bound by reading the rows (4 KE d bytes per token). The rows come by
+// bulk copies into a ring of three stages of 256 columns per warp (lane a fetches row a; the next token's rows follow without a
+// gap): with eight warps and 192 KB per SM twice the bytes are in flight that registers could hold beside the sums, and the
+// double-precision units work meanwhile. 8192 tokens x 8 rows x 2048 columns: a warp per ordered pair 619 us, rows through
+// registers with one chunk ahead 137 (134 alone
+// under a profiler), this 101 alone (98 without the atomics).
+constexpr int kRingWarps = 8;
+constexpr int kRingStages = 3;
+constexpr int kRingCols = 256;
+
+__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(ptx::smem_u32(dst)), "l"(src),
+                 "r"(bytes), "r"(ptx::smem_u32(bar))
+                 : "memory");
+}
+
 template <int KE>
-__global__ void __launch_bounds__(kStatsThreads) calib_stats_kernel(CalibStatsParams p) {
+__global__ void __launch_bounds__(32 * kRingWarps) calib_stats_kernel(CalibStatsParams p) {
     constexpr int NV = KE * (KE + 1) / 2;
-    __shared__ double s_gram[kStatsThreads / 32][NV];
+    extern __shared__ __align__(128) float ring_all[];
+    __shared__ double s_gram[kRingWarps][NV];
+    __shared__ __align__(8) uint64_t bars[kRingWarps][kRingStages];
+    __shared__ int abort_s;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    float* ring = ring_all + (size_t)warp * kRingStages * KE * kRingCols;
+    if (lane == 0) {
+        for (int s = 0; s < kRingStages; ++s) ptx::mbar_init(&bars[warp][s], 1);
+        ptx::fence_mbar_init();
+    }
+    if (threadIdx.x == 0) abort_s = 0;
+    __syncthreads();
     grid_dep_launch();
     grid_dep_wait();
-    const int64_t i = (int64_t)blockIdx.x * (kStatsThreads / 32) + warp;
-    if (i >= p.m) return;
-    const int d = p.d;
-    const float* row[KE];
-#pragma unroll
-    for (int a = 0; a < KE; ++a) row[a] = p.out + stats_row(p, i, a) * d;
-    double acc[NV];
-#pragma unroll
-    for (int v = 0; v < NV; ++v) acc[v] = 0.0;
-    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-    float4 nxt[KE];
-    int c = lane * 4;
-#pragma unroll
-    for (int a = 0; a < KE; ++a) nxt[a] = c < d ? __ldcs(reinterpret_cast<const float4*>(row[a] + c)) : zero;
-    for (; c < d; c += 128) {
-        float4 cur[KE];
-#pragma unroll
-        for (int a = 0; a < KE; ++a) {
-            cur[a] = nxt[a];
-            nxt[a] = c + 128 < d ? __ldcs(reinterpret_cast<const float4*>(row[a] + c + 128)) : zero;
+    const int d = p.d, n_chunks = (d + kRingCols - 1) / kRingCols;
+    const int64_t step = (int64_t)gridDim.x * kRingWarps, i0 = (int64_t)blockIdx.x * kRingWarps + warp;
+    // the loads run ahead of the sums: chunk lc of token li into stage ls
+    int64_t li = i0;
+    int lc = 0, ls = 0;
+    const float* row = li < p.m && lane < KE ? p.out + stats_row(p, li, lane) * d : nullptr;
+    auto load = [&]() {
+        if (li >= p.m) return;
+        const int c0 = lc * kRingCols, cols = min(kRingCols, d - c0);
+        if (lane == 0) ptx::mbar_expect_tx(&bars[warp][ls], (uint32_t)(KE * cols * 4));
+        __syncwarp();
+        if (lane < KE) bulk_load(ring + (ls * KE + lane) * kRingCols, row + c0, (uint32_t)cols * 4, &bars[warp][ls]);
+        if (++ls == kRingStages) ls = 0;
+        if (++lc == n_chunks) {
+            lc = 0;
+            li += step;
+            if (li < p.m && lane < KE) row = p.out + stats_row(p, li, lane) * d;
         }
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            double o[KE];
-#pragma unroll
-            for (int a = 0; a < KE; ++a)
-                o[a] = (double)(q == 0 ? cur[a].x : q == 1 ? cur[a].y : q == 2 ? cur[a].z : cur[a].w);
-            int v = 0;
-#pragma unroll
-            for (int a = 0; a < KE; ++a)
-#pragma unroll
-                for (int b = a; b < KE; ++b, ++v) acc[v] = fma(o[a], o[b], acc[v]);
-        }
-    }
-    double* g = s_gram[warp];
-    warp_sums<NV>(acc, g, lane);
-    __syncwarp();
-    auto at = [](int a, int b) {  // place of (a, b) in the upper triangle
-        const int lo = a < b ? a : b, hi = a < b ? b : a;
-        return lo * KE - lo * (lo - 1) / 2 + (hi - lo);
     };
-    const int32_t* ids = p.ids + i * KE;
-    for (int q = lane; q < KE * KE; q += 32) {
-        const int a = q / KE, b = q - a * KE;
-        const double uu = g[at(a, a)], wi = sqrt(uu);
-        if (a == b) {
-            atomicAdd(&p.H[ids[a]], wi);
-            atomicAdd(&p.hc[ids[a]], 1);
-        } else {
-            add_pair(p, ids[a], ids[b], wi, uu, g[at(a, b)], g[at(b, b)]);
+#pragma unroll
+    for (int s = 0; s < kRingStages; ++s) load();
+    int cs = 0, cphase = 0;
+    for (int64_t i = i0; i < p.m; i += step) {
+        double acc[NV];
+#pragma unroll
+        for (int v = 0; v < NV; ++v) acc[v] = 0.0;
+        for (int k = 0; k < n_chunks; ++k) {
+            const bool ok = ptx::mbar_wait(&bars[warp][cs], cphase, &abort_s, p.status, 9);
+            if (!__all_sync(0xffffffffu, ok)) {
+                __nanosleep(100000);  // let any copy still in flight land before shared memory is released
+                return;
+            }
+            const float* st = ring + cs * KE * kRingCols;
+            const int cols = min(kRingCols, d - k * kRingCols);
+            for (int c = lane * 4; c < cols; c += 128) {
+                float4 cur[KE];
+#pragma unroll
+                for (int a = 0; a < KE; ++a) cur[a] = *reinterpret_cast<const float4*>(st + a * kRingCols + c);
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    double o[KE];
+#pragma unroll
+                    for (int a = 0; a < KE; ++a)
+                        o[a] = (double)(q == 0 ? cur[a].x : q == 1 ? cur[a].y : q == 2 ? cur[a].z : cur[a].w);
+                    int v = 0;
+#pragma unroll
+                    for (int a = 0; a < KE; ++a)
+#pragma unroll
+                        for (int b = a; b < KE; ++b, ++v) acc[v] = fma(o[a], o[b], acc[v]);
+                }
+            }
+            __syncwarp();  // the stage is used up
+            load();
+            if (++cs == kRingStages) {
+                cs = 0;
+                cphase ^= 1;
+            }
         }
+        double* g = s_gram[warp];
+        warp_sums<NV>(acc, g, lane);
+        __syncwarp();
+        auto at = [](int a, int b) {  // place of (a, b) in the upper triangle
+            const int lo = a < b ? a : b, hi = a < b ? b : a;
+            return lo * KE - lo * (lo - 1) / 2 + (hi - lo);
+        };
+        const int32_t* ids = p.ids + i * KE;
+        for (int q = lane; q < KE * KE; q += 32) {
+            const int a = q / KE, b = q - a * KE;
+            const double uu = g[at(a, a)], wi = sqrt(uu);
+            if (a == b) {
+                atomicAdd(&p.H[ids[a]], wi);
+                atomicAdd(&p.hc[ids[a]], 1);
+            } else {
+                add_pair(p, ids[a], ids[b], wi, uu, g[at(a, b)], g[at(b, b)]);
+            }
+        }
+        __syncwarp();
     }
 }
 
@@ -400,7 +450,15 @@ cudaError_t launch_calib_stats_common(const CalibStatsParams& p, double* nrm, in
     return cudaGetLastError();
 }
 
-cudaError_t launch_calib_stats(const CalibStatsParams& p, cudaStream_t s) {
+template <int KE>
+static cudaError_t launch_stats(const CalibStatsParams& p, int sms, cudaStream_t s) {
+    const size_t smem = (size_t)kRingWarps * kRingStages * KE * kRingCols * sizeof(float);
+    cudaError_t err = ensure_smem(calib_stats_kernel<KE>, smem);
+    if (err != cudaSuccess) return err;
+    const int64_t blocks = std::min<int64_t>((p.m + kRingWarps - 1) / kRingWarps, sms);
+    return launch_pdl(calib_stats_kernel<KE>, (unsigned)blocks, 32 * kRingWarps, smem, s, p);
+}
+cudaError_t launch_calib_stats(const CalibStatsParams& p, int sms, cudaStream_t s) {
     if (p.m == 0) return cudaSuccess;
     constexpr int kWarps = kStatsThreads / 32;
     if (p.Ke > kStatsRows) {
@@ -408,16 +466,15 @@ cudaError_t launch_calib_stats(const CalibStatsParams& p, cudaStream_t s) {
         const int64_t warps = p.m * (nb * (nb + 1) / 2);
         return launch_pdl(calib_stats_tiled_kernel, (unsigned)((warps + kWarps - 1) / kWarps), kStatsThreads, 0, s, p, nb);
     }
-    const unsigned grid = (unsigned)((p.m + kWarps - 1) / kWarps);
     switch (p.Ke) {
-        case 1: return launch_pdl(calib_stats_kernel<1>, grid, kStatsThreads, 0, s, p);
-        case 2: return launch_pdl(calib_stats_kernel<2>, grid, kStatsThreads, 0, s, p);
-        case 3: return launch_pdl(calib_stats_kernel<3>, grid, kStatsThreads, 0, s, p);
-        case 4: return launch_pdl(calib_stats_kernel<4>, grid, kStatsThreads, 0, s, p);
-        case 5: return launch_pdl(calib_stats_kernel<5>, grid, kStatsThreads, 0, s, p);
-        case 6: return launch_pdl(calib_stats_kernel<6>, grid, kStatsThreads, 0, s, p);
-        case 7: return launch_pdl(calib_stats_kernel<7>, grid, kStatsThreads, 0, s, p);
-        default: return launch_pdl(calib_stats_kernel<8>, grid, kStatsThreads, 0, s, p);
+        case 1: return launch_stats<1>(p, sms, s);
+        case 2: return launch_stats<2>(p, sms, s);
+        case 3: return launch_stats<3>(p, sms, s);
+        case 4: return launch_stats<4>(p, sms, s);
+        case 5: return launch_stats<5>(p, sms, s);
+        case 6: return launch_stats<6>(p, sms, s);
+        case 7: return launch_stats<7>(p, sms, s);
+        default: return launch_stats<8>(p, sms, s);
     }
 }
 

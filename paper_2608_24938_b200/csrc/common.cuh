@@ -440,8 +440,9 @@ struct CalibStatsParams {
     int32_t* cnt;  // [N][N]
     double* H;     // [N]
     int32_t* hc;   // [N]
+    DeviceStatus* status;
 };
-cudaError_t launch_calib_stats(const CalibStatsParams& p, cudaStream_t s);
+cudaError_t launch_calib_stats(const CalibStatsParams& p, int sms, cudaStream_t s);
 // Common-input mode with identity slots (slot a = expert a, inv_pos unused): same sums via per-token Gram
 // products held in registers; nrm is scratch for m*Ke doubles
 cudaError_t launch_calib_stats_common(const CalibStatsParams& p, double* nrm, int sms, cudaStream_t s);
