@@ -294,7 +294,8 @@ bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 
 // Row tiles of a grouped GEMM over `rows` sorted rows of G groups: on average half a tile per group is a ragged last one
 int64_t expected_tiles(int64_t rows, int G) { return rows / kTileM + G / 2; }
 
-// Whether the two GEMMs run their whole pairs of row tiles on CTA pairs (gemm_pair.cu: a third less operand traffic per
+// For the calls that use_mixed (below) leaves to row tiles of 128 rows, and with a shared expert for its early pairs:
+// whether the two GEMMs run their whole pairs of row tiles on CTA pairs (gemm_pair.cu: a third less operand traffic per
 // SM, a deeper ring) with the groups' odd last tiles beside them, or every tile on the one-CTA kernel. The pairs pay once
 // a group owns a tile or more on average (before, most tiles are odd ones, and the weights of a group with three tiles
 // are read by both passes) and the GEMMs are long enough for the second stream's fork and join: from ~400 k-blocks per
@@ -560,8 +561,8 @@ int exfold_moe_prefill_ex(const exfold_layer* layer, const void* x, const float*
     prof_reset();
     // Calls without the CTA-pair passes (fp32 layers, shorter bf16 prompts) are a chain of short kernels on one stream:
     // programmatic dependent launch hides their launches and set-up (Qwen3 shape 20 tokens 66.8 -> 56.5 us, 777 tokens 279
-    // -> 270; Mixtral shape 200 tokens 532 -> 514). The large calls launch plainly: early-resident successors compete with
-    // the running kernels (19-32 us slower).
+    // -> 270; Mixtral shape 200 tokens 532 -> 514). So are the mixed kernel's calls (0.5-1 % of the call). The CTA-pair passes
+    // beside odd-tile passes launch plainly: early-resident successors compete with the running kernels (19-32 us slower).
     PdlScope pdl_scope(!pairs || mixed);
 
     PrefillRouteParams rp{};

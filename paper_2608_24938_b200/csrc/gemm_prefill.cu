@@ -30,7 +30,8 @@ constexpr int kATileBytes = kTileM * kBK * 2;  // 16 KB
 constexpr int kBTileBytes = 256 * kBK * 2;     // 32 KB
 constexpr int kStageBytes = kATileBytes + kBTileBytes;
 constexpr int kGemmSmem = kStages * kStageBytes + 4 * kStageOutBytes + 1024;
-// One thread's loop {wait for the stage, expect_tx, 2-3 TMA issues} takes ~600-700 cycles: longer than the 512
+// One thread's loop {wait for the stage, expect_tx, 2-3 TMA issues} took ~600-700 cycles (on an elected lane some 400): with
+// the copies' own backpressure longer than the 512
 // cycles the tensor pipe needs for a k-block. The k-blocks are therefore dealt round-robin over kProducers
 // one-thread producers in warps of their own (warp 0 and the warps after the epilogue warps).
 constexpr int kProducers = 2;

@@ -75,3 +75,38 @@ def test_calibration(mode, m):
     seen = (ref["n_obs"] > 0) | np.eye(N, dtype=bool)
     np.testing.assert_allclose(L.cpu().numpy()[seen], ref["L"][seen], rtol=5e-3, atol=5e-3)
     np.testing.assert_allclose(h.cpu().numpy(), ref["h"], rtol=3e-3)
+
+
+@pytest.mark.parametrize("ns", [0, 1])
+def test_two_streams_and_a_replayed_graph(ns):
+    """The work counters lie in the workspace and start at zero in every call: calls of one thread on two streams, and a captured
+    call replayed, give the bits of the one-CTA kernel."""
+    T, Kp = 2049, 2
+    case = Case(si.LayerConfig("graph", 8, ns, 1024, 7168, 3, "bf16", T, (Kp,), 4, (2,)))
+    ex, dev = case.ex, case.dev
+    want = case.run_prefill(Kp, with_meta=False, gemm_path=1)["y"]
+    need = ex.exfold_workspace_bytes(case.layer, T, Kp)
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    wss = [torch.full((need,), 0xFF, dtype=torch.uint8, device=dev) for _ in streams]
+    ys = [torch.full((T, 1024), float("nan"), dtype=torch.bfloat16, device=dev) for _ in streams]
+
+    def call(i):
+        ex.exfold_moe_prefill(case.layer, case.d_x, case.d_lg, case.d_wg, case.d_wu, case.d_wd, case.tables, Kp, ys[i], wss[i], stream=streams[i])
+
+    torch.cuda.synchronize()
+    for _ in range(2):
+        for i in (0, 1):
+            call(i)
+    for i in (0, 1):
+        assert ex.exfold_device_status(wss[i], streams[i]) == 0
+        assert np.array_equal(ys[i].float().cpu().numpy(), want)
+    with torch.cuda.stream(streams[0]):
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=streams[0]):
+            call(0)
+        ys[0].fill_(float("nan"))
+        for _ in range(3):
+            graph.replay()
+        streams[0].synchronize()
+    assert ex.exfold_device_status(wss[0], streams[0]) == 0
+    assert np.array_equal(ys[0].float().cpu().numpy(), want)
