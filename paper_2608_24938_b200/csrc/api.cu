@@ -627,16 +627,13 @@ int exfold_moe_prefill_ex(const exfold_layer* layer, const void* x, const float*
         sp.x = reinterpret_cast<const __nv_bfloat16*>(x); sp.wg = reinterpret_cast<const __nv_bfloat16*>(w_gate);
         sp.wu = reinterpret_cast<const __nv_bfloat16*>(w_up); sp.wd = reinterpret_cast<const __nv_bfloat16*>(w_down);
         sp.y = reinterpret_cast<__nv_bfloat16*>(y); sp.ids = rp.ids; sp.w_in = rp.w;
-        if (small_routed) {
-            sp.route = rp;
-            sp.status = rp.status;
-        }
+        if (small_routed) sp.status = rp.status;
         sp.B = (int)T; sp.N = N; sp.K = Kp; sp.M = N; sp.n_shared = l.n_shared; sp.d = d; sp.I = I;
         sp.max_groups = (int)std::min<int64_t>(N, R) + l.n_shared; sp.max_rows = (int)Rtot;
         sp.H = at<__nv_bfloat16>(ws, pl.H); sp.row_tok = cp.row_tok; sp.row_w = cp.row_w; sp.row_grp = at<int32_t>(ws, pl.row_grp);
         sp.grp_expert = at<int32_t>(ws, pl.grp_expert); sp.n_groups = at<int32_t>(ws, pl.n_groups);
         ProfScope ps(3, s);
-        EXFOLD_CUDA(launch_decode_small(sp, sm_count(), s));
+        EXFOLD_CUDA(launch_decode_small(sp, small_routed ? &rp : nullptr, sm_count(), s));
     } else if (bf16) {
         GroupedGemmParams g{};
         g.tm_a = tm_xs; g.tm_a2 = tm_x; g.tm_b0 = tm_wg; g.tm_b1 = tm_wu; g.x_rows = (int)T; g.o32 = nullptr;
@@ -773,7 +770,7 @@ static int decode_impl(const exfold_layer* layer, const void* x, const float* lo
             sp.H = at<__nv_bfloat16>(ws, pl.H); sp.row_tok = rp.row_tok; sp.row_w = rp.row_w;
             sp.row_grp = at<int32_t>(ws, pl.row_grp); sp.grp_expert = rp.grp_expert; sp.n_groups = rp.n_groups;
             sp.status = w_router == nullptr ? rp.status : nullptr;
-            { ProfScope ps(14, s); EXFOLD_CUDA(launch_decode_small(sp, sm_count(), s)); }
+            { ProfScope ps(14, s); EXFOLD_CUDA(launch_decode_small(sp, nullptr, sm_count(), s)); }
         } else {
             // Token-parallel Top-K (with the router scores when w_router is given) -> gate/up kernel that finishes the
             // routing in its prologue and streams the pool's gate and up weights against x in place -> grouped down

@@ -327,8 +327,7 @@ struct DecodeSmallParams {
     const float* logits;  // [B][N], or null: ids and w64 come from the top-k kernel
     const int32_t* ids;
     const double* w64;
-    const float* w_in;    // prefill: the routes' final weights [B][K]; ids are then executed as they are, no pool, no remap,
-    PrefillRouteParams route;  // or, with route.logits set, the kernel routes the tokens itself (no metadata)
+    const float* w_in;    // prefill: the routes' final weights [B][K]; ids are then executed as they are, no pool, no remap
     const float* S;
     const float* L;
     const float* h;
@@ -356,7 +355,8 @@ struct DecodeSmallParams {
     DeviceStatus* status; // cleared here when this is the call's first kernel (else null)
 };
 bool decode_small_fits(int B, int K, int d, const void* wg, const void* wu, const void* wd);
-cudaError_t launch_decode_small(DecodeSmallParams p, int sms, cudaStream_t s);
+// route: prefill whose tokens the gate/up kernel routes itself (no metadata; ids and w_in unused), or null
+cudaError_t launch_decode_small(DecodeSmallParams p, const PrefillRouteParams* route, int sms, cudaStream_t s);
 cudaError_t launch_static_pool(int N, int M, const float* S, const float* L, const float* h, int32_t* pool_ids,
                                int32_t* target, float* scale, cudaStream_t s);
 

@@ -123,8 +123,10 @@ __device__ __forceinline__ int compact_threads(bool flag, int* warp_cnt, int* li
 
 // GIVEN: prefill, the routes and their weights are final (or found here, a token per warp, as prefill does); else Top-K, pool and
 // remap happen here
-template <bool GIVEN>
-__global__ void __launch_bounds__(kThreads, 2) decode_small_gateup_kernel(DecodeSmallParams p) {
+struct NoRoute {};
+template <bool GIVEN, typename R>  // R: PrefillRouteParams where the kernel routes prefill tokens (an argument that decode does without)
+__global__ void __launch_bounds__(kThreads, 2) decode_small_gateup_kernel(DecodeSmallParams p, R route) {
+    constexpr bool kRoutes = sizeof(R) > sizeof(NoRoute);
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ float4 s_red[2][kWarps][32];
     SmallState& sc = *reinterpret_cast<SmallState*>(smem);
@@ -147,8 +149,9 @@ __global__ void __launch_bounds__(kThreads, 2) decode_small_gateup_kernel(Decode
 
     // ---- Eq. 2: a warp per token (or the result of the top-k kernel when that computed the scores)
     float v[8];
-    const float* logits = GIVEN ? p.route.logits : p.logits;
-    const bool ranks = logits != nullptr && warp < B;
+    const float* logits = p.logits;
+    if constexpr (kRoutes) logits = route.logits;
+    const bool ranks = (kRoutes || !GIVEN) && logits != nullptr && warp < B;
     if (ranks) {
 #pragma unroll
         for (int q = 0; q < 8; ++q) v[q] = lane + 32 * q < N ? logits[(size_t)warp * N + lane + 32 * q] : -INFINITY;
@@ -158,13 +161,15 @@ __global__ void __launch_bounds__(kThreads, 2) decode_small_gateup_kernel(Decode
     for (int t = 0; t < B; ++t)  // lands while the routing below runs
         for (int c = tid * 8; c < d; c += kThreads * 8) cp_async16(xs + t * xld + c, p.x + (size_t)t * d + c);
     asm volatile("cp.async.commit_group;" ::: "memory");
-    if (GIVEN && ranks) {
-        const TokenRoute r = route_token<8>(p.route, v, lane);
-        if (r.kept) {
-            ids[warp * K + r.rank] = r.id;
-            wrm[warp * K + r.rank] = r.w;
+    if constexpr (kRoutes) {
+        if (ranks) {
+            const TokenRoute r = route_token<8>(route, v, lane);
+            if (r.kept) {
+                ids[warp * K + r.rank] = r.id;
+                wrm[warp * K + r.rank] = r.w;
+            }
         }
-    } else if (ranks) {
+    } else if (!GIVEN && ranks) {
         int id;
         const double w = warp_topk_softmax<8>(v, N, K, lane, &id);
         if (lane < K) {
@@ -172,7 +177,7 @@ __global__ void __launch_bounds__(kThreads, 2) decode_small_gateup_kernel(Decode
             w64[warp * K + lane] = w;
         }
     }
-    if (logits == nullptr)
+    if ((GIVEN && !kRoutes) || logits == nullptr)
         for (int s = tid; s < BK; s += kThreads) {
             ids[s] = p.ids[s];
             if (GIVEN) wrm[s] = p.w_in[s];
@@ -578,12 +583,15 @@ bool decode_small_fits(int B, int K, int d, const void* wg, const void* wu, cons
     return B <= kSmallDecodeBatch && gateup_bytes(B, K, d) <= 100 * 1024 && a32(wg) && a32(wu) && a32(wd);
 }
 
-cudaError_t launch_decode_small(DecodeSmallParams p, int sms, cudaStream_t s) {
+cudaError_t launch_decode_small(DecodeSmallParams p, const PrefillRouteParams* route, int sms, cudaStream_t s) {
     const size_t smem = gateup_bytes(p.B, p.K, p.d);
-    const auto gateup = p.w_in != nullptr ? decode_small_gateup_kernel<true> : decode_small_gateup_kernel<false>;
-    cudaError_t err = ensure_smem(gateup, smem);
-    if (err != cudaSuccess) return err;
-    err = launch_pdl(gateup, std::min(2 * sms, p.max_groups * (p.I / 8)), kThreads, smem, s, p);
+    auto gateup = [&](auto kernel, const auto& r) {
+        const cudaError_t e = ensure_smem(kernel, smem);
+        return e != cudaSuccess ? e : launch_pdl(kernel, std::min(2 * sms, p.max_groups * (p.I / 8)), kThreads, smem, s, p, r);
+    };
+    cudaError_t err = route != nullptr ? gateup(decode_small_gateup_kernel<true, PrefillRouteParams>, *route)
+                      : p.w_in != nullptr ? gateup(decode_small_gateup_kernel<true, NoRoute>, NoRoute{})
+                                          : gateup(decode_small_gateup_kernel<false, NoRoute>, NoRoute{});
     if (err != cudaSuccess) return err;
     // Down kernel, 16 warps per SM: one CTA of 16 warps when there are no more items than SMs (a cluster per item when
     // there are at most half as many), else two CTAs of 8 warps
