@@ -54,11 +54,12 @@ __device__ __forceinline__ TokenRoute route_token(const PrefillRouteParams& p, c
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
     const float w = ex / sum;
-    // ---- Eq. 10 on log scale: key = logit + ln h (one fp32 add); rank by (key desc, id asc)
-    const float key = has ? __fadd_rn(my_r, p.lnh != nullptr ? p.lnh[my_id] : 0.f) : -INFINITY;
+    // ---- Eq. 10 on log scale: key = logit + ln h (one fp32 add); rank by (key desc, id asc). Ranked by the integer images, of
+    // which any two compare also where a score or a norm is NaN: the ranks are places in arrays, no two the same, none left out.
+    const uint32_t key = has ? float_order_key(__fadd_rn(my_r, p.lnh != nullptr ? p.lnh[my_id] : 0.f)) : 0u;
     int rank = 0;
     for (int j = 0; j < K; ++j) {
-        float kj = __shfl_sync(0xffffffffu, key, j);
+        const uint32_t kj = __shfl_sync(0xffffffffu, key, j);
         int ij = __shfl_sync(0xffffffffu, my_id, j);
         if (has && j != lane && (kj > key || (kj == key && ij < my_id))) rank++;
     }

@@ -64,3 +64,42 @@ def test_a_broken_expert_touches_its_own_tokens_only(T, dtype, ns, bad):
             if bad != bad or w is not case.d_wg:  # (an infinite gate may be silu(-inf) = 0 or x - inf)
                 assert not np.isfinite(got[mine]).all(axis=1).any()
         w[3, 5, 7] = keep
+
+
+def check_routing_is_whole(got, T, K, Kp, N):
+    """Whatever the scores: Kp distinct experts per token, the omitted ones beside them, every route sorted once."""
+    routes = np.concatenate([got["ids"], got["omit_src"]], axis=1)
+    assert routes.min() >= 0 and routes.max() < N
+    assert all(len(set(r)) == K for r in routes.tolist())
+    assert np.array_equal(np.diff(got["offsets"]), np.bincount(got["ids"].ravel(), minlength=N))
+    assert got["offsets"][0] == 0 and np.array_equal(np.sort(got["perm"]), np.arange(T * Kp))
+
+
+@pytest.mark.parametrize("dtype,ns,N", [("bf16", 0, 12), ("bf16", 1, 40), ("f32", 0, 12), ("f32", 1, 140)])
+@pytest.mark.parametrize("T,K,Kp", [(1, 4, 2), (3, 4, 4), (8, 6, 3), (9, 4, 3), (64, 5, 2), (128, 4, 4), (300, 4, 2), (2300, 3, 2)])
+def test_prefill_tokens_of_non_finite_scores(T, K, Kp, dtype, ns, N):
+    """Scores of every third token NaN (of either sign), infinite or one of them, and a NaN norm: each token has its K' distinct
+    retained routes and the others keep their bits, with the metadata and without."""
+    case = Case(si.LayerConfig("nanscore", N, ns, 128, 192, K, dtype, T, (Kp,), 4, (2,)))
+    lg = case.lg.clone()
+    want = case.run_prefill(Kp)
+    bad = np.arange(T) % 3 == 0
+    kinds = [torch.full((N,), float("nan")), torch.full((N,), -float("nan")), torch.full((N,), float("inf")),
+             torch.full((N,), float("-inf")), torch.where(torch.arange(N) % 2 == 0, float("nan"), 1.0),
+             torch.where(torch.arange(N) == 5, float("inf"), 0.0), torch.where(torch.arange(N) % 3 == 0, -float("nan"), float("nan"))]
+    for j, i in enumerate(np.flatnonzero(bad)):
+        case.lg[i] = kinds[(j + T) % len(kinds)]
+    case.d_lg = case.lg.to(case.dev)
+    got = case.run_prefill(Kp)
+    check_routing_is_whole(got, T, K, Kp, N)
+    assert np.array_equal(got["y"][~bad], want["y"][~bad])
+    assert np.array_equal(got["y"], case.run_prefill(Kp, with_meta=False)["y"], equal_nan=True)
+    # a norm: its expert's tokens are folded in some order, the others' bits stay
+    case.d_lg = lg.to(case.dev)
+    S, L, h, lnh = (t.clone() for t in case.tables_host)
+    h[2] = lnh[2] = float("nan")
+    case.set_tables((S, L, h, lnh))
+    got = case.run_prefill(Kp)
+    check_routing_is_whole(got, T, K, Kp, N)
+    clean = (lg.topk(K, dim=1).indices != 2).all(dim=1).numpy()
+    assert np.array_equal(got["y"][clean], want["y"][clean])
