@@ -72,6 +72,12 @@ __device__ __forceinline__ uint32_t float_order_key(float f) {
 __device__ __forceinline__ float float_from_order_key(uint32_t k) {
     return __uint_as_float((k & 0x80000000u) ? (k & 0x7fffffffu) : ~k);
 }
+// The same for the doubles that pools are ranked by. Any two images compare, those of NaN too, so ranks counted on them are
+// places that no two experts share and none leaves out.
+__device__ __forceinline__ long long score_order_key(double score) {
+    const long long b = __double_as_longlong(score + 0.0);  // -0.0 as +0.0
+    return b < 0 ? b ^ 0x7FFFFFFFFFFFFFFFll : b;            // negative: larger magnitude = smaller
+}
 // Warp-wide (value desc, id asc) arg-max. Lanes without a candidate pass has = false. Returns the
 // winning id to every lane and its key through *key_out. At least one lane must have a candidate.
 __device__ __forceinline__ int warp_argmax(bool has, uint32_t key, int id, uint32_t* key_out) {

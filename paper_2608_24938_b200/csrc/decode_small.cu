@@ -219,10 +219,7 @@ __global__ void __launch_bounds__(kThreads, 2) decode_small_gateup_kernel(Decode
                 const unsigned long long acc = (unsigned long long)sc.acc32[3 * tid] +
                                                ((unsigned long long)sc.acc32[3 * tid + 1] << 21) +
                                                ((unsigned long long)sc.acc32[3 * tid + 2] << 42);
-                const double score = (double)acc * (1.0 / 9007199254740992.0) * (double)h_e + 0.0;
-                long long key = __double_as_longlong(score);
-                if (key < 0) key ^= 0x7FFFFFFFFFFFFFFFll;  // negative doubles: larger magnitude = smaller
-                sc.key[mine] = key;
+                sc.key[mine] = score_order_key((double)acc * (1.0 / 9007199254740992.0) * (double)h_e);
             }
             __syncthreads();
             int lanes = 32;  // threads per member

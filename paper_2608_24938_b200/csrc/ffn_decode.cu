@@ -342,9 +342,8 @@ __global__ void __launch_bounds__(kFThreads, 1) decode_ffn_kernel(const __grid_c
                 const unsigned long long acc = (unsigned long long)sc.acc32[3 * e] +
                                                ((unsigned long long)sc.acc32[3 * e + 1] << 21) +
                                                ((unsigned long long)sc.acc32[3 * e + 2] << 42);
-                const double score = (double)acc * (1.0 / 9007199254740992.0) * (double)(c < kFThreads / 32 ? h_e[0] : h_e[1]) + 0.0;
-                long long key = __double_as_longlong(score);
-                if (key < 0) key ^= 0x7FFFFFFFFFFFFFFFll;  // negative doubles: larger magnitude = smaller
+                const long long key =
+                    score_order_key((double)acc * (1.0 / 9007199254740992.0) * (double)(c < kFThreads / 32 ? h_e[0] : h_e[1]));
                 member[pos] = e;
                 sc.key[pos] = key;
                 khi[pos] = (int)(key >> 32);

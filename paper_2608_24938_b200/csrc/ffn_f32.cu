@@ -234,7 +234,7 @@ __device__ __forceinline__ bool route_tile(const FfnF32Route& rt, cg::cluster_gr
 // decode_route_kernel's. Whole call before / now: tiny layer 16 tokens 16.1 / 12.7 us, one 15.5 / 12.3, 74 19.9 / 15.0.
 struct DecodeRouteSmem {
     double w64[kRoutedSlots];
-    double score[kRoutedExperts];
+    long long key[kRoutedExperts];           // order-preserving image of the expert's score
     unsigned long long acc[kRoutedExperts];  // sum_i w_{i,e} in 2^-53 units: exact, order-independent
     short id[kRoutedSlots];
     float wrm[kRoutedSlots];  // remapped weights
@@ -261,7 +261,6 @@ __device__ __forceinline__ bool route_tile(const DecodeRouteParams& p, cg::clust
         sm.acc[e] = 0ull;
         sm.in_union[e] = 0;
         sm.rank_of[e] = -1;
-        sm.pool[e] = 0;  // (a NaN norm leaves ranks that no expert has)
     }
     for (int i = tid; i < kRoutedExperts * (kRoutedTokens / 32); i += kThreads) (&sm.mask[0][0])[i] = 0u;
     if (tid == 0) st->g = -1;
@@ -310,14 +309,14 @@ __device__ __forceinline__ bool route_tile(const DecodeRouteParams& p, cg::clust
         int in = 0;
         if (tid < N) {
             in = sm.in_union[tid];
-            sm.score[tid] = (double)sm.acc[tid] * (1.0 / 9007199254740992.0) * (double)p.h[tid];
+            sm.key[tid] = score_order_key((double)sm.acc[tid] * (1.0 / 9007199254740992.0) * (double)p.h[tid]);
         }
         const int usz = __syncthreads_count(in);
         if (in) {
-            const double se = sm.score[tid];
+            const long long ke = sm.key[tid];
             int better = 0;
             for (int o = 0; o < N; ++o)
-                better += sm.in_union[o] && (sm.score[o] > se || (sm.score[o] == se && o < tid)) ? 1 : 0;
+                better += sm.in_union[o] && (sm.key[o] > ke || (sm.key[o] == ke && o < tid)) ? 1 : 0;
             if (better < M) {
                 sm.rank_of[tid] = better;
                 sm.pool[better] = tid;

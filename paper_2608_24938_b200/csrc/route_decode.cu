@@ -26,7 +26,7 @@ struct DecSmem {
     double w64[kDecMaxSlots];
     int ids[kDecMaxSlots];
     float wrm[kDecMaxSlots];  // remapped weights
-    double score[kMaxExperts];
+    long long key[kMaxExperts];           // order-preserving image of the expert's score
     unsigned long long acc[kMaxExperts];  // sum_i w_{i,e} in fixed point (2^-53 units): exact, order-independent
     int in_union[kMaxExperts];
     int rank_of[kMaxExperts];   // pool rank or -1
@@ -175,7 +175,7 @@ __global__ void __launch_bounds__(kDecThreads) decode_route_kernel(DecodeRoutePa
     // ---- Eq. 11: score_e = h_e * sum_i w_{i,e} (every CTA computes the same pool from the same sums)
     if (!is_static)
         for (int e = threadIdx.x; e < N; e += kDecThreads)
-            sm.score[e] = (double)sm.acc[e] * (1.0 / 9007199254740992.0) * (double)sm.hh[e];
+            sm.key[e] = score_order_key((double)sm.acc[e] * (1.0 / 9007199254740992.0) * (double)sm.hh[e]);
     __syncthreads();
     // pool = best min(M, |U|) experts of the union by (score desc, id asc): rank by counting. Experts are
     // dealt round-robin over the CTAs, one warp per expert; ranks are broadcast to every copy.
@@ -187,10 +187,10 @@ __global__ void __launch_bounds__(kDecThreads) decode_route_kernel(DecodeRoutePa
         if (threadIdx.x == 0) sm.P = usz < M ? usz : M;
         for (int e = rank + nct * warp; e < N; e += nct * kWarps) {
             if (!sm.in_union[e]) continue;  // warp-uniform
-            const double se = sm.score[e];
+            const long long ke = sm.key[e];
             int better = 0;
             for (int o = lane; o < N; o += 32)
-                if (sm.in_union[o] && (sm.score[o] > se || (sm.score[o] == se && o < e))) better++;
+                if (sm.in_union[o] && (sm.key[o] > ke || (sm.key[o] == ke && o < e))) better++;
 #pragma unroll
             for (int off = 16; off > 0; off >>= 1) better += __shfl_xor_sync(0xffffffffu, better, off);
             if (better < M && lane < nct) {

@@ -3,8 +3,9 @@ import numpy as np
 import pytest
 import torch
 
+import oracle
 import synth_inputs as si
-from harness import Case, check_decode_meta, check_output
+from harness import A, Case, check_decode_meta, check_output
 
 pytestmark = pytest.mark.gpu
 
@@ -103,3 +104,38 @@ def test_prefill_tokens_of_non_finite_scores(T, K, Kp, dtype, ns, N):
     check_routing_is_whole(got, T, K, Kp, N)
     clean = (lg.topk(K, dim=1).indices != 2).all(dim=1).numpy()
     assert np.array_equal(got["y"][clean], want["y"][clean])
+
+
+def bad_scores(lgd):
+    """Every fourth token's scores NaN or infinite, in part or in whole; which tokens."""
+    B, N = lgd.shape
+    kinds = [torch.full((N,), float("nan")), torch.full((N,), float("inf")), torch.full((N,), float("-inf")),
+             torch.where(torch.arange(N) % 2 == 0, -float("nan"), 1.0)]
+    bad = np.arange(B) % 4 == 2
+    for j, i in enumerate(np.flatnonzero(bad)):
+        lgd[i] = kinds[j % len(kinds)]
+    return bad
+
+
+@pytest.mark.parametrize("dtype,ns,N", [("bf16", 0, 24), ("bf16", 1, 200), ("f32", 0, 24), ("f32", 1, 120), ("f32", 0, 140)])
+@pytest.mark.parametrize("B", [1, 3, 8, 20, 60, 129, 200])
+@pytest.mark.parametrize("M", [1, 5, 20])
+def test_decode_pool_of_non_finite_norms(B, M, dtype, ns, N):
+    """A third of the norms NaN or infinite and some tokens' scores too: a pool of distinct experts of the batch, every route on one
+    of them, and the tokens of finite scores are the sums over the routes that the metadata names."""
+    K = 4
+    case = Case(si.LayerConfig("nannorm", N, ns, 128, 192, K, dtype, 8, (1,), B, (M,)))
+    S, L, h, lnh = (t.clone() for t in case.tables_host)
+    h[::3], h[1::7], h[2::11] = float("nan"), float("inf"), -float("nan")
+    case.set_tables((S, L, h, lnh))
+    bad = bad_scores(case.lgd)
+    case.d_lgd = case.lgd.to(case.dev)
+    got = case.run_decode(M)
+    P, pool = int(got["pool_size"][0]), got["pool_ids"]
+    assert 1 <= P <= M and len(set(pool[:P].tolist())) == P and pool[:P].min() >= 0 and pool[:P].max() < N and (pool[P:] == -1).all()
+    mask = got["pool_mask"].view(np.uint32)
+    assert sorted(pool[:P].tolist()) == [e for e in range(N) if mask[e >> 5] >> (e & 31) & 1]
+    assert np.isin(got["ids"], pool[:P]).all() and np.isin(got["target"], pool[:P]).all()
+    assert np.array_equal(got["y"], case.run_decode(M, with_meta=False)["y"], equal_nan=True)
+    yr = oracle.moe_apply(A(case.xd), A(case.wg), A(case.wu), A(case.wd), got["ids"], np.where(bad[:, None], 0, got["w"]).astype(np.float32), N, ns)
+    check_output(got["y"][~bad], yr[~bad], dtype)
