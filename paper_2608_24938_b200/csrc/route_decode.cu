@@ -463,10 +463,10 @@ __global__ void __launch_bounds__(256) static_pool_kernel(int N, int M, const fl
     grid_dep_launch();
     grid_dep_wait();
     for (int e = threadIdx.x; e < N; e += blockDim.x) {
-        const float he = h[e];
+        const uint32_t he = float_order_key(h[e]);  // (a NaN norm has its place among the others, so that no pool slot stays unwritten)
         int better = 0;
         for (int o = 0; o < N; ++o) {
-            const float ho = h[o];
+            const uint32_t ho = float_order_key(h[o]);
             if (ho > he || (ho == he && o < e)) better++;
         }
         rank_of[e] = better < M ? better : -1;

@@ -139,3 +139,28 @@ def test_decode_pool_of_non_finite_norms(B, M, dtype, ns, N):
     assert np.array_equal(got["y"], case.run_decode(M, with_meta=False)["y"], equal_nan=True)
     yr = oracle.moe_apply(A(case.xd), A(case.wg), A(case.wu), A(case.wd), got["ids"], np.where(bad[:, None], 0, got["w"]).astype(np.float32), N, ns)
     check_output(got["y"][~bad], yr[~bad], dtype)
+
+
+@pytest.mark.parametrize("dtype,N,B", [("bf16", 24, 5), ("bf16", 200, 40), ("bf16", 24, 200), ("f32", 24, 40), ("f32", 140, 40)])
+@pytest.mark.parametrize("M", [1, 5, 20])
+def test_static_pool_of_non_finite_norms(M, dtype, N, B):
+    """The static pool built from norms of which a third are NaN or infinite: M distinct experts, every target among them; a step on
+    it is the sum over the remapped routes."""
+    K, d = 4, 128
+    case = Case(si.LayerConfig("nanstat", N, 0, d, 192, K, dtype, 8, (1,), B, (M,)))
+    ex, dev = case.ex, case.dev
+    S, L, h, lnh = (t.clone() for t in case.tables_host)
+    h[::3], h[1::7], h[2::11] = float("nan"), float("inf"), -float("nan")
+    case.set_tables((S, L, h, lnh))
+    pool_t = [torch.full((M,), -7, dtype=torch.int32, device=dev), torch.full((N,), -7, dtype=torch.int32, device=dev), torch.empty(N, device=dev)]
+    pool = ex.exfold_static_pool_build(case.layer, case.tables, M, *pool_t)
+    ids, target, scale = (t.cpu().numpy() for t in pool_t)
+    assert len(set(ids.tolist())) == M and ids.min() >= 0 and ids.max() < N
+    assert np.isin(target, ids).all() and np.array_equal(target[ids], ids)
+    out, w = torch.empty((B, K), dtype=torch.int32, device=dev), torch.empty((B, K), device=dev)
+    y, ws = torch.full((B, d), float("nan"), dtype=case.d_wg.dtype, device=dev), case.workspace(B, K)
+    ex.exfold_moe_decode_static(case.layer, case.d_xd, case.d_lgd, case.d_wg, case.d_wu, case.d_wd, pool, y, ws, meta=dict(ids=out, w=w))
+    assert ex.exfold_device_status(ws) == 0
+    assert np.array_equal(out.cpu().numpy(), target[case.lgd.topk(K, dim=1).indices.numpy()])
+    yr = oracle.moe_apply(A(case.xd), A(case.wg), A(case.wu), A(case.wd), out.cpu().numpy(), w.cpu().numpy(), N, 0)
+    check_output(y.float().cpu().numpy(), yr, dtype)
