@@ -650,7 +650,7 @@ __global__ void __launch_bounds__(kFThreads, 1) decode_ffn_kernel(const __grid_c
                         }
                     }
                 }
-                if (NMT == 2) ok = __shfl_sync(0xffffffffu, ok, 0);
+                if (NMT == 2) ok = __all_sync(0xffffffffu, ok);  // (whichever lane was elected and gave up)
             }
         }
         __syncwarp();
