@@ -198,7 +198,8 @@ int exfold_moe_prefill(const exfold_layer *layer, const void *x, const float *lo
  *                     w_s c S[s][t] is folded onto t and w_s (1 - c) is spread over the retained
  *                     routes in proportion to their original router weights.
  *   gemm_path         0: the library chooses the tensor-core kernels (above); 1: one-CTA kernel only;
- *                     2: CTA pairs wherever a group has a pair of row tiles. Same results bit for bit.
+ *                     2: CTA pairs wherever a group has a pair of row tiles; 3: the one pass over whole and
+ *                     ragged tiles. Same results bit for bit.
  */
 typedef struct {
     float loss_threshold;

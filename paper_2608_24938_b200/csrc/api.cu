@@ -545,9 +545,9 @@ int exfold_moe_prefill_ex(const exfold_layer* layer, const void* x, const float*
     const bool direct = Kp == 1 && l.n_shared == 0;  // every token is written exactly once
 
     CUtensorMap tm_xs, tm_x, tm_wg, tm_wu, tm_h, tm_wd, tm_wd_half;
-    const int mode = opts == nullptr || opts->gemm_path < 0 || opts->gemm_path > 2 ? 0 : opts->gemm_path;
-    const bool pairs = bf16 && !small && (mode == 2 ? Rtot >= 2 * kTileM : mode == 0 && use_pairs(Rtot, G, d, I));
-    const bool mixed = bf16 && !small && mode == 0 && use_mixed(Rtot, G, d, I);
+    const int mode = opts == nullptr || opts->gemm_path < 0 || opts->gemm_path > 3 ? 0 : opts->gemm_path;
+    const bool pairs = bf16 && !small && (mode == 2 ? Rtot >= 2 * kTileM : mode != 1 && use_pairs(Rtot, G, d, I));
+    const bool mixed = bf16 && !small && (mode == 3 || (mode == 0 && use_mixed(Rtot, G, d, I)));
     const int sms = sm_count() & ~1;
     if (bf16 && !small) {
         const uint64_t E = (uint64_t)G;

@@ -1,5 +1,6 @@
 """Whole row tiles and ragged remainders in one pass (gemm_mixed.cu), at the group sizes where it can go wrong: against the
-one-CTA kernel bit for bit (the same products accumulated in the same order) and against the CPU oracle."""
+one-CTA kernel bit for bit (the same products accumulated in the same order) and against the CPU oracle. MIXED forces the pass, so
+that the sizes here do not hang on the library's choice."""
 import numpy as np
 import pytest
 import torch
@@ -9,16 +10,35 @@ import synth_inputs as si
 from harness import A, Case, check_output, check_prefill_meta
 
 pytestmark = pytest.mark.gpu
+ONE_CTA, PAIRS, MIXED = 1, 2, 3  # gemm_path
 
 EDGES = [0, 1, 2, 31, 32, 33, 63, 64, 65, 96, 97, 127, 128, 129, 160, 161, 192, 193, 223, 224, 225, 255, 256, 257, 288, 289, 383, 384,
          480, 481, 511, 512, 513, 767, 768, 769]
 
 
-@pytest.mark.parametrize("d,I", [(64, 896), (320, 832), (1088, 64 * 13)])
-def test_group_sizes_at_the_edges_of_tiles(d, I):
-    """One route per token, dealt so that the experts own exactly the sizes above: one k-block, K and N tails, column tiles of
-    which the second CTA has none, groups without rows."""
-    sizes = (EDGES * 2)[:64]
+def mixed_ran(case, Kp, gemm_path=0):
+    """Whether a call ran the pass: it draws its items from the two work counters in the status record (words 4 and 5), which the
+    other kernels leave as they were."""
+    ws = case.workspace(case.T, Kp)  # all bytes 0xFF
+    y = torch.empty((case.T, case.cfg.hidden), dtype=case.d_wg.dtype, device=case.dev)
+    case.ex.exfold_moe_prefill_ex(case.layer, case.d_x, case.d_lg, case.d_wg, case.d_wu, case.d_wd, case.tables, Kp, y, ws, gemm_path=gemm_path)
+    torch.cuda.synchronize()
+    return ws[16:24].view(torch.int32).tolist() != [-1, -1]
+
+
+@pytest.mark.parametrize("N,ns,d,I,K,Kp,T", [(64, 0, 192, 64, 2, 1, 200), (8, 1, 1024, 7168, 3, 2, 2100)])
+def test_gemm_path_forces_the_pass(N, ns, d, I, K, Kp, T):
+    """The counters move with MIXED, whatever the size, and with no other forced path."""
+    case = Case(si.LayerConfig("forced", N, ns, d, I, K, "bf16", T, (Kp,), 4, (2,)))
+    assert mixed_ran(case, Kp, MIXED) and not mixed_ran(case, Kp, ONE_CTA) and not mixed_ran(case, Kp, PAIRS)
+
+
+@pytest.mark.parametrize("n_groups", [5, 64])
+@pytest.mark.parametrize("d,I", [(64, 64), (64, 896), (320, 832), (1088, 64 * 13), (192, 128)])
+def test_group_sizes_at_the_edges_of_tiles(d, I, n_groups):
+    """One route per token, dealt so that the experts own exactly the sizes above: one k-block, K and N tails, one column tile, column
+    tiles of which the second CTA has none, groups without rows, fewer items than CTA pairs."""
+    sizes = EDGES[-5:] if n_groups == 5 else (EDGES * 2)[:64]
     T, N = sum(sizes), len(sizes)
     case = Case(si.LayerConfig("edges", N, 0, d, I, 2, "bf16", T, (1,), 4, (2,)))
     owner = np.repeat(np.arange(N), sizes)[np.random.default_rng(3).permutation(T)]
@@ -27,7 +47,7 @@ def test_group_sizes_at_the_edges_of_tiles(d, I):
     lg[torch.arange(T), torch.from_numpy((owner + 1) % N)] = -3.0
     case.lg, case.d_lg = lg, lg.to(case.dev)
     case.set_tables((case.tables_host[0], case.tables_host[1], torch.ones(N), torch.zeros(N)))
-    got, one = case.run_prefill(1), case.run_prefill(1, with_meta=False, gemm_path=1)["y"]
+    got, one = case.run_prefill(1, gemm_path=MIXED), case.run_prefill(1, with_meta=False, gemm_path=ONE_CTA)["y"]
     assert np.array_equal(np.diff(got["offsets"]), sizes)
     assert np.array_equal(got["y"], one)
     idx = np.random.default_rng(4).choice(T, 300, replace=False)
@@ -39,26 +59,27 @@ def test_shared_expert_beside_the_scatter_kernel(T):
     """A shared expert whose gate/up pairs run on the second stream: the pass takes what is left of its group (an odd last row
     tile, or nothing), and all of it in the down projection."""
     case = Case(si.LayerConfig("shared", 8, 1, 1024, 7168, 3, "bf16", T, (2,), 4, (2,)))
-    got, one = case.run_prefill(2), case.run_prefill(2, with_meta=False, gemm_path=1)["y"]
+    got, one = case.run_prefill(2, gemm_path=MIXED), case.run_prefill(2, with_meta=False, gemm_path=ONE_CTA)["y"]
     assert np.array_equal(got["y"], one)
     idx = np.random.default_rng(5).choice(T, 24, replace=False)
     check_output(got["y"][idx], case.oracle_prefill(2, tok_idx=idx)["y"], "bf16")
 
 
-@pytest.mark.parametrize("Kp,ns,T,d", [(2, 0, 4000, 192), (3, 1, 2500, 128), (3, 0, 40, 3136)])
+@pytest.mark.parametrize("Kp,ns,T,d", [(2, 0, 4000, 192), (3, 1, 2500, 128), (3, 0, 40, 3136), (4, 1, 9, 64)])
 def test_rows_of_several_routes(Kp, ns, T, d):
     """Several routes per token through the per-route buffer; few rows of a wide layer."""
     case = Case(si.LayerConfig("routes", 64, ns, d, 896, 4, "bf16", T, (Kp,), 4, (2,), logits="zipf"))
-    got, ref = case.run_prefill(Kp), case.oracle_prefill(Kp, tok_idx=np.arange(min(T, 200)))
+    got, ref = case.run_prefill(Kp, gemm_path=MIXED), case.oracle_prefill(Kp, tok_idx=np.arange(min(T, 200)))
     check_prefill_meta(got, ref)
     check_output(got["y"][:200], ref["y"], "bf16")
-    assert np.array_equal(got["y"], case.run_prefill(Kp, with_meta=False, gemm_path=1)["y"])
+    assert np.array_equal(got["y"], case.run_prefill(Kp, with_meta=False, gemm_path=ONE_CTA)["y"])
 
 
-@pytest.mark.parametrize("mode,m", [(0, 2000), (1, 130), (1, 225)])
+@pytest.mark.parametrize("mode,m", [(0, 1600), (1, 775), (1, 993)])
 def test_calibration(mode, m):
-    """fp32 rows of whole and ragged items: the oracle's tables, tolerances as in test_calibrate_bf16_on_tensor_cores."""
-    cfg = si.LayerConfig("calib", 64, 0, 128, 896, 4, "bf16", 64, (2,), 4, (2,))
+    """fp32 rows of whole and ragged items (775 = 3 x 256 + 7; 993: a rest of 225 rows, a whole item) in a calibration that takes the
+    pass: the oracle's tables, tolerances as in test_calibrate_bf16_on_tensor_cores."""
+    cfg = si.LayerConfig("calib", 8, 0, 256, 2432, 4, "bf16", 64, (2,), 4, (2,))
     case = Case(cfg, correlated=0.8)
     ex, dev, N = case.ex, case.dev, cfg.n_experts
     xc, lc = si.hidden_states(cfg, m, "x_cal"), si.router_logits(cfg, m, "logits_cal")
@@ -69,6 +90,7 @@ def test_calibration(mode, m):
     ws = ex.alloc_workspace(case.layer, m, N if mode else cfg.top_k)
     ws.fill_(0xFF)
     ex.exfold_calibrate(case.layer, xc.to(dev), lc.to(dev), case.d_wg, case.d_wu, case.d_wd, ex.make_tables(S, L, h, lnh, n_obs), ws, mode=mode)
+    assert min(ws[16:24].view(torch.int32).tolist()) > 0  # the pass's work counters
     assert ex.exfold_device_status(ws) == 0
     assert np.array_equal(n_obs.cpu().numpy(), ref["n_obs"])
     np.testing.assert_allclose(S.cpu().numpy(), ref["S"], rtol=5e-3, atol=5e-3)
@@ -84,14 +106,15 @@ def test_two_streams_and_a_replayed_graph(ns):
     T, Kp = 2049, 2
     case = Case(si.LayerConfig("graph", 8, ns, 1024, 7168, 3, "bf16", T, (Kp,), 4, (2,)))
     ex, dev = case.ex, case.dev
-    want = case.run_prefill(Kp, with_meta=False, gemm_path=1)["y"]
+    want = case.run_prefill(Kp, with_meta=False, gemm_path=ONE_CTA)["y"]
     need = ex.exfold_workspace_bytes(case.layer, T, Kp)
     streams = [torch.cuda.Stream(), torch.cuda.Stream()]
     wss = [torch.full((need,), 0xFF, dtype=torch.uint8, device=dev) for _ in streams]
     ys = [torch.full((T, 1024), float("nan"), dtype=torch.bfloat16, device=dev) for _ in streams]
 
     def call(i):
-        ex.exfold_moe_prefill(case.layer, case.d_x, case.d_lg, case.d_wg, case.d_wu, case.d_wd, case.tables, Kp, ys[i], wss[i], stream=streams[i])
+        ex.exfold_moe_prefill_ex(case.layer, case.d_x, case.d_lg, case.d_wg, case.d_wu, case.d_wd, case.tables, Kp, ys[i], wss[i],
+                                 gemm_path=MIXED, stream=streams[i])
 
     torch.cuda.synchronize()
     for _ in range(2):
