@@ -580,7 +580,7 @@ int exfold_moe_prefill_ex(const exfold_layer* layer, const void* x, const float*
     rp.queue = mixed ? at<DeviceStatus>(ws, pl.status)->queue : nullptr;
     // few tokens of an fp32 layer: its FFN kernel routes them itself
     const int tile_rows = mixed ? kMixedTiles : bf16 ? kTileM : ffn_f32_tile_rows(Rtot, G, d, I, sm_count());
-    const bool routed = !bf16 && ffn_f32_routes(T, Rtot, G, N, Kp, d, I, tile_rows, sm_count());
+    const bool routed = !bf16 && ffn_f32_routes(false, T, Rtot, G, N, Kp, d, I, tile_rows, sm_count());
     // (so do the small-batch kernels, unless the caller asks for the metadata, of which the scatter kernel writes a part)
     const bool small_routed = small && meta == nullptr;
     if (!routed && !small_routed) { ProfScope ps(0, s); EXFOLD_CUDA(launch_prefill_route(rp, s)); }
@@ -841,7 +841,7 @@ static int decode_impl(const exfold_layer* layer, const void* x, const float* lo
         // a token has at most as many rows as the pool has experts
         const int64_t rows = B * std::min(K, (int)pool_m) + B * l.n_shared;
         rp.tile_rows = ffn_f32_tile_rows(rows, max_groups, d, I, sm_count());
-        const bool routed = ffn_f32_routes(B, rows, max_groups, N, K, d, I, rp.tile_rows, sm_count());
+        const bool routed = ffn_f32_routes(true, B, rows, max_groups, N, K, d, I, rp.tile_rows, sm_count());
         if (!routed) { ProfScope ps(6, s); EXFOLD_CUDA(launch_decode_route(rp, s)); }
         FfnF32Params fp = f32_params(x, w_gate, w_up, w_down, d, I, max_groups, rp.tile_rows);
         fp.offsets = rp.grp_off; fp.tile_start = rp.grp_tiles; fp.grp_expert = rp.grp_expert; fp.n_groups_dev = rp.n_groups;

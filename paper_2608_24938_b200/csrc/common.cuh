@@ -397,8 +397,8 @@ struct FfnF32Route {
     int32_t* row_tok;
     float* row_w;
 };
-// rows: of all groups, at most; slots: routes per token that the kernel holds
-bool ffn_f32_routes(int64_t T, int64_t rows, int G, int N, int slots, int d, int I, int tile_rows, int sms);
+// rows: of all groups, at most; slots: routes per token that the kernel holds; decode: its routing (more state than prefill's)
+bool ffn_f32_routes(bool decode, int64_t T, int64_t rows, int G, int N, int slots, int d, int I, int tile_rows, int sms);
 cudaError_t launch_ffn_f32_routed(const FfnF32Params& p, const FfnF32Route& rt, int64_t rows, cudaStream_t s);
 // Decode of few tokens, likewise (the group tables of rt are not written)
 cudaError_t launch_ffn_f32_routed(const FfnF32Params& p, const DecodeRouteParams& rt, int64_t rows, cudaStream_t s);

@@ -774,6 +774,9 @@ __global__ void __launch_bounds__(kThreads, 2) ffn_f32_tall_kernel(FfnF32Params 
 constexpr size_t kSmemLimit = 227 * 1024 - 1024;
 int features_per_cta(int I, int cl) { return ((I + cl - 1) / cl + kKC - 1) / kKC * kKC; }
 size_t short_bytes(int d, int I) { return (size_t)kSR * ((d + 127) / 128 * 128 + (I + 127) / 128 * 128 + 4) * sizeof(float); }
+// CTAs of the short form that run at once, of `bytes` of shared memory each: two to an SM (what their registers allow) while an SM
+// holds twice the memory (d + I up to 3580, 3130 where decode is routed in it), else one; in clusters of eight some nine tenths
+int64_t short_wave(size_t bytes, int sms) { return (int64_t)sms * (2 * (bytes + 1024) <= 228 * 1024 ? 184 : 92) / 100; }
 size_t tall_bytes(int tile_rows, int I, int cl) {  // two stages of 128 weight rows and the form's token rows, then the slice of H
     const int form_rows = tile_rows > 16 ? 32 : 16;
     return ((size_t)2 * (128 + form_rows) * kLd + (size_t)tile_rows * (features_per_cta(I, cl) + 4)) * sizeof(float);
@@ -851,15 +854,28 @@ static int64_t short_tiles(int64_t rows, int G) { return std::min<int64_t>(rows,
 
 // Rows per tile: a tile computes all of its rows, so short groups want short tiles (and more of them to fill the SMs); a
 // tile's weights are read once per tile, so long groups want long ones. The short form is the faster one for as long as its
-// tiles are a few waves of clusters at most: five where the alternative is 16-row tiles or the layer is small, else three. Whole call with tall / short tiles: tiny layer prefill (K' = 1) 75 tokens
-// 20.3 / 12.0 us, 342 23.5 / 19.4, 509 35.0 / 22.8, (K' = 2) 456 40.4 / 28.3, 770 (6 waves) 34.6 / 39.2; decode of 116 tokens, pool
-// of 3 35.2 / 21.9; 28 experts of 320 x 960, 41 tokens, pool of 8 85 / 53; 9 of 384 x 736, 79 tokens 85 / 60; 30 + 1 of 96 x 128,
-// 871 tokens (K' = 3, 13 waves) 39 / 56; 83 + 1 of 160 x 480, decode of 159 tokens, pool of 6 (4.3 waves) 66 / 76. Short tiles need the tokens and H in shared memory
-// whole (d + I up to ~7000); tall ones are halved while the slice of H does not fit (32 rows: I above ~11 000).
+// tiles are a few waves of clusters at most: five where the alternative is 16-row tiles or the layer is small, else three (counted
+// with the K chunks that sizes between multiples of 128 compute in vain). Whole call with tall / short tiles: tiny layer prefill (K' = 1)
+// 75 tokens 20.3 / 12.0 us, 342 23.5 / 19.4, 509 35.0 / 22.8, (K' = 2) 456 40.4 / 28.3, 770 (6 waves) 34.6 / 39.2; decode of 116
+// tokens, pool of 3 35.2 / 21.9; 28 experts of 320 x 960, 41 tokens, pool of 8 85 / 53; 9 of 384 x 736, 79 tokens 85 / 60; 8 of
+// 2048 x 1536, 293 tokens (1.3 waves) 491 / 458; 8 + 1 of 160 x 480, 204 tokens x 2 (4.3 waves) 47.7 / 53.3; 30 + 1 of 96 x 128, 871
+// tokens (K' = 3, 13 waves) 39 / 56.
+// Where an SM holds one such CTA only, a wave is half as many tiles and a second one as long as a wave of 16-row tiles and a half: one
+// wave, two where the alternative is 32 rows. 8 experts of 2048 x 2048, 16 tiles 623 / 299, 22 tiles 438 / 523, 28 434 / 535; of 1024 x
+// 4096, 22 tiles 441 / 560; 2 of 2048 x 2048, 93 rows each 629 / 500, 6 of 1024 x 4096, 63 each (53 tiles) 637 / 958.
+// Short tiles need the tokens and H in shared memory whole (d + I up to ~7000); tall ones are halved while the slice of H does not
+// fit (32 rows: I above ~11 000).
 int ffn_f32_tile_rows(int64_t rows, int G, int d, int I, int sms) {
-    const int waves = rows <= (int64_t)48 * G || (int64_t)d * I <= 48 * 1024 ? 5 : 3;
-    if ((rows <= (int64_t)kSR * G || short_tiles(rows, G) * kMaxCl * 100 <= (int64_t)184 * waves * sms) && short_bytes(d, I) <= kSmemLimit) return kSR;
-    int tile_rows = rows > (int64_t)48 * G ? 32 : 16;
+    const size_t bytes = short_bytes(d, I);
+    const bool rows16 = rows <= (int64_t)48 * G;  // else the alternative is 32
+    if (bytes <= kSmemLimit) {
+        if (rows <= (int64_t)kSR * G) return kSR;
+        const int64_t wave = short_wave(bytes, sms);
+        const int waves = wave < sms ? (rows16 ? 1 : 2) : (rows16 || (int64_t)d * I <= 48 * 1024 ? 5 : 3);
+        const int64_t computed = (int64_t)((d + 127) / 128 * 128) * ((I + 127) / 128 * 128);  // K chunks are computed whole
+        if (short_tiles(rows, G) * kMaxCl * computed <= wave * waves * d * I) return kSR;
+    }
+    int tile_rows = rows16 ? 16 : 32;
     while (tile_rows > 1 && tall_bytes(tile_rows, I, kMaxCl) > kSmemLimit) tile_rows /= 2;
     return tile_rows;
 }
@@ -896,11 +912,12 @@ cudaError_t launch_ffn_f32(const FfnF32Params& p, int64_t rows, int sms, cudaStr
     return cl == 8 ? launch_cl<8>(p, tiles, s) : (cl == 4 ? launch_cl<4>(p, tiles, s) : launch_cl<2>(p, tiles, s));
 }
 
-// One wave of clusters (each repeats the routing), and the routes of all tokens in shared memory
-bool ffn_f32_routes(int64_t T, int64_t rows, int G, int N, int slots, int d, int I, int tile_rows, int sms) {
-    constexpr size_t route_bytes = std::max(sizeof(PrefillRouteSmem), sizeof(DecodeRouteSmem)) + 256;
-    return tile_rows == kSR && short_bytes(d, I) + route_bytes <= kSmemLimit && T <= kRoutedTokens && T * slots <= kRoutedSlots &&
-           N <= kRoutedExperts && short_tiles(rows, G) * kMaxCl * 100 <= (int64_t)184 * sms;
+// One wave of clusters (each repeats the routing), and the routes of all tokens in shared memory. (8 + 1 experts of 2048 x 1536, 93
+// tokens, 32 tiles: the state leaves one CTA to an SM, two waves, 402 us; lists from kernels of their own and two CTAs 273)
+bool ffn_f32_routes(bool decode, int64_t T, int64_t rows, int G, int N, int slots, int d, int I, int tile_rows, int sms) {
+    const size_t bytes = short_bytes(d, I) + (decode ? sizeof(DecodeRouteSmem) : sizeof(PrefillRouteSmem)) + 256;
+    return tile_rows == kSR && bytes <= kSmemLimit && T <= kRoutedTokens && T * slots <= kRoutedSlots && N <= kRoutedExperts &&
+           short_tiles(rows, G) * kMaxCl <= short_wave(bytes, sms);
 }
 cudaError_t launch_ffn_f32_routed(const FfnF32Params& p, const FfnF32Route& rt, int64_t rows, cudaStream_t s) {
     const int64_t tiles = short_tiles(rows, p.G);

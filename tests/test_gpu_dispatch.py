@@ -334,6 +334,20 @@ def test_fp32_prefill_that_routes_in_its_ffn_kernel(T, N, ns, d, I, K, Kp):
     assert np.array_equal(got["y"], case.run_prefill(Kp, with_meta=False)["y"])
 
 
+@pytest.mark.parametrize("T,ns,d,I,launches", [(93, 1, 1600, 1024, 2), (93, 1, 2048, 1536, 4), (60, 0, 2048, 1536, 1), (20, 1, 2048, 1536, 2)])
+def test_fp32_routing_where_a_wave_holds_the_tiles(T, ns, d, I, launches):
+    """The FFN kernel routes only where all its clusters run at once: two CTAs to an SM up to 3130 to 3500 of d + I, one above, where
+    its routing state does not fit twice. One launch (rows stored into y) or two, else four."""
+    case = Case(si.LayerConfig("f32w", 8, ns, d, I, 2, "f32", T, (1,), 4, (2,)))
+    before = case.ex.exfold_launch_count()
+    got = case.run_prefill(1)
+    assert case.ex.exfold_launch_count() - before == launches
+    idx = np.arange(0, T, 7)
+    ref = case.oracle_prefill(1, tok_idx=idx)
+    check_prefill_meta(got, ref)
+    assert check_output(got["y"][idx], ref["y"], "f32")[1] < 2e-6
+
+
 @pytest.mark.parametrize("T,B,N,ns,d,I,K,Kp,M", [(456, 116, 8, 0, 128, 256, 2, 2, 3), (600, 230, 8, 0, 64, 96, 2, 2, 2), (700, 33, 7, 1, 68, 90, 5, 5, 1)])
 def test_fp32_short_tiles_of_long_groups(T, B, N, ns, d, I, K, Kp, M):
     """Groups of many short tiles (a few waves of clusters, four or two CTAs each) and, last, the tall tiles beyond."""
