@@ -74,22 +74,33 @@ __device__ __forceinline__ void add_pair(const CalibStatsParams& p, int s, int t
 // Pair sums of a token per warp, KE = Top-K <= 8: the token's KE output rows are read once, converted to double once, and all
 // KE (KE + 1) / 2 inner products accumulate in registers. Bound by reading the rows (4 KE d bytes per token). The rows come by
 // bulk copies into a ring of three stages of 256 columns per warp (lane a fetches row a; the next token's rows follow without a
-// gap): with eight warps and 192 KB per SM twice the bytes are in flight that registers could hold beside the sums, and the
+// gap): with 192 KB per SM twice the bytes are in flight that registers could hold beside the sums, and the
 // double-precision units work meanwhile. 8192 tokens x 8 rows x 2048 columns: a warp per ordered pair 619 us, rows through
-// registers with one chunk ahead 137 (134 alone
-// under a profiler), this 101 alone (98 without the atomics).
-constexpr int kRingWarps = 8;
+// registers with one chunk ahead 137 (134 alone under a profiler), this 101 alone (98 without the atomics).
+constexpr int kRingWarps = 8;  // of a CTA, at most
 constexpr int kRingStages = 3;
 constexpr int kRingCols = 256;
+// CTAs per SM, as many as their rings leave room for. Whole calibration with one / these: 64 experts of 1024 x 512, 2048 tokens, Top-3
+// 95.1 / 93.3 us, 8 of 4096 x 1024, 2048 tokens, Top-4 249 / 245.
+template <int KE>
+constexpr int kRingCtas = KE == 2 ? 4 : KE == 3 ? 3 : KE == 4 ? 2 : 1;
 
-__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(ptx::smem_u32(dst)), "l"(src),
-                 "r"(bytes), "r"(ptx::smem_u32(bar))
+// The rows are read once: they are the first to leave L2, before the weights (a layer of 50 MB calibrated again and again, Top-1, 2048
+// tokens: 83.4 -> 75.3 us)
+__device__ __forceinline__ uint64_t evict_first_policy() {
+    uint64_t policy;
+    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
+    return policy;
+}
+__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* bar, uint64_t policy) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;" ::"r"(
+                     ptx::smem_u32(dst)),
+                 "l"(src), "r"(bytes), "r"(ptx::smem_u32(bar)), "l"(policy)
                  : "memory");
 }
 
 template <int KE>
-__global__ void __launch_bounds__(32 * kRingWarps) calib_stats_kernel(CalibStatsParams p) {
+__global__ void __launch_bounds__(32 * kRingWarps, kRingCtas<KE>) calib_stats_kernel(CalibStatsParams p) {
     constexpr int NV = KE * (KE + 1) / 2;
     extern __shared__ __align__(128) float ring_all[];
     __shared__ double s_gram[kRingWarps][NV];
@@ -106,7 +117,9 @@ __global__ void __launch_bounds__(32 * kRingWarps) calib_stats_kernel(CalibStats
     grid_dep_launch();
     grid_dep_wait();
     const int d = p.d, n_chunks = (d + kRingCols - 1) / kRingCols;
-    const int64_t step = (int64_t)gridDim.x * kRingWarps, i0 = (int64_t)blockIdx.x * kRingWarps + warp;
+    const int n_warps = (int)blockDim.x >> 5;
+    const uint64_t policy = evict_first_policy();
+    const int64_t step = (int64_t)gridDim.x * n_warps, i0 = (int64_t)blockIdx.x * n_warps + warp;
     // the loads run ahead of the sums: chunk lc of token li into stage ls
     int64_t li = i0;
     int lc = 0, ls = 0;
@@ -116,7 +129,7 @@ __global__ void __launch_bounds__(32 * kRingWarps) calib_stats_kernel(CalibStats
         const int c0 = lc * kRingCols, cols = min(kRingCols, d - c0);
         if (lane == 0) ptx::mbar_expect_tx(&bars[warp][ls], (uint32_t)(KE * cols * 4));
         __syncwarp();
-        if (lane < KE) bulk_load(ring + (ls * KE + lane) * kRingCols, row + c0, (uint32_t)cols * 4, &bars[warp][ls]);
+        if (lane < KE) bulk_load(ring + (ls * KE + lane) * kRingCols, row + c0, (uint32_t)cols * 4, &bars[warp][ls], policy);
         if (++ls == kRingStages) ls = 0;
         if (++lc == n_chunks) {
             lc = 0;
@@ -182,6 +195,72 @@ __global__ void __launch_bounds__(32 * kRingWarps) calib_stats_kernel(CalibStats
             }
         }
         __syncwarp();
+    }
+}
+
+// The same for one row per token, or two of at most 2048 columns: a warp per token, 16 bytes per lane and row with the next chunk in
+// flight, into registers. The ring's barriers and its walk over the tokens cost a token more than so few copies bring. Whole
+// calibration with the ring / this: 32 experts of 2048 x 128, Top-1, 2048 and 8192 tokens 75.3 / 67.9, 115.0 / 102.4 us, Top-2, 8192
+// 154 / 140; 64 of 1024 x 512, Top-2, 2048 tokens 92.7 / 88.4; the other way 8 of 4096 x 1024, Top-2, 64, 512 and 2048 tokens 91.6 /
+// 97.6, 102.6 / 107.0, 150.4 / 158.0.
+template <int KE>
+__global__ void __launch_bounds__(kStatsThreads) calib_stats_short_kernel(CalibStatsParams p) {
+    constexpr int NV = KE * (KE + 1) / 2;
+    __shared__ double s_gram[kStatsThreads / 32][NV];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    grid_dep_launch();
+    grid_dep_wait();
+    const int64_t i = (int64_t)blockIdx.x * (kStatsThreads / 32) + warp;
+    if (i >= p.m) return;
+    const int d = p.d;
+    const float* row[KE];
+#pragma unroll
+    for (int a = 0; a < KE; ++a) row[a] = p.out + stats_row(p, i, a) * d;
+    double acc[NV];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) acc[v] = 0.0;
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    float4 nxt[KE];
+    int c = lane * 4;
+#pragma unroll
+    for (int a = 0; a < KE; ++a) nxt[a] = c < d ? __ldcs(reinterpret_cast<const float4*>(row[a] + c)) : zero;
+    for (; c < d; c += 128) {
+        float4 cur[KE];
+#pragma unroll
+        for (int a = 0; a < KE; ++a) {
+            cur[a] = nxt[a];
+            nxt[a] = c + 128 < d ? __ldcs(reinterpret_cast<const float4*>(row[a] + c + 128)) : zero;
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            double o[KE];
+#pragma unroll
+            for (int a = 0; a < KE; ++a)
+                o[a] = (double)(q == 0 ? cur[a].x : q == 1 ? cur[a].y : q == 2 ? cur[a].z : cur[a].w);
+            int v = 0;
+#pragma unroll
+            for (int a = 0; a < KE; ++a)
+#pragma unroll
+                for (int b = a; b < KE; ++b, ++v) acc[v] = fma(o[a], o[b], acc[v]);
+        }
+    }
+    double* g = s_gram[warp];
+    warp_sums<NV>(acc, g, lane);
+    __syncwarp();
+    auto at = [](int a, int b) {  // place of (a, b) in the upper triangle
+        const int lo = a < b ? a : b, hi = a < b ? b : a;
+        return lo * KE - lo * (lo - 1) / 2 + (hi - lo);
+    };
+    const int32_t* ids = p.ids + i * KE;
+    for (int q = lane; q < KE * KE; q += 32) {
+        const int a = q / KE, b = q - a * KE;
+        const double uu = g[at(a, a)], wi = sqrt(uu);
+        if (a == b) {
+            atomicAdd(&p.H[ids[a]], wi);
+            atomicAdd(&p.hc[ids[a]], 1);
+        } else {
+            add_pair(p, ids[a], ids[b], wi, uu, g[at(a, b)], g[at(b, b)]);
+        }
     }
 }
 
@@ -452,23 +531,28 @@ cudaError_t launch_calib_stats_common(const CalibStatsParams& p, double* nrm, in
 
 template <int KE>
 static cudaError_t launch_stats(const CalibStatsParams& p, int sms, cudaStream_t s) {
-    const size_t smem = (size_t)kRingWarps * kRingStages * KE * kRingCols * sizeof(float);
+    // few tokens: fewer warps to a CTA, so that every SM has some
+    const int warps = (int)std::min<int64_t>((p.m + sms - 1) / sms, kRingWarps);
+    const size_t smem = (size_t)warps * kRingStages * KE * kRingCols * sizeof(float);
     cudaError_t err = ensure_smem(calib_stats_kernel<KE>, smem);
     if (err != cudaSuccess) return err;
-    const int64_t blocks = std::min<int64_t>((p.m + kRingWarps - 1) / kRingWarps, sms);
-    return launch_pdl(calib_stats_kernel<KE>, (unsigned)blocks, 32 * kRingWarps, smem, s, p);
+    const int64_t blocks = std::min<int64_t>((p.m + warps - 1) / warps, (int64_t)sms * kRingCtas<KE>);
+    return launch_pdl(calib_stats_kernel<KE>, (unsigned)blocks, 32 * warps, smem, s, p);
 }
 cudaError_t launch_calib_stats(const CalibStatsParams& p, int sms, cudaStream_t s) {
     if (p.m == 0) return cudaSuccess;
     constexpr int kWarps = kStatsThreads / 32;
+    const unsigned short_grid = (unsigned)((p.m + kWarps - 1) / kWarps);
     if (p.Ke > kStatsRows) {
         const int nb = (p.Ke + 3) / 4;
         const int64_t warps = p.m * (nb * (nb + 1) / 2);
         return launch_pdl(calib_stats_tiled_kernel, (unsigned)((warps + kWarps - 1) / kWarps), kStatsThreads, 0, s, p, nb);
     }
     switch (p.Ke) {
-        case 1: return launch_stats<1>(p, sms, s);
-        case 2: return launch_stats<2>(p, sms, s);
+        case 1: return launch_pdl(calib_stats_short_kernel<1>, short_grid, kStatsThreads, 0, s, p);
+        case 2:
+            if (p.d <= 2048) return launch_pdl(calib_stats_short_kernel<2>, short_grid, kStatsThreads, 0, s, p);
+            return launch_stats<2>(p, sms, s);
         case 3: return launch_stats<3>(p, sms, s);
         case 4: return launch_stats<4>(p, sms, s);
         case 5: return launch_stats<5>(p, sms, s);

@@ -10,16 +10,17 @@ from harness import A, Case, check_decode_meta, check_output, check_prefill_meta
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("K", [1, 2, 3, 4, 5, 6, 7, 8, 9, 13, 16])
-def test_calibration_sums_by_top_k(K):
+@pytest.mark.parametrize("K,m,d", [(K, 61, 132) for K in (1, 2, 3, 4, 5, 6, 7, 8, 9, 13, 16)] + [
+    (1, 1, 260), (2, 3, 2052), (2, 700, 2052), (2, 700, 2048), (3, 1, 516), (3, 3700, 260), (4, 149, 516), (4, 2400, 68), (8, 1200, 260), (8, 2, 1028)])
+def test_calibration_sums_by_top_k(K, m, d):
     """Pair sums: a kernel per Top-K up to 8, tiles of four slots above (9: a ragged last tile). d = 132 leaves a tail
     after whole 128-column steps; m is not a multiple of the tokens per block; odd K: x_cal 4 bytes off a 16-byte
     boundary (fp32 calibration takes any). fp32 outputs, double sums: the oracle's
-    tables to fp32 rounding of the outputs (2e-5, as in the other fp32 calibration tests)."""
+    tables to fp32 rounding of the outputs (2e-5, as in the other fp32 calibration tests). Then one token, one to a warp and one more,
+    several per warp in one, two and three CTAs to an SM, rows of one column chunk, a ragged one and several, the line of K = 2."""
     N = 16
-    cfg = si.LayerConfig("calk", N, 0, 132, 64, K, "f32", 16, (1,), 4, (2,))
+    cfg = si.LayerConfig("calk", N, 0, d, 64, K, "f32", 16, (1,), 4, (2,))
     case = Case(cfg, std=0.05, correlated=0.8)
-    m = 61
     xc, lc = si.hidden_states(cfg, m, "x_cal"), si.router_logits(cfg, m, "logits_cal")
     ref = oracle.calibrate(A(xc), lc.numpy(), A(case.wg), A(case.wu), A(case.wd), N, K, mode=0)
     dev, ex = case.dev, case.ex
