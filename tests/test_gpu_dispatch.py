@@ -327,7 +327,7 @@ def test_host_prefill_covers_every_token(T):
     (3, 100, 1, 96, 64, 32, 16), (20, 129, 0, 64, 64, 3, 1), (2, 8, 0, 3584, 3584, 2, 2)])
 def test_fp32_prefill_that_routes_in_its_ffn_kernel(T, N, ns, d, I, K, Kp):
     """Few tokens of an fp32 layer: routing inside the FFN kernel (up to 128 tokens, 128 experts, one wave of clusters) and the
-    kernels of its own beyond; metadata bit-exact, safeguards included, outputs to fp32 rounding."""
+    kernels of its own beyond; metadata bit-exact, outputs to fp32 rounding."""
     case = Case(si.LayerConfig("f32r", N, ns, d, I, K, "f32", T, (Kp,), 4, (2,)))
     got, ref = case.run_prefill(Kp), case.oracle_prefill(Kp)
     check_prefill_meta(got, ref)
@@ -347,6 +347,34 @@ def test_fp32_routing_where_a_wave_holds_the_tiles(T, ns, d, I, launches):
     ref = case.oracle_prefill(1, tok_idx=idx)
     check_prefill_meta(got, ref)
     assert check_output(got["y"][idx], ref["y"], "f32")[1] < 2e-6
+
+
+@pytest.mark.parametrize("thr,rescale,conf", [(0.6, False, False), (0.6, True, False), (float("inf"), False, True), (0.5, True, True), (-1.0, True, False)])
+@pytest.mark.parametrize("dtype,T,N,K,Kp", [("f32", 64, 8, 4, 2), ("f32", 128, 40, 4, 3), ("f32", 150, 8, 4, 2), ("bf16", 1, 16, 6, 3), ("bf16", 8, 40, 6, 2)])
+def test_safeguards_where_the_ffn_kernels_route(dtype, T, N, K, Kp, thr, rescale, conf):
+    """Loss threshold, rescale and confidence split of the calls whose FFN kernel routes its tokens itself (fp32 up to 128 tokens, and
+    150 beside it; bf16 up to 8 without metadata): metadata as the oracle's, the same bits without it."""
+    d = 128
+    case = Case(si.LayerConfig("safe", N, 1, d, 192, K, dtype, T, (Kp,), 4, (2,)))
+    ex, dev = case.ex, case.dev
+    S, L, h, lnh = case.np_tables()
+    ref = oracle.prefill_fold_safe(case.lg.numpy(), K, Kp, S, L, lnh, loss_thr=thr, rescale=rescale, confidence=conf)
+    yref = oracle.moe_apply(A(case.x), A(case.wg), A(case.wu), A(case.wd), ref["ids"], ref["w"], N, 1)
+    i32 = dict(dtype=torch.int32, device=dev)
+    meta = dict(ids=torch.full((T, Kp), -7, **i32), w=torch.full((T, Kp), float("nan"), device=dev),
+                omit_src=torch.full((T, K - Kp), -7, **i32), omit_tgt=torch.full((T, K - Kp), -7, **i32))
+    ys = []
+    for m in (meta, None):
+        ws, y = case.workspace(T, Kp), torch.full((T, d), float("nan"), dtype=case.d_wg.dtype, device=dev)
+        ex.exfold_moe_prefill_ex(case.layer, case.d_x, case.d_lg, case.d_wg, case.d_wu, case.d_wd, case.tables, Kp, y, ws,
+                                 loss_threshold=thr, rescale=rescale, confidence_split=conf, meta=m)
+        assert ex.exfold_device_status(ws) == 0
+        ys.append(y.float().cpu().numpy())
+    for k in ("ids", "omit_src", "omit_tgt"):
+        assert np.array_equal(meta[k].cpu().numpy(), ref[k]), k
+    np.testing.assert_allclose(meta["w"].cpu().numpy(), ref["w"], rtol=2e-5, atol=2e-5)  # as in test_prefill_safeguards
+    check_output(ys[0], yref, dtype)
+    assert np.array_equal(ys[0], ys[1])
 
 
 @pytest.mark.parametrize("T,B,N,ns,d,I,K,Kp,M", [(456, 116, 8, 0, 128, 256, 2, 2, 3), (600, 230, 8, 0, 64, 96, 2, 2, 2), (700, 33, 7, 1, 68, 90, 5, 5, 1)])
