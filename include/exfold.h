@@ -170,9 +170,10 @@ int exfold_calibrate_layers(const exfold_layer *layer, const exfold_calib_job *j
  * routes only). x [T][d], logits [T][N] -> y [T][d]. k_pre = K' in [1, K]; k_pre = K is the
  * unfolded layer. Each token executes exactly K' routed experts (+ the shared expert).
  * Ranking uses key = logit + lnh[e] (one fp32 add; same order as a_e h_e).
- * bf16 layers: the two grouped GEMMs of most calls run the experts' whole 256-row tiles and their ragged remainders in one
- * pass over pairs of CTAs; with eight row tiles of 128 sorted rows or more per expert, the row tiles two at a time on pairs of CTAs
- * and, beside them, the experts' odd last tiles on the one-CTA-per-tile kernel; calls of few or short work items use the latter
+ * bf16 layers: the two grouped GEMMs run the experts' whole 256-row tiles and their ragged remainders (of up to 224 rows) in one pass
+ * over pairs of CTAs where there are enough work items, fewer than eight row tiles of 128 sorted rows per expert and items long enough
+ * for the rows per expert. Other calls of a row tile or more per expert, and enough work, run the row tiles two at a time on pairs of CTAs
+ * and, beside them, the experts' odd last tiles on the one-CTA-per-tile kernel; what is left uses that kernel
  * alone. The results are bit-identical either way. The odd-tile kernels run on a
  * second stream (highest priority) that the library creates once per host thread; with a shared expert, the gate/up
  * projection of its whole row-tile pairs also runs there, beside the kernel that gathers the routed rows (its inputs

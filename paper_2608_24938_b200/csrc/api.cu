@@ -388,16 +388,29 @@ int enqueue_mixed_gemms(const GroupedGemmParams& g, const GroupedGemmParams& g2,
 
 // Whether they do. The mixed kernel computes and loads what a group's rows need, where row tiles of 128 rows waste half a tile
 // per group, and reads a weight tile once; but it has half as many workers (CTA pairs), and an item costs a pair more to hand over.
-// So it wants a few rounds of items, and long ones (48 k-blocks of GEMM-1 and more) or groups of a few rows and more.
-// With eight row tiles per group and more, the waste is small and the passes side by side on their own SMs are as fast.
-// Measured, whole prefill call on row tiles / mixed: GLM shape (K' = 4) 48 tokens 502 / 478 us, 768 768 / 727, 3072 972 / 863,
-// 12288 2391 / 2222; Mixtral shape (K' = 1) 192 tokens 466 / 443, 1536 750 / 567, 3072 1301 / 1231; Qwen3 shape, even / skewed
-// scores, 777 tokens (K' = 4) 228 / 221, 132 / 133, (K' = 6) 237 / 227, 182 / 178, 1536 tokens 253 / 249, 235 / 218; 64 experts of
-// 2048 x 1408 (K' = 3) 384 tokens 197 / 200, 1536 225 / 218; 160 of 1536 x 1024 200 tokens 229 / 231, 1536 285 / 273. Few items:
-// 64 experts of 1024 x 512 (K' = 4) 768 tokens 64 / 71; 11 of 2688 x 512 (K' = 3) 58 / 65.
+// So it wants a few rounds of items, and the more rows per group the shorter the items are (k-blocks of an item, the mean over both
+// GEMMs' work: a hand-over against that). Whole prefill call on row tiles / mixed, even and skewed scores, three layers in turn:
+//   12 k-blocks and more: 24 rows per group, any number from 48 k-blocks of GEMM-1 on. GLM shape (K' = 4) 59 tokens 552 / 518 us, 192 /
+//   187, 400 746 / 705, 349 / 336, 1200 802 / 757, 547 / 503; Qwen3 shape (K' = 6) 777 tokens 234 / 228, 185 / 180, 2200 285 / 276, 284 /
+//   268; Mixtral shape (K' = 2) 200 tokens 484 / 464, 489 / 476; 160 experts of 1024 x 1024 (K' = 4) 1300 tokens 216 / 205, 127 / 126,
+//   4000 265 / 248, 225 / 212; 128 of 768 x 1536 (K' = 4) 1500 tokens 192 / 190, 140 / 139; the line itself: 64 + 1 of 2048 x 1408 (K' = 2)
+//   800 tokens 218 / 216, 151 / 154, 96 + 1 of 1536 x 768 (K' = 3) 1500 tokens 165 / 169, 135 / 134.
+//   9: 144 rows. 160 of 1024 x 320 (K' = 4) 1800 tokens (45 rows) 102 / 105, 78 / 87, 8000 (200) 183 / 176, 173 / 165.
+//   8: 320 rows. 139 + 1 of 576 x 448 (K' = 3) 2102 tokens (60) 85 / 97, 71 / 79, 5000 (143) 115 / 125, 107 / 113, (K' = 2) 14000 (300)
+//   181 / 181, 169 / 166; 256 of 512 x 512 (K' = 3) 12600 tokens (148) 192 / 198, 162 / 169.
+//   Fewer: never. 200 of 320 x 1280 (K' = 4) 10000 tokens (200) 244 / 257, 234 / 231; 114 + 1 of 192 x 448 (K' = 5) 13328 tokens (695) skewed
+//   161 / 174; 64 of 128 x 1024 (K' = 3) 9000 tokens (422) 94 / 104, 94 / 105.
+// Where use_pairs would run pairs of row tiles beside odd ones, those / mixed: GLM shape 16384 tokens 2576 / 2423, Mixtral shape 2000
+// tokens 748 / 689, 4096 1271 / 1187 (8 experts of it, skewed, 3376 tokens 1123 / 1087), Qwen3 shape 8192 tokens 400 / 381; under the power
+// cap alike (2939 / 2757, 1455 / 1358). With eight row tiles per group and more there is little left to waste: 128 of 2048 x 768 (K' = 8)
+// 16384 tokens 1396 / 1375, 1408 / 1402, 64 of 2048 x 1408 (K' = 6) 12000 tokens 1245 / 1258, 1255 / 1250, GLM shape (K' = 8) 16000 tokens 4904 /
+// 4841, 4782 / 4873. Few items: 64 of 1024 x 512 (K' = 4) 768 tokens 64 / 71; 11 of 2688 x 512 (K' = 3) 58 / 65.
 bool use_mixed(int64_t rows, int G, int d, int I) {
     const int64_t items = (int64_t)G * ((I + 127) / 128) * std::max<int64_t>(1, rows / (256 * (int64_t)G));
-    return rows / kTileM < (int64_t)8 * G && items >= (int64_t)3 * sm_count() && (d >= 48 * kGemmBK || rows >= (int64_t)24 * G);
+    if (rows / kTileM >= (int64_t)8 * G || items < (int64_t)3 * sm_count()) return false;
+    const int64_t kblocks = (int64_t)3 * d * I / ((2 * (int64_t)I + d) * kGemmBK);  // GEMM-1 is two thirds of the work
+    if (kblocks >= 12) return d >= 48 * kGemmBK || rows >= (int64_t)24 * G;
+    return kblocks >= 8 && rows >= (int64_t)(kblocks >= 9 ? 144 : 320) * G;
 }
 
 struct PdlScope {  // programmatic dependent launch for the launches of this scope
@@ -785,10 +798,10 @@ static int decode_impl(const exfold_layer* layer, const void* x, const float* lo
             // and the unused gathered-rows region before it) and are summed, in order, by the kernel after.
             const int64_t row_tiles = (int64_t)max_groups * ((B + kTileM - 1) / kTileM), base_items = row_tiles * ((d + 255) / 256);
             const int ksplit = (2 * base_items < sms && I / 64 >= 8) ? kMaxDecodeKsplit : 1;
-            // Still few: narrower column tiles, as long as each has an SM to itself. (A k-block's MMAs take the same time for 64
-            // columns as for 256, so more rounds of narrower tiles lose.) Whole call, 256 columns / these: Qwen3 shape 128
-            // tokens, pool 2 29.2 / 27.2 us; GLM shape 100 tokens, pool 1 47.1 / 45.1; Mixtral shape 200 tokens, pool 1
-            // 152.8 / 144.3; 64 columns in three rounds: GLM shape 16 tokens, pool 4 50.4 / 60.0.
+            // Still few: narrower column tiles, as long as each has an SM to itself. (Fewer columns take the tensor pipe less time,
+            // but a k-block's copies and hand-over stay what they were: more rounds of narrower tiles lose.) Whole call, 256
+            // columns / these: Qwen3 shape 128 tokens, pool 2 29.2 / 27.2 us; GLM shape 100 tokens, pool 1 47.1 / 45.1; Mixtral
+            // shape 200 tokens, pool 1 152.8 / 144.3; 64 columns in three rounds: GLM shape 16 tokens, pool 4 50.4 / 60.0.
             int n_cols = 256;
             while (n_cols > 64 && base_items * (512 / n_cols) * ksplit <= sms) n_cols >>= 1;
             CUtensorMap tm_wd;

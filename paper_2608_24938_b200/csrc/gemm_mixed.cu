@@ -1,6 +1,7 @@
 // Expert GEMMs of prefill and calibration on CTA pairs, whole 256-row tiles and ragged remainders in one pass.
 //
-// A group of r rows is r / 256 whole items and one ragged item of the r % 256 rows left. Both kinds stage at most 32 KB per
+// A group of r rows is r / 256 whole items and one ragged item of the r % 256 rows left (a whole one of masked rows above
+// kRaggedMax = 224 of them, which take as long). Both kinds stage at most 32 KB per
 // CTA and k-block (16 KB of weight rows, up to 16 KB of token rows) and differ in which operand is which:
 //
 //   whole    A = 256 token rows (128 per CTA), B = 256 weight rows: accumulator lane = token row, column = feature.
@@ -17,9 +18,9 @@
 // index from a counter in memory, decodes it and puts it into a ring of slots in both CTAs' shared memory.
 //
 // What bounds it: an SM takes in 64 bytes per cycle, which a whole item needs (32 KB per 512 cycles), so whole items run at
-// 505-540 cycles per k-block; ragged items of 50 tokens at 510-530 where their weights come from memory. Whole prefill call
-// before (whole pairs of 128-row tiles and odd tiles in two passes side by side) / now: GLM shape 16384 tokens 3363 / 3047 us,
-// Mixtral shape 4096 tokens 1624 / 1497, Qwen3 shape 8192 tokens 511 / 474, its calibration 990 / 938.
+// 507-546 cycles per k-block; ragged items of 50 tokens at 530-570 where their weights come from memory. Whole prefill call on
+// whole pairs of 128-row tiles and odd tiles in two passes side by side / this: GLM shape 16384 tokens 2576 / 2423 us, Mixtral shape
+// 4096 tokens 1271 / 1187, Qwen3 shape 8192 tokens 400 / 381.
 //
 // Roles per CTA: warps 0 and 7 TMA producers (k-blocks dealt in turn; four of them are no faster: a k-block then takes each
 // 1500 instead of 750 cycles), warp 1 MMA issuer (leader), warps 2-5 epilogue, warp 6 item scheduler (leader) or, in the

@@ -1,6 +1,6 @@
 """Whole row tiles and ragged remainders in one pass (gemm_mixed.cu), at the group sizes where it can go wrong: against the
 one-CTA kernel bit for bit (the same products accumulated in the same order) and against the CPU oracle. MIXED forces the pass, so
-that the sizes here do not hang on the library's choice."""
+that the sizes here do not hang on the library's choice, which has a test of its own."""
 import numpy as np
 import pytest
 import torch
@@ -16,21 +16,45 @@ EDGES = [0, 1, 2, 31, 32, 33, 63, 64, 65, 96, 97, 127, 128, 129, 160, 161, 192, 
          480, 481, 511, 512, 513, 767, 768, 769]
 
 
-def mixed_ran(case, Kp, gemm_path=0):
+def mixed_ran(N, ns, d, I, K, Kp, T, gemm_path=0):
     """Whether a call ran the pass: it draws its items from the two work counters in the status record (words 4 and 5), which the
-    other kernels leave as they were."""
-    ws = case.workspace(case.T, Kp)  # all bytes 0xFF
-    y = torch.empty((case.T, case.cfg.hidden), dtype=case.d_wg.dtype, device=case.dev)
-    case.ex.exfold_moe_prefill_ex(case.layer, case.d_x, case.d_lg, case.d_wg, case.d_wu, case.d_wd, case.tables, Kp, y, ws, gemm_path=gemm_path)
+    other kernels leave as they were. (Zero weights: only the routing has to be real.)"""
+    from paper_2608_24938_b200 import binding as ex
+    dev = torch.device("cuda:0")
+    bf16 = dict(dtype=torch.bfloat16, device=dev)
+    layer = ex.make_layer(N, ns, d, I, K, "bf16")
+    tabs = [torch.zeros(s, device=dev) for s in ((N, N), (N, N), (N,), (N,))]
+    wg, wu, wd = torch.zeros((N + ns, I, d), **bf16), torch.zeros((N + ns, I, d), **bf16), torch.zeros((N + ns, d, I), **bf16)
+    ws = ex.alloc_workspace(layer, T, Kp).fill_(0xFF)
+    ex.exfold_moe_prefill_ex(layer, torch.zeros((T, d), **bf16), torch.randn((T, N), device=dev), wg, wu, wd, ex.make_tables(*tabs), Kp,
+                             torch.empty((T, d), **bf16), ws, gemm_path=gemm_path)
     torch.cuda.synchronize()
     return ws[16:24].view(torch.int32).tolist() != [-1, -1]
 
 
-@pytest.mark.parametrize("N,ns,d,I,K,Kp,T", [(64, 0, 192, 64, 2, 1, 200), (8, 1, 1024, 7168, 3, 2, 2100)])
-def test_gemm_path_forces_the_pass(N, ns, d, I, K, Kp, T):
+@pytest.mark.parametrize("shape", [(64, 0, 192, 64, 2, 1, 200), (8, 1, 1024, 7168, 3, 2, 2100)])
+def test_gemm_path_forces_the_pass(shape):
     """The counters move with MIXED, whatever the size, and with no other forced path."""
-    case = Case(si.LayerConfig("forced", N, ns, d, I, K, "bf16", T, (Kp,), 4, (2,)))
-    assert mixed_ran(case, Kp, MIXED) and not mixed_ran(case, Kp, ONE_CTA) and not mixed_ran(case, Kp, PAIRS)
+    assert mixed_ran(*shape, MIXED) and not mixed_ran(*shape, ONE_CTA) and not mixed_ran(*shape, PAIRS)
+
+
+@pytest.mark.parametrize("shape,want", [
+    # N, shared, d, I, K, K', T
+    ((64, 0, 2048, 896, 2, 1, 1536), True),   # 24 rows per expert
+    ((64, 0, 2048, 896, 2, 1, 1535), False),
+    ((64, 0, 2048, 768, 2, 1, 1536), False),  # fewer than three items per SM
+    ((64, 0, 3072, 896, 2, 1, 20), True),     # 48 k-blocks: any number of rows
+    ((150, 0, 1024, 320, 2, 1, 21600), True), # 9 k-blocks: 144 rows
+    ((150, 0, 1024, 320, 2, 1, 21599), False),
+    ((112, 0, 512, 512, 2, 1, 35840), True),  # 8: 320 rows
+    ((112, 0, 512, 512, 2, 1, 35839), False),
+    ((64, 0, 192, 896, 2, 1, 32000), False),  # fewer: 500 rows are not enough
+    ((8, 1, 1024, 7168, 3, 2, 3071), True),   # fewer than eight row tiles per expert
+    ((8, 1, 1024, 7168, 3, 2, 3072), False),
+])
+def test_the_librarys_choice(shape, want):
+    """use_mixed on both sides of each of its lines (148 SMs)."""
+    assert mixed_ran(*shape) == want
 
 
 @pytest.mark.parametrize("n_groups", [5, 64])
@@ -75,11 +99,11 @@ def test_rows_of_several_routes(Kp, ns, T, d):
     assert np.array_equal(got["y"], case.run_prefill(Kp, with_meta=False, gemm_path=ONE_CTA)["y"])
 
 
-@pytest.mark.parametrize("mode,m", [(0, 1600), (1, 775), (1, 993)])
+@pytest.mark.parametrize("mode,m", [(0, 1660), (1, 820), (1, 993)])
 def test_calibration(mode, m):
-    """fp32 rows of whole and ragged items (775 = 3 x 256 + 7; 993: a rest of 225 rows, a whole item) in a calibration that takes the
+    """fp32 rows of whole and ragged items (820 = 3 x 256 + 52; 993: a rest of 225 rows, a whole item) in a calibration that takes the
     pass: the oracle's tables, tolerances as in test_calibrate_bf16_on_tensor_cores."""
-    cfg = si.LayerConfig("calib", 8, 0, 256, 2432, 4, "bf16", 64, (2,), 4, (2,))
+    cfg = si.LayerConfig("calib", 8, 0, 384, 2432, 4, "bf16", 64, (2,), 4, (2,))
     case = Case(cfg, correlated=0.8)
     ex, dev, N = case.ex, case.dev, cfg.n_experts
     xc, lc = si.hidden_states(cfg, m, "x_cal"), si.router_logits(cfg, m, "logits_cal")
