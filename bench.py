@@ -45,13 +45,13 @@ NOMINAL = {"hbm_gbs": 8000.0, "bf16_tflops": 2250.0}  # the figures the task sta
 # DRAM bytes measured by ncu (dram__bytes_read.sum + dram__bytes_write.sum) divided by the algorithmic
 # bytes of the same launch, from the reduced-case ncu captures whose summaries are under profiles/
 # (same rows per expert as the full-size workload, fewer experts or a shorter intermediate size so that
-# the capture stays small). Traffic grows with the weights, so the full-size figure is this ratio times
+# the capture stays small; the kernels that the full size runs). Traffic grows with the weights, so the full-size figure is this ratio times
 # the full-size algorithmic bytes. A shape without a capture reports traffic = null.
 NCU_TRAFFIC_RATIO = {
     # profiles/kernels_mixtral_reduced.md, kernels_qwen3_full.md, kernels_glm45air_reduced.md
-    "mixtral": {"gemm1": 528.6 / 390.1, "decode_ffn": 171.8 / 168.3},
-    "qwen3": {"gemm1": 902.5 / 820.0, "decode_ffn": 104.0 / 101.7},
-    "glm45air": {"gemm1": 1346.9 / 986.7, "decode_ffn": 770.5 / 765.6},
+    "mixtral": {"gemm1": 542.2 / 532.7, "decode_ffn": 235.4 / 235.4},
+    "qwen3": {"gemm1": 811.4 / 820.0, "decode_ffn": 101.2 / 101.7},
+    "glm45air": {"gemm1": 997.9 / 986.7, "decode_ffn": 767.8 / 765.6},
 }
 
 
