@@ -1,5 +1,6 @@
 // Routing of one prefill token by one warp: Top-K gate (Eq. 2), retained set (Eq. 10), minimum-loss targets (Eq. 12) and the
-// folded weights (Eq. 13). Used by the route kernel and by the fp32 kernel that routes in its prologue.
+// folded weights (Eq. 13). Used by the route kernel and by the two kernels that route in their prologue
+// (fp32 FFN, few-token gate/up).
 #pragma once
 #include "common.cuh"
 
